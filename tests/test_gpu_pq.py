@@ -51,6 +51,54 @@ def test_encode_ragged_and_small_codebooks(ifvs, orc):
         np.testing.assert_array_equal(dmin, rd)
 
 
+def _hard_rows(rng, n, M, ds):
+    """Rows of every scale the tensor-core ranking has a rule for: ordinary,
+    far from the origin (many candidates), tiny, huge, zero, not finite."""
+    X = rng.standard_normal((n, M * ds)).astype(np.float32)
+    kind = rng.integers(0, 40, n)
+    X[kind == 0] += 1000.0
+    X[kind == 1] *= 1e-15
+    X[kind == 2] *= 1e18
+    X[kind == 3] = 0.0
+    X[kind == 4, ::7] = np.nan
+    X[kind == 5, ::5] = np.inf
+    X[kind == 6] += 30.0
+    return X
+
+
+@pytest.mark.parametrize("ds", [4, 8, 16])
+@pytest.mark.parametrize("n,M,K", [(1, 1, 1), (127, 2, 5), (128, 3, 32), (129, 5, 33), (2049, 16, 256), (300, 33, 100),
+                                   (40_000, 3, 255)])
+def test_encode_edges_of_the_tensor_core_path(ifvs, orc, ds, n, M, K):
+    rng = np.random.default_rng(n * ds + K)
+    X = _hard_rows(rng, n, M, ds)
+    C = rng.standard_normal((M, K, ds)).astype(np.float32)
+    C[:, -1] = C[:, 0]                           # duplicate codeword: ties go to 0
+    if M > 2:
+        C[1] += 500.0                            # a subspace far from the origin
+        C[2, K // 2] = np.inf                    # one whose error bound does not hold
+        X[:, ds:2 * ds] += 500.0
+    codes, dmin = ifvs.ifvs_pq_encode(X, C, want_dmin=True)
+    rc, rd = orc.pq_encode_f32(X, C)
+    np.testing.assert_array_equal(codes, rc)
+    np.testing.assert_array_equal(dmin, rd)
+    np.testing.assert_array_equal(ifvs.ifvs_pq_encode(X, C), rc)   # without distances: fewer exact evaluations
+
+
+def test_encode_unaligned_device_pointers(ifvs, orc):
+    import torch
+    rng = np.random.default_rng(9)
+    n, M, K, ds = 700, 4, 64, 8
+    X = rng.standard_normal((n, M * ds)).astype(np.float32)
+    C = rng.standard_normal((M, K, ds)).astype(np.float32)
+    x = torch.zeros(X.size + 1, device="cuda")[1:].view(n, M * ds)
+    x.copy_(torch.from_numpy(X))
+    c = torch.from_numpy(C).cuda()
+    codes = torch.empty((n * M + 3,), dtype=torch.uint8, device="cuda")[3:].view(n, M)
+    ifvs.ifvs_pq_encode(x, c, codes=codes, flags=ifvs.IFVS_F_DEVICE_IO)
+    np.testing.assert_array_equal(codes.cpu().numpy(), orc.pq_encode_f32(X, C)[0])
+
+
 def _ulp_close(a, b):
     a = np.asarray(a, np.float32)
     b = np.asarray(b, np.float32)
