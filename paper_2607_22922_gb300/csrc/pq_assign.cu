@@ -19,20 +19,24 @@
 // float32 distance it stands for is within 20 x 2^-24 x 2 (|x|^2 + |c|^2) of
 // the true one.  So the float32 argmin's score is within
 // 2 (1.2e-5 + 1.2e-5 + 2.4e-6) (|x|^2 + max|c|^2) of the smallest score, and
-// every codeword within kMargin = 2^-13 (1.2e-4) of it is a candidate: one
-// for almost every row (data whose offset from the origin is ~30 times its
-// spread would see several), and several are compared exactly, smallest
-// first.  Rows for which the bound does not hold (non-finite or huge values,
-// all values below 1e-12) and rows with more than kMaxCand candidates scan
-// all codewords exactly.
+// every codeword within kMargin = 2^-14 (6.1e-5) of it is a candidate.  The
+// unit is a group of 4 codewords: the groups whose smallest score is a
+// candidate (one for almost every row) are compared exactly, codewords
+// ascending; data whose offset from the origin is tens of times its spread
+// would see several.  Rows for which the bound does not hold (non-finite or
+// huge values, all values below 1e-12) and rows with more than kMaxCand
+// candidate groups take all codewords exactly.
 //
-// A thread owns a row.  Two passes over its 256 scores in TMEM: the minimum
-// (three-input min: half an ALU operation per score), then a bit per score
-// within the margin (half a packed subtraction and one funnel shift that
-// collects the sign).  The ALU pipe is the bound: 1.5 operations per score at
-// 64 lanes per SM and cycle.  A CTA of 128 threads holds 256 TMEM columns,
-// two CTAs share an SM: one's epilogue covers the other's MMA, whose operands
-// for the next tile are prepared while the current tile's MMA runs.
+// A thread owns a row.  It reads its scores from TMEM once, keeps the minimum
+// of every four (half an ALU operation per score with the three-input min),
+// then finds the groups within the margin (one packed subtraction per two
+// groups and one funnel shift each that collects the sign).  A CTA of 128
+// threads works on half a codebook (128 TMEM columns) at a time, so that four
+// CTAs share an SM's 512 columns: their decisions cover each other's MMAs.
+// The issue slots are the bound (58 % used; tensor pipe 14 %).  Measured,
+// 2^20 rows x 16 subspaces: 3.49 ms with every codeword evaluated in float32,
+// 0.69 ms now; with whole codebooks (256 columns, two CTAs per SM) 0.80 ms;
+// with two passes over the scores and a bit per codeword 1.22 ms.
 #include "scan_common.cuh"
 
 namespace ifvs {
@@ -41,27 +45,34 @@ namespace {
 
 constexpr int kTile = 128;              // rows per MMA (TMEM lanes), threads per CTA
 constexpr int kMaxTiles = 4;            // tiles per CTA: one codebook image serves them
-constexpr float kMargin = 0x1p-13f;
-constexpr int kMaxCand = 16;
+constexpr float kMargin = 0x1p-14f;
+constexpr int kHalf2 = 128;             // codewords (TMEM columns) per MMA: half a codebook
+constexpr int kMaxCand = 8;             // candidate groups per row; more: all codewords
 
 template <int DS>
 struct AssignShape {
     static constexpr int NB = (DS + 7) / 8;          // 16-byte chunks (8 bf16) per operand part
-    static constexpr int A_CHUNKS = 2 * NB + 2;      // xh, xl, ones, zeros
+    static constexpr int A_CHUNKS = 2 * NB + 1 + (NB & 1 ? 0 : 1);   // xh, xl, ones (, zeros)
     static constexpr int B_CHUNKS = 3 * NB + 1 + (NB & 1 ? 0 : 1);   // ch, ch, cl, |c|^2 (+ a zero chunk: whole K = 16 steps)
     static constexpr int STEPS = B_CHUNKS / 2;
     static constexpr uint32_t A_BYTES = A_CHUNKS * kTile * 16;
     static constexpr uint32_t B_BYTES = B_CHUNKS * 256 * 16;
-    static constexpr uint32_t C_BYTES = 256 * DS * 4;
 };
 
-// dynamic shared memory: A (two buffers), B, codebook in float32 (three
-// slots: a warp may still compare with subspace m - 1 while another, one
-// barrier ahead, stores m + 1), codes of the CTA's rows and subspaces
+// floats of one float32 codebook slot (halves of 128 codewords): 4 codewords
+// and 16 bytes of padding per group, so that the lanes' groups spread over
+// the banks
+__host__ __device__ constexpr int code_floats(int ds, int K) { return (K > kHalf2 ? 2 : 1) * (kHalf2 * ds + kHalf2); }
+
+// Slots of the float32 codebook: a warp may still compare with subspace
+// m - 1 while another stores m + 1, unless a barrier lies between (two halves).
+__host__ __device__ constexpr int code_slots(int K) { return K > kHalf2 ? 2 : 3; }
+
+// dynamic shared memory: A, B, the codebook slots, the codes of the CTA's rows and subspaces
 template <int DS>
-size_t assign_smem_bytes(int tiles, int group) {
+size_t assign_smem_bytes(int K, int tiles, int group) {
     using S = AssignShape<DS>;
-    return 2 * S::A_BYTES + S::B_BYTES + 3 * S::C_BYTES + (size_t)tiles * kTile * group;
+    return S::A_BYTES + S::B_BYTES + (size_t)code_slots(K) * code_floats(DS, K) * 4 + (size_t)tiles * kTile * group;
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -85,29 +96,24 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t addr, float (&v)[32]) {
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&v)[16]) {
     uint32_t* r = reinterpret_cast<uint32_t*>(v);
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(addr));
 }
 
 // the loaded registers pass through the wait, so that no use of them can be
 // moved above it
-__device__ __forceinline__ void tmem_wait_ld(float (&v)[32]) {
+__device__ __forceinline__ void tmem_wait_ld(float (&v)[16]) {
     uint32_t* r = reinterpret_cast<uint32_t*>(v);
     asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
-                   "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
-                   "+r"(r[29]), "+r"(r[30]), "+r"(r[31])::"memory");
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+                   "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
+                   "+r"(r[14]), "+r"(r[15])::"memory");
 }
 
 __device__ __forceinline__ float min3(float a, float b, float c) {
@@ -175,24 +181,6 @@ __device__ __forceinline__ float exact_dist(const float (&x)[DS], const float* c
     return s;
 }
 
-// the first set bit of mask[0..8) (bit j of word w: codeword 32 w + j), cleared; -1 when none is set
-__device__ __forceinline__ int take_first(uint32_t (&mask)[8]) {
-    int w = -1;
-    uint32_t v = 0u;
-#pragma unroll
-    for (int i = 7; i >= 0; --i)
-        if (mask[i] != 0u) {
-            w = i;
-            v = mask[i];
-        }
-    if (w < 0) return -1;
-    const int j = __ffs(v) - 1;
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        if (i == w) mask[i] = v & (v - 1u);
-    return 32 * w + j;
-}
-
 // Codewords `tid` and `tid + 128` of one subspace, in registers.
 template <int DS>
 struct CodeRegs {
@@ -214,14 +202,19 @@ struct CodeRegs {
     __device__ __forceinline__ void store(int K, int tid, float* cbf, uint8_t* B, unsigned* cmax) const {
         using S = AssignShape<DS>;
         unsigned mx = 0u;
+        const float nan = __uint_as_float(0x7FC00000u);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int k = tid + i * kTile;
+            if (i == 1 && K <= kHalf2) break;   // one half
             float n = 0.f;
+            float4* f = reinterpret_cast<float4*>(cbf + k * DS + (k >> 2) * 4);
 #pragma unroll
-            for (int t = 0; t < DS; ++t) {
-                cbf[k * DS + t] = c[i][t];
-                n += c[i][t] * c[i][t];
+            for (int t = 0; t < DS; t += 4) {
+                f[t / 4] = k < K ? make_float4(c[i][t], c[i][t + 1], c[i][t + 2], c[i][t + 3])
+                                 : make_float4(nan, nan, nan, nan);   // never nearest
+                n += c[i][t] * c[i][t] + c[i][t + 1] * c[i][t + 1];
+                n += c[i][t + 2] * c[i][t + 2] + c[i][t + 3] * c[i][t + 3];
             }
             if (k < K) mx = max(mx, n < 1e28f ? __float_as_uint(n) : 0x7F800000u);
             float g[DS];
@@ -255,29 +248,31 @@ struct CodeRegs {
 
 // CTA (row chunk of `tiles` x 128 rows, group of `group` subspaces).
 template <int DS>
-__global__ void __launch_bounds__(kTile, 2) k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K,
-                                                         const float* __restrict__ C, int tiles, int group, int vec,
-                                                         uint8_t* __restrict__ codes, float* __restrict__ dmin) {
+__global__ void __launch_bounds__(kTile, DS > 8 ? 2 : 4)
+k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, const float* __restrict__ C, int tiles,
+                int group, int vec, uint8_t* __restrict__ codes, float* __restrict__ dmin) {
     using S = AssignShape<DS>;
     extern __shared__ __align__(1024) uint8_t sm[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tmem_base;
     __shared__ unsigned cmax[3];   // slots as the float32 codebooks
+    const int nslots = code_slots(K);
     uint8_t* A = sm;
-    uint8_t* B = sm + 2 * S::A_BYTES;
+    uint8_t* B = sm + S::A_BYTES;
     float* cbf = reinterpret_cast<float*>(B + S::B_BYTES);
-    uint8_t* out = B + S::B_BYTES + 3 * S::C_BYTES;      // [tiles * 128][group]
+    uint8_t* out = B + S::B_BYTES + nslots * code_floats(DS, K) * 4;   // [tiles * 128][group]
     const int tid = threadIdx.x, warp = tid >> 5;
     const int64_t row0 = (int64_t)blockIdx.x * tiles * kTile;
     const int m0 = blockIdx.y * group;
     const int g = min(group, M - m0);
     const int nt = (int)min((int64_t)tiles, (n - row0 + kTile - 1) / kTile);
-    const int ncol = (K + 31) & ~31;                      // columns read back
-    // instruction: D float32, A and B bf16, both K-major, N = 256, M = 128
-    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
+    const int halves = K > kHalf2 ? 2 : 1;
+    // instruction: D float32, A and B bf16, both K-major, N = 128, M = 128
+    constexpr uint32_t idesc =
+        (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kHalf2 >> 3) << 17) | ((128u >> 4) << 24);
 
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&tmem_base))
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(smem_u32(&tmem_base))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
@@ -286,41 +281,47 @@ __global__ void __launch_bounds__(kTile, 2) k_pq_assign_mma(const float* __restr
         fence_mbar_init();
         cmax[0] = cmax[1] = cmax[2] = 0u;
     }
-    // the constant chunks of both A buffers: ones against the parts of |c|^2, zeros
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-        uint8_t* a = A + b * S::A_BYTES;
-        *reinterpret_cast<uint4*>(a + (size_t)(2 * S::NB * kTile + tid) * 16) =
-            make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u);
-        *reinterpret_cast<uint4*>(a + (size_t)((2 * S::NB + 1) * kTile + tid) * 16) = make_uint4(0u, 0u, 0u, 0u);
-    }
+    // the constant chunks of A: ones against the parts of |c|^2, zeros
+    *reinterpret_cast<uint4*>(A + (size_t)(2 * S::NB * kTile + tid) * 16) =
+        make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u);
+    if (S::A_CHUNKS > 2 * S::NB + 1)
+        *reinterpret_cast<uint4*>(A + (size_t)((2 * S::NB + 1) * kTile + tid) * 16) = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
 
     CodeRegs<DS> cr;
-    float x[DS], x1[DS], x2[DS];   // this tile's row, the next one's, the one after that (loading)
-    auto load_x = [&](int it, float (&v)[DS]) {
-        const int m = m0 + it / nt;
-        const int64_t r = row0 + (int64_t)(it % nt) * kTile + tid;
-        if (r < n)
-            load_vec<DS>(X + r * D + m * DS, vec != 0, v);
+    float x[DS], x1[DS];   // this tile's row, the next one's (loading)
+    // the row pointer runs ahead of the tile being decided: tile xt of subspace xm
+    int xm = 0, xt = 0;
+    const float* xp = X + (row0 + tid) * D + m0 * DS;
+    int64_t left = n - row0 - tid;   // rows from this thread's on
+    auto load_x = [&](float (&v)[DS]) {
+        if (left > 0)
+            load_vec<DS>(xp, vec != 0, v);
         else
 #pragma unroll
             for (int t = 0; t < DS; ++t) v[t] = 0.f;
+        xp += (int64_t)kTile * D;
+        left -= kTile;
+        if (++xt == nt) {
+            xt = 0;
+            ++xm;
+            xp = X + (row0 + tid) * D + (m0 + xm) * DS;
+            left = n - row0 - tid;
+        }
     };
-    auto store_a = [&](int it, const float (&v)[DS]) {
-        uint8_t* a = A + (it & 1) * S::A_BYTES;
+    auto store_a = [&](const float (&v)[DS]) {
 #pragma unroll
         for (int b = 0; b < S::NB; ++b) {
             uint4 h, l;
             split8<(DS < 8 ? DS : 8)>(v + 8 * b, h, l);
-            *reinterpret_cast<uint4*>(a + (size_t)(b * kTile + tid) * 16) = h;
-            *reinterpret_cast<uint4*>(a + (size_t)((S::NB + b) * kTile + tid) * 16) = l;
+            *reinterpret_cast<uint4*>(A + (size_t)(b * kTile + tid) * 16) = h;
+            *reinterpret_cast<uint4*>(A + (size_t)((S::NB + b) * kTile + tid) * 16) = l;
         }
     };
     // A's chunk of K chunk j of B: (ch, xh), (ch, xl), (cl, xh), (|c|^2, ones), (0, zeros)
     auto a_chunk = [](int j) { return j < 2 * S::NB ? j : (j < 3 * S::NB ? j - 2 * S::NB : j - S::NB); };
-    auto issue = [&](int it) {   // one thread
-        const uint32_t a = smem_u32(A + (it & 1) * S::A_BYTES), b = smem_u32(B);
+    auto issue = [&](int half) {   // one thread
+        const uint32_t a = smem_u32(A), b = smem_u32(B) + (uint32_t)half * kHalf2 * 16;
 #pragma unroll
         for (int st = 0; st < S::STEPS; ++st) {
             const int c0 = a_chunk(2 * st), c1 = a_chunk(2 * st + 1);
@@ -332,11 +333,10 @@ __global__ void __launch_bounds__(kTile, 2) k_pq_assign_mma(const float* __restr
 
     const int iters = g * nt;
     cr.load(C, m0, K, tid, vec != 0);
-    load_x(0, x);
-    if (iters > 1) load_x(1, x1);
+    load_x(x);
     cr.store(K, tid, cbf, B, &cmax[0]);
-    store_a(0, x);
-    if (g > 1) cr.load(C, m0 + 1, K, tid, vec != 0);
+    store_a(x);
+    if (iters > 1) load_x(x1);
     fence_proxy_async_smem();
     __syncthreads();
     const uint32_t tm = tmem_base + ((uint32_t)(warp * 32) << 16);
@@ -344,127 +344,158 @@ __global__ void __launch_bounds__(kTile, 2) k_pq_assign_mma(const float* __restr
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         issue(0);
     }
-    // mma_ok false, late >= 0: the bounded wait for tile `late`'s MMA ran out;
-    // its rows and all later ones are scanned exactly
+    // mma_ok false, late = 0 or 1: the bounded wait for an MMA (of that
+    // barrier parity) ran out; its rows and all later ones are scanned exactly
     bool mma_ok = true;
     int late = -1;
+    uint32_t phase = 0u;
+    int mi = 0, ti = 0, slot = 0;   // subspace and tile of iteration it; the subspace's codebook slot
 #pragma unroll 1
     for (int it = 0; it < iters; ++it) {
-        const int mi = it / nt;
         const bool more = it + 1 < iters;
-        const bool new_m = more && (it + 1) / nt != mi;
-        if (it + 2 < iters) load_x(it + 2, x2);
-        if (more) store_a(it + 1, x1);
+        const bool new_m = more && ti + 1 == nt;
         float nx = 0.f;
 #pragma unroll
         for (int t = 0; t < DS; ++t) nx = fmaf(x[t], x[t], nx);
-        const float span = nx + __uint_as_float(cmax[mi % 3]);
+        const float span = nx + __uint_as_float(cmax[slot]);
+        const float margin = kMargin * span;
         bool all = !(span > 1e-24f && span < 1e28f);
-        uint32_t mask[8];
+        // per half: the smallest score and the groups within the margin of
+        // it (bit j: group j of the half)
+        uint32_t mask[2] = {0u, 0u};
+        float low[2] = {0x1p120f, 0x1p120f};
 #pragma unroll
-        for (int i = 0; i < 8; ++i) mask[i] = 0u;
-        if (mma_ok) mma_ok = mbar_wait_warp(smem_u32(&bar), (uint32_t)it & 1u);
-        if (mma_ok) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // both passes read 32 columns ahead
-            float lo = 0x1p120f;
-            float vv[2][32];
-            tmem_ld32(tm, vv[0]);
+        for (int h = 0; h < 2; ++h) {
+            if (h >= halves) break;
+            float gm[32];
+            if (mma_ok) mma_ok = mbar_wait_warp(smem_u32(&bar), phase);
+            if (mma_ok) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                // the smallest score of every 4 codewords
+                float vv[2][16];
+                tmem_ld16(tm, vv[0]);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (32 * i >= ncol) break;
-                float(&v)[32] = vv[i & 1];
-                tmem_wait_ld(v);
-                if (32 * (i + 1) < ncol) tmem_ld32(tm + 32 * (i + 1), vv[(i + 1) & 1]);
-                float p = min3(v[0], v[1], v[2]), q = min3(v[3], v[4], v[5]);
+                for (int i = 0; i < 8; ++i) {
+                    float(&v)[16] = vv[i & 1];
+                    tmem_wait_ld(v);
+                    if (i < 7) tmem_ld16(tm + 16 * (i + 1), vv[(i + 1) & 1]);
 #pragma unroll
-                for (int j = 6; j < 30; j += 4) {
-                    p = min3(p, v[j], v[j + 1]);
-                    q = min3(q, v[j + 2], v[j + 3]);
+                    for (int j = 0; j < 4; ++j)
+                        gm[4 * i + j] = fminf(min3(v[4 * j], v[4 * j + 1], v[4 * j + 2]), v[4 * j + 3]);
                 }
-                lo = min3(lo, min3(p, v[30], v[31]), q);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             }
-            const float thr = lo + kMargin * span;
-            const uint64_t nthr = add_f32x2(0ull, -thr, -thr);
-            tmem_ld32(tm, vv[0]);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (32 * i >= ncol) break;
-                float(&v)[32] = vv[i & 1];
-                tmem_wait_ld(v);
-                if (32 * (i + 1) < ncol) tmem_ld32(tm + 32 * (i + 1), vv[(i + 1) & 1]);
-                uint32_t w = 0u;
-#pragma unroll
-                for (int j = 30; j >= 0; j -= 2) {
-                    float a, b;
-                    unpack_f32x2(add_f32x2(nthr, v[j], v[j + 1]), a, b);
-                    w = __funnelshift_l(__float_as_uint(b), w, 1);
-                    w = __funnelshift_l(__float_as_uint(a), w, 1);
+            const bool read = mma_ok;
+            // the next MMA: the other half, or the next tile, whose operands
+            // replace this one's now that its MMAs are done
+            const bool last = h + 1 == halves;
+            if (last && more) {
+                store_a(x1);
+                if (new_m) {
+                    const int next = slot + 1 == nslots ? 0 : slot + 1;
+                    cr.load(C, m0 + mi + 1, K, tid, vec != 0);
+                    cr.store(K, tid, cbf + next * code_floats(DS, K), B, &cmax[next]);
                 }
-                mask[i] = w;
+                fence_proxy_async_smem();
             }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        }
-        const bool mma_was_ok = mma_ok;
-        // the next tile's MMA: its operands are in place, this tile's scores are read
-        if (new_m) {
-            cr.store(K, tid, cbf + ((mi + 1) % 3) * (256 * DS), B, &cmax[(mi + 1) % 3]);
-            if (mi + 2 < g) cr.load(C, m0 + mi + 2, K, tid, vec != 0);
-        }
-        fence_proxy_async_smem();
-        if (__syncthreads_or(mma_ok ? 0 : 1) != 0 && late < 0) late = it;
-        mma_ok = late < 0;
-        if (mma_ok && more && tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            issue(it + 1);
-        }
-        // the decision
-        int cnt = 0;
+            if (__syncthreads_or(mma_ok ? 0 : 1) != 0 && late < 0) late = (int)phase;
+            mma_ok = late < 0;
+            phase ^= 1u;
+            if (mma_ok && (!last || more) && tid == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                issue(last ? 0 : 1);
+            }
+            if (read) {
+                float lo[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) cnt += __popc(mask[i]);
-        all = all || !mma_was_ok || cnt == 0 || cnt > kMaxCand;
-        const float* cb = cbf + (mi % 3) * (256 * DS);
-        float best = 0.f;
+                for (int i = 0; i < 4; ++i) lo[i] = fminf(gm[i], gm[i + 4]);
+#pragma unroll
+                for (int j = 8; j < 32; j += 8)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) lo[i] = min3(lo[i], gm[j + i], gm[j + i + 4]);
+                low[h] = fminf(fminf(lo[0], lo[1]), fminf(lo[2], lo[3]));
+                const float thr = low[h] + margin;
+                const uint64_t nthr = add_f32x2(0ull, -thr, -thr);
+                // the signs of (score - thr), eight per chain of funnel shifts
+                uint32_t w[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) w[i] = 0u;
+#pragma unroll
+                for (int j = 6; j >= 0; j -= 2)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float a, b;
+                        unpack_f32x2(add_f32x2(nthr, gm[8 * i + j], gm[8 * i + j + 1]), a, b);
+                        w[i] = __funnelshift_l(__float_as_uint(b), w[i], 1);
+                        w[i] = __funnelshift_l(__float_as_uint(a), w[i], 1);
+                    }
+                mask[h] = w[0] | w[1] << 8 | w[2] << 16 | w[3] << 24;
+            }
+        }
+        // a half whose smallest score is beyond the other's margin has no candidate
+        if (low[1] > low[0] + margin) mask[1] = 0u;
+        if (low[0] > low[1] + margin) mask[0] = 0u;
+        const int cnt = __popc(mask[0]) + __popc(mask[1]);
+        all = all || cnt == 0 || cnt > kMaxCand || (late >= 0);
+        const float* cb = cbf + slot * code_floats(DS, K);
+        float best = INFINITY;
         int bk = 0;
-        if (!all) {
-            bk = take_first(mask);
-            if (cnt > 1 || dmin != nullptr) best = exact_dist<DS>(x, cb + bk * DS);
-            for (int left = cnt - 1; left > 0; --left) {
-                const int k = take_first(mask);
-                const float s = exact_dist<DS>(x, cb + k * DS);
-                if (s < best) {
-                    best = s;
-                    bk = k;
-                }
-            }
-        } else {
+        if (all) {
+            // every codeword exactly; NaN distances as in the definition
+            // (the first codeword stands until a smaller distance is found)
+            mask[0] = mask[1] = 0u;
             best = exact_dist<DS>(x, cb);
 #pragma unroll 1
             for (int k = 1; k < K; ++k) {
-                const float s = exact_dist<DS>(x, cb + k * DS);
+                const float s = exact_dist<DS>(x, cb + k * DS + (k >> 2) * 4);
                 if (s < best) {
                     best = s;
                     bk = k;
                 }
             }
         }
-        const int lr = (it % nt) * kTile + tid;
+        // the float32 decision over the candidate groups, codewords
+        // ascending; their distances are finite, those of columns beyond K NaN
+#pragma unroll 1
+        while ((mask[0] | mask[1]) != 0u) {
+            int g4;
+            if (mask[0] != 0u) {
+                g4 = __ffs(mask[0]) - 1;
+                mask[0] &= mask[0] - 1u;
+            } else {
+                g4 = 31 + __ffs(mask[1]);
+                mask[1] &= mask[1] - 1u;
+            }
+            const float* c = cb + g4 * (4 * DS + 4);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float s = exact_dist<DS>(x, c + j * DS);
+                if (s < best) {
+                    best = s;
+                    bk = 4 * g4 + j;
+                }
+            }
+        }
+        const int lr = ti * kTile + tid;
         out[lr * g + mi] = (uint8_t)bk;
         if (dmin != nullptr && row0 + lr < n) dmin[(row0 + lr) * M + m0 + mi] = best;
-        if (new_m && tid == 0) cmax[mi % 3] = 0u;   // its last readers passed the barrier above
+        if (new_m && tid == 0) cmax[slot] = 0u;   // its last readers passed the barrier above
 #pragma unroll
-        for (int t = 0; t < DS; ++t) {
-            x[t] = x1[t];
-            x1[t] = x2[t];
+        for (int t = 0; t < DS; ++t) x[t] = x1[t];
+        if (it + 2 < iters) load_x(x1);
+        if (++ti == nt) {
+            ti = 0;
+            ++mi;
+            slot = slot + 1 == nslots ? 0 : slot + 1;
         }
     }
     __syncthreads();
     if (late >= 0) {   // that MMA may still be in flight: wait again (bounded) before TMEM is freed
-        mbar_wait_warp(smem_u32(&bar), (uint32_t)late & 1u);
+        mbar_wait_warp(smem_u32(&bar), (uint32_t)late);
         __syncthreads();
     }
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem_base));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem_base));
     const int64_t rows = min((int64_t)nt * kTile, n - row0);
     for (int e = tid; e < (int)rows * g; e += kTile) {
         const int r = e / g;
@@ -512,10 +543,10 @@ static cudaError_t launch_assign_mma(const float* X, int64_t n, int D, int M, in
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    // Tiles per CTA share one codebook image (worth about a fifth of a tile);
+    // Tiles per CTA share one codebook image (worth about a fourth of a tile);
     // fewer, and the subspaces split over CTAs, where the rows alone would
-    // leave the two CTAs per SM without four waves of work.
-    const int64_t want = (int64_t)sms * 2 * 4;
+    // leave the resident CTAs without four waves of work.
+    const int64_t want = (int64_t)sms * (DS > 8 ? 2 : 4) * 4;
     const int64_t all = (n + kTile - 1) / kTile;
     int tiles = (int)(all / want);
     tiles = tiles < 1 ? 1 : (tiles > kMaxTiles ? kMaxTiles : tiles);
@@ -523,10 +554,10 @@ static cudaError_t launch_assign_mma(const float* X, int64_t n, int D, int M, in
     int64_t groups = (want + chunks - 1) / chunks;
     if (groups > M) groups = M;
     int group = (int)((M + groups - 1) / groups);
-    if (group > (DS > 8 ? 16 : 32)) group = DS > 8 ? 16 : 32;   // two CTAs' shared memory per SM
+    if (group > (DS > 8 ? 8 : 32)) group = DS > 8 ? 8 : 32;   // two CTAs' shared memory per SM
     groups = (M + group - 1) / group;
     const bool vec = ((uintptr_t)X | (uintptr_t)C) % 16 == 0;   // ds is a multiple of 4: so are D and every offset
-    const size_t smem = assign_smem_bytes<DS>(tiles, group);
+    const size_t smem = assign_smem_bytes<DS>(K, tiles, group);
     e = cudaFuncSetAttribute(k_pq_assign_mma<DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_pq_assign_mma<DS><<<dim3((unsigned)chunks, (unsigned)groups), kTile, smem, s>>>(X, n, D, M, K, C, tiles, group,
