@@ -358,8 +358,7 @@ int ifvs_pq_encode(int32_t device, const float* X, int64_t n, int32_t D, int32_t
  *   objective  [iters][M] fp64 out (sum of the assignment's minimum
  *              distances at each iteration, before its update), or NULL
  *   stream     cudaStream_t for the work, or NULL (a stream of the call's own)
- * The call returns when C_out (and objective) are written; it reads the
- * per-codeword counts back to the host once per iteration.  Errors as
+ * The call returns when C_out (and objective) are written.  Errors as
  * ifvs_pq_encode, plus IFVS_ERR_ARG for iters < 0.
  */
 int ifvs_pq_train(int32_t device, const float* X, int64_t n, int32_t D, int32_t M, int32_t K,

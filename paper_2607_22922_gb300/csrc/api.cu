@@ -1453,7 +1453,7 @@ extern "C" int ifvs_pq_encode(int32_t device, const float* X, int64_t n, int32_t
             ddmin = (float*)p;
         }
     }
-    CUDA_TRY(launch_pq_assign((const float*)dX, n, D, M, K, (const float*)dC, dcodes, ddmin, a.s));
+    CUDA_TRY(launch_pq_assign((const float*)dX, n, D, M, K, (const float*)dC, dcodes, ddmin, false, a.s));
     if (!dio) {
         CUDA_TRY(cudaMemcpyAsync(codes, dcodes, (size_t)n * M, cudaMemcpyDeviceToHost, a.s));
         if (dmin) CUDA_TRY(cudaMemcpyAsync(dmin, ddmin, sizeof(float) * n * M, cudaMemcpyDeviceToHost, a.s));
@@ -1476,39 +1476,28 @@ extern "C" int ifvs_pq_train(int32_t device, const float* X, int64_t n, int32_t 
     const void *dX = nullptr, *dC0;
     if (n > 0) TRY(a.input(X, sizeof(float) * n * D, dio, &dX));
     TRY(a.input(C_init, cb_bytes, dio, &dC0));
-    void *cA, *cB, *codes, *dmin, *sums, *counts, *best, *obj;
-    TRY(a.alloc(&cA, cb_bytes));
-    TRY(a.alloc(&cB, cb_bytes));
-    TRY(a.alloc(&codes, (size_t)(n > 0 ? n : 1) * M));
-    TRY(a.alloc(&dmin, sizeof(float) * (size_t)(n > 0 ? n : 1) * M));
-    TRY(a.alloc(&sums, sizeof(double) * (size_t)M * K * ds));
-    TRY(a.alloc(&counts, sizeof(unsigned long long) * (size_t)M * K));
-    TRY(a.alloc(&best, sizeof(unsigned long long)));
-    TRY(a.alloc(&obj, sizeof(double) * M));
+    // one allocation: two codebooks, every iteration's objective, the update's buffers
+    LloydBufs lb{};
+    size_t lb_bytes = 0;
+    lloyd_plan(n, M, K, ds, a.num_sms, &lb, &lb_bytes);
+    auto padded = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t obj_bytes = objective && !dio ? sizeof(double) * (size_t)M * iters : 0;
+    void* base;
+    TRY(a.alloc(&base, 2 * padded(cb_bytes) + padded(obj_bytes) + lb_bytes));
+    float* cA = (float*)base;
+    float* cB = (float*)((uint8_t*)base + padded(cb_bytes));
+    double* obj = dio ? objective : (double*)((uint8_t*)base + 2 * padded(cb_bytes));
+    lb.base = (uint8_t*)base + 2 * padded(cb_bytes) + padded(obj_bytes);
+    lloyd_plan(n, M, K, ds, a.num_sms, &lb, &lb_bytes);
     CUDA_TRY(cudaMemcpyAsync(cA, dC0, cb_bytes, cudaMemcpyDeviceToDevice, a.s));
-    std::vector<unsigned long long> cnt((size_t)M * K);
     for (int it = 0; it < iters && n > 0; ++it) {
-        CUDA_TRY(launch_pq_assign((const float*)dX, n, D, M, K, (const float*)cA, (uint8_t*)codes,
-                                  (float*)dmin, a.s));
-        if (objective) {
-            CUDA_TRY(launch_pq_objective((const float*)dmin, n, M, (double*)obj, a.num_sms, a.s));
-            CUDA_TRY(cudaMemcpyAsync(objective + (size_t)it * M, obj, sizeof(double) * M,
-                                     dio ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, a.s));
-        }
-        CUDA_TRY(launch_pq_update((const float*)dX, n, D, M, K, (const uint8_t*)codes, (double*)sums,
-                                  (unsigned long long*)counts, (const float*)cA, (float*)cB,
-                                  a.num_sms, a.s));
-        CUDA_TRY(cudaMemcpyAsync(cnt.data(), counts, sizeof(unsigned long long) * cnt.size(),
-                                 cudaMemcpyDeviceToHost, a.s));
-        CUDA_TRY(cudaStreamSynchronize(a.s));
-        for (int m = 0; m < M; ++m)
-            for (int c = 0; c < K; ++c)
-                if (cnt[(size_t)m * K + c] == 0)
-                    CUDA_TRY(launch_pq_reseed((const float*)dX, n, D, M, K, m, c,
-                                              (unsigned long long*)best, (float*)cB, (float*)dmin,
-                                              a.num_sms, a.s));
+        CUDA_TRY(launch_pq_assign((const float*)dX, n, D, M, K, cA, lb.codes, lb.dmin, true, a.s));
+        CUDA_TRY(launch_pq_update((const float*)dX, n, D, M, K, lb, cA, cB,
+                                  objective ? obj + (size_t)it * M : nullptr, a.s));
         std::swap(cA, cB);
     }
+    if (obj_bytes && n > 0)
+        CUDA_TRY(cudaMemcpyAsync(objective, obj, obj_bytes, cudaMemcpyDeviceToHost, a.s));
     CUDA_TRY(cudaMemcpyAsync(C_out, cA, cb_bytes, dio ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, a.s));
     CUDA_TRY(cudaStreamSynchronize(a.s));
     return IFVS_OK;

@@ -252,19 +252,29 @@ cudaError_t launch_relayout_codes(const uint8_t* src, int64_t N, int M, int K, i
                                   int64_t n_rows_pad, uint8_t* dst, int* bad, cudaStream_t s);
 
 // ---- PQ construction (csrc/pq.cu) --------------------------------------
-// codes [n][M] and optional dmin [n][M] (float32 argmin, fixed order)
+// codes [n][M] and optional dmin [n][M] (float32 argmin, fixed order); by
+// subspace ([M][n]) when `by_subspace`
 cudaError_t launch_pq_assign(const float* X, int64_t n, int D, int M, int K, const float* C,
-                             uint8_t* codes, float* dmin, cudaStream_t s);
-// Lloyd update: fp64 means of the members (sums [M][K][ds], counts [M][K])
-cudaError_t launch_pq_update(const float* X, int64_t n, int D, int M, int K, const uint8_t* codes,
-                             double* sums, unsigned long long* counts, const float* C_in,
-                             float* C_out, int num_sms, cudaStream_t s);
-// empty codeword c of subspace m <- the farthest row (best: 8-byte scratch)
-cudaError_t launch_pq_reseed(const float* X, int64_t n, int D, int M, int K, int m, int c,
-                             unsigned long long* best, float* C_out, float* dmin, int num_sms,
-                             cudaStream_t s);
-cudaError_t launch_pq_objective(const float* dmin, int64_t n, int M, double* objective, int num_sms,
-                                cudaStream_t s);
+                             uint8_t* codes, float* dmin, bool by_subspace, cudaStream_t s);
+// Buffers of Lloyd training, carved from one allocation at `base`
+struct LloydBufs {
+    uint8_t* base;
+    int64_t rows_per_chunk;
+    int chunks;
+    float2* sums;               // [chunks][M][K][ds] member sums (value + error)
+    double* obj;                // [chunks][M] sums of distances
+    unsigned long long* far;    // [chunks][M] farthest row: distance bits << 32 | ~row
+    unsigned* counts;           // [chunks][M][K] members
+    float* dmin;                // [M][n]
+    uint8_t* codes;             // [M][n]
+    uint8_t* used;              // [M][K]
+};
+// sets the plan and the pointers (relative to b->base, which may be null) and the bytes needed
+void lloyd_plan(int64_t n, int M, int K, int ds, int num_sms, LloydBufs* b, size_t* bytes);
+// Lloyd update from b's codes and dmin: fp64 means of the members, unused
+// codewords on the farthest rows; objective [M] (may be null)
+cudaError_t launch_pq_update(const float* X, int64_t n, int D, int M, int K, const LloydBufs& b, const float* C_in,
+                             float* C_out, double* objective, cudaStream_t s);
 
 // ---- training of bank, W, w_f (csrc/train.cu) --------------------------
 constexpr int kTrainMaxR = 32;     // r per subspace handled by the gradient kernels

@@ -246,8 +246,9 @@ struct CodeRegs {
 
 }  // namespace
 
-// CTA (row chunk of `tiles` x 128 rows, group of `group` subspaces).
-template <int DS>
+// CTA (row chunk of `tiles` x 128 rows, group of `group` subspaces).  Codes
+// and distances [n][M], or [M][n] (BY_SUBSPACE).
+template <int DS, bool BY_SUBSPACE>
 __global__ void __launch_bounds__(kTile, DS > 8 ? 2 : 4)
 k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, const float* __restrict__ C, int tiles,
                 int group, int vec, uint8_t* __restrict__ codes, float* __restrict__ dmin) {
@@ -477,8 +478,9 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
             }
         }
         const int lr = ti * kTile + tid;
-        out[lr * g + mi] = (uint8_t)bk;
-        if (dmin != nullptr && row0 + lr < n) dmin[(row0 + lr) * M + m0 + mi] = best;
+        out[BY_SUBSPACE ? mi * (nt * kTile) + lr : lr * g + mi] = (uint8_t)bk;
+        if (dmin != nullptr && row0 + lr < n)
+            dmin[BY_SUBSPACE ? (m0 + mi) * n + row0 + lr : (row0 + lr) * M + m0 + mi] = best;
         if (new_m && tid == 0) cmax[slot] = 0u;   // its last readers passed the barrier above
 #pragma unroll
         for (int t = 0; t < DS; ++t) x[t] = x1[t];
@@ -497,9 +499,15 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem_base));
     const int64_t rows = min((int64_t)nt * kTile, n - row0);
-    for (int e = tid; e < (int)rows * g; e += kTile) {
-        const int r = e / g;
-        codes[(row0 + r) * M + m0 + (e - r * g)] = out[e];
+    if (BY_SUBSPACE) {
+        for (int j = 0; j < g; ++j)
+            for (int r = tid; r < (int)rows; r += kTile)
+                codes[(m0 + j) * n + row0 + r] = out[j * nt * kTile + r];
+    } else {
+        for (int e = tid; e < (int)rows * g; e += kTile) {
+            const int r = e / g;
+            codes[(row0 + r) * M + m0 + (e - r * g)] = out[e];
+        }
     }
 }
 
@@ -507,8 +515,8 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
 constexpr int kPqThreads = 256;
 __global__ void __launch_bounds__(kPqThreads) k_pq_assign_any(const float* __restrict__ X, int64_t n,
                                                               int D, int M, int K, int ds,
-                                                              const float* __restrict__ C,
-                                                              uint8_t* __restrict__ codes,
+                                                              const float* __restrict__ C, int64_t row_stride,
+                                                              int64_t sub_stride, uint8_t* __restrict__ codes,
                                                               float* __restrict__ dmin) {
     extern __shared__ __align__(16) float cb[];
     const int64_t i = (int64_t)blockIdx.x * kPqThreads + threadIdx.x;
@@ -531,14 +539,15 @@ __global__ void __launch_bounds__(kPqThreads) k_pq_assign_any(const float* __res
                 bk = k;
             }
         }
-        codes[i * M + m] = (uint8_t)bk;
-        if (dmin != nullptr) dmin[i * M + m] = best;
+        const int64_t at = i * row_stride + m * sub_stride;
+        codes[at] = (uint8_t)bk;
+        if (dmin != nullptr) dmin[at] = best;
     }
 }
 
 template <int DS>
 static cudaError_t launch_assign_mma(const float* X, int64_t n, int D, int M, int K, const float* C, uint8_t* codes,
-                                     float* dmin, cudaStream_t s) {
+                                     float* dmin, bool by_subspace, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -558,25 +567,27 @@ static cudaError_t launch_assign_mma(const float* X, int64_t n, int D, int M, in
     groups = (M + group - 1) / group;
     const bool vec = ((uintptr_t)X | (uintptr_t)C) % 16 == 0;   // ds is a multiple of 4: so are D and every offset
     const size_t smem = assign_smem_bytes<DS>(K, tiles, group);
-    e = cudaFuncSetAttribute(k_pq_assign_mma<DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = by_subspace ? k_pq_assign_mma<DS, true> : k_pq_assign_mma<DS, false>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_pq_assign_mma<DS><<<dim3((unsigned)chunks, (unsigned)groups), kTile, smem, s>>>(X, n, D, M, K, C, tiles, group,
-                                                                                    vec ? 1 : 0, codes, dmin);
+    kern<<<dim3((unsigned)chunks, (unsigned)groups), kTile, smem, s>>>(X, n, D, M, K, C, tiles, group, vec ? 1 : 0,
+                                                                       codes, dmin);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pq_assign(const float* X, int64_t n, int D, int M, int K, const float* C,
-                             uint8_t* codes, float* dmin, cudaStream_t s) {
+                             uint8_t* codes, float* dmin, bool by_subspace, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int ds = D / M;
-    if (ds == 4) return launch_assign_mma<4>(X, n, D, M, K, C, codes, dmin, s);
-    if (ds == 8) return launch_assign_mma<8>(X, n, D, M, K, C, codes, dmin, s);
-    if (ds == 16) return launch_assign_mma<16>(X, n, D, M, K, C, codes, dmin, s);
+    const int64_t rs = by_subspace ? 1 : M, ss = by_subspace ? n : 1;
+    if (ds == 4) return launch_assign_mma<4>(X, n, D, M, K, C, codes, dmin, by_subspace, s);
+    if (ds == 8) return launch_assign_mma<8>(X, n, D, M, K, C, codes, dmin, by_subspace, s);
+    if (ds == 16) return launch_assign_mma<16>(X, n, D, M, K, C, codes, dmin, by_subspace, s);
     const size_t smem = (size_t)K * ds * sizeof(float);
     const int64_t blocks = (n + kPqThreads - 1) / kPqThreads;
     cudaError_t e = cudaFuncSetAttribute(k_pq_assign_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_pq_assign_any<<<(unsigned)blocks, kPqThreads, smem, s>>>(X, n, D, M, K, ds, C, codes, dmin);
+    k_pq_assign_any<<<(unsigned)blocks, kPqThreads, smem, s>>>(X, n, D, M, K, ds, C, rs, ss, codes, dmin);
     return cudaGetLastError();
 }
 

@@ -114,6 +114,25 @@ def test_one_lloyd_step(ifvs, orc, name, n):
     np.testing.assert_allclose(obj[0], robj, rtol=1e-12)
 
 
+@pytest.mark.parametrize("n,M,K,ds", [(1, 3, 2, 8), (1023, 16, 256, 8), (40_003, 64, 32, 4), (9001, 2, 256, 12)])
+def test_one_lloyd_step_edges(ifvs, orc, n, M, K, ds):
+    """One row, one short chunk, chunks of several sorted runs, a generic
+    sub-vector length; some codewords start unused."""
+    rng = np.random.default_rng(n)
+    X = rng.standard_normal((n, M * ds)).astype(np.float32)
+    C0 = rng.standard_normal((M, K, ds)).astype(np.float32)
+    C0[:, K // 2] += 50.0
+    C0[:, K - 1] -= 50.0
+    if n == 40_003:
+        X[::7, :4] *= 1e37                       # member sums beyond float32
+        X[3, 5] = np.inf
+    C1, obj = ifvs.ifvs_pq_train(X, C0, 1)
+    R1, _, robj = orc.lloyd_step(X, C0)
+    with np.errstate(invalid="ignore"):
+        assert (_ulp_close(C1, R1) | (C1 == R1) | (np.isnan(C1) & np.isnan(R1))).all()
+    np.testing.assert_allclose(obj[0], robj, rtol=1e-12)
+
+
 def test_empty_codewords_take_the_farthest_points(ifvs, orc):
     rng = np.random.default_rng(5)
     X = rng.standard_normal((4000, 16)).astype(np.float32)
