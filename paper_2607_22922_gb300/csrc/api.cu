@@ -484,16 +484,43 @@ ScanShape scan_shape(const ifvs_index* ix, int64_t n, int kk, int64_t chunk_bloc
     return sh;
 }
 
+// Arguments of launch_prepare: the predicates alone, and with the
+// conditioning into the index's workspace (w_idx, w_alpha, w_wf).
+PrepareArgs prepare_args(const ifvs_index* ix, const ifvs_predicate* dp, CanonPred* canon) {
+    PrepareArgs a{};
+    a.preds = dp;
+    a.cols = ix->cols();
+    a.canon = canon;
+    a.err = ix->w_err.as<int>();
+    return a;
+}
+
+void prepare_condition(const ifvs_index* ix, const float* dq, const float* dwz, int64_t wz_stride, bool cond,
+                       PrepareArgs* a) {
+    a->q = dq;
+    a->D = ix->D;
+    a->seeds = ix->d_seeds;
+    a->h = ix->h;
+    a->B = ix->B;
+    a->bank = cond ? ix->d_bank : nullptr;
+    a->Mr = ix->M * ix->r;
+    a->wz = dwz;
+    a->wz_stride = wz_stride;
+    a->idx = ix->w_idx.as<uint32_t>();
+    a->alpha = ix->w_alpha.as<float>();
+    a->wf = ix->w_wf.as<float>();
+}
+
 // The query path for one sub-batch of n queries whose inputs are on the
-// device.  Writes k ids / dists per query to out_ids / out_dists (device)
-// and the pass counts to npass_u64 (device, zeroed here).
+// device (w_z of query i at dwz + i * wz_stride).  Writes k ids / dists per query to out_ids / out_dists (device)
+// and the pass counts to npass_u64 (device).
 int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
-             const ifvs_predicate* dp, const float* dwz, int64_t n, int k, int64_t* out_ids,
+             const ifvs_predicate* dp, const float* dwz, int64_t wz_stride, int64_t n, int k, int64_t* out_ids,
              float* out_dists, unsigned long long* npass_u64) {
     const int kk = o.R > 0 ? o.R : k;
     const int Mr = ix->M * ix->r;
     const bool cond = !o.plain && ix->d_bank != nullptr;
-    // Which queries take the bitmap path is decided on the device (k_plan),
+    // Which queries take the bitmap path is decided on the device (k_prepare),
     // but with the sorted-copy path on for every pool size and one attribute
     // column none can: every predicate then constrains at most that column.
     // Such batches need no bitmap workspace (N / 8 bytes per query) and no
@@ -514,34 +541,39 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
         TRY(ensure(ix->w_cand, sizeof(int64_t) * n * kk));
         TRY(ensure(ix->w_cdist, sizeof(float) * n * kk));
     }
-    CUDA_TRY(cudaMemsetAsync(npass_u64, 0, sizeof(unsigned long long) * n, s));
-    {
-        Stage st(ix, s, o.timing, IFVS_STAGE_PREDICATE);
-        CUDA_TRY(st.end(launch_canonicalize(dp, n, ix->cols(), ix->w_canon.as<CanonPred>(),
-                                            ix->w_err.as<int>(), s)));
-    }
     // one-column predicates take the sorted-copy scan (up to the threshold)
     const ScanPlan* plan = nullptr;
+    PrepareArgs pa = prepare_args(ix, dp, ix->w_canon.as<CanonPred>());
+    if (o.timing) {   // every stage in a launch of its own, to be timed by itself
+        Stage st(ix, s, true, IFVS_STAGE_PREDICATE);
+        CUDA_TRY(st.end(launch_prepare(pa, n, s)));
+    }
     if (list_on) {
-        const int64_t max_rows = ppm >= 1000000 ? ix->N : ix->N * ppm / 1000000;
         TRY(ensure(ix->w_plan, sizeof(ScanPlan) * n));
         TRY(ensure(ix->w_items, scan_list_workspace_bytes(n)));   // query groups of the sorted-copy scan
-        Stage st(ix, s, o.timing, IFVS_STAGE_FILTER);
-        CUDA_TRY(st.end(launch_plan(ix->w_canon.as<CanonPred>(), n, ix->sorted(), ix->N, max_rows,
-                                    ix->w_plan.as<ScanPlan>(), npass_u64, s)));
-        plan = ix->w_plan.as<ScanPlan>();
+        pa.sorted = ix->sorted();
+        pa.N = ix->N;
+        pa.max_rows = ppm >= 1000000 ? ix->N : ix->N * ppm / 1000000;
+        pa.plan = ix->w_plan.as<ScanPlan>();
+        pa.npass = npass_u64;
+        plan = pa.plan;
+        if (o.timing) {
+            Stage st(ix, s, true, IFVS_STAGE_FILTER);
+            CUDA_TRY(st.end(launch_prepare(pa, n, s)));
+            pa.plan = nullptr;
+        }
+    } else {
+        CUDA_TRY(cudaMemsetAsync(npass_u64, 0, sizeof(unsigned long long) * n, s));
+    }
+    prepare_condition(ix, dq, dwz, wz_stride, cond, &pa);
+    {
+        Stage st(ix, s, o.timing, IFVS_STAGE_CONDITION);
+        CUDA_TRY(st.end(launch_prepare(pa, n, s)));
     }
     if (bitmaps) {
         Stage st(ix, s, o.timing, IFVS_STAGE_FILTER);
         CUDA_TRY(st.end(launch_filter(ix->cols(), ix->N, ix->n_blocks, ix->w_canon.as<CanonPred>(),
                                       plan, n, ix->w_bm.as<uint32_t>(), npass_u64, ix->num_sms, s)));
-    }
-    {
-        Stage st(ix, s, o.timing, IFVS_STAGE_CONDITION);
-        CUDA_TRY(st.end(launch_condition(dq, dp, n, ix->D, ix->d_seeds, ix->h, ix->B,
-                                         cond ? ix->d_bank : nullptr, Mr, dwz,
-                                         ix->w_idx.as<uint32_t>(), ix->w_alpha.as<float>(),
-                                         ix->w_wf.as<float>(), s)));
     }
     {
         Stage st(ix, s, o.timing, IFVS_STAGE_LUT);
@@ -705,8 +737,7 @@ int train_check(ifvs_index* ix, const ifvs_train_params* tp, int64_t nq, bool st
     return 0;
 }
 
-// Stages queries, predicates and the shared w_z (a device copy in t_wz and a
-// per-query broadcast in w_wz), and validates the predicates.
+// Stages queries, predicates and the shared w_z (a device copy in t_wz).
 int train_stage(ifvs_index* ix, cudaStream_t s, const Opts& o, int64_t n, const float* queries,
                 const ifvs_predicate* preds, const float* wz, const float** dq,
                 const ifvs_predicate** dp) {
@@ -714,14 +745,6 @@ int train_stage(ifvs_index* ix, cudaStream_t s, const Opts& o, int64_t n, const 
     TRY(ensure(ix->t_wz, sizeof(float) * ix->D));
     CUDA_TRY(cudaMemcpyAsync(ix->t_wz.p, wz, sizeof(float) * ix->D,
                              o.dio ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-    TRY(ensure(ix->w_wz, sizeof(float) * n * ix->D));
-    CUDA_TRY(launch_broadcast_wz(ix->t_wz.as<float>(), ix->D, n, ix->w_wz.as<float>(), s));
-    TRY(ensure(ix->w_canon, sizeof(CanonPred) * n));
-    {
-        Stage st(ix, s, o.timing, IFVS_STAGE_PREDICATE);
-        CUDA_TRY(st.end(launch_canonicalize(*dp, n, ix->cols(), ix->w_canon.as<CanonPred>(),
-                                            ix->w_err.as<int>(), s)));
-    }
     return 0;
 }
 
@@ -1087,7 +1110,7 @@ int ifvs_search_batch(ifvs_index* ix, const float* queries, const ifvs_predicate
         TRY(stage_inputs(ix, s, o, q0, n, queries, preds, wz, &dq, &dp, &dwz));
         int64_t* oid = o.dio ? ids + q0 * k : ix->w_ids.as<int64_t>();
         float* odi = o.dio ? dists + q0 * k : ix->w_dists.as<float>();
-        TRY(run_path(ix, s, o, dq, dp, dwz, n, k, oid, odi, ix->w_npass.as<unsigned long long>()));
+        TRY(run_path(ix, s, o, dq, dp, dwz, ix->D, n, k, oid, odi, ix->w_npass.as<unsigned long long>()));
         if (!o.dio) {
             TRY(copy_out(s, false, ids + q0 * k, oid, sizeof(int64_t) * n * k));
             TRY(copy_out(s, false, dists + q0 * k, odi, sizeof(float) * n * k));
@@ -1122,8 +1145,7 @@ int ifvs_filter(ifvs_index* ix, const ifvs_predicate* preds, int64_t nq, const i
         CUDA_TRY(cudaMemsetAsync(ix->w_npass.p, 0, sizeof(unsigned long long) * n, s));
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_PREDICATE);
-            CUDA_TRY(st.end(launch_canonicalize(dp, n, ix->cols(), ix->w_canon.as<CanonPred>(),
-                                                ix->w_err.as<int>(), s)));
+            CUDA_TRY(st.end(launch_prepare(prepare_args(ix, dp, ix->w_canon.as<CanonPred>()), n, s)));
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_FILTER);
@@ -1159,7 +1181,6 @@ int ifvs_condition(ifvs_index* ix, const float* queries, const ifvs_predicate* p
     const int Mr = ix->M * ix->r;
     const int64_t sb = nq < 1024 ? nq : 1024;
     TRY(reset_err_flag(ix, s));
-    TRY(ensure(ix->w_canon, sizeof(CanonPred) * sb));
     TRY(ensure(ix->w_idx, sizeof(uint32_t) * sb * (ix->h > 0 ? ix->h : 1)));
     TRY(ensure(ix->w_alpha, sizeof(float) * sb * (Mr > 0 ? Mr : 1)));
     TRY(ensure(ix->w_wf, sizeof(float) * sb * ix->D));
@@ -1170,21 +1191,15 @@ int ifvs_condition(ifvs_index* ix, const float* queries, const ifvs_predicate* p
         const float *dq, *dwz;
         const ifvs_predicate* dp;
         TRY(stage_inputs(ix, s, o, q0, n, queries, preds, wz, &dq, &dp, &dwz));
-        {
-            Stage st(ix, s, o.timing, IFVS_STAGE_PREDICATE);
-            CUDA_TRY(st.end(launch_canonicalize(dp, n, ix->cols(), ix->w_canon.as<CanonPred>(),
-                                                ix->w_err.as<int>(), s)));
-        }
         if (!cond) {
             CUDA_TRY(cudaMemsetAsync(ix->w_idx.p, 0, sizeof(uint32_t) * n * (ix->h > 0 ? ix->h : 1), s));
             CUDA_TRY(cudaMemsetAsync(ix->w_alpha.p, 0, sizeof(float) * n * (Mr > 0 ? Mr : 1), s));
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_CONDITION);
-            CUDA_TRY(st.end(launch_condition(dq, dp, n, ix->D, ix->d_seeds, ix->h, ix->B,
-                                             cond ? ix->d_bank : nullptr, Mr, dwz,
-                                             ix->w_idx.as<uint32_t>(), ix->w_alpha.as<float>(),
-                                             ix->w_wf.as<float>(), s)));
+            PrepareArgs pa = prepare_args(ix, dp, nullptr);
+            prepare_condition(ix, dq, dwz, ix->D, cond, &pa);
+            CUDA_TRY(st.end(launch_prepare(pa, n, s)));
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_LUT);
@@ -1530,9 +1545,9 @@ int ifvs_train_grad(ifvs_index* ix, const float* queries, const ifvs_predicate* 
     }
     {
         Stage st(ix, s, o.timing, IFVS_STAGE_CONDITION);
-        CUDA_TRY(st.end(launch_condition(dq, dp, nq, ix->D, ix->d_seeds, ix->h, ix->B, ix->d_bank,
-                                         (int)Mr, ix->w_wz.as<float>(), ix->w_idx.as<uint32_t>(),
-                                         ix->w_alpha.as<float>(), ix->w_wf.as<float>(), s)));
+        PrepareArgs pa = prepare_args(ix, dp, nullptr);
+        prepare_condition(ix, dq, ix->t_wz.as<float>(), 0, true, &pa);
+        CUDA_TRY(st.end(launch_prepare(pa, nq, s)));
     }
     TrainQueryArgs a = train_args(ix, tp, nq, dq);
     a.pos = dcand;
@@ -1586,7 +1601,7 @@ int ifvs_train_step(ifvs_index* ix, const float* queries, const ifvs_predicate* 
     mo.R = 0;
     mo.sub_batch = 0;
     mo.chunk_blocks = 0;
-    TRY(run_path(ix, s, mo, dq, dp, ix->w_wz.as<float>(), nq, kk, ix->t_mined.as<int64_t>(),
+    TRY(run_path(ix, s, mo, dq, dp, ix->t_wz.as<float>(), 0, nq, kk, ix->t_mined.as<int64_t>(),
                  ix->t_mdist.as<float>(), ix->w_npass.as<unsigned long long>()));
     TRY(ensure(ix->t_neg, sizeof(int64_t) * nq * (tp->n_neg > 0 ? tp->n_neg : 1)));
     TrainQueryArgs a = train_args(ix, tp, nq, dq);

@@ -1,11 +1,11 @@
 // Conditioning and table build of §2.
 //
-// k_condition (one CTA per query): the pair <q, f> is fingerprinted by h
-// hash functions into the memory bank (FNV-1a-64 of the key bytes, then the
-// SplitMix64 finalizer of base XOR seed_i, mod B — the paper names no hash
-// function), alpha = sum of the h fetched bank rows, and the filter weights
-// w_f = softplus(w_z) (w_f = 1 when no w_z is given: the paper's initial
-// state).
+// k_prepare (one CTA per query): the predicate's canonical form and scan plan;
+// the pair <q, f> is fingerprinted by h hash functions into the memory bank
+// (FNV-1a-64 of the key bytes, then the SplitMix64 finalizer of base XOR
+// seed_i, mod B — the paper names no hash function), alpha = sum of the h
+// fetched bank rows, and the filter weights w_f = softplus(w_z) (w_f = 1 when
+// no w_z is given: the paper's initial state).
 //
 // k_lut (grid: subspace m x query group; thread = codeword k): the
 // adjustment Delta[m][k][:] = sum_j alpha[m][j] W[m][j][k][:] is formed with
@@ -18,14 +18,23 @@
 
 namespace ifvs {
 
-__device__ __forceinline__ uint64_t fnv_byte(uint64_t h, uint32_t byte) {
-    return (h ^ (uint64_t)byte) * 1099511628211ull;
-}
+// ---- fingerprint ----------------------------------------------------------
+//
+// FNV-1a-64 (h <- (h xor byte) P for every byte) by one warp instead of one
+// thread, whose chain of 64-bit multiplications took 11 us for a 532-byte key
+// and 86 us for a 3868-byte one.  Three facts make it parallel:
+//  * The low byte evolves by itself: l <- ((l xor b) 0xb3) mod 256, and bit j
+//    of the product is bit j of x = l xor b (0xb3 is odd) xor a carry c_j of
+//    the lower bits of x.  So bit j of every l in a run of bytes is a prefix
+//    xor of (b_j xor c_j), once the bits below j are known: eight rounds of
+//    bitwise work on 32 bytes per lane, a ballot each.
+//  * 0xb3 x = s + 16 s + 128 x with s = 3 x: two ripple carries.
+//  * From a start value whose low byte is known the run is affine in the rest:
+//    F(h) = F(l) + (h - l) P^len; every lane hashes its 32 bytes from its l and
+//    five combinations join the lanes.
 
-__device__ __forceinline__ uint64_t fnv_word(uint64_t h, uint64_t v, int nbytes) {
-    for (int b = 0; b < nbytes; ++b) h = fnv_byte(h, (uint32_t)(v >> (8 * b)) & 0xFFu);
-    return h;
-}
+constexpr uint64_t kFnvPrime = 1099511628211ull;
+constexpr uint64_t kFnvBasis = 14695981039346656037ull;
 
 __device__ __forceinline__ uint64_t splitmix64_finalizer(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
@@ -33,57 +42,248 @@ __device__ __forceinline__ uint64_t splitmix64_finalizer(uint64_t z) {
     return z ^ (z >> 31);
 }
 
+// bit 8 i + j <-> bit 8 j + i: the 8 x 8 bit matrix of 8 bytes, transposed
+__device__ __forceinline__ uint64_t transpose8(uint64_t x) {
+    uint64_t t = (x ^ (x >> 7)) & 0x00AA00AA00AA00AAull;
+    x ^= t ^ (t << 7);
+    t = (x ^ (x >> 14)) & 0x0000CCCC0000CCCCull;
+    x ^= t ^ (t << 14);
+    t = (x ^ (x >> 28)) & 0x00000000F0F0F0F0ull;
+    return x ^ t ^ (t << 28);
+}
+
+__device__ __forceinline__ uint32_t majority(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (c & (a | b)); }
+
+// h after the key's words [first, first + 256), word(i) giving word i (words
+// before 0 are absent: the run is right-aligned); every lane takes 8 words
+template <class Word>
+__device__ __forceinline__ uint64_t fnv_run(uint64_t h, int first, const Word& word, int lane) {
+    uint32_t w[8];
+    uint32_t mask = 0u;    // bytes present
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int at = first + lane * 8 + i;
+        w[i] = at >= 0 ? word(at) : 0u;
+        mask |= at >= 0 ? 0xFu << (4 * i) : 0u;
+    }
+    uint32_t b[8];         // bit i of b[j]: bit j of byte i
+    {
+        uint32_t lo[4], hi[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const uint64_t t = transpose8((uint64_t)w[2 * g + 1] << 32 | w[2 * g]);
+            lo[g] = (uint32_t)t;
+            hi[g] = (uint32_t)(t >> 32);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t sel = (uint32_t)(j | (j + 4) << 4);
+            b[j] = __byte_perm(__byte_perm(lo[0], lo[1], sel), __byte_perm(lo[2], lo[3], sel), 0x5410);
+            b[j + 4] = __byte_perm(__byte_perm(hi[0], hi[1], sel), __byte_perm(hi[2], hi[3], sel), 0x5410);
+        }
+    }
+    uint32_t x[8], s[8], k1 = 0u, k2 = 0u, start = 0u;
+    const uint32_t before = (1u << lane) - 1u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const uint32_t below = j > 0 ? x[j - 1] : 0u;
+        uint32_t c = below ^ k1 ^ k2;
+        if (j >= 4) c ^= s[j - 4];
+        if (j == 7) c ^= x[0];
+        uint32_t t = (b[j] ^ c) & mask;
+        t ^= t << 1;
+        t ^= t << 2;
+        t ^= t << 4;
+        t ^= t << 8;
+        t ^= t << 16;
+        const unsigned odd = __ballot_sync(0xFFFFFFFFu, (t >> 31) != 0u);
+        const uint32_t flip = (uint32_t)(__popc(odd & before) & 1) ^ (uint32_t)(h >> j & 1u);
+        const uint32_t l = (t << 1) ^ (0u - flip);
+        start |= (l & 1u) << j;
+        x[j] = l ^ b[j];
+        s[j] = x[j] ^ below ^ k1;
+        k1 = majority(x[j], below, k1);
+        if (j >= 4) k2 = majority(s[j], s[j - 4], k2);
+    }
+    uint64_t r = start, A = 1ull;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (first + lane * 8 + i >= 0) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) r = (r ^ (uint64_t)(w[i] >> (8 * e) & 0xFFu)) * kFnvPrime;
+            A *= kFnvPrime * kFnvPrime * kFnvPrime * kFnvPrime;
+        }
+    uint64_t C = r - start * A;     // h -> A h + C
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t A2 = __shfl_down_sync(0xFFFFFFFFu, A, o), C2 = __shfl_down_sync(0xFFFFFFFFu, C, o);
+        C = A2 * C + C2;            // lanes that are multiples of 2 o hold their group's map
+        A *= A2;
+    }
+    return __shfl_sync(0xFFFFFFFFu, A * h + C, 0);
+}
+
 __device__ __forceinline__ float softplus_f32(float x) {
     // log(1 + e^x) without overflow on either side
     return x > 0.f ? x + log1pf(expf(-x)) : log1pf(expf(x));
 }
 
-__global__ void k_condition(const float* __restrict__ q, const ifvs_predicate* __restrict__ preds,
-                            int64_t nq, int D, const uint64_t* __restrict__ seeds, int h,
-                            int64_t B, const float* __restrict__ bank, int Mr,
-                            const float* __restrict__ wz, uint32_t* __restrict__ idx_out,
-                            float* __restrict__ alpha, float* __restrict__ wf) {
-    const int64_t qi = blockIdx.x;
-    __shared__ uint32_t s_idx[64];
-    const float* qv = q + qi * D;
-    if (bank != nullptr) {
-        if (threadIdx.x == 0) {
-            uint64_t hsh = 14695981039346656037ull;
-            for (int d = 0; d < D; ++d) hsh = fnv_word(hsh, __float_as_uint(qv[d]), 4);
-            const ifvs_predicate& p = preds[qi];
-            int nc = p.n_clauses;
-            hsh = fnv_word(hsh, (uint32_t)nc, 4);
-            if (nc < 0) nc = 0;
-            if (nc > IFVS_MAX_CLAUSES) nc = IFVS_MAX_CLAUSES;
-            for (int i = 0; i < nc; ++i) {
-                hsh = fnv_word(hsh, (uint32_t)p.c[i].col, 4);
-                hsh = fnv_word(hsh, (uint32_t)p.c[i].op, 4);
-                hsh = fnv_word(hsh, (uint64_t)p.c[i].lo, 8);
-                hsh = fnv_word(hsh, (uint64_t)p.c[i].hi, 8);
-            }
-            for (int i = 0; i < h; ++i)
-                s_idx[i] = (uint32_t)(splitmix64_finalizer(hsh ^ seeds[i]) % (uint64_t)B);
-        }
-        __syncthreads();
-        if (idx_out != nullptr)
-            for (int i = threadIdx.x; i < h; i += blockDim.x) idx_out[qi * h + i] = s_idx[i];
-        for (int t = threadIdx.x; t < Mr; t += blockDim.x) {
-            float a = 0.f;
-            for (int i = 0; i < h; ++i) a += bank[(int64_t)s_idx[i] * Mr + t];
-            alpha[qi * Mr + t] = a;
-        }
+// ---- scan plan --------------------------------------------------------------
+//
+// A predicate that constrains one column selects, for that column's canonical
+// interval [lo, lo + wm1], a contiguous segment of the rows sorted by (value,
+// row): two searches give it, and its length is the exact pool size.  On an
+// index with composite copies a predicate that fixes one of the two columns
+// and bounds the other does the same.  Pools up to max_rows take the
+// row-list scan (no filter pass, no bitmap); empty and malformed predicates
+// take it with an empty segment, and a predicate that constrains no column
+// (every row passes) takes it with all N positions of column 0's copy; every
+// other query takes the bitmap path.
+
+// first index in [0, n] whose value is not below x; the warp probes 32 places
+// a round (5 rounds at 10^7 values, against 24 dependent loads of a thread)
+template <class T>
+__device__ __forceinline__ int64_t first_not_below(const T* __restrict__ v, int64_t n, T x, int lane) {
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int64_t step = (hi - lo) <= 32 ? 1 : (hi - lo) / 33 + 1;
+        const int64_t at = lo + (lane + 1) * step - 1;
+        const bool below = at < hi && __ldg(v + at) < x;
+        const int64_t cnt = __popc(__ballot_sync(0xFFFFFFFFu, below));
+        const int64_t top = lo + (cnt + 1) * step - 1;   // probe cnt, if there is one, is not below
+        lo += cnt * step;
+        if (step == 1) break;
+        hi = top < hi ? top : hi;
     }
-    for (int d = threadIdx.x; d < D; d += blockDim.x)
-        wf[qi * D + d] = wz != nullptr ? softplus_f32(wz[qi * D + d]) : 1.0f;
+    return lo;
 }
 
-cudaError_t launch_condition(const float* q, const ifvs_predicate* preds, int64_t nq, int D,
-                             const uint64_t* seeds, int h, int64_t B, const float* bank, int Mr,
-                             const float* wz, uint32_t* idx, float* alpha, float* wf,
-                             cudaStream_t s) {
+// Where a predicate's segment starts (end = 0) or ends (end = 1): the copy and
+// the value (or composite key) to search for; false: no search is needed
+// (*edge is the answer) or there is no segment (*copy < 0).
+__device__ __forceinline__ bool segment_bound(const CanonPred& cp, const SortedCols& sc, int64_t N, int end, int* copy,
+                                              int64_t* value, uint64_t* key, int64_t* edge) {
+    *copy = -1;
+    *edge = 0;
+    if (cp.empty) {
+        *copy = 0;
+        return false;
+    }
+    if (cp.used == 0u) {
+        if (sc.n > 0 && sc.vals_of(0) != nullptr) *copy = 0;
+        *edge = end ? N : 0;
+        return false;
+    }
+    if (__popc(cp.used) == 1) {
+        const int c = __ffs(cp.used) - 1;
+        if (c >= sc.n || sc.vals_of(c) == nullptr) return false;
+        int64_t lo = 0, wm1 = 0;
+#pragma unroll
+        for (int i = 0; i < IFVS_MAX_ATTRS; ++i)
+            if (c == i) {
+                lo = cp.lo[i];
+                wm1 = cp.wm1[i];
+            }
+        *copy = c;
+        *value = end ? lo + wm1 + 1 : lo;
+        *edge = N;
+        return *value <= 2147483647ll;     // above every value: N
+    }
+    if (cp.used == 3u && sc.ckeys[0] != nullptr && (cp.wm1[0] == 0u || cp.wm1[1] == 0u)) {
+        // columns 0 and 1, one of them fixed to a value: a position range of
+        // the composite copy keyed by that column first
+        const int j = cp.wm1[0] == 0u ? 0 : 1;
+        const int32_t v = cp.lo[j], lo2 = cp.lo[1 - j];
+        *copy = kComposite + j;
+        // one past (v, lo2 + w2) is the next composite key (it carries into
+        // the primary half when the secondary value is the largest int32)
+        const uint64_t k = ckey(v, (int32_t)((uint32_t)lo2 + (end ? cp.wm1[1 - j] : 0u)));
+        *key = k + (end ? 1ull : 0ull);
+        *edge = N;
+        return !(end && k == ~0ull);
+    }
+    return false;
+}
+
+// Everything about a query that comes before its tables, one CTA each: the
+// predicate's canonical form, its scan plan (warps 0 and 1 search the two ends
+// of the segment), the fingerprint of <q, f> (warp 2) and from it alpha, and
+// the filter weights.  One launch for what took three and a memset, 28 us for
+// one query on 10^6 rows and 40 us on 10^7.
+constexpr int kPrepThreads = 128;
+
+__global__ void __launch_bounds__(kPrepThreads) k_prepare(PrepareArgs a) {
+    const int64_t qi = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ uint32_t s_idx[64];
+    __shared__ int64_t s_end[2];
+    __shared__ CanonPred s_cp;
+    if (tid == 0) {
+        const ifvs_predicate p = a.preds[qi];
+        CanonPred cp;
+        if (canonicalize(p, a.cols.type, a.cols.n, &cp) != 0) atomicOr(a.err, 1);
+        if (a.canon != nullptr) a.canon[qi] = cp;
+        s_cp = cp;
+    }
+    if (a.plan != nullptr) __syncthreads();
+    if (a.plan != nullptr && warp < 2) {
+        int copy = -1;
+        int64_t value = 0, at = 0;
+        uint64_t key = 0ull;
+        if (segment_bound(s_cp, a.sorted, a.N, warp, &copy, &value, &key, &at))
+            at = copy >= kComposite ? first_not_below<uint64_t>(a.sorted.ckeys_of(copy - kComposite), a.N, key, lane)
+                                    : first_not_below<int32_t>(a.sorted.vals_of(copy), a.N, (int32_t)value, lane);
+        if (lane == 0) s_end[warp] = at;
+    }
+    if (a.bank != nullptr && warp == 2) {
+        const uint32_t* qw = reinterpret_cast<const uint32_t*>(a.q + qi * a.D);
+        const uint32_t* pw = reinterpret_cast<const uint32_t*>(a.preds + qi);
+        int nc = (int)pw[0];
+        nc = nc < 0 ? 0 : (nc > IFVS_MAX_CLAUSES ? IFVS_MAX_CLAUSES : nc);
+        // the key: q, n_clauses, then each clause's col, op, lo, hi (24 bytes)
+        const int D = a.D, nw = D + 1 + 6 * nc;
+        auto word = [&](int i) { return __ldg(i < D ? qw + i : (i == D ? pw : pw + (i - D + 1))); };
+        uint64_t h = kFnvBasis;
+        for (int first = nw - (nw + 255) / 256 * 256; first < nw; first += 256) h = fnv_run(h, first, word, lane);
+        for (int i = lane; i < a.h; i += 32)
+            s_idx[i] = (uint32_t)(splitmix64_finalizer(h ^ a.seeds[i]) % (uint64_t)a.B);
+    }
+    if (a.wf != nullptr)
+        for (int d = tid; d < a.D; d += kPrepThreads)
+            a.wf[qi * a.D + d] = a.wz != nullptr ? softplus_f32(a.wz[qi * a.wz_stride + d]) : 1.0f;
+    __syncthreads();
+    if (a.plan != nullptr && tid == 0) {
+        ScanPlan p;
+        p.a = p.b = 0;
+        p.col = p.list = 0;
+        int copy;
+        int64_t value, at;
+        uint64_t key;
+        segment_bound(s_cp, a.sorted, a.N, 0, &copy, &value, &key, &at);
+        const int64_t len = s_end[1] - s_end[0];
+        if (copy >= 0 && len <= a.max_rows) {
+            p.a = s_end[0];
+            p.b = s_end[1];
+            p.col = copy;
+            p.list = 1;
+        }
+        a.plan[qi] = p;
+        a.npass[qi] = p.list ? (unsigned long long)len : 0ull;   // the filter adds to the others
+    }
+    if (a.bank != nullptr) {
+        if (a.idx != nullptr)
+            for (int i = tid; i < a.h; i += kPrepThreads) a.idx[qi * a.h + i] = s_idx[i];
+        for (int t = tid; t < a.Mr; t += kPrepThreads) {
+            float s = 0.f;
+            for (int i = 0; i < a.h; ++i) s += a.bank[(int64_t)s_idx[i] * a.Mr + t];
+            a.alpha[qi * a.Mr + t] = s;
+        }
+    }
+}
+
+cudaError_t launch_prepare(const PrepareArgs& a, int64_t nq, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
-    k_condition<<<(unsigned)nq, 128, 0, s>>>(q, preds, nq, D, seeds, h, B, bank, Mr, wz, idx,
-                                             alpha, wf);
+    k_prepare<<<(unsigned)nq, kPrepThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -13,127 +13,6 @@
 
 namespace ifvs {
 
-__global__ void k_canonicalize(const ifvs_predicate* __restrict__ preds, int64_t nq,
-                               AttrCols cols, CanonPred* __restrict__ out, int* __restrict__ err) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nq) return;
-    ifvs_predicate p = preds[i];
-    CanonPred c;
-    if (canonicalize(p, cols.type, cols.n, &c) != 0) atomicOr(err, 1);
-    out[i] = c;
-}
-
-cudaError_t launch_canonicalize(const ifvs_predicate* preds, int64_t nq, AttrCols cols,
-                                CanonPred* out, int* err, cudaStream_t s) {
-    if (nq <= 0) return cudaSuccess;
-    int threads = 128;
-    int64_t blocks = (nq + threads - 1) / threads;
-    k_canonicalize<<<(unsigned)blocks, threads, 0, s>>>(preds, nq, cols, out, err);
-    return cudaGetLastError();
-}
-
-// Scan plan.  A predicate that constrains one column selects, for that
-// column's canonical interval [lo, lo + wm1], a contiguous segment of the
-// rows sorted by (value, row): two binary searches give it, and its length
-// is the exact pool size.  Pools up to max_rows take the row-list scan (no
-// filter pass, no bitmap); empty and malformed predicates take it with an
-// empty segment, and a predicate that constrains no column (every row
-// passes) takes it with all N positions of column 0's copy; every other
-// query takes the bitmap path.
-__device__ __forceinline__ int64_t first_not_below(const int32_t* __restrict__ v, int64_t n, int64_t x) {
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((int64_t)v[mid] < x)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ int64_t first_key_not_below(const uint64_t* __restrict__ v, int64_t n, uint64_t x) {
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (v[mid] < x)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-__global__ void k_plan(const CanonPred* __restrict__ canon, int64_t nq, SortedCols sc, int64_t N,
-                       int64_t max_rows, ScanPlan* __restrict__ plan,
-                       unsigned long long* __restrict__ npass) {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nq) return;
-    const CanonPred cp = canon[q];
-    ScanPlan p;
-    p.a = 0;
-    p.b = 0;
-    p.col = 0;
-    p.list = 0;
-    if (cp.empty) {
-        p.list = 1;
-    } else if (cp.used == 0u) {
-        if (sc.n > 0 && sc.vals_of(0) != nullptr && N <= max_rows) {
-            p.b = N;
-            p.list = 1;
-        }
-    } else if (__popc(cp.used) == 1) {
-        const int c = __ffs(cp.used) - 1;
-        const int32_t* vals = sc.vals_of(c);
-        if (c < sc.n && vals != nullptr) {
-            int64_t lo = 0, wm1 = 0;
-#pragma unroll
-            for (int i = 0; i < IFVS_MAX_ATTRS; ++i)
-                if (c == i) {
-                    lo = cp.lo[i];
-                    wm1 = cp.wm1[i];
-                }
-            const int64_t hi = lo + wm1;
-            const int64_t a = first_not_below(vals, N, lo);
-            const int64_t b = first_not_below(vals, N, hi + 1);
-            if (b - a <= max_rows) {
-                p.a = a;
-                p.b = b;
-                p.col = c;
-                p.list = 1;
-            }
-        }
-    } else if (cp.used == 3u && sc.ckeys[0] != nullptr && (cp.wm1[0] == 0u || cp.wm1[1] == 0u)) {
-        // columns 0 and 1, one of them fixed to a value: a position range of
-        // the composite copy keyed by that column first
-        const int j = cp.wm1[0] == 0u ? 0 : 1;
-        const int32_t v = cp.lo[j];
-        const int32_t lo2 = cp.lo[1 - j];
-        const uint32_t w2 = cp.wm1[1 - j];
-        const uint64_t* keys = sc.ckeys_of(j);
-        const int64_t a = first_key_not_below(keys, N, ckey(v, lo2));
-        // one past (v, lo2 + w2): the next composite key (carries into the
-        // primary half when the secondary value is the largest int32)
-        const uint64_t kh = ckey(v, (int32_t)((uint32_t)lo2 + w2));
-        const int64_t b = kh == ~0ull ? N : first_key_not_below(keys, N, kh + 1ull);
-        if (b - a <= max_rows) {
-            p.a = a;
-            p.b = b;
-            p.col = kComposite + j;
-            p.list = 1;
-        }
-    }
-    plan[q] = p;
-    if (p.list) npass[q] = (unsigned long long)(p.b - p.a);
-}
-
-cudaError_t launch_plan(const CanonPred* canon, int64_t nq, SortedCols sc, int64_t N, int64_t max_rows,
-                        ScanPlan* plan, unsigned long long* npass, cudaStream_t s) {
-    if (nq <= 0) return cudaSuccess;
-    k_plan<<<(unsigned)((nq + 127) / 128), 128, 0, s>>>(canon, nq, sc, N, max_rows, plan, npass);
-    return cudaGetLastError();
-}
-
 // Fail bits of 8 rows against one interval, shifted into `fail` (row j0 + 7
 // first, so that after four calls bit j is row j).  For each row:
 // off = v - lo (mod 2^32); the carry out of off + ~wm1 is 1 exactly when

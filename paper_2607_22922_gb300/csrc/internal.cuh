@@ -96,10 +96,6 @@ struct AttrCols {
 // ---- kernel launchers (one per translation unit) -----------------------
 // Every launcher returns the cudaError_t of its launch.
 
-// predicates -> canonical intervals; *err |= 1 for any malformed predicate
-cudaError_t launch_canonicalize(const ifvs_predicate* preds, int64_t nq, AttrCols cols,
-                                CanonPred* out, int* err, cudaStream_t s);
-
 // Per-query scan plan: a predicate whose pool is one position range [a, b)
 // of a sorted copy (one constrained column; or, with composite copies, one
 // column fixed to a value and the other bounded) with at most max_rows rows,
@@ -156,9 +152,33 @@ struct SortedCols {
     }
     __host__ __device__ const uint64_t* ckeys_of(int j) const { return j == 0 ? ckeys[0] : ckeys[1]; }
 };
-// plan [nq]; writes npass of the list-path queries
-cudaError_t launch_plan(const CanonPred* canon, int64_t nq, SortedCols sc, int64_t N, int64_t max_rows,
-                        ScanPlan* plan, unsigned long long* npass, cudaStream_t s);
+// What precedes the tables, per query (condition.cu).  Parts whose outputs
+// are null are left out.
+struct PrepareArgs {
+    const ifvs_predicate* preds;
+    AttrCols cols;
+    CanonPred* canon;              // canonical predicates, or null (checked all the same)
+    int* err;                      // |= 1 for any malformed predicate
+    // scan plan
+    SortedCols sorted;
+    int64_t N, max_rows;
+    ScanPlan* plan;                // or null
+    unsigned long long* npass;     // with plan: pool sizes of list-path queries, 0 for the others
+    // fingerprint, alpha (when bank is not null), w_f (when wf is not null)
+    const float* q;                // [nq][D]
+    int D;
+    const uint64_t* seeds;
+    int h;
+    int64_t B;
+    const float* bank;             // [B][Mr]
+    int Mr;
+    const float* wz;               // w_z of query i at wz + i * wz_stride; null: w_f = 1
+    int64_t wz_stride;
+    uint32_t* idx;                 // [nq][h], or null
+    float* alpha;                  // [nq][Mr]
+    float* wf;                     // [nq][D]
+};
+cudaError_t launch_prepare(const PrepareArgs& a, int64_t nq, cudaStream_t s);
 
 // Filter: lane-major pass bitmaps [nq][n_blocks * 32] + popcounts (added to
 // npass) for the bitmap-path queries of `plan` (all queries when plan is null)
@@ -171,12 +191,6 @@ cudaError_t launch_filter(AttrCols cols, int64_t N, int64_t n_blocks, const Cano
 cudaError_t launch_bitmap_layout(const uint32_t* src, uint32_t* dst, int64_t nq,
                                  int64_t n_blocks, int64_t n_words_rows, bool to_rows,
                                  cudaStream_t s);
-
-// fingerprint + alpha (when bank != nullptr) and w_f
-cudaError_t launch_condition(const float* q, const ifvs_predicate* preds, int64_t nq, int D,
-                             const uint64_t* seeds, int h, int64_t B, const float* bank, int Mr,
-                             const float* wz, uint32_t* idx, float* alpha, float* wf,
-                             cudaStream_t s);
 
 // Delta, C_iFVS (optional output) and the weighted ADC tables
 cudaError_t launch_lut(const float* cpq, const float* W, const float* alpha, const float* q,
@@ -322,7 +336,6 @@ cudaError_t launch_train_bank(const uint32_t* idx, int64_t n, int h, int Mr, con
                               float inv_n, float* gbank, cudaStream_t s);
 cudaError_t launch_train_wz(const float* gw, int64_t n, int D, const float* wz, float inv_n, float* gwz,
                             cudaStream_t s);
-cudaError_t launch_broadcast_wz(const float* wz, int D, int64_t n, float* out, cudaStream_t s);
 cudaError_t launch_sgd(float* theta, const float* g, int64_t n, float lr, cudaStream_t s);
 
 // Read-only view of a loaded index, for entry points defined outside api.cu.

@@ -36,11 +36,6 @@ __device__ __forceinline__ double warp_min(double v) {
 }
 }  // namespace
 
-__global__ void k_broadcast_wz(const float* __restrict__ wz, int D, int64_t n, float* __restrict__ out) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n * D) out[e] = wz[e % D];
-}
-
 // G[m][j][j'] = sum over (k, t) of W[m][j][k][t] W[m][j'][k][t]; one CTA per entry
 __global__ void __launch_bounds__(kTrainThreads) k_train_gram(const float* __restrict__ W, int M,
                                                               int r, int KD, float* __restrict__ G) {
@@ -454,12 +449,6 @@ cudaError_t launch_train_bank(const uint32_t* idx, int64_t n, int h, int Mr, con
 cudaError_t launch_train_wz(const float* gw, int64_t n, int D, const float* wz, float inv_n, float* gwz,
                             cudaStream_t s) {
     k_train_wz<<<(unsigned)((D + 31) / 32), dim3(32, 32), 0, s>>>(gw, n, D, wz, inv_n, gwz);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_broadcast_wz(const float* wz, int D, int64_t n, float* out, cudaStream_t s) {
-    const int64_t total = n * D;
-    k_broadcast_wz<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(wz, D, n, out);
     return cudaGetLastError();
 }
 
