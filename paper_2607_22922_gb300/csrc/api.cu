@@ -533,7 +533,6 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     TRY(ensure(ix->w_idx, sizeof(uint32_t) * n * (ix->h > 0 ? ix->h : 1)));
     TRY(ensure(ix->w_alpha, sizeof(float) * n * (Mr > 0 ? Mr : 1)));
     TRY(ensure(ix->w_wf, sizeof(float) * n * ix->D));
-    TRY(ensure(ix->w_lut, sizeof(float) * n * ix->M * ix->K));
     TRY(ensure(ix->w_tab, sizeof(float) * n * 256 * ix->tab_words));
     const ScanShape sh = scan_shape(ix, n, kk, o.chunk_blocks);
     TRY(ensure(ix->w_part, sizeof(uint64_t) * n * sh.n_chunks * kk));
@@ -575,13 +574,18 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
         CUDA_TRY(st.end(launch_filter(ix->cols(), ix->N, ix->n_blocks, ix->w_canon.as<CanonPred>(),
                                       plan, n, ix->w_bm.as<uint32_t>(), npass_u64, ix->num_sms, s)));
     }
-    {
-        Stage st(ix, s, o.timing, IFVS_STAGE_LUT);
-        CUDA_TRY(st.end(launch_lut(ix->d_cpq, ix->d_W, cond ? ix->w_alpha.as<float>() : nullptr,
-                                   dq, ix->w_wf.as<float>(), n, ix->M, ix->K, ix->ds, ix->r,
-                                   ix->w_lut.as<float>(), nullptr, ix->num_sms, s)));
-    }
-    {
+    const float* alpha = cond ? ix->w_alpha.as<float>() : nullptr;
+    if (!o.timing && cond_tables_fit(ix->ds, ix->r, cond)) {
+        Stage st(ix, s, false, IFVS_STAGE_LUT);
+        CUDA_TRY(st.end(launch_cond_tables(ix->d_cpq, ix->d_W, alpha, dq, ix->w_wf.as<float>(), n, ix->M, ix->K,
+                                           ix->ds, ix->tab_words, ix->w_tab.as<float>(), ix->num_sms, s)));
+    } else {
+        TRY(ensure(ix->w_lut, sizeof(float) * n * ix->M * ix->K));
+        {
+            Stage st(ix, s, o.timing, IFVS_STAGE_LUT);
+            CUDA_TRY(st.end(launch_lut(ix->d_cpq, ix->d_W, alpha, dq, ix->w_wf.as<float>(), n, ix->M, ix->K, ix->ds,
+                                       ix->r, ix->w_lut.as<float>(), nullptr, ix->num_sms, s)));
+        }
         Stage st(ix, s, o.timing, IFVS_STAGE_LUT);
         CUDA_TRY(st.end(launch_tables(ix->w_lut.as<float>(), n, ix->M, ix->K, ix->tab_words,
                                       ix->w_tab.as<float>(), s)));

@@ -399,6 +399,164 @@ cudaError_t launch_lut(const float* cpq, const float* W, const float* alpha, con
     return cudaGetLastError();
 }
 
+// ---- tables in the scan's layout, straight from the conditioning ---------------
+//
+// For ds = 4, 8, 16 and r = 8 (or no bank) a query's weighted tables are
+// formed and written in the scan's layout (below) by one kernel, without the
+// [M][K] table in between.  CTA (8 subspaces x 32 codewords, query group):
+// warp m, lane c keeps W[m][:][c][:] and C_PQ[m][c] in registers across the
+// group.  alpha, q and w_f of 8 queries at a time arrive in shared memory by
+// asynchronous copies, one stage ahead, and are read as broadcasts: fetched by
+// every lane for itself they filled the L1 data pipe (78 % busy).  The entries
+// pass through shared memory so that 8 lanes write a codeword's 8 words as one
+// sector, to each of their places in row c.  The arithmetic is k_lut_fixed's.
+// Words from M + 31 on are never read and stay unwritten.  1024 queries at
+// M = 16 took 95 us as two kernels, 28 us here; 256 queries at M = 120 145 us,
+// 59 us here.
+constexpr int kTabM = 8, kTabC = 32, kTabQ = 8;
+constexpr int kTabThreads = kTabM * kTabC;
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+template <int DS, bool COND>
+__global__ void __launch_bounds__(kTabThreads, DS > 8 ? 1 : 2)
+k_cond_tables(const float* __restrict__ cpq, const float* __restrict__ W, const float* __restrict__ alpha,
+              const float* __restrict__ q, const float* __restrict__ wf, int64_t nq, int M, int K, int S,
+              int q_per_cta, int vec, float* __restrict__ tab) {
+    constexpr int R = 8, NX = kTabM * DS, NA = kTabM * R, NP = NA + 2 * NX;   // floats per query of a stage
+    __shared__ __align__(16) float par[2][kTabQ][NP];                         // alpha, q, w_f
+    __shared__ float st[kTabQ][kTabC * (kTabM + 1)];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m0 = (int)(blockIdx.x / (256 / kTabC)) * kTabM, c0 = (int)(blockIdx.x % (256 / kTabC)) * kTabC;
+    const int D = M * DS, mg = min(kTabM, M - m0);
+    const int64_t q0 = (int64_t)blockIdx.y * q_per_cta;
+    const int64_t q1 = min(nq, q0 + (int64_t)q_per_cta);
+    auto stage = [&](int64_t s0, int b) {   // queries [s0, s0 + kTabQ)
+        const int ns = (int)min((int64_t)kTabQ, q1 - s0);
+        if (COND)
+            for (int e = tid; e < ns * (NA / 4); e += kTabThreads) {
+                const int i = e / (NA / 4), o = (e - i * (NA / 4)) * 4;
+                if (o < mg * R) cp_async16(&par[b][i][o], alpha + ((s0 + i) * M + m0) * R + o);
+            }
+        for (int e = tid; e < ns * (NX / 4); e += kTabThreads) {
+            const int i = e / (NX / 4), o = (e - i * (NX / 4)) * 4;
+            if (o >= mg * DS) continue;
+            const int64_t at = (s0 + i) * D + m0 * DS + o;
+            cp_async16(&par[b][i][NA + NX + o], wf + at);
+            if (vec)
+                cp_async16(&par[b][i][NA + o], q + at);
+            else
+#pragma unroll
+                for (int u = 0; u < 4; ++u) cp_async4(&par[b][i][NA + o + u], q + at + u);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(q0, 0);
+    const int m = m0 + warp, c = c0 + lane;
+    const bool real = m < M && c < K;
+    float base[DS], w[R][DS];
+#pragma unroll
+    for (int t = 0; t < DS; ++t) base[t] = real ? __ldg(cpq + ((int64_t)m * K + c) * DS + t) : 0.f;
+    if (COND) {
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+#pragma unroll
+            for (int t = 0; t < DS; t += 4) {
+                const float4 v =
+                    real ? __ldg(reinterpret_cast<const float4*>(W + (((int64_t)m * R + j) * K + c) * DS + t))
+                         : make_float4(0.f, 0.f, 0.f, 0.f);
+                w[j][t] = v.x, w[j][t + 1] = v.y, w[j][t + 2] = v.z, w[j][t + 3] = v.w;
+            }
+    }
+    // where this thread writes: codeword wc, subspace wm
+    const int wc = tid / kTabM, wm = tid % kTabM;
+    float* out = tab + (q0 * 256 + c0 + wc) * (int64_t)S;
+    int b = 0;
+#pragma unroll 1
+    for (int64_t s0 = q0; s0 < q1; s0 += kTabQ, b ^= 1) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();   // the stage is here, the other buffer and the entries are read
+        if (s0 + kTabQ < q1) stage(s0 + kTabQ, b ^ 1);
+        const int ns = (int)min((int64_t)kTabQ, q1 - s0);
+#pragma unroll 1
+        for (int i = 0; i < ns; ++i) {
+            const float4* pa = reinterpret_cast<const float4*>(&par[b][i][warp * R]);
+            const float4* px = reinterpret_cast<const float4*>(&par[b][i][NA + warp * DS]);
+            const float4* pf = reinterpret_cast<const float4*>(&par[b][i][NA + NX + warp * DS]);
+            float a[R];
+            if (COND) {
+                const float4 v0 = pa[0], v1 = pa[1];
+                a[0] = v0.x, a[1] = v0.y, a[2] = v0.z, a[3] = v0.w;
+                a[4] = v1.x, a[5] = v1.y, a[6] = v1.z, a[7] = v1.w;
+            }
+            float s = 0.f;
+#pragma unroll
+            for (int t = 0; t < DS; t += 4) {
+                const float4 x4 = px[t / 4], f4 = pf[t / 4];
+                const float x[4] = {x4.x, x4.y, x4.z, x4.w}, f[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    float cv = base[t + u];
+                    if (COND) {
+                        float delta = 0.f;
+#pragma unroll
+                        for (int j = 0; j < R; ++j) delta = fmaf(a[j], w[j][t + u], delta);
+                        cv += delta;
+                    }
+                    const float diff = x[u] - cv;
+                    s = fmaf(f[u] * diff, diff, s);
+                }
+            }
+            st[i][lane * (kTabM + 1) + warp] = real ? s : 0.f;
+        }
+        __syncthreads();
+        for (int i = 0; i < ns; ++i, out += (int64_t)256 * S)
+            if (wm < mg) {
+                const float s = st[i][wc * (kTabM + 1) + wm];
+                for (int o = m0 + wm; o < M + 31; o += M) out[o] = s;
+            }
+    }
+}
+
+template <int DS>
+static void start_cond_tables(dim3 grid, const float* cpq, const float* W, const float* alpha, const float* q,
+                              const float* wf, int64_t nq, int M, int K, int S, int qpc, int vec, float* tab,
+                              cudaStream_t s) {
+    if (alpha != nullptr)
+        k_cond_tables<DS, true><<<grid, kTabThreads, 0, s>>>(cpq, W, alpha, q, wf, nq, M, K, S, qpc, vec, tab);
+    else
+        k_cond_tables<DS, false><<<grid, kTabThreads, 0, s>>>(cpq, W, alpha, q, wf, nq, M, K, S, qpc, vec, tab);
+}
+
+bool cond_tables_fit(int ds, int r, bool cond) { return (ds == 4 || ds == 8 || ds == 16) && (!cond || r == 8); }
+
+cudaError_t launch_cond_tables(const float* cpq, const float* W, const float* alpha, const float* q, const float* wf,
+                               int64_t nq, int M, int K, int ds, int S, float* tab, int num_sms, cudaStream_t s) {
+    if (nq <= 0) return cudaSuccess;
+    const int tiles = (M + kTabM - 1) / kTabM * (256 / kTabC);
+    // two CTAs per SM; a group of queries shares a CTA's registers
+    int64_t groups = ((int64_t)num_sms * 2 + tiles - 1) / tiles;
+    if (groups > nq) groups = nq;
+    const int64_t qpc = (nq + groups - 1) / groups;
+    groups = (nq + qpc - 1) / qpc;
+    const dim3 grid((unsigned)tiles, (unsigned)groups);
+    const int vec = (uintptr_t)q % 16 == 0;
+    if (ds == 4)
+        start_cond_tables<4>(grid, cpq, W, alpha, q, wf, nq, M, K, S, (int)qpc, vec, tab, s);
+    else if (ds == 8)
+        start_cond_tables<8>(grid, cpq, W, alpha, q, wf, nq, M, K, S, (int)qpc, vec, tab, s);
+    else
+        start_cond_tables<16>(grid, cpq, W, alpha, q, wf, nq, M, K, S, (int)qpc, vec, tab, s);
+    return cudaGetLastError();
+}
+
 // ---- scan tables -------------------------------------------------------------
 //
 // The scan keeps each query's table in shared memory as 256 rows (one per

@@ -202,6 +202,12 @@ cudaError_t launch_lut(const float* cpq, const float* W, const float* alpha, con
 cudaError_t launch_tables(const float* lut, int64_t nq, int M, int K, int S, float* tab,
                           cudaStream_t s);
 
+// the same layout straight from the conditioning (alpha null: no bank), for
+// the shapes that cond_tables_fit names
+bool cond_tables_fit(int ds, int r, bool cond);
+cudaError_t launch_cond_tables(const float* cpq, const float* W, const float* alpha, const float* q, const float* wf,
+                               int64_t nq, int M, int K, int ds, int S, float* tab, int num_sms, cudaStream_t s);
+
 struct ScanShape {
     int64_t n_blocks;      // bitmap blocks (rows padded to n_blocks * 1024)
     int M, K;

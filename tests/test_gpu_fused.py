@@ -1,0 +1,46 @@
+"""The fused launches of an ordinary search against the same stages as
+launches of their own (a search with stage timing), bit for bit: canonical
+predicates, plan, fingerprint, alpha and w_f in one kernel, and the tables
+straight from the conditioning, at the edges of their tiles."""
+import numpy as np
+import pytest
+
+from paper_2607_22922_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ifvs():
+    from paper_2607_22922_gb300 import build
+    build.build()
+    from paper_2607_22922_gb300 import ifvs as mod
+    return mod
+
+
+@pytest.mark.parametrize("M,K,ds", [(1, 256, 4), (5, 100, 8), (8, 256, 16), (12, 256, 8), (16, 1, 8), (16, 256, 8),
+                                    (16, 255, 4), (24, 256, 16), (33, 16, 4), (120, 256, 8), (128, 100, 4)])
+@pytest.mark.parametrize("cond", [True, False])
+def test_fused_tables_equal_separate_stages(ifvs, M, K, ds, cond):
+    rng = np.random.default_rng(M * K + ds)
+    N, nq = 3001, 70
+    codes = rng.integers(0, K, (N, M), dtype=np.uint8)
+    attr = rng.integers(0, 1000, N, dtype=np.int32)
+    Cpq = rng.standard_normal((M, K, ds)).astype(np.float32)
+    bank = rng.standard_normal((64, M * 8)).astype(np.float32)
+    W = (0.1 * rng.standard_normal((M, 8, K, ds))).astype(np.float32)
+    g = ifvs.Index(codes, [attr], D=M * ds, K=K)
+    g.load_codebooks(Cpq, **(dict(bank=bank, W=W, hash_seeds=np.array([3, 5], np.uint64)) if cond else {}))
+    q = rng.standard_normal((nq, M * ds)).astype(np.float32)
+    wz = rng.standard_normal((nq, M * ds)).astype(np.float32)
+    p = synth.empty_predicates(nq)
+    p["n_clauses"] = 1
+    p["c"][:, 0]["op"] = synth.OP_LT
+    p["c"][:, 0]["lo"] = rng.integers(0, 1100, nq)
+    for n in (1, nq):
+        for w in (None, wz):
+            a = g.search(q[:n], p[:n], 10, wz=None if w is None else w[:n])
+            b = g.search(q[:n], p[:n], 10, wz=None if w is None else w[:n], flags=ifvs.IFVS_F_STAGE_TIMING)
+            for x, y in zip(a, b):
+                np.testing.assert_array_equal(x, y)
+    g.close()
