@@ -123,9 +123,8 @@ typedef struct {
     int32_t sub_batch;  /* queries per filter/scan pass; bounds the bitmap
                            workspace to sub_batch * ceil(N/1024) * 128 bytes.
                            0: automatic (at most 1024).                        */
-    int32_t chunk_blocks; /* rows per scan CTA in units of 1024 (0: automatic);
-                           a tuning knob: CTAs of different queries that walk
-                           the same chunk together share its codes in L2     */
+    int32_t chunk_blocks; /* rows per scan work item in units of 1024 (0:
+                           automatic); a tuning knob                         */
     int32_t list_max_ppm; /* a query whose predicate constrains one column,
                            or, on an index of two columns, fixes one column
                            to a single value and bounds the other, takes the
@@ -156,7 +155,8 @@ enum {
     IFVS_STAGE_SCAN = 4,       /* Rank: code scan + per-CTA top-k             */
     IFVS_STAGE_MERGE = 5,      /* Select: merge of the per-CTA top-k lists    */
     IFVS_STAGE_RERANK = 6,     /* exact fp32 rerank                           */
-    IFVS_STAGE_LAYOUT = 7,     /* bitmap layout conversions                   */
+    IFVS_STAGE_LAYOUT = 7,     /* bitmap layout conversions; work lists of
+                                  batches without pairs                       */
     IFVS_STAGE_TRAIN = 8       /* training: loss, gradient and SGD kernels    */
 };
 
@@ -274,8 +274,8 @@ int ifvs_scan_topk(ifvs_index* ix, const float* lut, const uint32_t* bitmaps, in
  *   stream                    cudaStream_t to enqueue on (NULL: legacy stream)
  * The call only enqueues work on `stream` and returns; results are ready
  * when the stream reaches them.  Its scratch is a file-scope device array of
- * IFVS_STATIC_SCRATCH_BYTES that every GPU running the library holds until
- * the process exits; queries are processed in sub-batches that fit it.
+ * IFVS_STATIC_SCRATCH_BYTES (and 64 KB for the scan's work lists) that every
+ * GPU running the library holds until the process exits; queries are processed in sub-batches that fit it.
  * Sizes beyond it (one query's lane-major bitmap, N / 8 bytes rounded up to
  * 128-byte blocks, plus its 64 KB scan table (160 KB for M > 33) and k keys,
  * above the array) return
@@ -439,7 +439,9 @@ int ifvs_get_conditioning(ifvs_index* ix, float* bank, float* W, uint32_t flags)
 /*
  * ifvs_stage_times — device time (ms, from CUDA events recorded on the
  * launching stream around each launch) and launch counts per stage,
- * accumulated over calls made with IFVS_F_STAGE_TIMING.  Either array may be
+ * accumulated over calls made with IFVS_F_STAGE_TIMING.  Those calls run every
+ * stage as launches of its own; without the flag several stages share a
+ * launch, with the same results.  Either array may be
  * NULL; reset != 0 zeroes the counters after reading.
  */
 int ifvs_stage_times(ifvs_index* ix, double* ms, int64_t* launches, int32_t reset);

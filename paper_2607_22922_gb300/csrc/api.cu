@@ -162,7 +162,7 @@ struct ifvs_index {
     size_t bytes = 0;
     // workspace
     DevBuf w_q, w_wz, w_preds, w_canon, w_err, w_bm, w_rows, w_npass, w_idx, w_alpha, w_wf,
-        w_lut, w_cifvs, w_part, w_ids, w_dists, w_cand, w_cdist, w_tab, w_plan, w_items;
+        w_lut, w_cifvs, w_part, w_ids, w_dists, w_cand, w_cdist, w_tab, w_plan;
     // training workspace
     DevBuf t_cand, t_pos, t_mined, t_mdist, t_gC, t_gw, t_loss, t_G, t_gW, t_gWpart, t_galpha,
         t_gbank, t_gwz, t_wz, t_neg;
@@ -238,7 +238,7 @@ void free_index(ifvs_index* ix) {
     DevBuf* bufs[] = {&ix->w_q, &ix->w_wz, &ix->w_preds, &ix->w_canon, &ix->w_err, &ix->w_bm,
                       &ix->w_rows, &ix->w_npass, &ix->w_idx, &ix->w_alpha, &ix->w_wf,
                       &ix->w_lut, &ix->w_cifvs, &ix->w_part, &ix->w_ids, &ix->w_dists,
-                      &ix->w_cand, &ix->w_cdist, &ix->w_tab, &ix->w_plan, &ix->w_items, &ix->t_cand, &ix->t_pos,
+                      &ix->w_cand, &ix->w_cdist, &ix->w_tab, &ix->w_plan, &ix->t_cand, &ix->t_pos,
                       &ix->t_mined, &ix->t_mdist, &ix->t_gC, &ix->t_gw, &ix->t_loss, &ix->t_G,
                       &ix->t_gW, &ix->t_gWpart, &ix->t_galpha, &ix->t_gbank, &ix->t_gwz, &ix->t_wz, &ix->t_neg};
     for (DevBuf* b : bufs) release(*b);
@@ -447,7 +447,7 @@ int64_t pick_sub_batch(const ifvs_index* ix, const Opts& o, int64_t nq) {
     return sb < nq ? sb : nq;
 }
 
-ScanShape scan_shape(const ifvs_index* ix, int64_t n, int kk, int64_t chunk_blocks) {
+ScanShape scan_shape(const ifvs_index* ix) {
     ScanShape sh;
     sh.n_blocks = ix->n_blocks;
     sh.n_rows = ix->N;
@@ -455,33 +455,20 @@ ScanShape scan_shape(const ifvs_index* ix, int64_t n, int kk, int64_t chunk_bloc
     sh.K = ix->K;
     sh.row_bytes = ix->row_bytes;
     sh.tab_words = ix->tab_words;
-    // Rows per scan CTA.  Every CTA pays a fixed cost (its table, its
-    // lists and their merge, one more partial list per query for k_merge),
-    // so a batch takes as few chunks as keep the GPU busy: about two waves
-    // of CTAs from the queries alone, and chunks of at most 65 536 blocks
-    // (6.7e7 rows), which keeps the long CTAs of 10^8-row dense bins from
-    // leaving a ragged last wave.  Measured with 1024-query batches:
-    // 10^8 rows 2 chunks 28.1k queries/s (1: 25.3k, 3: 27.2k, 4: 27.5k,
-    // 12 L2-sized chunks, the earlier rule: 25.4k); 10^6 rows 1 chunk 795k
-    // (2: 723k, 3: 693k).
-    const int64_t resident = (int64_t)ix->num_sms * scan_ctas_per_sm(ix->tab_words, scan_kp(kk));
-    int64_t chunks = (resident * 2 + n - 1) / n;
-    const int64_t by_rows = (ix->n_blocks + 65535) / 65536;
-    if (chunks < by_rows) chunks = by_rows;
-    int64_t max_chunks = ix->n_blocks / 16;
-    if (max_chunks < 1) max_chunks = 1;
-    const int64_t key_cap = 32768 / kk;  // bounds the merge's input per query
-    if (max_chunks > key_cap) max_chunks = key_cap > 0 ? key_cap : 1;
-    if (max_chunks > 65535) max_chunks = 65535;
-    if (chunks > max_chunks) chunks = max_chunks;
-    if (chunks < 1) chunks = 1;
-    if (chunk_blocks > 0) {
-        chunks = (ix->n_blocks + chunk_blocks - 1) / chunk_blocks;
-        if (chunks > 65535) chunks = 65535;
-    }
-    sh.blocks_per_chunk = (ix->n_blocks + chunks - 1) / chunks;
-    sh.n_chunks = (int)((ix->n_blocks + sh.blocks_per_chunk - 1) / sh.blocks_per_chunk);
     return sh;
+}
+
+// Work lists of n queries (k keys per list) in w_part; groups that the batch
+// cannot use get no room.
+int make_sched(ifvs_index* ix, const ScanShape& sh, int64_t n, int k, const Opts& o, bool lists, bool bitmaps,
+               bool pairs, ScanSched* s) {
+    const int slots[3] = {ix->num_sms * scan_list_ctas_per_sm(sh, k, !o.plain_loads),
+                          ix->num_sms * scan_ctas_per_sm(ix->tab_words, scan_kp(k)), ix->num_sms};
+    const int64_t any = (int64_t)1 << 40;
+    const int64_t most[3] = {lists ? any : 0, bitmaps ? any : 0, pairs ? any : 0};
+    TRY(ensure(ix->w_part, scan_sched_layout(n, k, ix->n_blocks, slots, o.chunk_blocks, most, nullptr, s)));
+    scan_sched_layout(n, k, ix->n_blocks, slots, o.chunk_blocks, most, ix->w_part.as<uint8_t>(), s);
+    return 0;
 }
 
 // Arguments of launch_prepare: the predicates alone, and with the
@@ -534,8 +521,14 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     TRY(ensure(ix->w_alpha, sizeof(float) * n * (Mr > 0 ? Mr : 1)));
     TRY(ensure(ix->w_wf, sizeof(float) * n * ix->D));
     TRY(ensure(ix->w_tab, sizeof(float) * n * 256 * ix->tab_words));
-    const ScanShape sh = scan_shape(ix, n, kk, o.chunk_blocks);
-    TRY(ensure(ix->w_part, sizeof(uint64_t) * n * sh.n_chunks * kk));
+    const ScanShape sh = scan_shape(ix);
+    // pairs need two queries that together span pair_min_rows of the index's
+    // rows; with stage timing every kernel of the path is launched
+    const int64_t pair_min = o.pair_min_rows > 0 ? o.pair_min_rows : kPairDefaultMinRows;
+    const bool pairs = list_on && o.pair_min_rows >= 0 && scan_pairs_fit(sh, kk) &&
+                       (o.timing || (n > 1 && ix->N >= pair_min));
+    ScanSched sched;
+    TRY(make_sched(ix, sh, n, kk, o, list_on, bitmaps, pairs, &sched));
     if (o.R > 0) {
         TRY(ensure(ix->w_cand, sizeof(int64_t) * n * kk));
         TRY(ensure(ix->w_cdist, sizeof(float) * n * kk));
@@ -549,7 +542,6 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     }
     if (list_on) {
         TRY(ensure(ix->w_plan, sizeof(ScanPlan) * n));
-        TRY(ensure(ix->w_items, scan_list_workspace_bytes(n)));   // query groups of the sorted-copy scan
         pa.sorted = ix->sorted();
         pa.N = ix->N;
         pa.max_rows = ppm >= 1000000 ? ix->N : ix->N * ppm / 1000000;
@@ -590,30 +582,31 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
         CUDA_TRY(st.end(launch_tables(ix->w_lut.as<float>(), n, ix->M, ix->K, ix->tab_words,
                                       ix->w_tab.as<float>(), s)));
     }
+    {
+        Stage st(ix, s, o.timing, pairs ? IFVS_STAGE_SCAN : IFVS_STAGE_LAYOUT);
+        CUDA_TRY(st.end(launch_schedule(plan, npass_u64, n, ix->n_blocks, pairs ? pair_min : -1, sched, s)));
+    }
     if (bitmaps) {
         Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
-        CUDA_TRY(st.end(launch_scan(ix->d_codes, ix->w_tab.as<float>(), ix->w_bm.as<uint32_t>(), plan,
-                                    n, kk, sh, ix->w_part.as<uint64_t>(), s)));
+        CUDA_TRY(st.end(launch_scan(ix->d_codes, ix->w_tab.as<float>(), ix->w_bm.as<uint32_t>(), n, kk, sh, sched, s)));
+    }
+    if (pairs) {
+        Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
+        CUDA_TRY(st.end(launch_scan_pairs(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, s)));
     }
     if (plan) {
         Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
-        int nl = 0;
         ListOpts lo;
-        lo.pair_min_rows = o.pair_min_rows > 0 ? o.pair_min_rows : kPairDefaultMinRows;
         lo.bulk = !o.plain_loads;
         lo.tx_extra = stall_copies_for_tests() ? 16u : 0u;
         lo.err = ix->w_err.as<int>();
-        const cudaError_t e = launch_scan_list(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh,
-                                               ix->w_part.as<uint64_t>(),
-                                               o.pair_min_rows < 0 ? nullptr : ix->w_items.as<uint8_t>(),
-                                               lo, s, &nl);
-        CUDA_TRY(st.end(e, nl));
+        CUDA_TRY(st.end(launch_scan_list(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, lo, s)));
     }
     int64_t* m_ids = o.R > 0 ? ix->w_cand.as<int64_t>() : out_ids;
     float* m_dists = o.R > 0 ? ix->w_cdist.as<float>() : out_dists;
     {
         Stage st(ix, s, o.timing, IFVS_STAGE_MERGE);
-        CUDA_TRY(st.end(launch_merge(ix->w_part.as<uint64_t>(), n, sh.n_chunks, kk, m_ids, m_dists, s)));
+        CUDA_TRY(st.end(launch_merge(sched, n, kk, m_ids, m_dists, s)));
     }
     if (o.R > 0) {
         Stage st(ix, s, o.timing, IFVS_STAGE_RERANK);
@@ -1263,23 +1256,28 @@ int ifvs_scan_topk(ifvs_index* ix, const float* lut, const uint32_t* bitmaps, in
             CUDA_TRY(st.end(launch_bitmap_layout(drows, ix->w_bm.as<uint32_t>(), n, ix->n_blocks, wrows,
                                                  false, s)));
         }
-        const ScanShape sh = scan_shape(ix, n, k, o.chunk_blocks);
-        TRY(ensure(ix->w_part, sizeof(uint64_t) * n * sh.n_chunks * k));
+        const ScanShape sh = scan_shape(ix);
+        ScanSched sched;
+        TRY(make_sched(ix, sh, n, k, o, false, true, false, &sched));
         TRY(ensure(ix->w_tab, sizeof(float) * n * 256 * ix->tab_words));
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_LUT);
             CUDA_TRY(st.end(launch_tables(dl, n, ix->M, ix->K, ix->tab_words, ix->w_tab.as<float>(), s)));
         }
         {
+            Stage st(ix, s, o.timing, IFVS_STAGE_LAYOUT);
+            CUDA_TRY(st.end(launch_schedule(nullptr, nullptr, n, ix->n_blocks, -1, sched, s)));
+        }
+        {
             Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
-            CUDA_TRY(st.end(launch_scan(ix->d_codes, ix->w_tab.as<float>(), ix->w_bm.as<uint32_t>(), nullptr,
-                                        n, k, sh, ix->w_part.as<uint64_t>(), s)));
+            CUDA_TRY(st.end(launch_scan(ix->d_codes, ix->w_tab.as<float>(), ix->w_bm.as<uint32_t>(), n, k, sh, sched,
+                                        s)));
         }
         int64_t* oid = o.dio ? ids + q0 * k : ix->w_ids.as<int64_t>();
         float* odi = o.dio ? dists + q0 * k : ix->w_dists.as<float>();
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_MERGE);
-            CUDA_TRY(st.end(launch_merge(ix->w_part.as<uint64_t>(), n, sh.n_chunks, k, oid, odi, s)));
+            CUDA_TRY(st.end(launch_merge(sched, n, k, oid, odi, s)));
         }
         if (!o.dio) {
             TRY(copy_out(s, false, ids + q0 * k, oid, sizeof(int64_t) * n * k));

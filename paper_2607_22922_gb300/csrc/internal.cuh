@@ -113,7 +113,9 @@ struct ScanPlan {
 // ckey(v_j, v_{1-j}) of each position: a predicate fixing column j to one
 // value and bounding the other column to an interval selects one contiguous
 // position range of that copy.  Every copy: position p holds row rows[p]'s
-// codes, rotated by (p mod 32) mod M, row_bytes apart, padded like the index.
+// codes, rotated by (p mod 32) mod M, padded like the index: row_bytes apart for
+// M = 12 and 16, by groups of 32 positions word by word for other M
+// (sorted_byte, scan.cu).
 constexpr int kComposite = IFVS_MAX_ATTRS;
 constexpr int kSortedCopies = IFVS_MAX_ATTRS + 2;
 
@@ -213,53 +215,76 @@ struct ScanShape {
     int M, K;
     int row_bytes;         // code row stride in bytes (M rounded up to 4)
     int tab_words;         // LUT table stride in words per codeword
-    int64_t blocks_per_chunk;
-    int n_chunks;
     int64_t n_rows;        // N (rows of the index)
 };
 size_t scan_smem_bytes(int tab_words, int kp);
-// CTAs of the scan resident per SM for this table stride and list size
+// CTAs resident per SM: of the bitmap scan, and of the one-query sorted-copy
+// scan, for this shape and k
 int scan_ctas_per_sm(int tab_words, int kp);
+int scan_list_ctas_per_sm(const ScanShape& sh, int k, bool bulk);
 int scan_kp(int k);
-// Rank: per (query, chunk) CTA, the k best keys (dist bits << 32 | row) of
-// the chunk's passing rows -> partials [nq][n_chunks][k]; `tab` holds the
-// tables written by launch_tables
-cudaError_t launch_scan(const uint8_t* codes, const float* tab, const uint32_t* bm,
-                        const ScanPlan* plan, int64_t nq, int k, const ScanShape& sh,
-                        uint64_t* partials, cudaStream_t s);
-// One CTA's work in the M = 16 sorted-copy scan: queries qa and qb share
-// it (qb = -1: qa alone; qa = -1: no work).
-struct PairItem {
-    int32_t qa, qb;
+
+// ---- work lists of a batch (scan_sched.cu) -------------------------------
+constexpr int kRoundRows = 256;   // positions of a warp's round on a sorted copy
+// One CTA's work: query qa (with qb when >= 0) on units [a, b): rounds of a
+// sorted copy (list group), blocks (bitmap and pair groups); writes list la
+// (and lb) of k keys.
+struct ScanItem {
+    int32_t qa, qb, la, lb;
+    uint32_t a, b;
 };
-// the list-path queries of `plan`: their pool is the position range [a, b)
-// of a column's sorted copy (same grid and partial layout as launch_scan).
-// For M = 16, `work` (scan_list_workspace_bytes(nq) bytes) receives the
-// pairs of overlapping ranges that together span at least pair_min_rows
-// positions, served by a two-query kernel; a one-query kernel serves the
-// other queries (all of them when work is null or M != 16).  *launches =
-// kernels launched.
-// M = 16 one-query CTAs bring their code rows in by bulk copies into shared
-// memory when `bulk` (else by per-lane vector loads); a bounded wait that
-// runs out sets bit 4 of *err.  tx_extra: bytes added to what each copy's
-// barrier expects (0; positive only to exercise the timeout path).
+struct SchedGroup {
+    int64_t slots;     // CTAs resident on the device
+    int64_t least;     // fewest units per item
+    int64_t fixed;     // units per item set by the caller (0: automatic)
+    int64_t cap;       // most items
+};
+// Groups 0, 1, 2: one-query sorted-copy scan, bitmap scan, pairs.
+struct ScanSched {
+    SchedGroup group[3];
+    ScanItem* items[3];
+    int* ctl;              // [0, 3): items per group; [3, 6): work counters
+    int2* qlist;           // [nq] (first list, lists) of a query
+    int2* pairs;           // pairs of queries
+    uint8_t* paired;       // [nq]
+    uint64_t* partials;    // [lists][k]
+};
+// fills s (pointers from `base`, which may be null); returns the bytes needed.
+// most[g] bounds group g's items (0: the group is not used).
+size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)[3], int64_t chunk_blocks,
+                         const int64_t (&most)[3], uint8_t* base, ScanSched* s);
+// plan null: every query on the bitmap path; npass null: pass counts unknown;
+// pair_min_rows < 0: no pairs
+cudaError_t launch_schedule(const ScanPlan* plan, const unsigned long long* npass, int64_t nq, int64_t n_blocks,
+                            int64_t pair_min_rows, const ScanSched& s, cudaStream_t st);
+
+// Rank over the bitmap group's items: per item, the k best keys (dist bits <<
+// 32 | row) of its blocks' passing rows; `tab` holds the tables written by
+// launch_tables
+cudaError_t launch_scan(const uint8_t* codes, const float* tab, const uint32_t* bm, int64_t nq, int k,
+                        const ScanShape& sh, const ScanSched& sched, cudaStream_t s);
+// Rank over the list group's items: a query's pool is the position range
+// [a, b) of a sorted copy.  Code rows arrive by bulk copies into shared memory
+// when `bulk` and the shape allows it (else by per-lane loads); a bounded wait
+// that runs out sets bit 4 of *err.  tx_extra: bytes added to what each
+// copy's barrier expects (0; positive only to exercise the timeout path).
 struct ListOpts {
-    int64_t pair_min_rows;
     bool bulk;
     uint32_t tx_extra;
     int* err;
 };
-size_t scan_list_workspace_bytes(int64_t nq);
 cudaError_t launch_scan_list(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                             const ScanShape& sh, uint64_t* partials, uint8_t* work, const ListOpts& lo,
-                             cudaStream_t s, int* launches);
+                             const ScanShape& sh, const ScanSched& sched, const ListOpts& lo, cudaStream_t s);
+// Rank over the pair group's items (M = 16): two queries per CTA
+bool scan_pairs_fit(const ScanShape& sh, int k);
+cudaError_t launch_scan_pairs(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
+                              const ScanShape& sh, const ScanSched& sched, cudaStream_t s);
 // the sorted copy of the codes: dst position p <- row rows[p] of the index
 // layout `src`, re-rotated by (p mod 32) mod M; positions >= N are zero
 cudaError_t launch_relayout_sorted(const uint8_t* src, const uint32_t* rows, int64_t N, int M,
                                    int row_bytes, int64_t n_rows_pad, uint8_t* dst, cudaStream_t s);
-// Select: merge [nq][n_lists][k] partial keys -> ids / dists
-cudaError_t launch_merge(const uint64_t* partials, int64_t nq, int n_lists, int k,
-                         int64_t* ids, float* dists, cudaStream_t s);
+// Select: a query's lists -> ids / dists
+cudaError_t launch_merge(const ScanSched& sched, int64_t nq, int k, int64_t* ids, float* dists, cudaStream_t s);
 // exact fp32 rerank of cand [nq][R] -> k best
 // Select across row shards: [G][nq][k] (dist, global id) -> [nq][k]
 int shard_merge_cap();

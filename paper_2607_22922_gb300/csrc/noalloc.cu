@@ -27,7 +27,10 @@
 namespace ifvs {
 namespace {
 
-constexpr size_t kScratchBytes = (size_t)IFVS_STATIC_SCRATCH_BYTES;
+// room for a single query's work lists beside the documented bytes, so that
+// they take nothing from the sizes that fit
+constexpr size_t kListBytes = 64 << 10;
+constexpr size_t kScratchBytes = (size_t)IFVS_STATIC_SCRATCH_BYTES + kListBytes;
 __device__ __align__(256) unsigned char g_scan_scratch[kScratchBytes];
 
 // Device address of g_scan_scratch on the current device.
@@ -43,27 +46,21 @@ int scratch_address(unsigned char** out) {
     return 0;
 }
 
-// Chunks per query for n queries: the allocating path's rule (about two
-// waves of CTAs from the queries alone, chunks of at most 65 536 blocks, at
-// least 16 blocks per chunk, at most 32768 keys per query for the merge).
-int64_t chunks_for(const IndexView& v, int64_t n, int k) {
-    const int64_t resident = (int64_t)v.num_sms * scan_ctas_per_sm(v.tab_words, scan_kp(k));
-    int64_t c = (resident * 2 + n - 1) / n;
-    const int64_t by_rows = (v.n_blocks + 65535) / 65536;
-    if (c < by_rows) c = by_rows;
-    int64_t cap = v.n_blocks / 16;
-    if (cap < 1) cap = 1;
-    if (cap > 32768 / k) cap = 32768 / k > 0 ? 32768 / k : 1;
-    if (cap > 65535) cap = 65535;
-    if (c > cap) c = cap;
-    if (c < 1) c = 1;
-    return c;
+// What one query needs at least: its lane-major bitmap, its table and one
+// list of k keys.
+size_t one_query(const IndexView& v, int k) {
+    return (size_t)v.n_blocks * 128 + (size_t)256 * v.tab_words * sizeof(float) + (size_t)k * sizeof(uint64_t);
 }
 
-size_t footprint(const IndexView& v, int64_t n, int64_t chunks, int k) {
+// Layout of n queries: lane-major bitmaps, tables, the scan's work lists with
+// at most `items` items (n <= items).  Returns the bytes.
+size_t layout(const IndexView& v, int64_t n, int64_t items, int k, uint8_t* base, ScanSched* s) {
     const size_t bm = (size_t)n * v.n_blocks * 128;
     const size_t tab = (size_t)n * 256 * v.tab_words * sizeof(float);
-    return bm + tab + (size_t)n * chunks * k * sizeof(uint64_t);
+    const int slots[3] = {1, v.num_sms * scan_ctas_per_sm(v.tab_words, scan_kp(k)), 1};
+    const int64_t most[3] = {0, items, 0};
+    const size_t head = (bm + tab + 255) / 256 * 256;
+    return head + scan_sched_layout(n, k, v.n_blocks, slots, 0, most, base ? base + head : nullptr, s);
 }
 
 }  // namespace
@@ -86,12 +83,12 @@ extern "C" int ifvs_scan_topk_static(ifvs_index* ix, const float* lut, const uin
                             k, v.M, scan_smem_bytes(v.tab_words, scan_kp(k)), v.max_smem);
     if (nq == 0) return IFVS_OK;
     if (!lut || !bitmaps || !ids || !dists) return report_error(IFVS_ERR_ARG, "an array argument is NULL");
-    // one query must fit: its lane-major bitmap, its table and one list of k keys
-    if (footprint(v, 1, 1, k) > kScratchBytes)
+    ScanSched sched;
+    if (one_query(v, k) > (size_t)IFVS_STATIC_SCRATCH_BYTES)
         return report_error(IFVS_ERR_UNSUPPORTED,
                             "N = %lld needs %zu bytes of scratch per query; the static scratch "
                             "holds %zu (IFVS_STATIC_SCRATCH_BYTES)",
-                            (long long)v.N, footprint(v, 1, 1, k), kScratchBytes);
+                            (long long)v.N, one_query(v, k), (size_t)IFVS_STATIC_SCRATCH_BYTES);
     int prev = -1;
     if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
     if (prev != v.device && cudaSetDevice(v.device) != cudaSuccess) {
@@ -104,19 +101,23 @@ extern "C" int ifvs_scan_topk_static(ifvs_index* ix, const float* lut, const uin
     const int64_t wrows = (v.N + 31) / 32;
     const size_t lut_n = (size_t)v.M * v.K;
     // largest sub-batch (halving from nq) whose bitmaps, tables and lists fit
-    // the scratch with the allocating path's chunk split
+    // the scratch with the allocating path's number of items
+    const int64_t any = (int64_t)1 << 40;
     int64_t sb = nq;
-    while (rc == 0 && sb > 1 && footprint(v, sb, chunks_for(v, sb, k), k) > kScratchBytes) sb = (sb + 1) / 2;
+    while (rc == 0 && sb > 1 && layout(v, sb, any, k, nullptr, &sched) > kScratchBytes) sb = (sb + 1) / 2;
     for (int64_t q0 = 0; rc == 0 && q0 < nq; q0 += sb) {
         const int64_t n = sb < nq - q0 ? sb : nq - q0;
         // where even one query's lists with that split overflow, use fewer
-        // chunks (one chunk always fits: checked above)
-        int64_t chunks = chunks_for(v, n, k);
-        while (chunks > 1 && footprint(v, n, chunks, k) > kScratchBytes) chunks = (chunks + 1) / 2;
+        // items (one always fits: checked above)
+        int64_t items = any;
+        if (layout(v, n, items, k, nullptr, &sched) > kScratchBytes) {
+            items = sched.group[1].cap;
+            while (items > n && layout(v, n, items, k, nullptr, &sched) > kScratchBytes)
+                items = items / 2 > n ? items / 2 : n;
+        }
+        layout(v, n, items, k, base, &sched);
         uint32_t* bm = reinterpret_cast<uint32_t*>(base);
         float* tab = reinterpret_cast<float*>(base + (size_t)n * v.n_blocks * 128);
-        uint64_t* part = reinterpret_cast<uint64_t*>(base + (size_t)n * v.n_blocks * 128 +
-                                                     (size_t)n * 256 * v.tab_words * sizeof(float));
         ScanShape sh;
         sh.n_blocks = v.n_blocks;
         sh.n_rows = v.N;
@@ -124,12 +125,11 @@ extern "C" int ifvs_scan_topk_static(ifvs_index* ix, const float* lut, const uin
         sh.K = v.K;
         sh.row_bytes = v.row_bytes;
         sh.tab_words = v.tab_words;
-        sh.blocks_per_chunk = (v.n_blocks + chunks - 1) / chunks;
-        sh.n_chunks = (int)((v.n_blocks + sh.blocks_per_chunk - 1) / sh.blocks_per_chunk);
         cudaError_t e = launch_bitmap_layout(bitmaps + q0 * wrows, bm, n, v.n_blocks, wrows, false, s);
         if (e == cudaSuccess) e = launch_tables(lut + q0 * lut_n, n, v.M, v.K, v.tab_words, tab, s);
-        if (e == cudaSuccess) e = launch_scan(v.codes, tab, bm, nullptr, n, k, sh, part, s);
-        if (e == cudaSuccess) e = launch_merge(part, n, sh.n_chunks, k, ids + q0 * k, dists + q0 * k, s);
+        if (e == cudaSuccess) e = launch_schedule(nullptr, nullptr, n, v.n_blocks, -1, sched, s);
+        if (e == cudaSuccess) e = launch_scan(v.codes, tab, bm, n, k, sh, sched, s);
+        if (e == cudaSuccess) e = launch_merge(sched, n, k, ids + q0 * k, dists + q0 * k, s);
         if (e != cudaSuccess) {
             cudaGetLastError();
             rc = report_error(IFVS_ERR_CUDA, "ifvs_scan_topk_static launch failed: %s", cudaGetErrorString(e));

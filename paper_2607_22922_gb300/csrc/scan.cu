@@ -10,14 +10,14 @@ int scan_kp(int k) { return k <= 32 ? 32 : (k <= 64 ? 64 : (k <= 128 ? 128 : 256
 
 size_t scan_smem_bytes(int tab_words, int kp) {
     return (size_t)256 * tab_words * 4 + (size_t)kScanWarps * 2 * kp * 8 +
-           (size_t)kScanWarps * kRing * 32 * 4;
+           (size_t)kScanWarps * kRing * 32 * 4 + 16;
 }
 
 int scan_ctas_per_sm(int tab_words, int kp) {
     const size_t per_cta = scan_smem_bytes(tab_words, kp) + 1024;
     const int by_smem = (int)((size_t)233472 / per_cta);
-    const int by_threads = 2048 / kScanThreads;
-    int n = by_smem < by_threads ? by_smem : by_threads;
+    const int by_regs = 2;   // 128 registers
+    int n = by_smem < by_regs ? by_smem : by_regs;
     return n < 1 ? 1 : n;
 }
 
@@ -164,8 +164,7 @@ __device__ __forceinline__ void scan_chunk(const uint8_t* __restrict__ codes,
 template <int KP, int MM, int MINB>
 __global__ void __launch_bounds__(kScanThreads, MINB)
 k_scan(const uint8_t* __restrict__ codes, const float* __restrict__ tables,
-       const uint32_t* __restrict__ bm, const ScanPlan* __restrict__ plan, int64_t nq, int k,
-       ScanShape sh, uint64_t* __restrict__ partials) {
+       const uint32_t* __restrict__ bm, int k, ScanShape sh, ScanSched sched) {
     extern __shared__ __align__(256) uint8_t smem[];
     const int S = MM > 0 ? 64 : sh.tab_words;
     float* tab = reinterpret_cast<float*>(smem);
@@ -173,9 +172,12 @@ k_scan(const uint8_t* __restrict__ codes, const float* __restrict__ tables,
     uint32_t* ringbase = reinterpret_cast<uint32_t*>(smem + (size_t)256 * S * 4 +
                                                      (size_t)kScanWarps * 2 * KP * 8);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t q = blockIdx.x;
-    const int chunk = blockIdx.y;
-    if (plan != nullptr && plan[q].list) return;   // k_scan_list covers this query
+    uint32_t* ring = ringbase + warp * kRing * 32;
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab);
+    const bool fast = base == kDynSmemBase;
+    for (ItemLoop loop(sched, 1, ringbase + kScanWarps * kRing * 32); loop.more(); loop.next()) {
+    const ScanItem item = loop.items[loop.at];
+    const int64_t q = item.qa;
 
     // 1) the query's table, replicated and rotated (see the file comment),
     //    as written by k_tables: a straight 16-byte-wide copy
@@ -188,13 +190,9 @@ k_scan(const uint8_t* __restrict__ codes, const float* __restrict__ tables,
     tk.init(tkbuf + warp * 2 * KP, k, lane);
     __syncthreads();
 
-    // 2) the chunk's blocks
-    const int64_t b0 = (int64_t)chunk * sh.blocks_per_chunk;
-    const int64_t b1 = min(sh.n_blocks, b0 + sh.blocks_per_chunk);
+    // 2) the item's blocks
+    const int64_t b0 = item.a, b1 = item.b;
     const uint32_t* bmq = bm + q * sh.n_blocks * 32;
-    uint32_t* ring = ringbase + warp * kRing * 32;
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab);
-    const bool fast = base == kDynSmemBase;
     if constexpr (MM > 0) {
         if (fast)
             scan_chunk<KP, MM, true>(codes, bmq, sh, b0, b1, tab, ring, tk, lane, warp);
@@ -204,75 +202,63 @@ k_scan(const uint8_t* __restrict__ codes, const float* __restrict__ tables,
         scan_chunk<KP, 0, false>(codes, bmq, sh, b0, b1, tab, ring, tk, lane, warp);
     }
 
-    // 3) merge the warps' lists pairwise (4 levels); warp 0 writes the
-    //    CTA's k best keys
-    tk.flush(lane);
-#pragma unroll 1
-    for (int step = 1; step < kScanWarps; step <<= 1) {
-        __syncthreads();
-        if ((warp & (2 * step - 1)) == 0) {
-            const uint64_t* other = tkbuf + (warp + step) * 2 * KP;
-            for (int i = lane; i < k; i += 32) tk.buf[KP + i] = other[i];
-            __syncwarp();
-            tk.flush(lane);
-        }
-    }
-    if (warp == 0) {
-        uint64_t* out = partials + (q * sh.n_chunks + chunk) * (int64_t)k;
-        for (int i = lane; i < k; i += 32) out[i] = tk.buf[i];
+    // 3) merge the warps' lists pairwise; warp 0 writes the k best keys
+    merge_warps<KP, kScanWarps>(tk, tkbuf, k, lane, warp, sched.partials + (int64_t)item.la * k);
     }
 }
 
 template <int KP, int MM, int MINB>
-static cudaError_t launch_one(const uint8_t* codes, const float* tab, const uint32_t* bm,
-                              const ScanPlan* plan, int64_t nq, int k, const ScanShape& sh,
-                              uint64_t* partials, size_t smem, cudaStream_t s) {
+static cudaError_t launch_one(const uint8_t* codes, const float* tab, const uint32_t* bm, int k, const ScanShape& sh,
+                              const ScanSched& sched, size_t smem, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_scan<KP, MM, MINB>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)nq, (unsigned)sh.n_chunks);
-    k_scan<KP, MM, MINB><<<grid, kScanThreads, smem, s>>>(codes, tab, bm, plan, nq, k, sh, partials);
+    k_scan<KP, MM, MINB><<<item_grid(sched.group[1]), kScanThreads, smem, s>>>(codes, tab, bm, k, sh, sched);
     return cudaGetLastError();
 }
 
 template <int KP>
-static cudaError_t launch_scan_kp(const uint8_t* codes, const float* tab, const uint32_t* bm,
-                                  const ScanPlan* plan, int64_t nq, int k, const ScanShape& sh,
-                                  uint64_t* partials, cudaStream_t s) {
+static cudaError_t launch_scan_kp(const uint8_t* codes, const float* tab, const uint32_t* bm, int k,
+                                  const ScanShape& sh, const ScanSched& sched, cudaStream_t s) {
     const int mm = fixed_m(sh);
     const size_t smem = scan_smem_bytes(sh.tab_words, KP);
     const bool two = scan_ctas_per_sm(sh.tab_words, KP) >= 2;
     if (mm == 16)
-        return two ? launch_one<KP, 16, 2>(codes, tab, bm, plan, nq, k, sh, partials, smem, s)
-                   : launch_one<KP, 16, 1>(codes, tab, bm, plan, nq, k, sh, partials, smem, s);
+        return two ? launch_one<KP, 16, 2>(codes, tab, bm, k, sh, sched, smem, s)
+                   : launch_one<KP, 16, 1>(codes, tab, bm, k, sh, sched, smem, s);
     if (mm == 12)
-        return two ? launch_one<KP, 12, 2>(codes, tab, bm, plan, nq, k, sh, partials, smem, s)
-                   : launch_one<KP, 12, 1>(codes, tab, bm, plan, nq, k, sh, partials, smem, s);
-    return launch_one<KP, 0, 1>(codes, tab, bm, plan, nq, k, sh, partials, smem, s);
+        return two ? launch_one<KP, 12, 2>(codes, tab, bm, k, sh, sched, smem, s)
+                   : launch_one<KP, 12, 1>(codes, tab, bm, k, sh, sched, smem, s);
+    return launch_one<KP, 0, 1>(codes, tab, bm, k, sh, sched, smem, s);
 }
 
-cudaError_t launch_scan(const uint8_t* codes, const float* tab, const uint32_t* bm,
-                        const ScanPlan* plan, int64_t nq, int k, const ScanShape& sh,
-                        uint64_t* partials, cudaStream_t s) {
+cudaError_t launch_scan(const uint8_t* codes, const float* tab, const uint32_t* bm, int64_t nq, int k,
+                        const ScanShape& sh, const ScanSched& sched, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     switch (scan_kp(k)) {
-        case 32: return launch_scan_kp<32>(codes, tab, bm, plan, nq, k, sh, partials, s);
-        case 64: return launch_scan_kp<64>(codes, tab, bm, plan, nq, k, sh, partials, s);
-        case 128: return launch_scan_kp<128>(codes, tab, bm, plan, nq, k, sh, partials, s);
-        default: return launch_scan_kp<256>(codes, tab, bm, plan, nq, k, sh, partials, s);
+        case 32: return launch_scan_kp<32>(codes, tab, bm, k, sh, sched, s);
+        case 64: return launch_scan_kp<64>(codes, tab, bm, k, sh, sched, s);
+        case 128: return launch_scan_kp<128>(codes, tab, bm, k, sh, sched, s);
+        default: return launch_scan_kp<256>(codes, tab, bm, k, sh, sched, s);
     }
+}
+
+// Byte of a sorted copy that holds byte s of position p's row: rows one after
+// the other (16-byte rows of the loops compiled for M = 12 and 16), or by
+// groups of 32 positions, word by word (k_scan_list_gen).
+__device__ __forceinline__ int64_t sorted_byte(int64_t p, int s, int row_bytes, bool by_word) {
+    return by_word ? ((p >> 5) * (row_bytes >> 2) + (s >> 2)) * 128 + (p & 31) * 4 + (s & 3) : p * row_bytes + s;
 }
 
 // sorted copy: position p <- row rows[p] (stored rotated by (row mod 32) mod M)
 // re-rotated by (p mod 32) mod M
 __global__ void k_relayout_sorted(const uint8_t* __restrict__ src, const uint32_t* __restrict__ rows,
-                                  int64_t N, int M, int row_bytes, int64_t n_rows_pad,
+                                  int64_t N, int M, int row_bytes, int64_t n_rows_pad, bool by_word,
                                   uint8_t* __restrict__ dst) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n_rows_pad) return;
-    uint8_t* out = dst + p * row_bytes;
     if (p >= N) {
-        for (int s = 0; s < row_bytes; ++s) out[s] = 0;
+        for (int s = 0; s < row_bytes; ++s) dst[sorted_byte(p, s, row_bytes, by_word)] = 0;
         return;
     }
     const uint32_t row = rows[p];
@@ -289,7 +275,7 @@ __global__ void k_relayout_sorted(const uint8_t* __restrict__ src, const uint32_
             if (t < 0) t += M;
             v = in[t];
         }
-        out[s] = v;
+        dst[sorted_byte(p, s, row_bytes, by_word)] = v;
     }
 }
 
@@ -297,7 +283,12 @@ cudaError_t launch_relayout_sorted(const uint8_t* src, const uint32_t* rows, int
                                    int row_bytes, int64_t n_rows_pad, uint8_t* dst, cudaStream_t s) {
     const int threads = 256;
     const int64_t blocks = (n_rows_pad + threads - 1) / threads;
-    k_relayout_sorted<<<(unsigned)blocks, threads, 0, s>>>(src, rows, N, M, row_bytes, n_rows_pad, dst);
+    ScanShape sh{};
+    sh.M = M;
+    sh.row_bytes = row_bytes;
+    sh.tab_words = (M + 31 + 31) / 32 * 32;
+    k_relayout_sorted<<<(unsigned)blocks, threads, 0, s>>>(src, rows, N, M, row_bytes, n_rows_pad, fixed_m(sh) == 0,
+                                                           dst);
     return cudaGetLastError();
 }
 

@@ -3,11 +3,11 @@
 // form of the printed score), and each CTA keeps the k smallest
 // (dist, row id) of its chunk exactly.
 //
-// Work split.  CTA (query q, chunk c), 8 warps; blockIdx.x runs over the
-// queries so that the CTAs resident together walk the same code chunk and
-// share it through L2.  Warp w of the CTA owns bitmap blocks c0 + w,
-// c0 + w + 8, ...; lane l owns, in each of them, the 32 rows
-// b*1024 + 32*j + l, whose pass bits form its lane-major bitmap word.
+// Work split.  A CTA of 8 warps takes items, parts of a query's rows, from a
+// list made on the device (scan_sched.cu).  Warp w of the bitmap path owns
+// the item's bitmap blocks b0 + w, b0 + w + 8, ...; lane l owns, in each of
+// them, the 32 rows b*1024 + 32*j + l, whose pass bits form its lane-major
+// bitmap word.
 //
 // LUT placement.  The scan issues one shared-memory load per code byte, so
 // bank conflicts set its speed.  The table of query q is stored as 256 rows
@@ -117,27 +117,16 @@ __device__ __forceinline__ void warp_merge_low(uint64_t* a, int n, int lane) {
 
 // Merges a warp's candidates [KP, 2KP) of buf into its sorted list [0, KP),
 // clears the candidates, publishes the new k-th key to the CTA's bound (if
-// any) and returns it.  For KP >= 64 the candidates are sorted and the KP
-// smallest of both runs kept by one bitonic merge (half the compare-
-// exchanges of one sort of 2 KP); for KP = 32 both take the same number of
-// steps and one sort of 64 measured faster (sift1m 693k against 599k
-// queries/s; 10^8 rows at KP = 128: 0.1 % and 1 % bins 1.51 -> 1.41 and
-// 4.33 -> 4.04 ms with the merge).  Out of line: the scan loops offer keys
-// at many sites and flush rarely, and one copy of the sort keeps their code
-// small (instruction-fetch stalls led the two-query kernel's profile).
+// any) and returns it.  The candidates are sorted and the KP smallest of both
+// runs kept by one bitonic merge (half the compare-exchanges of one sort of
+// 2 KP; 10^8 rows at KP = 128: 0.1 % and 1 % bins 1.51 -> 1.41 and 4.33 ->
+// 4.04 ms).  Out of line: the scan loops offer keys at many sites and flush
+// rarely, and one copy of the sort keeps their code small (instruction-fetch
+// stalls led the two-query kernel's profile).
 template <int KP>
-#ifndef IFVS_FLUSH_INLINE
-__device__ __noinline__
-#else
-__device__ __forceinline__
-#endif
-uint64_t flush_list(uint64_t* buf, int k, uint64_t* cta, int lane) {
-    if constexpr (KP <= 32) {
-        warp_sort(buf, 2 * KP, lane);
-    } else {
-        warp_sort(buf + KP, KP, lane);
-        warp_merge_low(buf, KP, lane);
-    }
+__device__ __noinline__ uint64_t flush_list(uint64_t* buf, int k, uint64_t* cta, int lane) {
+    warp_sort(buf + KP, KP, lane);
+    warp_merge_low(buf, KP, lane);
     const uint64_t thr = buf[k - 1];
     for (int i = KP + lane; i < 2 * KP; i += 32) buf[i] = ~0ull;
     if (cta != nullptr && lane == 0 && thr != ~0ull) atomicMin(reinterpret_cast<unsigned long long*>(cta), thr);
@@ -191,6 +180,73 @@ struct WarpTopK {
             __syncwarp();
             flush(lane);
         }
+    }
+};
+
+// k <= 32: the sorted list is one key per lane, in registers, and up to 63
+// candidates wait in shared memory; every 32 of them are sorted and merged
+// across the lanes by shuffles (15 + 6 steps of about 25 cycles; the sort of 64
+// keys in shared memory took three times as long and ran for every offer).
+// Out of line, as flush_list.
+__device__ __forceinline__ uint64_t min_max_step(uint64_t x, int j, bool low) {
+    const uint64_t y = __shfl_xor_sync(0xFFFFFFFFu, x, j);
+    return (x < y) == low ? x : y;
+}
+// `mine` ascending over the lanes, `c` any: the 32 smallest keys of both, ascending
+static __device__ __noinline__ uint64_t absorb32(uint64_t mine, uint64_t c, int lane) {
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+        for (int j = size >> 1; j > 0; j >>= 1)
+            c = min_max_step(c, j, ((lane & j) == 0) != ((lane & size) == 0));   // descending in the end
+    mine = c < mine ? c : mine;
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) mine = min_max_step(mine, j, (lane & j) == 0);
+    return mine;
+}
+
+template <>
+struct WarpTopK<32> {
+    uint64_t* buf;   // candidates, 64 slots
+    uint64_t* cta;   // as above
+    int cnt;
+    int k;
+    uint64_t thr;
+    uint64_t mine;   // the lane's key of the sorted list
+
+    __device__ __forceinline__ void init(uint64_t* b, int k_, int, uint64_t* cta_ = nullptr) {
+        buf = b;
+        cta = cta_;
+        k = k_;
+        cnt = 0;
+        thr = ~0ull;
+        mine = ~0ull;
+    }
+    __device__ __forceinline__ void refresh(int) {
+        if (cta == nullptr) return;
+        const uint64_t t = *reinterpret_cast<volatile uint64_t*>(cta);
+        if (t < thr) thr = t;
+    }
+    __device__ __forceinline__ void drain(int n, int lane) {
+        cnt -= n;
+        __syncwarp();
+        const uint64_t c = lane < n ? buf[cnt + lane] : ~0ull;
+        __syncwarp();   // the drained slots take the next candidates
+        mine = absorb32(mine, c, lane);
+        thr = __shfl_sync(0xFFFFFFFFu, mine, k - 1);
+        if (cta != nullptr && lane == 0 && thr != ~0ull)
+            atomicMin(reinterpret_cast<unsigned long long*>(cta), thr);
+        refresh(lane);
+    }
+    __device__ __forceinline__ void flush(int lane) {
+        if (cnt > 0) drain(cnt, lane);
+    }
+    __device__ __forceinline__ void offer(uint64_t key, bool want, int lane) {
+        const unsigned ball = __ballot_sync(0xFFFFFFFFu, want);
+        if (ball == 0) return;
+        if (want) buf[cnt + __popc(ball & ((1u << lane) - 1u))] = key;
+        cnt += __popc(ball);
+        if (cnt >= 32) drain(32, lane);
     }
 };
 
@@ -341,23 +397,41 @@ __device__ __forceinline__ void lookup_rows(const uint8_t* __restrict__ codes, c
     for (int u = 0; u < NU; u += 2) unpack_f32x2(acc[u / 2], d[u], d[u + 1]);
 }
 
-// merge the warps' lists of one query pairwise; warp 0 writes k keys
+// merge the warps' lists of one query pairwise (both sorted: one bitonic merge
+// per level); warp 0 writes k keys
 template <int KP, int WARPS>
 __device__ __forceinline__ void merge_warps(WarpTopK<KP>& tk, uint64_t* tkbuf, int k, int lane, int warp,
                                             uint64_t* out) {
     tk.flush(lane);
+    if constexpr (KP == 32) {
+        __syncwarp();
+        tk.buf[lane] = tk.mine;
+    }
 #pragma unroll 1
     for (int step = 1; step < WARPS; step <<= 1) {
         __syncthreads();
         if ((warp & (2 * step - 1)) == 0 && warp + step < WARPS) {
             const uint64_t* other = tkbuf + (warp + step) * 2 * KP;
-            for (int i = lane; i < k; i += 32) tk.buf[KP + i] = other[i];
-            __syncwarp();
-            tk.flush(lane);
+            if constexpr (KP == 32) {
+                const uint64_t o = other[31 - lane];
+                uint64_t m = o < tk.mine ? o : tk.mine;
+#pragma unroll
+                for (int j = 16; j > 0; j >>= 1) m = min_max_step(m, j, (lane & j) == 0);
+                tk.mine = m;
+                tk.buf[lane] = m;
+            } else {
+                for (int i = lane; i < KP; i += 32) tk.buf[KP + i] = other[i];
+                warp_merge_low(tk.buf, KP, lane);
+            }
         }
     }
-    if (warp == 0 && out != nullptr)
-        for (int i = lane; i < k; i += 32) out[i] = tk.buf[i];
+    if (warp == 0 && out != nullptr) {
+        if constexpr (KP == 32) {
+            if (lane < k) out[lane] = tk.mine;
+        } else {
+            for (int i = lane; i < k; i += 32) out[i] = tk.buf[i];
+        }
+    }
 }
 
 // ---- bulk copies into shared memory (cp.async.bulk) and their mbarriers ----
@@ -456,12 +530,30 @@ inline int fixed_m(const ScanShape& sh) {
     return (sh.M == 16 || sh.M == 12) ? sh.M : 0;
 }
 
-// Two-query scan of the sorted copy (scan_pair.cu): pairs the list-path
-// queries of `plan` whose ranges overlap enough (k_pair_items) and serves
-// the pairs; `work` receives the pair items and a flag per query, *paired
-// points at the flags (null when no pair kernel ran), *launches += kernels.
-cudaError_t launch_pairs(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                         const ScanShape& sh, uint64_t* partials, uint8_t* work, int64_t pair_min_rows,
-                         cudaStream_t s, const uint8_t** paired, int* launches);
+// A scan kernel's CTA takes items from its group's list until it is empty: the
+// first by its block index, the others from the work counter.  `slot`: a word
+// of the CTA's dynamic shared memory (static shared memory would move the
+// dynamic window off the base that the look-ups' immediate offsets assume).
+struct ItemLoop {
+    const ScanItem* items;
+    int n;
+    int* counter;
+    volatile int* slot;
+    int at;
+    __device__ __forceinline__ ItemLoop(const ScanSched& s, int group, void* slot_)
+        : items(s.items[group]), n(s.ctl[group]), counter(s.ctl + 3 + group),
+          slot(reinterpret_cast<volatile int*>(slot_)), at((int)blockIdx.x) {}
+    __device__ __forceinline__ bool more() const { return at < n; }
+    // all threads; a barrier on both sides: shared memory may be reused after it
+    __device__ __forceinline__ void next() {
+        if (threadIdx.x == 0) *slot = (int)gridDim.x + atomicAdd(counter, 1);
+        __syncthreads();
+        at = *slot;
+        __syncthreads();
+    }
+};
+
+// CTAs to launch for a group: all that fit the device, or the items there can be
+inline unsigned item_grid(const SchedGroup& g) { return (unsigned)(g.cap < g.slots ? (g.cap < 1 ? 1 : g.cap) : g.slots); }
 
 }  // namespace ifvs

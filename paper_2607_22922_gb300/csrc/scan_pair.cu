@@ -1,13 +1,13 @@
 // Rank (§2 stage 2) for two queries per CTA on the sorted copy of the codes
-// (M = 16): the pairing kernel k_pair_items and the two-query kernel
-// k_scan_list_pair.  Design notes in scan_common.cuh.
+// (M = 16): the two-query kernel k_scan_list_pair.  Design notes in
+// scan_common.cuh.
 #include "scan_common.cuh"
 
 namespace ifvs {
 
 // ---- two queries per CTA on the sorted copy --------------------------------
 //
-// When k_pair_items (below) pairs two queries on the sorted copy of the same
+// When k_schedule pairs two queries on the sorted copy of the same
 // column (M = 16), one CTA serves both, and one shared-memory load serves
 // both queries' look-ups.  A 64 KB table with the rows, replication and rotation
 // of the float32 one holds, in word w of codeword row c, the pair
@@ -364,112 +364,12 @@ __device__ __forceinline__ void quant_params(const float* lo, const float* hi, f
     sl = s;
 }
 
-// ---- pairing of the sorted-copy queries of a batch -------------------------
-//
 // Two queries are worth one CTA when they read the same column's copy, their
 // ranges mostly coincide (at least 3/4 of the longer range is common to both;
 // the rows of only one range then run with the other query masked) and the
 // two ranges together span at least min_rows positions (the caller's choice:
 // for short ranges the one-query kernel, with two or three CTAs per SM, was
-// measured faster).
-// k_pair_items sorts the list-path queries of each segment of kPairSeg by
-// (column, range start, query) and pairs sorted neighbours (2j, 2j + 1) that
-// qualify.  Pairs fill the segment's item slots in sorted order and the
-// unused slots get qa = -1, so the pair kernel's CTA x serves item x (or
-// nothing); `paired` marks the queries of the pairs, and k_scan_list serves
-// every other list-path query.
-constexpr int kPairSeg = 2048;
-static_assert(kSortedCopies <= 8, "the pairing key keeps 3 bits of the sorted copy");
-constexpr int kPairSortThreads = 1024;
-
-__device__ __forceinline__ bool pairable(const ScanPlan& x, const ScanPlan& y, int64_t min_rows) {
-    if (!x.list || !y.list || x.col != y.col) return false;
-    const int64_t lx = x.b - x.a, ly = y.b - y.a;
-    if (lx <= 0 || ly <= 0) return false;
-    const int64_t common = min(x.b, y.b) - max(x.a, y.a);
-    const int64_t span = max(x.b, y.b) - min(x.a, y.a);
-    return 4 * common >= 3 * max(lx, ly) && span >= min_rows;
-}
-
-// exclusive prefix of v over the block's threads (in thread order) and the
-// total; wsum holds one int per warp
-__device__ __forceinline__ int block_prefix(int v, int* wsum, int& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    __syncthreads();
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    int before = 0;
-    total = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        const int t = wsum[w];
-        before += w < warp ? t : 0;
-        total += t;
-    }
-    return before + incl - v;
-}
-
-__global__ void __launch_bounds__(kPairSortThreads)
-k_pair_items(const ScanPlan* __restrict__ plan, int64_t nq, int64_t min_rows, PairItem* __restrict__ items,
-             uint8_t* __restrict__ paired, unsigned* __restrict__ counter) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;   // work counter of the two-query kernel
-    __shared__ uint64_t key[kPairSeg];
-    __shared__ int wsum[kPairSortThreads / 32];
-    const int64_t q0 = (int64_t)blockIdx.x * kPairSeg;
-    const int n = (int)min((int64_t)kPairSeg, nq - q0);
-    // key = copy (3 bits) | range start (32 bits) | index in the segment (11 bits);
-    // queries of the bitmap path sort last as all ones
-    for (int i = threadIdx.x; i < kPairSeg; i += kPairSortThreads) {
-        uint64_t kk = ~0ull;
-        if (i < n) {
-            const ScanPlan p = plan[q0 + i];
-            if (p.list) kk = ((uint64_t)(p.col & 7) << 43) | ((uint64_t)(uint32_t)p.a << 11) | (uint64_t)i;
-        }
-        key[i] = kk;
-    }
-    // block bitonic sort, ascending
-    for (int size = 2; size <= kPairSeg; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            __syncthreads();
-            for (int t = threadIdx.x; t < kPairSeg / 2; t += kPairSortThreads) {
-                const int i = 2 * t - (t & (stride - 1));
-                const int j = i + stride;
-                const bool up = (i & size) == 0;
-                const uint64_t x = key[i], y = key[j];
-                if ((x > y) == up) {
-                    key[i] = y;
-                    key[j] = x;
-                }
-            }
-        }
-    __syncthreads();
-    // sorted neighbours (2j, 2j + 1) that qualify make an item; positions by
-    // a block-wide exclusive scan of the counts, in sorted order
-    static_assert(kPairSeg == 2 * kPairSortThreads, "one neighbour pair per thread");
-    const int j = threadIdx.x;
-    const uint64_t ka = key[2 * j], kb = key[2 * j + 1];
-    int qa = -1, qb = -1, cnt = 0;
-    if (ka != ~0ull && kb != ~0ull) {
-        qa = (int)(q0 + (int64_t)(ka & 2047u));
-        qb = (int)(q0 + (int64_t)(kb & 2047u));
-        cnt = pairable(plan[qa], plan[qb], min_rows) ? 1 : 0;
-    }
-    for (int i = j; i < n; i += kPairSortThreads) paired[q0 + i] = 0;
-    __syncthreads();
-    if (cnt) paired[qa] = paired[qb] = 1;
-    // segment s owns item slots [s kPairSeg / 2, + ceil(n / 2)): at most one
-    // pair per two of its queries
-    int total = 0;
-    const int at = block_prefix(cnt, wsum, total);
-    PairItem* its = items + q0 / 2;
-    if (cnt) its[at] = PairItem{qa, qb};
-    for (int i = total + j; i < (n + 1) / 2; i += kPairSortThreads) its[i] = PairItem{-1, -1};
-}
+// measured faster).  k_schedule makes the pairs (scan_sched.cu).
 
 // Offset of the current work item in the two-query kernel's shared memory.
 __host__ __device__ constexpr size_t scan_pair_item_offset(int kp) {
@@ -477,12 +377,11 @@ __host__ __device__ constexpr size_t scan_pair_item_offset(int kp) {
            (pair_defers(kp) ? (size_t)kPairWarps * kCandWarpBytes : 0);
 }
 
-// One work item of the two-query kernel: pair slot `slot` on chunk `chunk`.
+// One work item of the two-query kernel.
 template <int KP>
 __device__ __forceinline__ void pair_item(uint8_t* smem, const float* __restrict__ tables, const SortedCols& sc,
-                                          const ScanPlan* __restrict__ plan, const PairItem* __restrict__ items,
-                                          int k, const ScanShape& sh, uint64_t* __restrict__ partials, int slot,
-                                          int chunk) {
+                                          const ScanPlan* __restrict__ plan, const ScanItem& it, int k,
+                                          uint64_t* __restrict__ partials) {
     uint32_t* ptab = reinterpret_cast<uint32_t*>(smem);
     float* exA = reinterpret_cast<float*>(smem + kTabBytes16);
     float* exB = reinterpret_cast<float*>(smem + kTabBytes16 + kExactBytes16);
@@ -493,33 +392,10 @@ __device__ __forceinline__ void pair_item(uint8_t* smem, const float* __restrict
     float* red = reinterpret_cast<float*>(tkbufA);   // [warp][4][16], before the lists are set up
     uint8_t* cand_base = reinterpret_cast<uint8_t*>(tkbufB + kPairWarps * 2 * KP);   // 16-byte aligned
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const PairItem it = items[slot];
-    if (it.qa < 0) return;
-    const int64_t qA = it.qa;
-    const bool hasB = it.qb >= 0;
-    const int64_t qB = hasB ? it.qb : it.qa;   // a single query: B mirrors A's table, with no range
-    const ScanPlan pA = plan[qA];
-    ScanPlan pB = plan[qB];
-    if (!hasB) pB.a = pB.b = 0;
-    const int64_t c0 = (int64_t)chunk * sh.blocks_per_chunk;
-    const int64_t c1 = min(sh.n_blocks, c0 + sh.blocks_per_chunk);
-    auto range = [&](const ScanPlan& p, int64_t& lo, int64_t& hi) {
-        lo = max(c0, p.a / kBlockRows);
-        hi = min(c1, (p.b + kBlockRows - 1) / kBlockRows);
-        if (p.a >= p.b || lo >= hi) lo = hi = 0;
-    };
-    int64_t lA, hA, lB, hB;
-    range(pA, lA, hA);
-    range(pB, lB, hB);
-    uint64_t* outA = partials + (qA * sh.n_chunks + chunk) * (int64_t)k;
-    uint64_t* outB = hasB ? partials + (qB * sh.n_chunks + chunk) * (int64_t)k : nullptr;
-    if (lA == hA && lB == hB) {
-        for (int i = threadIdx.x; i < k; i += kPairThreads) {
-            outA[i] = ~0ull;
-            if (outB) outB[i] = ~0ull;
-        }
-        return;
-    }
+    const int64_t qA = it.qa, qB = it.qb;
+    const ScanPlan pA = plan[qA], pB = plan[qB];
+    uint64_t* outA = partials + (int64_t)it.la * k;
+    uint64_t* outB = partials + (int64_t)it.lb * k;
     // 1) unreplicated float32 tables ex[c * 16 + m] (from the replicated
     //    tables of k_tables: word m < 16 of row c is LUT[m][c]) and the
     //    extremes of each subspace; a thread keeps one subspace m
@@ -572,8 +448,7 @@ __device__ __forceinline__ void pair_item(uint8_t* smem, const float* __restrict
     tkA.init(tkbufA + warp * 2 * KP, k, lane, ctab);
     tkB.init(tkbufB + warp * 2 * KP, k, lane, ctab + 1);
     __syncthreads();
-    const int64_t lo = (lA == hA) ? lB : ((lB == hB) ? lA : min(lA, lB));
-    const int64_t hi = max(hA, hB);
+    const int64_t lo = it.a, hi = it.b;
     CandBuf cbuf;
     {
         uint8_t* wb = cand_base + (size_t)warp * kCandWarpBytes;
@@ -593,77 +468,41 @@ __device__ __forceinline__ void pair_item(uint8_t* smem, const float* __restrict
     merge_warps<KP, kPairWarps>(tkB, tkbufB, k, lane, warp, outB);
 }
 
-// Persistent: one CTA per SM takes work items (pair slot, chunk) in the
-// order of a (slot, chunk) grid, chunk-major, from a counter that
-// k_pair_items zeroes: the CTAs that run together still walk the same chunk,
-// and no SM idles through a ragged last wave of long items (a 1024-CTA grid
-// over 152 SMs left 0.26 of its last wave empty on the dense bin).
+// Persistent: one CTA per SM takes work items, so no SM idles through a ragged
+// last wave of long ones (512 pairs as one item each over 152 SMs left the last
+// of 3.4 waves 0.6 empty).
 template <int KP>
 __global__ void __launch_bounds__(kPairThreads, 1)
-k_scan_list_pair(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __restrict__ plan,
-                 const PairItem* __restrict__ items, int n_slots, unsigned* __restrict__ counter, int k,
-                 ScanShape sh, uint64_t* __restrict__ partials) {
+k_scan_list_pair(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __restrict__ plan, int k,
+                 ScanSched sched) {
     extern __shared__ __align__(256) uint8_t smem[];
-    volatile unsigned* s_item = reinterpret_cast<volatile unsigned*>(smem + scan_pair_item_offset(KP));
-    const unsigned total = (unsigned)n_slots * (unsigned)sh.n_chunks;
-    for (;;) {
-        if (threadIdx.x == 0) *s_item = atomicAdd(counter, 1u);
-        __syncthreads();
-        const unsigned w = *s_item;
-        __syncthreads();   // read by all before thread 0 takes the next item
-        if (w >= total) break;
-        pair_item<KP>(smem, tables, sc, plan, items, k, sh, partials, (int)(w % (unsigned)n_slots),
-                      (int)(w / (unsigned)n_slots));
-        __syncthreads();   // the next item reuses the shared memory
-    }
-}
-
-size_t scan_list_workspace_bytes(int64_t nq) {
-    // pair slots (each segment rounds its count up), a flag per query, the
-    // two-query kernel's work counter
-    return (size_t)(nq + 2 * kPairSeg) * sizeof(PairItem) + (size_t)nq + 64;
+    for (ItemLoop loop(sched, 2, smem + scan_pair_item_offset(KP)); loop.more(); loop.next())
+        pair_item<KP>(smem, tables, sc, plan, loop.items[loop.at], k, sched.partials);
 }
 
 template <int KP>
-static cudaError_t launch_pairs_kp(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                                   const ScanShape& sh, uint64_t* partials, uint8_t* work, int64_t pair_min_rows,
-                                   cudaStream_t s, const uint8_t** paired, int* launches) {
+static cudaError_t launch_pairs_kp(const float* tab, SortedCols sc, const ScanPlan* plan, int k,
+                                   const ScanSched& sched, cudaStream_t s) {
     const size_t ps = scan_pair_smem_bytes(KP);
-    if (ps > (size_t)max_smem_optin()) return cudaSuccess;   // no pairs: one query per CTA
-    PairItem* items = reinterpret_cast<PairItem*>(work);
-    uint8_t* pd = reinterpret_cast<uint8_t*>(items + nq + 2 * kPairSeg);
-    unsigned* counter = reinterpret_cast<unsigned*>(work + (((size_t)(nq + 2 * kPairSeg) * sizeof(PairItem) +
-                                                             (size_t)nq + 15) / 16) * 16);
-    const unsigned segs = (unsigned)((nq + kPairSeg - 1) / kPairSeg);
-    k_pair_items<<<segs, kPairSortThreads, 0, s>>>(plan, nq, pair_min_rows, items, pd, counter);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_scan_list_pair<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps);
     if (e != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_scan_list_pair<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps)) !=
-        cudaSuccess)
-        return e;
-    int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int n_slots = (int)((nq + 1) / 2);   // at most nq / 2 pairs
-    const long long items_total = (long long)n_slots * sh.n_chunks;
-    const int grid = (int)(items_total < sms ? items_total : sms);   // one CTA per SM
-    k_scan_list_pair<KP><<<grid, kPairThreads, ps, s>>>(tab, sc, plan, items, n_slots, counter, k, sh, partials);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    *paired = pd;
-    *launches += 2;
-    return cudaSuccess;
+    k_scan_list_pair<KP><<<item_grid(sched.group[2]), kPairThreads, ps, s>>>(tab, sc, plan, k, sched);
+    return cudaGetLastError();
 }
 
-cudaError_t launch_pairs(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                         const ScanShape& sh, uint64_t* partials, uint8_t* work, int64_t pair_min_rows,
-                         cudaStream_t s, const uint8_t** paired, int* launches) {
-    *paired = nullptr;
+bool scan_pairs_fit(const ScanShape& sh, int k) {
+    return fixed_m(sh) == 16 && scan_pair_smem_bytes(scan_kp(k)) <= (size_t)max_smem_optin();
+}
+
+cudaError_t launch_scan_pairs(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
+                              const ScanShape&, const ScanSched& sched, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     switch (scan_kp(k)) {
-        case 32: return launch_pairs_kp<32>(tab, sc, plan, nq, k, sh, partials, work, pair_min_rows, s, paired, launches);
-        case 64: return launch_pairs_kp<64>(tab, sc, plan, nq, k, sh, partials, work, pair_min_rows, s, paired, launches);
-        case 128: return launch_pairs_kp<128>(tab, sc, plan, nq, k, sh, partials, work, pair_min_rows, s, paired, launches);
-        default: return launch_pairs_kp<256>(tab, sc, plan, nq, k, sh, partials, work, pair_min_rows, s, paired, launches);
+        case 32: return launch_pairs_kp<32>(tab, sc, plan, k, sched, s);
+        case 64: return launch_pairs_kp<64>(tab, sc, plan, k, sched, s);
+        case 128: return launch_pairs_kp<128>(tab, sc, plan, k, sched, s);
+        default: return launch_pairs_kp<256>(tab, sc, plan, k, sched, s);
     }
 }
 

@@ -44,3 +44,40 @@ def test_fused_tables_equal_separate_stages(ifvs, M, K, ds, cond):
             for x, y in zip(a, b):
                 np.testing.assert_array_equal(x, y)
     g.close()
+
+
+@pytest.mark.parametrize("M,k", [(16, 10), (16, 100), (16, 200), (12, 32), (12, 33), (8, 1), (10, 64), (34, 10),
+                                 (120, 128)])
+def test_results_do_not_depend_on_the_split(ifvs, M, k):
+    """Work items of any size, pairs or none, one query or more than a sorting
+    segment per batch: the same ids, distances and counts."""
+    rng = np.random.default_rng(M + k)
+    N, nq, ds = 70_001, 2300, 4
+    codes = rng.integers(0, 256, (N, M), dtype=np.uint8)
+    attr = rng.integers(0, 1000, N, dtype=np.int32)
+    other = rng.integers(0, 50, N).astype(np.int16)
+    g = ifvs.Index(codes, [attr, other, attr], D=M * ds)
+    g.load_codebooks(rng.standard_normal((M, 256, ds)).astype(np.float32))
+    q = rng.standard_normal((nq, M * ds)).astype(np.float32)
+    p = synth.empty_predicates(nq)
+    for i in range(nq):
+        lo = int(rng.integers(0, 1000))
+        width = int(rng.choice([0, 1, 3, 30, 300, 1000]))       # empty to all rows
+        synth.set_clause(p[i], 0, 0, synth.OP_RANGE, max(0, lo - width // 2), lo + width - width // 2)
+        p[i]["n_clauses"] = 1
+        if i % 5 == 0:                                            # the bitmap path
+            synth.set_clause(p[i], 1, 1, synth.OP_LT, int(rng.integers(0, 60)))
+            p[i]["n_clauses"] = 2
+    p[1]["n_clauses"] = 0
+    base = g.search(q, p, k, sub_batch=nq)
+    few = slice(0, 40)
+    for kw in (dict(sub_batch=152), dict(sub_batch=7), dict(chunk_blocks=1, sub_batch=300),
+               dict(pair_min_rows=1, sub_batch=nq), dict(pair_min_rows=1, chunk_blocks=9),
+               dict(flags=ifvs.IFVS_F_PLAIN_LOADS, sub_batch=600)):
+        got = g.search(q, p, k, **kw)
+        for x, y in zip(base, got):
+            np.testing.assert_array_equal(x, y)
+    one = [g.search(q[i:i + 1], p[i:i + 1], k) for i in range(nq)[few]]
+    for j in range(3):
+        np.testing.assert_array_equal(base[j][few], np.concatenate([o[j] for o in one]))
+    g.close()
