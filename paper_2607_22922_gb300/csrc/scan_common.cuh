@@ -115,45 +115,97 @@ __device__ __forceinline__ void warp_merge_low(uint64_t* a, int n, int lane) {
     __syncwarp();
 }
 
+__device__ __forceinline__ uint64_t min_max_step(uint64_t x, int j, bool low) {
+    const uint64_t y = __shfl_xor_sync(0xFFFFFFFFu, x, j);
+    return (x < y) == low ? x : y;
+}
+
+// 32 keys, one per lane, descending
+__device__ __forceinline__ uint64_t sort32_down(uint64_t c, int lane) {
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+        for (int j = size >> 1; j > 0; j >>= 1) c = min_max_step(c, j, ((lane & j) == 0) != ((lane & size) == 0));
+    return c;
+}
+
+// ---- the bound shared by a CTA's warps ----------------------------------------
+//
+// NW warps of a CTA serve one query.  share[0] is the bound, share[1 + w] the
+// smallest (kw + 1)-th key that warp w has published, kw + 1 = ceil(k / NW).
+// Two kinds of key bound the CTA's k-th from above: any warp's own k-th key
+// (it holds k distinct rows), and, once every warp has published, the largest
+// of the published keys (NW ceil(k / NW) >= k distinct rows are at or below
+// it).  The second is close to the CTA's true k-th key, as a warp's own k-th
+// over an NW-th of the rows is not: a warp then offers about ceil(k / NW)
+// rows per e-fold of rows instead of k.  A row above the bound cannot be in the
+// CTA's top-k, so the lists still hold every row of it; the rows at the bound
+// are in a list already.
+template <int NW>
+__device__ __forceinline__ void share_publish(uint64_t* share, uint64_t own_kth, uint64_t own_kw, int lane) {
+    const int warp = (int)(threadIdx.x >> 5);
+    if (lane == 0) *reinterpret_cast<volatile uint64_t*>(share + 1 + warp) = own_kw;
+    __syncwarp();
+    uint64_t b = lane < NW ? *reinterpret_cast<volatile uint64_t*>(share + 1 + lane) : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t y = __shfl_xor_sync(0xFFFFFFFFu, b, o);
+        b = y > b ? y : b;
+    }
+    b = own_kth < b ? own_kth : b;
+    if (lane == 0 && b != ~0ull) atomicMin(reinterpret_cast<unsigned long long*>(share), b);
+}
+
+constexpr size_t share_bytes(int warps) { return (size_t)(1 + warps) * 8; }
+
+// before a barrier, by the CTA's first threads
+template <int NW>
+__device__ __forceinline__ void share_init(uint64_t* share) {
+    if (threadIdx.x <= NW) share[threadIdx.x] = ~0ull;
+}
+
 // Merges a warp's candidates [KP, 2KP) of buf into its sorted list [0, KP),
-// clears the candidates, publishes the new k-th key to the CTA's bound (if
-// any) and returns it.  The candidates are sorted and the KP smallest of both
-// runs kept by one bitonic merge (half the compare-exchanges of one sort of
-// 2 KP; 10^8 rows at KP = 128: 0.1 % and 1 % bins 1.51 -> 1.41 and 4.33 ->
-// 4.04 ms).  Out of line: the scan loops offer keys at many sites and flush
-// rarely, and one copy of the sort keeps their code small (instruction-fetch
-// stalls led the two-query kernel's profile).
-template <int KP>
-__device__ __noinline__ uint64_t flush_list(uint64_t* buf, int k, uint64_t* cta, int lane) {
+// clears the candidates, publishes (NW > 0) and returns the new k-th key.  The
+// candidates are sorted and the KP smallest of both runs kept by one bitonic
+// merge (half the compare-exchanges of one sort of 2 KP; 10^8 rows at KP = 128:
+// 0.1 % and 1 % bins 1.51 -> 1.41 and 4.33 -> 4.04 ms).  Out of line: the scan
+// loops offer keys at many sites and flush rarely, and one copy of the sort
+// keeps their code small (instruction-fetch stalls led the two-query kernel's
+// profile).
+template <int KP, int NW>
+__device__ __noinline__ uint64_t flush_list(uint64_t* buf, int k, int kw, uint64_t* share, int lane) {
     warp_sort(buf + KP, KP, lane);
     warp_merge_low(buf, KP, lane);
     const uint64_t thr = buf[k - 1];
     for (int i = KP + lane; i < 2 * KP; i += 32) buf[i] = ~0ull;
-    if (cta != nullptr && lane == 0 && thr != ~0ull) atomicMin(reinterpret_cast<unsigned long long*>(cta), thr);
+    if constexpr (NW > 0) share_publish<NW>(share, thr, buf[kw], lane);
     __syncwarp();
     return thr;
 }
 
-// The warps of a CTA that serve one query share a bound `cta` (shared
-// memory): the smallest k-th key any of them has published.  A warp's list
-// holds k distinct rows, so its k-th key is at least the CTA's true k-th
-// key, and a row whose key is above some warp's k-th key cannot be in the
-// CTA's top-k: each warp offers only keys below min(own k-th, cta).  The
-// warps' lists then still contain every row of the CTA's top-k, and the
-// shared bound lets every warp drop rows as early as the whole CTA could.
-template <int KP>
+// A warp's first 32 candidates: enough for a first published key.
+template <int NW>
+__device__ __noinline__ void publish_first(const uint64_t* cand, int kw, uint64_t* share, int lane) {
+    const uint64_t c = sort32_down(cand[lane], lane);
+    share_publish<NW>(share, ~0ull, __shfl_sync(0xFFFFFFFFu, c, 31 - kw), lane);
+}
+
+template <int KP, int NW = 0>
 struct WarpTopK {
     uint64_t* buf;   // [0, KP): sorted best keys; [KP, 2KP): candidates
-    uint64_t* cta;   // shared bound of the CTA's warps for this query, or null
+    uint64_t* share; // the CTA's shared bound for this query (NW > 0)
     int cnt;
-    int k;
-    uint64_t thr;    // keys below thr are offered: min(own k-th key, *cta)
+    int k, kw;
+    bool first;      // nothing published yet
+    uint64_t thr;    // keys below thr are offered: min(own k-th key, shared bound)
 
-    __device__ __forceinline__ void init(uint64_t* b, int k_, int lane, uint64_t* cta_ = nullptr) {
+    __device__ __forceinline__ void init(uint64_t* b, int k_, int lane, uint64_t* share_ = nullptr) {
         buf = b;
-        cta = cta_;
+        share = share_;
         k = k_;
+        kw = NW > 0 ? (k_ + NW - 1) / (NW > 0 ? NW : 1) - 1 : 0;
         cnt = 0;
+        first = NW > 0;
         thr = ~0ull;
         for (int i = lane; i < 2 * KP; i += 32) buf[i] = ~0ull;
         __syncwarp();
@@ -162,13 +214,14 @@ struct WarpTopK {
     // broadcast (measured faster than a lane-0 load and a shuffle); any value
     // a lane sees is a valid bound, so thr stays correct in every lane
     __device__ __forceinline__ void refresh(int) {
-        if (cta == nullptr) return;
-        const uint64_t t = *reinterpret_cast<volatile uint64_t*>(cta);
+        if (NW == 0) return;
+        const uint64_t t = *reinterpret_cast<volatile uint64_t*>(share);
         if (t < thr) thr = t;
     }
     __device__ __forceinline__ void flush(int lane) {
-        thr = flush_list<KP>(buf, k, cta, lane);
+        thr = flush_list<KP, NW>(buf, k, kw, share, lane);
         cnt = 0;
+        first = false;
         refresh(lane);
     }
     __device__ __forceinline__ void offer(uint64_t key, bool want, int lane) {
@@ -176,6 +229,12 @@ struct WarpTopK {
         if (ball == 0) return;
         if (want) buf[KP + cnt + __popc(ball & ((1u << lane) - 1u))] = key;
         cnt += __popc(ball);
+        if (NW > 0 && first && cnt >= 32) {
+            __syncwarp();
+            publish_first<NW>(buf + KP, kw, share, lane);
+            first = false;
+            refresh(lane);
+        }
         if (cnt > KP - 32) {
             __syncwarp();
             flush(lane);
@@ -188,43 +247,36 @@ struct WarpTopK {
 // across the lanes by shuffles (15 + 6 steps of about 25 cycles; the sort of 64
 // keys in shared memory took three times as long and ran for every offer).
 // Out of line, as flush_list.
-__device__ __forceinline__ uint64_t min_max_step(uint64_t x, int j, bool low) {
-    const uint64_t y = __shfl_xor_sync(0xFFFFFFFFu, x, j);
-    return (x < y) == low ? x : y;
-}
 // `mine` ascending over the lanes, `c` any: the 32 smallest keys of both, ascending
 static __device__ __noinline__ uint64_t absorb32(uint64_t mine, uint64_t c, int lane) {
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1)
-#pragma unroll
-        for (int j = size >> 1; j > 0; j >>= 1)
-            c = min_max_step(c, j, ((lane & j) == 0) != ((lane & size) == 0));   // descending in the end
+    c = sort32_down(c, lane);
     mine = c < mine ? c : mine;
 #pragma unroll
     for (int j = 16; j > 0; j >>= 1) mine = min_max_step(mine, j, (lane & j) == 0);
     return mine;
 }
 
-template <>
-struct WarpTopK<32> {
+template <int NW>
+struct WarpTopK<32, NW> {
     uint64_t* buf;   // candidates, 64 slots
-    uint64_t* cta;   // as above
+    uint64_t* share;
     int cnt;
-    int k;
+    int k, kw;
     uint64_t thr;
     uint64_t mine;   // the lane's key of the sorted list
 
-    __device__ __forceinline__ void init(uint64_t* b, int k_, int, uint64_t* cta_ = nullptr) {
+    __device__ __forceinline__ void init(uint64_t* b, int k_, int, uint64_t* share_ = nullptr) {
         buf = b;
-        cta = cta_;
+        share = share_;
         k = k_;
+        kw = NW > 0 ? (k_ + NW - 1) / (NW > 0 ? NW : 1) - 1 : 0;
         cnt = 0;
         thr = ~0ull;
         mine = ~0ull;
     }
     __device__ __forceinline__ void refresh(int) {
-        if (cta == nullptr) return;
-        const uint64_t t = *reinterpret_cast<volatile uint64_t*>(cta);
+        if (NW == 0) return;
+        const uint64_t t = *reinterpret_cast<volatile uint64_t*>(share);
         if (t < thr) thr = t;
     }
     __device__ __forceinline__ void drain(int n, int lane) {
@@ -234,8 +286,7 @@ struct WarpTopK<32> {
         __syncwarp();   // the drained slots take the next candidates
         mine = absorb32(mine, c, lane);
         thr = __shfl_sync(0xFFFFFFFFu, mine, k - 1);
-        if (cta != nullptr && lane == 0 && thr != ~0ull)
-            atomicMin(reinterpret_cast<unsigned long long*>(cta), thr);
+        if (NW > 0) share_publish<(NW > 0 ? NW : 1)>(share, thr, __shfl_sync(0xFFFFFFFFu, mine, kw), lane);
         refresh(lane);
     }
     __device__ __forceinline__ void flush(int lane) {
@@ -399,9 +450,8 @@ __device__ __forceinline__ void lookup_rows(const uint8_t* __restrict__ codes, c
 
 // merge the warps' lists of one query pairwise (both sorted: one bitonic merge
 // per level); warp 0 writes k keys
-template <int KP, int WARPS>
-__device__ __forceinline__ void merge_warps(WarpTopK<KP>& tk, uint64_t* tkbuf, int k, int lane, int warp,
-                                            uint64_t* out) {
+template <int KP, int WARPS, class TK>
+__device__ __forceinline__ void merge_warps(TK& tk, uint64_t* tkbuf, int k, int lane, int warp, uint64_t* out) {
     tk.flush(lane);
     if constexpr (KP == 32) {
         __syncwarp();

@@ -20,13 +20,13 @@ namespace ifvs {
 // bitmap path's, so the two agree to float32 rounding.
 
 size_t scan_list_smem_bytes(int tab_words, int kp) {
-    return (size_t)256 * tab_words * 4 + (size_t)kScanWarps * 2 * kp * 8 + 32;
+    return (size_t)256 * tab_words * 4 + (size_t)kScanWarps * 2 * kp * 8 + share_bytes(kScanWarps) + 24;
 }
 
-template <int KP, int MM, bool FAST>
+template <int KP, int MM, bool FAST, class TK>
 __device__ __forceinline__ void scan_positions(const uint8_t* __restrict__ codes, const uint32_t* __restrict__ rows,
                                                int64_t a, int64_t b, uint32_t r0, uint32_t r1, uint32_t base,
-                                               WarpTopK<KP>& tk, int lane, int warp) {
+                                               TK& tk, int lane, int warp) {
     const uint32_t tb = 4u * (uint32_t)lane;
     const uint64_t keep = policy_evict_last();
     // positions fit in 32 bits: N < 2^32 - 2048
@@ -75,10 +75,10 @@ k_scan_list(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __r
     constexpr int S = 64;
     float* tab = reinterpret_cast<float*>(smem);
     uint64_t* tkbuf = reinterpret_cast<uint64_t*>(smem + (size_t)256 * S * 4);
-    uint64_t* cta = tkbuf + kScanWarps * 2 * KP;
+    uint64_t* share = tkbuf + kScanWarps * 2 * KP;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab);
-    for (ItemLoop loop(sched, 0, cta + 2); loop.more(); loop.next()) {
+    for (ItemLoop loop(sched, 0, share + 1 + kScanWarps); loop.more(); loop.next()) {
         const ScanItem item = loop.items[loop.at];
         const ScanPlan p = plan[item.qa];
         {
@@ -86,9 +86,9 @@ k_scan_list(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __r
             float4* dst = reinterpret_cast<float4*>(tab);
             for (int i = threadIdx.x; i < 64 * S; i += kScanThreads) dst[i] = __ldg(src + i);
         }
-        if (threadIdx.x == 0) *cta = ~0ull;
-        WarpTopK<KP> tk;
-        tk.init(tkbuf + warp * 2 * KP, k, lane, cta);
+        share_init<kScanWarps>(share);
+        WarpTopK<KP, kScanWarps> tk;
+        tk.init(tkbuf + warp * 2 * KP, k, lane, share);
         __syncthreads();
         const uint8_t* codes = sc.codes_of(p.col);
         const uint32_t* rows = sc.rows_of(p.col);
@@ -124,7 +124,7 @@ static_assert(32 % kU == 0, "whole rounds per block");
 static_assert(32 * kU == kRoundRows, "a warp's round is the unit of the work lists");
 
 __host__ __device__ constexpr size_t bulk_ring_offset(int kp) {
-    return ((size_t)256 * 64 * 4 + (size_t)kScanWarps * 2 * kp * 8 + 16 + 127) / 128 * 128;
+    return ((size_t)256 * 64 * 4 + (size_t)kScanWarps * 2 * kp * 8 + (1 + kScanWarps) * 8 + 127) / 128 * 128;
 }
 
 // tiles, one barrier per tile, and the barrier of the table copy
@@ -134,12 +134,12 @@ size_t scan_bulk_smem_bytes(int kp) {
 
 // `phase`: the tile barrier's parity before this item, updated; false when a
 // wait ran out (the barrier must not be used again)
-template <int KP, int MM, bool FAST>
+template <int KP, int MM, bool FAST, class TK>
 __device__ __forceinline__ bool scan_positions_bulk(const uint8_t* __restrict__ codes,
                                                     const uint32_t* __restrict__ rows, int64_t a, int64_t b,
                                                     uint32_t r0, uint32_t r1, const float* tab, uint8_t* tile_mem,
                                                     uint32_t bar_s, uint32_t& phase, uint32_t tx_extra, int* err,
-                                                    WarpTopK<KP>& tk, int lane, int warp) {
+                                                    TK& tk, int lane, int warp) {
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab);
     const uint32_t tb = 4u * (uint32_t)lane;
     const uint64_t keep = policy_evict_last();
@@ -219,7 +219,7 @@ k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan
         if (threadIdx.x == 0) mbar_init(tbar, 1u);
         fence_mbar_init();
     }
-    uint64_t* cta = tkbuf + kScanWarps * 2 * KP;
+    uint64_t* share = tkbuf + kScanWarps * 2 * KP;
     uint32_t phase = 0u, tphase = 0u;
     for (ItemLoop loop(sched, 0, bars_all + kScanWarps + 1); loop.more(); loop.next()) {
         const ScanItem item = loop.items[loop.at];
@@ -230,11 +230,11 @@ k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan
             mbar_arrive_expect_tx(tbar, 256u * 64u * 4u);
             bulk_g2s((uint32_t)__cvta_generic_to_shared(tab), tables + item.qa * (int64_t)256 * 64, 256u * 64u * 4u,
                      tbar, policy_evict_first());
-            *cta = ~0ull;
         }
+        share_init<kScanWarps>(share);
         const ScanPlan p = plan[item.qa];
-        WarpTopK<KP> tk;
-        tk.init(tkbuf + warp * 2 * KP, k, lane, cta);
+        WarpTopK<KP, kScanWarps> tk;
+        tk.init(tkbuf + warp * 2 * KP, k, lane, share);
         __syncthreads();
         bool ok = mbar_wait_warp(tbar, tphase);
         if (!ok) {
@@ -272,7 +272,7 @@ k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan
 // 256 queries on 5 x 10^5 rows at M = 120, pools of 10 %: 866 us with tiles, 370 us
 // here.
 size_t scan_gen_smem_bytes(int tab_words, int kp, int warps) {
-    return (size_t)256 * tab_words * 4 + (size_t)warps * 2 * kp * 8 + 32;
+    return (size_t)256 * tab_words * 4 + (size_t)warps * 2 * kp * 8 + share_bytes(warps) + 24;
 }
 
 constexpr int kGenWords = 4;   // words per block: 16 codes of each row
@@ -309,11 +309,11 @@ __device__ __forceinline__ uint64_t gen_block(const uint32_t (&wa)[kGenWords], c
     return acc;
 }
 
-template <int KP, int WARPS>
+template <int KP, int WARPS, class TK>
 __device__ __forceinline__ void scan_positions_gen(const uint32_t* __restrict__ codes,
                                                    const uint32_t* __restrict__ rows, int64_t a, int64_t b,
                                                    uint32_t r0, uint32_t r1, const ScanShape& sh, uint32_t base,
-                                                   WarpTopK<KP>& tk, int lane, int warp) {
+                                                   TK& tk, int lane, int warp) {
     const int M = sh.M, nw = sh.row_bytes / 4, nblk = (nw + kGenWords - 1) / kGenWords;
     const uint32_t S4 = 4u * (uint32_t)sh.tab_words, a32 = (uint32_t)a, b32 = (uint32_t)b;
     const uint64_t keep = policy_evict_last();
@@ -382,10 +382,10 @@ k_scan_list_gen(const float* __restrict__ tables, SortedCols sc, const ScanPlan*
     const int S = sh.tab_words;
     float* tab = reinterpret_cast<float*>(smem);
     uint64_t* tkbuf = reinterpret_cast<uint64_t*>(smem + (size_t)256 * S * 4);
-    uint64_t* cta = tkbuf + WARPS * 2 * KP;
+    uint64_t* share = tkbuf + WARPS * 2 * KP;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab);
-    for (ItemLoop loop(sched, 0, cta + 2); loop.more(); loop.next()) {
+    for (ItemLoop loop(sched, 0, share + 1 + WARPS); loop.more(); loop.next()) {
         const ScanItem item = loop.items[loop.at];
         const ScanPlan p = plan[item.qa];
         {
@@ -394,9 +394,9 @@ k_scan_list_gen(const float* __restrict__ tables, SortedCols sc, const ScanPlan*
 #pragma unroll 4
             for (int i = threadIdx.x; i < 64 * S; i += WARPS * 32) dst[i] = __ldg(src + i);
         }
-        if (threadIdx.x == 0) *cta = ~0ull;
-        WarpTopK<KP> tk;
-        tk.init(tkbuf + warp * 2 * KP, k, lane, cta);
+        share_init<WARPS>(share);
+        WarpTopK<KP, WARPS> tk;
+        tk.init(tkbuf + warp * 2 * KP, k, lane, share);
         __syncthreads();
         scan_positions_gen<KP, WARPS>(reinterpret_cast<const uint32_t*>(sc.codes_of(p.col)), sc.rows_of(p.col), p.a,
                                       p.b, item.a, item.b, sh, base, tk, lane, warp);

@@ -30,6 +30,7 @@ constexpr int kPairWarps = 16;
 constexpr int kPairThreads = kPairWarps * 32;
 constexpr uint32_t kTabBytes16 = 256u * 64u * 4u;    // one replicated M = 16 table
 constexpr uint32_t kExactBytes16 = 256u * 16u * 4u;  // one unreplicated table, [c][m]
+constexpr size_t kPairShare = 2 * share_bytes(kPairWarps);   // both queries' shared bounds
 constexpr int kQMax = 2047;                           // 16 * 2047 < 2^15
 
 // Deferred rescoring.  The rows of a round that pass a query's quantised
@@ -49,12 +50,15 @@ constexpr size_t kCandWarpBytes = (size_t)kCandCap * (16 + 4 + 4);
 
 __host__ __device__ constexpr bool pair_defers(int kp) { return IFVS_PAIR_DEFER != 0 && kp <= 128; }
 
+template <int KP>
+using PairTopK = WarpTopK<KP, kPairWarps>;
+
 // packed table, two exact tables, extremes + the two shared bounds, lists,
 // the candidate buffers, the current work item (no static shared memory:
 // it would move the dynamic window off the base the look-ups' immediate
 // offsets assume)
 size_t scan_pair_smem_bytes(int kp) {
-    return (size_t)kTabBytes16 + 2 * (size_t)kExactBytes16 + 64 * 4 + 16 + (size_t)kPairWarps * 2 * 2 * kp * 8 +
+    return (size_t)kTabBytes16 + 2 * (size_t)kExactBytes16 + 64 * 4 + kPairShare + (size_t)kPairWarps * 2 * 2 * kp * 8 +
            (pair_defers(kp) ? (size_t)kPairWarps * kCandWarpBytes : 0) + 16;
 }
 
@@ -184,8 +188,8 @@ struct CandBuf {
 // offers (warp-collective).
 template <int KP>
 __device__ __forceinline__ void rescore_entries(const CandBuf& cbuf, int first, int n,
-                                                const uint32_t* __restrict__ rows, WarpTopK<KP>& tkA,
-                                                WarpTopK<KP>& tkB, const float* exA, const float* exB, int lane) {
+                                                const uint32_t* __restrict__ rows, PairTopK<KP>& tkA,
+                                                PairTopK<KP>& tkB, const float* exA, const float* exB, int lane) {
     uint4 c = make_uint4(0, 0, 0, 0);
     uint32_t pos = 0u, f = 0u;
     if (lane < n) {
@@ -226,8 +230,8 @@ __device__ __forceinline__ void pair_load(const uint8_t* __restrict__ codes, uin
 // distances and top-k offers for the candidates.
 template <int KP, bool FAST, bool MASKED>
 __device__ __forceinline__ void pair_round(const uint4 (&c)[kU2], const uint32_t* __restrict__ rows,
-                                           uint32_t pos0, const uint32_t (&mask)[kU2], WarpTopK<KP>& tkA,
-                                           WarpTopK<KP>& tkB, const float* exA, const float* exB, float slA,
+                                           uint32_t pos0, const uint32_t (&mask)[kU2], PairTopK<KP>& tkA,
+                                           PairTopK<KP>& tkB, const float* exA, const float* exB, float slA,
                                            float invA, float slB, float invB, uint32_t tb, uint32_t base,
                                            int rot, int lane, uint32_t& Tpk, CandBuf& cbuf) {
     {
@@ -293,7 +297,7 @@ template <int KP, bool FAST>
 __device__ __forceinline__ void scan_positions_pair(const uint8_t* __restrict__ codes,
                                                     const uint32_t* __restrict__ rows, int64_t aA,
                                                     int64_t bA, int64_t aB, int64_t bB, int64_t blk0,
-                                                    int64_t blk1, WarpTopK<KP>& tkA, WarpTopK<KP>& tkB,
+                                                    int64_t blk1, PairTopK<KP>& tkA, PairTopK<KP>& tkB,
                                                     const float* exA, const float* exB, float slA, float invA,
                                                     float slB, float invB, uint32_t base, int lane, int warp,
                                                     CandBuf& cbuf) {
@@ -373,7 +377,7 @@ __device__ __forceinline__ void quant_params(const float* lo, const float* hi, f
 
 // Offset of the current work item in the two-query kernel's shared memory.
 __host__ __device__ constexpr size_t scan_pair_item_offset(int kp) {
-    return (size_t)kTabBytes16 + 2 * (size_t)kExactBytes16 + 64 * 4 + 16 + (size_t)kPairWarps * 2 * 2 * kp * 8 +
+    return (size_t)kTabBytes16 + 2 * (size_t)kExactBytes16 + 64 * 4 + kPairShare + (size_t)kPairWarps * 2 * 2 * kp * 8 +
            (pair_defers(kp) ? (size_t)kPairWarps * kCandWarpBytes : 0);
 }
 
@@ -386,8 +390,9 @@ __device__ __forceinline__ void pair_item(uint8_t* smem, const float* __restrict
     float* exA = reinterpret_cast<float*>(smem + kTabBytes16);
     float* exB = reinterpret_cast<float*>(smem + kTabBytes16 + kExactBytes16);
     float* prm = reinterpret_cast<float*>(smem + kTabBytes16 + 2 * kExactBytes16);   // lo/hi of A, lo/hi of B
-    uint64_t* ctab = reinterpret_cast<uint64_t*>(smem + kTabBytes16 + 2 * kExactBytes16 + 64 * 4);   // A, B
-    uint64_t* tkbufA = reinterpret_cast<uint64_t*>(smem + kTabBytes16 + 2 * kExactBytes16 + 64 * 4 + 16);
+    uint64_t* shareA = reinterpret_cast<uint64_t*>(smem + kTabBytes16 + 2 * kExactBytes16 + 64 * 4);
+    uint64_t* shareB = shareA + 1 + kPairWarps;
+    uint64_t* tkbufA = reinterpret_cast<uint64_t*>(smem + kTabBytes16 + 2 * kExactBytes16 + 64 * 4 + kPairShare);
     uint64_t* tkbufB = tkbufA + kPairWarps * 2 * KP;
     float* red = reinterpret_cast<float*>(tkbufA);   // [warp][4][16], before the lists are set up
     uint8_t* cand_base = reinterpret_cast<uint8_t*>(tkbufB + kPairWarps * 2 * KP);   // 16-byte aligned
@@ -443,10 +448,11 @@ __device__ __forceinline__ void pair_item(uint8_t* smem, const float* __restrict
         ptab[i] = quant12(exA[c * 16 + m], prm[m], invA) | quant12(exB[c * 16 + m], prm[32 + m], invB) << 16;
     }
     __syncthreads();   // the reduction scratch becomes the lists
-    if (threadIdx.x < 2) ctab[threadIdx.x] = ~0ull;
-    WarpTopK<KP> tkA, tkB;
-    tkA.init(tkbufA + warp * 2 * KP, k, lane, ctab);
-    tkB.init(tkbufB + warp * 2 * KP, k, lane, ctab + 1);
+    share_init<kPairWarps>(shareA);
+    share_init<kPairWarps>(shareB);
+    PairTopK<KP> tkA, tkB;
+    tkA.init(tkbufA + warp * 2 * KP, k, lane, shareA);
+    tkB.init(tkbufB + warp * 2 * KP, k, lane, shareB);
     __syncthreads();
     const int64_t lo = it.a, hi = it.b;
     CandBuf cbuf;
