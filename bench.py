@@ -47,7 +47,9 @@ if ROOT not in sys.path:
 
 WORKLOAD = "gmm100m-d128-m16"
 LIST_DEFAULT_PPM = 1000000   # the library's default sorted-copy threshold (always)
-PAIR_DEFAULT_ROWS = 1 << 22  # the library's default span from which ranges pair
+# the library's automatic pairing: rows a pair spans and rows a batch's ranges
+# hold together, at least, for k <= 32 and above
+PAIR_AUTO = {True: (160_000, 30_000_000), False: (300_000, 90_000_000)}
 TRAIN_WORKLOAD = "sift1m-d128-m16"
 CPU_SAMPLE_ROWS = 10_000_000
 
@@ -506,12 +508,13 @@ def sorted_path(preds, attrs, npass, list_rows):
     return out
 
 
-def scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, seg=2048):
+def scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, pair_total=0, seg=2048):
     """Shared-memory look-ups the scan stage executes for one batch, by the
     library's pairing rule for one-column ranges of the sorted copy (M = 16;
     sort by (column, range start, query) per 2048-query segment; neighbours
     2j, 2j+1 pair when 3/4 of the longer range is common and the two span at
-    least pair_rows): a pair costs the union of its ranges x M (one load
+    least pair_rows, in batches whose ranges hold pair_total rows or more): a
+    pair costs the union of its ranges x M (one load
     serves both queries), any other query its pool x M."""
     n = len(qs.q)
     a = np.zeros(n, np.int64)
@@ -540,7 +543,7 @@ def scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, seg=2048):
         span = max(b[x], b[y]) - min(a[x], a[y])
         return 4 * common >= 3 * max(lx, ly) and span >= pair_rows
 
-    if w.M == 16 and pair_rows >= 0:
+    if w.M == 16 and pair_rows >= 0 and (b - a).sum() >= pair_total:
         for s0 in range(0, n, seg):
             idx = [i for i in range(s0, min(n, s0 + seg)) if on_list[i]]
             idx.sort(key=lambda i: (col[i], a[i], i))
@@ -656,7 +659,7 @@ def run_ifvs(args):
     n_blocks = (w.N + 1023) // 1024
     ppm = args.list_max_ppm if args.list_max_ppm != 0 else LIST_DEFAULT_PPM
     list_rows = -1 if ppm < 0 else w.N * ppm // 1000000
-    pair_rows = args.pair_min_rows if args.pair_min_rows != 0 else PAIR_DEFAULT_ROWS
+    pair_rows, pair_total = (args.pair_min_rows, 0) if args.pair_min_rows != 0 else PAIR_AUTO[w.k <= 32]
     lookups_total = code_bytes_total = 0.0
     sorted_vals = [np.sort(a) for a in ix.attrs]
     for b, qs in enumerate(batches):
@@ -664,7 +667,7 @@ def run_ifvs(args):
         npass = dev_out[b][2].cpu().numpy().astype(np.float64)
         nsteps_b = len(ms_b)
         on_list = sorted_path(qs.preds, ix.attrs, npass, list_rows)
-        lk = scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows)
+        lk = scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, pair_total)
         lookups_total += nsteps_b * lk["lookups"]
         code_bytes_total += nsteps_b * float(npass.sum()) * w.M
         per_bin[str(qs.sel)] = {

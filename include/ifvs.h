@@ -142,7 +142,9 @@ typedef struct {
                            (tables quantised to 11 bits; every row that can
                            reach a top-k is rescored exactly, so results
                            equal those of one query per CTA bit for bit).
-                           0: default (4194304); -1: never pair.             */
+                           0: automatic (spans of at least 160000 rows in
+                           batches whose ranges hold 3e7 together, 300000
+                           and 9e7 for k > 32); -1: never pair.            */
     void* stream;       /* cudaStream_t to run on; NULL: the index's stream   */
 } ifvs_search_params;
 

@@ -407,11 +407,22 @@ struct Opts {
 // generic-M loop (10^6 x 120 codes)
 constexpr int32_t kListDefaultPpm = 1000000;
 
-// two-query CTAs for ranges that together span at least 2^22 rows: on the
-// 10^8-row workload pairs were faster at 10 % and 100 % of the rows
-// (10^7, 10^8) and slower at 0.1 % and 1 % (10^5, 10^6) than one query per
-// CTA, which holds two or three CTAs per SM
-constexpr int64_t kPairDefaultMinRows = int64_t(1) << 22;
+// Which ranges share a CTA when the caller sets no span.  A pair item costs
+// more to start than a single one (two tables quantised, twice the lists) and
+// one of its CTAs fills an SM, so it needs long ranges and enough of them to
+// fill the GPU.  Measured (us per batch, single / paired): k = 10, 1024
+// queries: spans of 10^5 407 / 408, 2 x 10^5 648 / 533, 4 x 10^5 1158 / 846;
+// 64 queries: 4 x 10^5 165 / 174, 5 x 10^5 170 / 156, 10^6 262 / 193.
+// k = 100, 1024 queries: 2 x 10^5 912 / 985, 4 x 10^5 1541 / 1443; 64
+// queries: 4 x 10^5 233 / 320, 10^6 337 / 325, 2 x 10^6 561 / 466.
+struct PairRule {
+    int64_t span;      // rows a pair spans, at least
+    int64_t total;     // rows of the batch's ranges together, at least
+};
+PairRule pair_rule(int32_t pair_min_rows, int k) {
+    if (pair_min_rows > 0) return {pair_min_rows, 0};
+    return k <= 32 ? PairRule{160000, 30000000} : PairRule{300000, 90000000};
+}
 
 int parse_opts(const ifvs_search_params* p, Opts* o) {
     if (!p) return 0;
@@ -522,11 +533,11 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     TRY(ensure(ix->w_wf, sizeof(float) * n * ix->D));
     TRY(ensure(ix->w_tab, sizeof(float) * n * 256 * ix->tab_words));
     const ScanShape sh = scan_shape(ix);
-    // pairs need two queries that together span pair_min_rows of the index's
-    // rows; with stage timing every kernel of the path is launched
-    const int64_t pair_min = o.pair_min_rows > 0 ? o.pair_min_rows : kPairDefaultMinRows;
+    // where no pair can arise its kernel is not launched (with stage timing
+    // every kernel of the path is)
+    const PairRule pr = pair_rule(o.pair_min_rows, kk);
     const bool pairs = list_on && o.pair_min_rows >= 0 && scan_pairs_fit(sh, kk) &&
-                       (o.timing || (n > 1 && ix->N >= pair_min));
+                       (o.timing || (n > 1 && ix->N >= pr.span && n * ix->N >= pr.total));
     ScanSched sched;
     TRY(make_sched(ix, sh, n, kk, o, list_on, bitmaps, pairs, &sched));
     if (o.R > 0) {
@@ -584,7 +595,7 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     }
     {
         Stage st(ix, s, o.timing, pairs ? IFVS_STAGE_SCAN : IFVS_STAGE_LAYOUT);
-        CUDA_TRY(st.end(launch_schedule(plan, npass_u64, n, ix->n_blocks, pairs ? pair_min : -1, sched, s)));
+        CUDA_TRY(st.end(launch_schedule(plan, npass_u64, n, ix->n_blocks, pairs ? pr.span : -1, pr.total, sched, s)));
     }
     if (bitmaps) {
         Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
@@ -600,6 +611,7 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
         lo.bulk = !o.plain_loads;
         lo.tx_extra = stall_copies_for_tests() ? 16u : 0u;
         lo.err = ix->w_err.as<int>();
+        lo.after_pairs = pairs && !o.timing;
         CUDA_TRY(st.end(launch_scan_list(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, lo, s)));
     }
     int64_t* m_ids = o.R > 0 ? ix->w_cand.as<int64_t>() : out_ids;
@@ -1266,7 +1278,7 @@ int ifvs_scan_topk(ifvs_index* ix, const float* lut, const uint32_t* bitmaps, in
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_LAYOUT);
-            CUDA_TRY(st.end(launch_schedule(nullptr, nullptr, n, ix->n_blocks, -1, sched, s)));
+            CUDA_TRY(st.end(launch_schedule(nullptr, nullptr, n, ix->n_blocks, -1, 0, sched, s)));
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);

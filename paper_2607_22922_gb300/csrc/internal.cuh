@@ -254,9 +254,10 @@ struct ScanSched {
 size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)[3], int64_t chunk_blocks,
                          const int64_t (&most)[3], uint8_t* base, ScanSched* s);
 // plan null: every query on the bitmap path; npass null: pass counts unknown;
-// pair_min_rows < 0: no pairs
+// pair_min_rows < 0: no pairs; nor where the sorted-copy ranges together hold
+// fewer than pair_min_total rows
 cudaError_t launch_schedule(const ScanPlan* plan, const unsigned long long* npass, int64_t nq, int64_t n_blocks,
-                            int64_t pair_min_rows, const ScanSched& s, cudaStream_t st);
+                            int64_t pair_min_rows, int64_t pair_min_total, const ScanSched& s, cudaStream_t st);
 
 // Rank over the bitmap group's items: per item, the k best keys (dist bits <<
 // 32 | row) of its blocks' passing rows; `tab` holds the tables written by
@@ -272,6 +273,7 @@ struct ListOpts {
     bool bulk;
     uint32_t tx_extra;
     int* err;
+    bool after_pairs;   // launched right after launch_scan_pairs: may overlap it
 };
 cudaError_t launch_scan_list(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
                              const ScanShape& sh, const ScanSched& sched, const ListOpts& lo, cudaStream_t s);

@@ -603,6 +603,14 @@ struct ItemLoop {
     }
 };
 
+// The one-query scan overlaps the two-query scan before it in the stream: they
+// share no data, and the second fills the SMs that the first leaves at its end
+// (one CTA of the first fills an SM).  The first lets the second start
+// (start_dependents), the second's CTAs end only after the first (wait_before),
+// so that what follows the second sees both.
+__device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // CTAs to launch for a group: all that fit the device, or the items there can be
 inline unsigned item_grid(const SchedGroup& g) { return (unsigned)(g.cap < g.slots ? (g.cap < 1 ? 1 : g.cap) : g.slots); }
 

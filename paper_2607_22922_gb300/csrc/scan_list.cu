@@ -98,6 +98,7 @@ k_scan_list(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __r
             scan_positions<KP, MM, false>(codes, rows, p.a, p.b, item.a, item.b, base, tk, lane, warp);
         merge_warps<KP, kScanWarps>(tk, tkbuf, k, lane, warp, sched.partials + (int64_t)item.la * k);
     }
+    wait_before();
 }
 
 // ---- sorted-copy scan with bulk-copied code tiles (M = 16) ------------------
@@ -253,8 +254,9 @@ k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan
                                                         tx_extra, err, tk, lane, warp);
         }
         merge_warps<KP, kScanWarps>(tk, tkbuf, k, lane, warp, sched.partials + (int64_t)item.la * k);
-        if (__syncthreads_or(ok ? 0 : 1)) return;   // the search reports a timeout; its lists are incomplete
+        if (__syncthreads_or(ok ? 0 : 1)) break;   // the search reports a timeout; its lists are incomplete
     }
+    wait_before();
 }
 
 // ---- generic M ----------------------------------------------------------------
@@ -405,12 +407,21 @@ k_scan_list_gen(const float* __restrict__ tables, SortedCols sc, const ScanPlan*
 }
 
 template <class Kernel, class... Args>
-static cudaError_t launch_items(Kernel kern, const ScanSched& sched, int threads, size_t smem, cudaStream_t s,
-                                Args... args) {
+static cudaError_t launch_items(Kernel kern, const ScanSched& sched, int threads, size_t smem, bool overlap,
+                                cudaStream_t s, Args... args) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<item_grid(sched.group[0]), threads, smem, s>>>(args...);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(item_grid(sched.group[0]));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 // The kernel for a shape.  M = 12 and 16: bulk copies where asked for, else
@@ -458,17 +469,17 @@ static cudaError_t launch_list_kp(const float* tab, SortedCols sc, const ScanPla
     if (lk.kind == ListKernel::kBulk) {
         auto kern = mm == 16 ? (two ? k_scan_list_bulk<KP, 16, 2> : k_scan_list_bulk<KP, 16, 1>)
                              : (two ? k_scan_list_bulk<KP, 12, 2> : k_scan_list_bulk<KP, 12, 1>);
-        return launch_items(kern, sched, threads, lk.smem, s, tab, sc, plan, k, sched, lo.tx_extra, lo.err);
+        return launch_items(kern, sched, threads, lk.smem, lo.after_pairs, s, tab, sc, plan, k, sched, lo.tx_extra, lo.err);
     }
     if (lk.kind == ListKernel::kPlain) {
         auto kern = mm == 16 ? (two ? k_scan_list<KP, 16, 2> : k_scan_list<KP, 16, 1>)
                              : (two ? k_scan_list<KP, 12, 2> : k_scan_list<KP, 12, 1>);
-        return launch_items(kern, sched, threads, lk.smem, s, tab, sc, plan, k, sched);
+        return launch_items(kern, sched, threads, lk.smem, lo.after_pairs, s, tab, sc, plan, k, sched);
     }
     auto kern = lk.warps == 24   ? k_scan_list_gen<KP, 24>
                 : lk.warps == 12 ? k_scan_list_gen<KP, 12>
                                  : k_scan_list_gen<KP, 8>;
-    return launch_items(kern, sched, threads, lk.smem, s, tab, sc, plan, k, sh, sched);
+    return launch_items(kern, sched, threads, lk.smem, lo.after_pairs, s, tab, sc, plan, k, sh, sched);
 }
 
 cudaError_t launch_scan_list(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,

@@ -371,9 +371,8 @@ __device__ __forceinline__ void quant_params(const float* lo, const float* hi, f
 // Two queries are worth one CTA when they read the same column's copy, their
 // ranges mostly coincide (at least 3/4 of the longer range is common to both;
 // the rows of only one range then run with the other query masked) and the
-// two ranges together span at least min_rows positions (the caller's choice:
-// for short ranges the one-query kernel, with two or three CTAs per SM, was
-// measured faster).  k_schedule makes the pairs (scan_sched.cu).
+// two ranges together span at least min_rows positions (pair_rule, api.cu).
+// k_schedule makes the pairs (scan_sched.cu).
 
 // Offset of the current work item in the two-query kernel's shared memory.
 __host__ __device__ constexpr size_t scan_pair_item_offset(int kp) {
@@ -482,6 +481,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
 k_scan_list_pair(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __restrict__ plan, int k,
                  ScanSched sched) {
     extern __shared__ __align__(256) uint8_t smem[];
+    start_dependents();
     for (ItemLoop loop(sched, 2, smem + scan_pair_item_offset(KP)); loop.more(); loop.next())
         pair_item<KP>(smem, tables, sc, plan, loop.items[loop.at], k, sched.partials);
 }

@@ -118,13 +118,29 @@ __device__ __forceinline__ Cut cut_of(int64_t work, int64_t n, const SchedGroup&
 
 __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __restrict__ plan,
                                                             const unsigned long long* __restrict__ npass, int64_t nq,
-                                                            int64_t n_blocks, int64_t pair_min_rows, ScanSched s) {
+                                                            int64_t n_blocks, int64_t pair_min_rows,
+                                                            int64_t pair_min_total, ScanSched s) {
     __shared__ uint64_t key[kSeg];          // pairing; then the items' prefix counts
     __shared__ int wsum[32];
     __shared__ int64_t wsum64[32];
     int* pre = reinterpret_cast<int*>(key);
     const int tid = threadIdx.x, nt = blockDim.x;
     int n_pairs = 0;
+
+    // no sort for a batch that cannot pair: 3/4 in common, a pair spans at most
+    // 5/4 of its longer range
+    if (pair_min_rows >= 0) {
+        int64_t rows = 0, wide = 0;
+        for (int64_t q = tid; q < nq; q += nt)
+            if (plan[q].list) {
+                const int64_t len = plan[q].b - plan[q].a;
+                rows += len;
+                wide += 5 * len >= 4 * pair_min_rows;
+            }
+        rows = block_sum(rows, wsum64);
+        wide = block_sum(wide, wsum64);
+        if (rows < pair_min_total || wide == 0) pair_min_rows = -1;
+    }
 
     // ---- pairs: sorted by (copy, range start, query), neighbours (2j, 2j + 1)
     if (pair_min_rows >= 0) {
@@ -349,11 +365,11 @@ size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)
 }
 
 cudaError_t launch_schedule(const ScanPlan* plan, const unsigned long long* npass, int64_t nq, int64_t n_blocks,
-                            int64_t pair_min_rows, const ScanSched& s, cudaStream_t st) {
+                            int64_t pair_min_rows, int64_t pair_min_total, const ScanSched& s, cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
     int threads = 128;
     while (threads < kSchedThreads && threads < nq) threads <<= 1;
-    k_schedule<<<1, threads, 0, st>>>(plan, npass, nq, n_blocks, plan ? pair_min_rows : -1, s);
+    k_schedule<<<1, threads, 0, st>>>(plan, npass, nq, n_blocks, plan ? pair_min_rows : -1, pair_min_total, s);
     return cudaGetLastError();
 }
 
