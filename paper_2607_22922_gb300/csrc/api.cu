@@ -161,11 +161,19 @@ struct ifvs_index {
     int h = 0, r = 0;
     size_t bytes = 0;
     // workspace
-    DevBuf w_q, w_wz, w_preds, w_canon, w_err, w_bm, w_rows, w_npass, w_idx, w_alpha, w_wf,
+    DevBuf w_q, w_wz, w_preds, w_canon, w_in, w_bm, w_rows, w_npass, w_idx, w_alpha, w_wf,
         w_lut, w_cifvs, w_part, w_ids, w_dists, w_cand, w_cdist, w_tab, w_plan;
     // training workspace
     DevBuf t_cand, t_pos, t_mined, t_mdist, t_gC, t_gw, t_loss, t_G, t_gW, t_gWpart, t_galpha,
         t_gbank, t_gwz, t_wz, t_neg;
+    // One page-locked block the device can address: the error word (kernels
+    // write it only when they find an error, so a call neither clears nor
+    // fetches one on the device), then room for the inputs and the results of
+    // small host calls, which would take three pageable copies each way.
+    uint8_t* page = nullptr;
+    uint8_t* page_dev = nullptr;
+    bool open = false;      // a call began and did not reach its synchronisation
+    int* err() const { return reinterpret_cast<int*>(page_dev); }
     // timing
     double stage_ms[IFVS_N_STAGES] = {0};
     int64_t stage_launches[IFVS_N_STAGES] = {0};
@@ -235,13 +243,14 @@ void free_index(ifvs_index* ix) {
     void* ptrs[] = {ix->d_codes, ix->d_vec, ix->d_cpq, ix->d_bank, ix->d_W, ix->d_seeds};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    DevBuf* bufs[] = {&ix->w_q, &ix->w_wz, &ix->w_preds, &ix->w_canon, &ix->w_err, &ix->w_bm,
+    DevBuf* bufs[] = {&ix->w_q, &ix->w_wz, &ix->w_preds, &ix->w_canon, &ix->w_in, &ix->w_bm,
                       &ix->w_rows, &ix->w_npass, &ix->w_idx, &ix->w_alpha, &ix->w_wf,
                       &ix->w_lut, &ix->w_cifvs, &ix->w_part, &ix->w_ids, &ix->w_dists,
                       &ix->w_cand, &ix->w_cdist, &ix->w_tab, &ix->w_plan, &ix->t_cand, &ix->t_pos,
                       &ix->t_mined, &ix->t_mdist, &ix->t_gC, &ix->t_gw, &ix->t_loss, &ix->t_G,
                       &ix->t_gW, &ix->t_gWpart, &ix->t_galpha, &ix->t_gbank, &ix->t_gwz, &ix->t_wz, &ix->t_neg};
     for (DevBuf* b : bufs) release(*b);
+    if (ix->page) cudaFreeHost(ix->page);
     for (auto& pr : ix->pending) {
         ix->ev_free.push_back(pr.second.first);
         ix->ev_free.push_back(pr.second.second);
@@ -250,6 +259,27 @@ void free_index(ifvs_index* ix) {
         if (e) cudaEventDestroy(e);
     if (ix->stream) cudaStreamDestroy(ix->stream);
     delete ix;
+}
+
+constexpr size_t kPageHead = 256;          // the error word
+constexpr size_t kPageHalf = 128 << 10;    // inputs, then results
+
+// the index's page-locked block; the error word is 0
+int make_page(ifvs_index* ix) {
+    void *h = nullptr, *d = nullptr;
+    cudaError_t e = cudaHostAlloc(&h, kPageHead + 2 * kPageHalf, cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e == cudaSuccess) {
+        ix->page = (uint8_t*)h;
+        e = cudaHostGetDevicePointer(&d, h, 0);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return set_err(IFVS_ERR_OOM, "page-locked allocation of %zu bytes failed: %s", kPageHead + 2 * kPageHalf,
+                       cudaGetErrorString(e));
+    }
+    ix->page_dev = (uint8_t*)d;
+    memset(h, 0, kPageHead);
+    return 0;
 }
 
 int dev_alloc(ifvs_index* ix, void** p, size_t bytes) {
@@ -489,7 +519,7 @@ PrepareArgs prepare_args(const ifvs_index* ix, const ifvs_predicate* dp, CanonPr
     a.preds = dp;
     a.cols = ix->cols();
     a.canon = canon;
-    a.err = ix->w_err.as<int>();
+    a.err = ix->err();
     return a;
 }
 
@@ -511,10 +541,11 @@ void prepare_condition(const ifvs_index* ix, const float* dq, const float* dwz, 
 
 // The query path for one sub-batch of n queries whose inputs are on the
 // device (w_z of query i at dwz + i * wz_stride).  Writes k ids / dists per query to out_ids / out_dists (device)
-// and the pass counts to npass_u64 (device).
+// and the pass counts to npass_u64 (device), from there to npass_copy unless
+// that is null.
 int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
              const ifvs_predicate* dp, const float* dwz, int64_t wz_stride, int64_t n, int k, int64_t* out_ids,
-             float* out_dists, unsigned long long* npass_u64) {
+             float* out_dists, unsigned long long* npass_u64, int64_t* npass_copy) {
     const int kk = o.R > 0 ? o.R : k;
     const int Mr = ix->M * ix->r;
     const bool cond = !o.plain && ix->d_bank != nullptr;
@@ -610,7 +641,7 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
         ListOpts lo;
         lo.bulk = !o.plain_loads;
         lo.tx_extra = stall_copies_for_tests() ? 16u : 0u;
-        lo.err = ix->w_err.as<int>();
+        lo.err = ix->err();
         lo.after_pairs = pairs && !o.timing;
         CUDA_TRY(st.end(launch_scan_list(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, lo, s)));
     }
@@ -618,7 +649,7 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     float* m_dists = o.R > 0 ? ix->w_cdist.as<float>() : out_dists;
     {
         Stage st(ix, s, o.timing, IFVS_STAGE_MERGE);
-        CUDA_TRY(st.end(launch_merge(sched, n, kk, m_ids, m_dists, s)));
+        CUDA_TRY(st.end(launch_merge(sched, n, kk, m_ids, m_dists, npass_u64, npass_copy, s)));
     }
     if (o.R > 0) {
         Stage st(ix, s, o.timing, IFVS_STAGE_RERANK);
@@ -696,10 +727,10 @@ int copy_out(cudaStream_t s, bool dio, void* dst, const void* src, size_t bytes)
 // Synchronise, fold the timing events, and report a malformed predicate.
 int finish(ifvs_index* ix, cudaStream_t s, bool check_preds) {
     CUDA_TRY(cudaStreamSynchronize(s));
+    ix->open = false;
     ix->collect();
     if (check_preds) {
-        int err = 0;
-        CUDA_TRY(cudaMemcpy(&err, ix->w_err.p, sizeof(int), cudaMemcpyDeviceToHost));
+        const int err = *reinterpret_cast<volatile int*>(ix->page);
         if (err & 4)
             return set_err(IFVS_ERR_TIMEOUT, "a bounded wait of the scan for its bulk-copied code tiles ran out; "
                                              "the results are incomplete");
@@ -710,9 +741,12 @@ int finish(ifvs_index* ix, cudaStream_t s, bool check_preds) {
     return 0;
 }
 
-int reset_err_flag(ifvs_index* ix, cudaStream_t s) {
-    TRY(ensure(ix->w_err, sizeof(int)));
-    CUDA_TRY(cudaMemsetAsync(ix->w_err.p, 0, sizeof(int), s));
+// A call that reads the error word begins.  Work of an earlier call that failed
+// midway may still be running and may still write the word.
+int reset_err_flag(ifvs_index* ix, cudaStream_t) {
+    if (ix->open) CUDA_TRY(cudaDeviceSynchronize());
+    *reinterpret_cast<volatile int*>(ix->page) = 0;
+    ix->open = true;
     return 0;
 }
 
@@ -830,7 +864,7 @@ TrainQueryArgs train_args(ifvs_index* ix, const ifvs_train_params* tp, int64_t n
     a.lambda = tp->lambda;
     a.n = n;
     a.N = ix->N;
-    a.err = ix->w_err.as<int>();
+    a.err = ix->err();
     a.gC = ix->t_gC.as<float>();
     a.gw = ix->t_gw.as<float>();
     a.galpha = ix->t_galpha.as<float>();
@@ -838,16 +872,22 @@ TrainQueryArgs train_args(ifvs_index* ix, const ifvs_train_params* tp, int64_t n
     return a;
 }
 
-// Mean of the per-query losses, summed in query order on the host.
-int train_loss_out(ifvs_index* ix, cudaStream_t s, int64_t n, double* loss) {
-    if (!loss) return 0;
-    std::vector<double> l((size_t)n);
-    CUDA_TRY(cudaMemcpyAsync(l.data(), ix->t_loss.p, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    double t = 0.0;
-    for (double v : l) t += v;
-    *loss = t / (double)n;
+// The per-query losses on their way to the host (at most 1024), and, after the
+// call's synchronisation, their mean, summed in query order.
+int train_loss_fetch(ifvs_index* ix, cudaStream_t s, int64_t n, const double* loss) {
+    if (loss)
+        CUDA_TRY(cudaMemcpyAsync(ix->page + kPageHead, ix->t_loss.p, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
     return 0;
+}
+void train_loss_mean(const ifvs_index* ix, int64_t n, double* loss) {
+    if (!loss) return;
+    double t = 0.0;
+    for (int64_t i = 0; i < n; ++i) {
+        double v;
+        memcpy(&v, ix->page + kPageHead + sizeof(double) * i, sizeof v);
+        t += v;
+    }
+    *loss = t / (double)n;
 }
 
 }  // namespace
@@ -984,20 +1024,17 @@ int ifvs_load_index(ifvs_index** out, int32_t device, const uint8_t* codes, int6
         return fail(rc);
     }
     ix->d_codes = (uint8_t*)dcodes;
-    if ((rc = ensure(ix->w_err, sizeof(int)))) {
+    if ((rc = make_page(ix))) {
         if (tmp) cudaFree(tmp);
         return fail(rc);
     }
-    cudaMemsetAsync(ix->w_err.p, 0, sizeof(int), s);
     cudaError_t e = launch_relayout_codes(src, N, M, K, ix->row_bytes, ix->n_rows_pad, ix->d_codes,
-                                          ix->w_err.as<int>(), s);
+                                          ix->err(), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (tmp) cudaFree(tmp);
     if (e != cudaSuccess) return fail(cuda_fail(e, "code re-layout", __LINE__));
-    int bad = 0;
-    if (cudaMemcpy(&bad, ix->w_err.p, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return fail(cuda_fail(cudaGetLastError(), "cudaMemcpy(flag)", __LINE__));
-    if (bad) return fail(set_err(IFVS_ERR_ARG, "a code is >= K = %d", K));
+    if (*reinterpret_cast<volatile int*>(ix->page) != 0)
+        return fail(set_err(IFVS_ERR_ARG, "a code is >= K = %d", K));
 
     // attribute columns, padded with zeros to n_rows_pad
     ix->n_attrs = n_attrs;
@@ -1107,6 +1144,35 @@ int ifvs_search_batch(ifvs_index* ix, const float* queries, const ifvs_predicate
     cudaStream_t s = o.stream ? o.stream : ix->stream;
     const int64_t sb = pick_sub_batch(ix, o, nq);
     TRY(reset_err_flag(ix, s));
+    if (!o.dio && nq <= sb) {
+        // a small host call: its inputs go over in one copy from the index's
+        // page-locked block and the kernels write the results into it
+        auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
+        const size_t bq = sizeof(float) * nq * ix->D, bp = sizeof(ifvs_predicate) * nq, bw = wz ? bq : 0;
+        const size_t bi = sizeof(int64_t) * nq * k, bd = sizeof(float) * nq * k, bn = sizeof(int64_t) * nq;
+        const size_t in = pad(bq) + pad(bp) + pad(bw), out = pad(bi) + pad(bd) + pad(bn);
+        if (in <= kPageHalf && out <= kPageHalf) {
+            uint8_t* hi = ix->page + kPageHead;
+            memcpy(hi, queries, bq);
+            memcpy(hi + pad(bq), preds, bp);
+            if (wz) memcpy(hi + pad(bq) + pad(bp), wz, bw);
+            TRY(ensure(ix->w_in, in));
+            CUDA_TRY(cudaMemcpyAsync(ix->w_in.p, hi, in, cudaMemcpyHostToDevice, s));
+            uint8_t* di = ix->w_in.as<uint8_t>();
+            uint8_t* od = ix->page_dev + kPageHead + kPageHalf;
+            TRY(ensure(ix->w_npass, bn));
+            TRY(run_path(ix, s, o, (const float*)di, (const ifvs_predicate*)(di + pad(bq)),
+                         wz ? (const float*)(di + pad(bq) + pad(bp)) : nullptr, ix->D, nq, k, (int64_t*)od,
+                         (float*)(od + pad(bi)), ix->w_npass.as<unsigned long long>(),
+                         npass ? (int64_t*)(od + pad(bi) + pad(bd)) : nullptr));
+            TRY(finish(ix, s, true));
+            const uint8_t* ho = ix->page + kPageHead + kPageHalf;
+            memcpy(ids, ho, bi);
+            memcpy(dists, ho + pad(bi), bd);
+            if (npass) memcpy(npass, ho + pad(bi) + pad(bd), bn);
+            return IFVS_OK;
+        }
+    }
     TRY(ensure(ix->w_npass, sizeof(unsigned long long) * sb));
     if (!o.dio) {
         TRY(ensure(ix->w_ids, sizeof(int64_t) * sb * k));
@@ -1119,13 +1185,16 @@ int ifvs_search_batch(ifvs_index* ix, const float* queries, const ifvs_predicate
         TRY(stage_inputs(ix, s, o, q0, n, queries, preds, wz, &dq, &dp, &dwz));
         int64_t* oid = o.dio ? ids + q0 * k : ix->w_ids.as<int64_t>();
         float* odi = o.dio ? dists + q0 * k : ix->w_dists.as<float>();
-        TRY(run_path(ix, s, o, dq, dp, dwz, ix->D, n, k, oid, odi, ix->w_npass.as<unsigned long long>()));
+        // with device I/O the counts are formed in the caller's array
+        auto* np = o.dio && npass ? reinterpret_cast<unsigned long long*>(npass + q0)
+                                  : ix->w_npass.as<unsigned long long>();
+        TRY(run_path(ix, s, o, dq, dp, dwz, ix->D, n, k, oid, odi, np, nullptr));
         if (!o.dio) {
             TRY(copy_out(s, false, ids + q0 * k, oid, sizeof(int64_t) * n * k));
             TRY(copy_out(s, false, dists + q0 * k, odi, sizeof(float) * n * k));
+            if (npass) TRY(copy_out(s, false, npass + q0, np, sizeof(int64_t) * n));
+            if (q0 + sb < nq) CUDA_TRY(cudaStreamSynchronize(s));
         }
-        if (npass) TRY(copy_out(s, o.dio, npass + q0, ix->w_npass.p, sizeof(int64_t) * n));
-        if (!o.dio && q0 + sb < nq) CUDA_TRY(cudaStreamSynchronize(s));
     }
     return finish(ix, s, true);
 }
@@ -1289,7 +1358,7 @@ int ifvs_scan_topk(ifvs_index* ix, const float* lut, const uint32_t* bitmaps, in
         float* odi = o.dio ? dists + q0 * k : ix->w_dists.as<float>();
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_MERGE);
-            CUDA_TRY(st.end(launch_merge(sched, n, k, oid, odi, s)));
+            CUDA_TRY(st.end(launch_merge(sched, n, k, oid, odi, nullptr, nullptr, s)));
         }
         if (!o.dio) {
             TRY(copy_out(s, false, ids + q0 * k, oid, sizeof(int64_t) * n * k));
@@ -1575,8 +1644,10 @@ int ifvs_train_grad(ifvs_index* ix, const float* queries, const ifvs_predicate* 
     if (g_bank) TRY(copy_out(s, o.dio, g_bank, ix->t_gbank.p, sizeof(float) * ix->B * Mr));
     if (g_W) TRY(copy_out(s, o.dio, g_W, ix->t_gW.p, nW));
     if (g_wz) TRY(copy_out(s, o.dio, g_wz, ix->t_gwz.p, sizeof(float) * ix->D));
-    TRY(train_loss_out(ix, s, nq, loss));
-    return finish(ix, s, true);
+    TRY(train_loss_fetch(ix, s, nq, loss));
+    const int rc = finish(ix, s, true);
+    train_loss_mean(ix, nq, loss);
+    return rc;
 }
 
 int ifvs_train_step(ifvs_index* ix, const float* queries, const ifvs_predicate* preds, int64_t nq,
@@ -1616,7 +1687,7 @@ int ifvs_train_step(ifvs_index* ix, const float* queries, const ifvs_predicate* 
     mo.sub_batch = 0;
     mo.chunk_blocks = 0;
     TRY(run_path(ix, s, mo, dq, dp, ix->t_wz.as<float>(), 0, nq, kk, ix->t_mined.as<int64_t>(),
-                 ix->t_mdist.as<float>(), ix->w_npass.as<unsigned long long>()));
+                 ix->t_mdist.as<float>(), ix->w_npass.as<unsigned long long>(), nullptr));
     TRY(ensure(ix->t_neg, sizeof(int64_t) * nq * (tp->n_neg > 0 ? tp->n_neg : 1)));
     TrainQueryArgs a = train_args(ix, tp, nq, dq);
     a.pos = dpos;
@@ -1644,8 +1715,10 @@ int ifvs_train_step(ifvs_index* ix, const float* queries, const ifvs_predicate* 
     TRY(copy_out(s, o.dio, wz, ix->t_wz.p, sizeof(float) * ix->D));
     if (negatives && tp->n_neg > 0)
         TRY(copy_out(s, o.dio, negatives, ix->t_neg.p, sizeof(int64_t) * nq * tp->n_neg));
-    TRY(train_loss_out(ix, s, nq, loss));
-    return finish(ix, s, true);
+    TRY(train_loss_fetch(ix, s, nq, loss));
+    const int rc = finish(ix, s, true);
+    train_loss_mean(ix, nq, loss);
+    return rc;
 }
 
 int ifvs_get_conditioning(ifvs_index* ix, float* bank, float* W, uint32_t flags) {

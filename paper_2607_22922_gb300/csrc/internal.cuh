@@ -285,8 +285,9 @@ cudaError_t launch_scan_pairs(const float* tab, SortedCols sc, const ScanPlan* p
 // layout `src`, re-rotated by (p mod 32) mod M; positions >= N are zero
 cudaError_t launch_relayout_sorted(const uint8_t* src, const uint32_t* rows, int64_t N, int M,
                                    int row_bytes, int64_t n_rows_pad, uint8_t* dst, cudaStream_t s);
-// Select: a query's lists -> ids / dists
-cudaError_t launch_merge(const ScanSched& sched, int64_t nq, int k, int64_t* ids, float* dists, cudaStream_t s);
+// Select: a query's lists -> ids / dists; npass to npass_copy unless null
+cudaError_t launch_merge(const ScanSched& sched, int64_t nq, int k, int64_t* ids, float* dists,
+                         const unsigned long long* npass, int64_t* npass_copy, cudaStream_t s);
 // exact fp32 rerank of cand [nq][R] -> k best
 // Select across row shards: [G][nq][k] (dist, global id) -> [nq][k]
 int shard_merge_cap();

@@ -129,7 +129,7 @@ extern "C" int ifvs_scan_topk_static(ifvs_index* ix, const float* lut, const uin
         if (e == cudaSuccess) e = launch_tables(lut + q0 * lut_n, n, v.M, v.K, v.tab_words, tab, s);
         if (e == cudaSuccess) e = launch_schedule(nullptr, nullptr, n, v.n_blocks, -1, 0, sched, s);
         if (e == cudaSuccess) e = launch_scan(v.codes, tab, bm, n, k, sh, sched, s);
-        if (e == cudaSuccess) e = launch_merge(sched, n, k, ids + q0 * k, dists + q0 * k, s);
+        if (e == cudaSuccess) e = launch_merge(sched, n, k, ids + q0 * k, dists + q0 * k, nullptr, nullptr, s);
         if (e != cudaSuccess) {
             cudaGetLastError();
             rc = report_error(IFVS_ERR_CUDA, "ifvs_scan_topk_static launch failed: %s", cudaGetErrorString(e));

@@ -56,11 +56,14 @@ __device__ __forceinline__ void write_key(uint64_t key, int64_t* id, float* d) {
 template <int KP, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32) k_merge(const uint64_t* __restrict__ partials,
                                                       const int2* __restrict__ qlist, int k,
-                                                      int64_t* __restrict__ ids, float* __restrict__ dists) {
+                                                      int64_t* __restrict__ ids, float* __restrict__ dists,
+                                                      const unsigned long long* __restrict__ npass,
+                                                      int64_t* __restrict__ npass_copy) {
     __shared__ uint64_t a[WARPS * 2 * KP];
     const int64_t q = blockIdx.x;
     const int2 ql = qlist[q];
     const uint64_t* src = partials + (int64_t)ql.x * k;
+    if (npass_copy != nullptr && threadIdx.x == 0) npass_copy[q] = (int64_t)npass[q];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (ql.y > 1) {
         uint64_t* buf = a + warp * 2 * KP;
@@ -88,17 +91,22 @@ __global__ void __launch_bounds__(WARPS * 32) k_merge(const uint64_t* __restrict
     }
 }
 
-cudaError_t launch_merge(const ScanSched& sched, int64_t nq, int k, int64_t* ids, float* dists, cudaStream_t s) {
+cudaError_t launch_merge(const ScanSched& sched, int64_t nq, int k, int64_t* ids, float* dists,
+                         const unsigned long long* npass, int64_t* npass_copy, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     const unsigned g = (unsigned)nq;
     if (k <= 32)
-        k_merge<32, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists);
+        k_merge<32, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists, npass,
+                                                npass_copy);
     else if (k <= 64)
-        k_merge<64, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists);
+        k_merge<64, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists, npass,
+                                                npass_copy);
     else if (k <= 128)
-        k_merge<128, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists);
+        k_merge<128, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists, npass,
+                                                npass_copy);
     else
-        k_merge<256, 8><<<g, 256, 0, s>>>(sched.partials, sched.qlist, k, ids, dists);
+        k_merge<256, 8><<<g, 256, 0, s>>>(sched.partials, sched.qlist, k, ids, dists, npass,
+                                                npass_copy);
     return cudaGetLastError();
 }
 

@@ -109,7 +109,7 @@ def _ptr(a):
     if isinstance(a, np.ndarray):
         if not a.flags.c_contiguous:
             raise ValueError("arrays must be C-contiguous")
-        return a.ctypes.data
+        return a.__array_interface__["data"][0]
     if hasattr(a, "data_ptr"):
         if hasattr(a, "is_contiguous") and not a.is_contiguous():
             raise ValueError("tensors must be contiguous")
