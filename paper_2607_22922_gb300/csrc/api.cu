@@ -606,13 +606,19 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     if (bitmaps) {
         Stage st(ix, s, o.timing, IFVS_STAGE_FILTER);
         CUDA_TRY(st.end(launch_filter(ix->cols(), ix->N, ix->n_blocks, ix->w_canon.as<CanonPred>(),
-                                      plan, n, ix->w_bm.as<uint32_t>(), npass_u64, ix->num_sms, s)));
+                                      plan, n, ix->w_bm.as<uint32_t>(), npass_u64, ix->num_sms, !o.timing, s)));
+    }
+    const bool chain = !o.timing && cond_tables_fit(ix->ds, ix->r, cond);
+    {
+        Stage st(ix, s, o.timing, pairs ? IFVS_STAGE_SCAN : IFVS_STAGE_LAYOUT);
+        CUDA_TRY(st.end(launch_schedule(plan, npass_u64, n, ix->n_blocks, pairs ? pr.span : -1, pr.total, sched, chain,
+                                        s)));
     }
     const float* alpha = cond ? ix->w_alpha.as<float>() : nullptr;
-    if (!o.timing && cond_tables_fit(ix->ds, ix->r, cond)) {
+    if (chain) {
         Stage st(ix, s, false, IFVS_STAGE_LUT);
         CUDA_TRY(st.end(launch_cond_tables(ix->d_cpq, ix->d_W, alpha, dq, ix->w_wf.as<float>(), n, ix->M, ix->K,
-                                           ix->ds, ix->tab_words, ix->w_tab.as<float>(), ix->num_sms, s)));
+                                           ix->ds, ix->tab_words, ix->w_tab.as<float>(), ix->num_sms, true, s)));
     } else {
         TRY(ensure(ix->w_lut, sizeof(float) * n * ix->M * ix->K));
         {
@@ -624,17 +630,17 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
         CUDA_TRY(st.end(launch_tables(ix->w_lut.as<float>(), n, ix->M, ix->K, ix->tab_words,
                                       ix->w_tab.as<float>(), s)));
     }
-    {
-        Stage st(ix, s, o.timing, pairs ? IFVS_STAGE_SCAN : IFVS_STAGE_LAYOUT);
-        CUDA_TRY(st.end(launch_schedule(plan, npass_u64, n, ix->n_blocks, pairs ? pr.span : -1, pr.total, sched, s)));
-    }
+    ScanOrder order{chain, true};
     if (bitmaps) {
         Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
-        CUDA_TRY(st.end(launch_scan(ix->d_codes, ix->w_tab.as<float>(), ix->w_bm.as<uint32_t>(), n, kk, sh, sched, s)));
+        CUDA_TRY(st.end(launch_scan(ix->d_codes, ix->w_tab.as<float>(), ix->w_bm.as<uint32_t>(), n, kk, sh, sched,
+                                    order, s)));
+        order.first = false;
     }
     if (pairs) {
         Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
-        CUDA_TRY(st.end(launch_scan_pairs(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, s)));
+        CUDA_TRY(st.end(launch_scan_pairs(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, order, s)));
+        order.first = false;
     }
     if (plan) {
         Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
@@ -642,19 +648,18 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
         lo.bulk = !o.plain_loads;
         lo.tx_extra = stall_copies_for_tests() ? 16u : 0u;
         lo.err = ix->err();
-        lo.after_pairs = pairs && !o.timing;
-        CUDA_TRY(st.end(launch_scan_list(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, lo, s)));
+        CUDA_TRY(st.end(launch_scan_list(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, lo, order, s)));
     }
     int64_t* m_ids = o.R > 0 ? ix->w_cand.as<int64_t>() : out_ids;
     float* m_dists = o.R > 0 ? ix->w_cdist.as<float>() : out_dists;
     {
         Stage st(ix, s, o.timing, IFVS_STAGE_MERGE);
-        CUDA_TRY(st.end(launch_merge(sched, n, kk, m_ids, m_dists, npass_u64, npass_copy, s)));
+        CUDA_TRY(st.end(launch_merge(sched, n, kk, m_ids, m_dists, npass_u64, npass_copy, chain, s)));
     }
     if (o.R > 0) {
         Stage st(ix, s, o.timing, IFVS_STAGE_RERANK);
         CUDA_TRY(st.end(launch_rerank(ix->d_vec, ix->N, ix->D, dq, m_ids, n, o.R, k, out_ids,
-                                      out_dists, s)));
+                                      out_dists, chain, s)));
     }
     return 0;
 }
@@ -1229,7 +1234,7 @@ int ifvs_filter(ifvs_index* ix, const ifvs_predicate* preds, int64_t nq, const i
             Stage st(ix, s, o.timing, IFVS_STAGE_FILTER);
             CUDA_TRY(st.end(launch_filter(ix->cols(), ix->N, ix->n_blocks, ix->w_canon.as<CanonPred>(),
                                           nullptr, n, ix->w_bm.as<uint32_t>(),
-                                          ix->w_npass.as<unsigned long long>(), ix->num_sms, s)));
+                                          ix->w_npass.as<unsigned long long>(), ix->num_sms, false, s)));
         }
         uint32_t* rows = o.dio ? bitmaps + q0 * wrows : ix->w_rows.as<uint32_t>();
         {
@@ -1347,18 +1352,18 @@ int ifvs_scan_topk(ifvs_index* ix, const float* lut, const uint32_t* bitmaps, in
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_LAYOUT);
-            CUDA_TRY(st.end(launch_schedule(nullptr, nullptr, n, ix->n_blocks, -1, 0, sched, s)));
+            CUDA_TRY(st.end(launch_schedule(nullptr, nullptr, n, ix->n_blocks, -1, 0, sched, false, s)));
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
             CUDA_TRY(st.end(launch_scan(ix->d_codes, ix->w_tab.as<float>(), ix->w_bm.as<uint32_t>(), n, k, sh, sched,
-                                        s)));
+                                        ScanOrder{false, true}, s)));
         }
         int64_t* oid = o.dio ? ids + q0 * k : ix->w_ids.as<int64_t>();
         float* odi = o.dio ? dists + q0 * k : ix->w_dists.as<float>();
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_MERGE);
-            CUDA_TRY(st.end(launch_merge(sched, n, k, oid, odi, nullptr, nullptr, s)));
+            CUDA_TRY(st.end(launch_merge(sched, n, k, oid, odi, nullptr, nullptr, false, s)));
         }
         if (!o.dio) {
             TRY(copy_out(s, false, ids + q0 * k, oid, sizeof(int64_t) * n * k));
@@ -1401,7 +1406,7 @@ int ifvs_rerank(ifvs_index* ix, const float* queries, const int64_t* cand, int64
     }
     {
         Stage st(ix, s, o.timing, IFVS_STAGE_RERANK);
-        CUDA_TRY(st.end(launch_rerank(ix->d_vec, ix->N, ix->D, dq, dc, nq, R, k, oid, odi, s)));
+        CUDA_TRY(st.end(launch_rerank(ix->d_vec, ix->N, ix->D, dq, dc, nq, R, k, oid, odi, false, s)));
     }
     if (!o.dio) {
         TRY(copy_out(s, false, ids, oid, sizeof(int64_t) * nq * k));

@@ -218,6 +218,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(PrepareArgs a) {
     __shared__ uint32_t s_idx[64];
     __shared__ int64_t s_end[2];
     __shared__ CanonPred s_cp;
+    start_dependents();
     if (tid == 0) {
         const ifvs_predicate p = a.preds[qi];
         CanonPred cp;
@@ -438,6 +439,7 @@ k_cond_tables(const float* __restrict__ cpq, const float* __restrict__ W, const 
     const int D = M * DS, mg = min(kTabM, M - m0);
     const int64_t q0 = (int64_t)blockIdx.y * q_per_cta;
     const int64_t q1 = min(nq, q0 + (int64_t)q_per_cta);
+    start_dependents();
     auto stage = [&](int64_t s0, int b) {   // queries [s0, s0 + kTabQ)
         const int ns = (int)min((int64_t)kTabQ, q1 - s0);
         if (COND)
@@ -523,22 +525,22 @@ k_cond_tables(const float* __restrict__ cpq, const float* __restrict__ W, const 
                 for (int o = m0 + wm; o < M + 31; o += M) out[o] = s;
             }
     }
+    wait_before();
 }
 
 template <int DS>
-static void start_cond_tables(dim3 grid, const float* cpq, const float* W, const float* alpha, const float* q,
-                              const float* wf, int64_t nq, int M, int K, int S, int qpc, int vec, float* tab,
-                              cudaStream_t s) {
-    if (alpha != nullptr)
-        k_cond_tables<DS, true><<<grid, kTabThreads, 0, s>>>(cpq, W, alpha, q, wf, nq, M, K, S, qpc, vec, tab);
-    else
-        k_cond_tables<DS, false><<<grid, kTabThreads, 0, s>>>(cpq, W, alpha, q, wf, nq, M, K, S, qpc, vec, tab);
+static cudaError_t start_cond_tables(dim3 grid, bool chain, cudaStream_t s, const float* cpq, const float* W,
+                                     const float* alpha, const float* q, const float* wf, int64_t nq, int M, int K,
+                                     int S, int qpc, int vec, float* tab) {
+    auto kern = alpha != nullptr ? k_cond_tables<DS, true> : k_cond_tables<DS, false>;
+    return launch_kernel(kern, grid, dim3(kTabThreads), 0, chain, s, cpq, W, alpha, q, wf, nq, M, K, S, qpc, vec, tab);
 }
 
 bool cond_tables_fit(int ds, int r, bool cond) { return (ds == 4 || ds == 8 || ds == 16) && (!cond || r == 8); }
 
 cudaError_t launch_cond_tables(const float* cpq, const float* W, const float* alpha, const float* q, const float* wf,
-                               int64_t nq, int M, int K, int ds, int S, float* tab, int num_sms, cudaStream_t s) {
+                               int64_t nq, int M, int K, int ds, int S, float* tab, int num_sms, bool chain,
+                               cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     const int tiles = (M + kTabM - 1) / kTabM * (256 / kTabC);
     // two CTAs per SM; a group of queries shares a CTA's registers
@@ -548,13 +550,8 @@ cudaError_t launch_cond_tables(const float* cpq, const float* W, const float* al
     groups = (nq + qpc - 1) / qpc;
     const dim3 grid((unsigned)tiles, (unsigned)groups);
     const int vec = (uintptr_t)q % 16 == 0;
-    if (ds == 4)
-        start_cond_tables<4>(grid, cpq, W, alpha, q, wf, nq, M, K, S, (int)qpc, vec, tab, s);
-    else if (ds == 8)
-        start_cond_tables<8>(grid, cpq, W, alpha, q, wf, nq, M, K, S, (int)qpc, vec, tab, s);
-    else
-        start_cond_tables<16>(grid, cpq, W, alpha, q, wf, nq, M, K, S, (int)qpc, vec, tab, s);
-    return cudaGetLastError();
+    auto start = ds == 4 ? start_cond_tables<4> : (ds == 8 ? start_cond_tables<8> : start_cond_tables<16>);
+    return start(grid, chain, s, cpq, W, alpha, q, wf, nq, M, K, S, (int)qpc, vec, tab);
 }
 
 // ---- scan tables -------------------------------------------------------------

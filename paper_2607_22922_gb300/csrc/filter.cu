@@ -80,6 +80,8 @@ __global__ void __launch_bounds__(kThreads) k_filter(AttrCols cols, int64_t N, i
         }
     }
 
+    wait_before();         // the columns are the index's; what follows is prepare's
+    start_dependents();
     const int64_t words = n_blocks * 32;
     const int warp = threadIdx.x >> 5;
     for (int64_t g0 = q0; g0 < q1; g0 += kFilterQ) {
@@ -129,7 +131,7 @@ __global__ void __launch_bounds__(kThreads) k_filter(AttrCols cols, int64_t N, i
 
 cudaError_t launch_filter(AttrCols cols, int64_t N, int64_t n_blocks, const CanonPred* canon,
                           const ScanPlan* plan, int64_t nq, uint32_t* bm, unsigned long long* npass,
-                          int num_sms, cudaStream_t s) {
+                          int num_sms, bool chain, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     const int64_t tiles = (n_blocks + kWarps - 1) / kWarps;
     // enough CTAs to fill the GPU a few times over; each CTA walks a group
@@ -143,13 +145,9 @@ cudaError_t launch_filter(AttrCols cols, int64_t N, int64_t n_blocks, const Cano
     groups = (nq + qpc - 1) / qpc;
     dim3 grid((unsigned)tiles, (unsigned)groups);
     int na = cols.n < 1 ? 1 : cols.n;
-    switch (na) {
-        case 1: k_filter<1><<<grid, kThreads, 0, s>>>(cols, N, n_blocks, canon, plan, nq, (int)qpc, bm, npass); break;
-        case 2: k_filter<2><<<grid, kThreads, 0, s>>>(cols, N, n_blocks, canon, plan, nq, (int)qpc, bm, npass); break;
-        case 3: k_filter<3><<<grid, kThreads, 0, s>>>(cols, N, n_blocks, canon, plan, nq, (int)qpc, bm, npass); break;
-        default: k_filter<4><<<grid, kThreads, 0, s>>>(cols, N, n_blocks, canon, plan, nq, (int)qpc, bm, npass); break;
-    }
-    return cudaGetLastError();
+    auto kern = na == 1 ? k_filter<1> : (na == 2 ? k_filter<2> : (na == 3 ? k_filter<3> : k_filter<4>));
+    return launch_kernel(kern, grid, dim3(kThreads), 0, chain, s, cols, N, n_blocks, canon, plan, nq, (int)qpc, bm,
+                         npass);
 }
 
 // ---- layout conversion ---------------------------------------------------

@@ -93,6 +93,38 @@ struct AttrCols {
     int32_t n;
 };
 
+// ---- overlapping launches ----------------------------------------------
+//
+// The kernels of a search follow each other in one stream.  Launched with
+// `chain`, a kernel may start while the one before it still runs (programmatic
+// launch), once all of that one's CTAs have called start_dependents:
+//   prepare [-> filter] -> schedule -> tables -> scans -> merge [-> rerank]
+// A kernel either waits for the one before it at its start (wait_before, after
+// reading only what no kernel of the path writes), or, where it needs nothing
+// of it, at its end: schedule starts the tables once prepare and filter are
+// complete, the first scan waits for the tables, and the other scans start
+// with it.  Since every kernel waits before it completes, a kernel that has
+// waited sees all that came earlier.  Without `chain` (stage timing, shapes
+// with separate table kernels) launches are ordinary and the calls do nothing.
+__device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+inline cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, bool chain, cudaStream_t s,
+                                 A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chain ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // ---- kernel launchers (one per translation unit) -----------------------
 // Every launcher returns the cudaError_t of its launch.
 
@@ -186,7 +218,7 @@ cudaError_t launch_prepare(const PrepareArgs& a, int64_t nq, cudaStream_t s);
 // npass) for the bitmap-path queries of `plan` (all queries when plan is null)
 cudaError_t launch_filter(AttrCols cols, int64_t N, int64_t n_blocks, const CanonPred* canon,
                           const ScanPlan* plan, int64_t nq, uint32_t* bm, unsigned long long* npass,
-                          int num_sms, cudaStream_t s);
+                          int num_sms, bool chain, cudaStream_t s);
 
 // 32x32 bit transposes between the lane-major layout and the row-ordered
 // layout of the ABI ([nq][ceil(N/32)]).  to_rows = true: lane-major -> rows.
@@ -208,7 +240,8 @@ cudaError_t launch_tables(const float* lut, int64_t nq, int M, int K, int S, flo
 // the shapes that cond_tables_fit names
 bool cond_tables_fit(int ds, int r, bool cond);
 cudaError_t launch_cond_tables(const float* cpq, const float* W, const float* alpha, const float* q, const float* wf,
-                               int64_t nq, int M, int K, int ds, int S, float* tab, int num_sms, cudaStream_t s);
+                               int64_t nq, int M, int K, int ds, int S, float* tab, int num_sms, bool chain,
+                               cudaStream_t s);
 
 struct ScanShape {
     int64_t n_blocks;      // bitmap blocks (rows padded to n_blocks * 1024)
@@ -257,13 +290,18 @@ size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)
 // pair_min_rows < 0: no pairs; nor where the sorted-copy ranges together hold
 // fewer than pair_min_total rows
 cudaError_t launch_schedule(const ScanPlan* plan, const unsigned long long* npass, int64_t nq, int64_t n_blocks,
-                            int64_t pair_min_rows, int64_t pair_min_total, const ScanSched& s, cudaStream_t st);
+                            int64_t pair_min_rows, int64_t pair_min_total, const ScanSched& s, bool chain, cudaStream_t st);
 
+// How a scan is launched: `chain` as above; first: it is the batch's first scan
+// (waits at its start, the others at their end)
+struct ScanOrder {
+    bool chain, first;
+};
 // Rank over the bitmap group's items: per item, the k best keys (dist bits <<
 // 32 | row) of its blocks' passing rows; `tab` holds the tables written by
 // launch_tables
 cudaError_t launch_scan(const uint8_t* codes, const float* tab, const uint32_t* bm, int64_t nq, int k,
-                        const ScanShape& sh, const ScanSched& sched, cudaStream_t s);
+                        const ScanShape& sh, const ScanSched& sched, ScanOrder o, cudaStream_t s);
 // Rank over the list group's items: a query's pool is the position range
 // [a, b) of a sorted copy.  Code rows arrive by bulk copies into shared memory
 // when `bulk` and the shape allows it (else by per-lane loads); a bounded wait
@@ -273,28 +311,28 @@ struct ListOpts {
     bool bulk;
     uint32_t tx_extra;
     int* err;
-    bool after_pairs;   // launched right after launch_scan_pairs: may overlap it
 };
 cudaError_t launch_scan_list(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                             const ScanShape& sh, const ScanSched& sched, const ListOpts& lo, cudaStream_t s);
+                             const ScanShape& sh, const ScanSched& sched, const ListOpts& lo, ScanOrder o,
+                             cudaStream_t s);
 // Rank over the pair group's items (M = 16): two queries per CTA
 bool scan_pairs_fit(const ScanShape& sh, int k);
 cudaError_t launch_scan_pairs(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                              const ScanShape& sh, const ScanSched& sched, cudaStream_t s);
+                              const ScanShape& sh, const ScanSched& sched, ScanOrder o, cudaStream_t s);
 // the sorted copy of the codes: dst position p <- row rows[p] of the index
 // layout `src`, re-rotated by (p mod 32) mod M; positions >= N are zero
 cudaError_t launch_relayout_sorted(const uint8_t* src, const uint32_t* rows, int64_t N, int M,
                                    int row_bytes, int64_t n_rows_pad, uint8_t* dst, cudaStream_t s);
 // Select: a query's lists -> ids / dists; npass to npass_copy unless null
 cudaError_t launch_merge(const ScanSched& sched, int64_t nq, int k, int64_t* ids, float* dists,
-                         const unsigned long long* npass, int64_t* npass_copy, cudaStream_t s);
+                         const unsigned long long* npass, int64_t* npass_copy, bool chain, cudaStream_t s);
 // exact fp32 rerank of cand [nq][R] -> k best
 // Select across row shards: [G][nq][k] (dist, global id) -> [nq][k]
 int shard_merge_cap();
 cudaError_t launch_merge_shards(const float* dists, const int64_t* ids, int64_t nq, int G, int k,
                                 float* dists_out, int64_t* ids_out, cudaStream_t s);
 cudaError_t launch_rerank(const float* X, int64_t N, int D, const float* q, const int64_t* cand,
-                          int64_t nq, int R, int k, int64_t* ids, float* dists, cudaStream_t s);
+                          int64_t nq, int R, int k, int64_t* ids, float* dists, bool chain, cudaStream_t s);
 // codes [N][M] -> rotated rows [n_rows_pad][row_bytes]; *bad = 1 if a code >= K
 cudaError_t launch_relayout_codes(const uint8_t* src, int64_t N, int M, int K, int row_bytes,
                                   int64_t n_rows_pad, uint8_t* dst, int* bad, cudaStream_t s);

@@ -127,9 +127,9 @@ extern "C" int ifvs_scan_topk_static(ifvs_index* ix, const float* lut, const uin
         sh.tab_words = v.tab_words;
         cudaError_t e = launch_bitmap_layout(bitmaps + q0 * wrows, bm, n, v.n_blocks, wrows, false, s);
         if (e == cudaSuccess) e = launch_tables(lut + q0 * lut_n, n, v.M, v.K, v.tab_words, tab, s);
-        if (e == cudaSuccess) e = launch_schedule(nullptr, nullptr, n, v.n_blocks, -1, 0, sched, s);
-        if (e == cudaSuccess) e = launch_scan(v.codes, tab, bm, n, k, sh, sched, s);
-        if (e == cudaSuccess) e = launch_merge(sched, n, k, ids + q0 * k, dists + q0 * k, nullptr, nullptr, s);
+        if (e == cudaSuccess) e = launch_schedule(nullptr, nullptr, n, v.n_blocks, -1, 0, sched, false, s);
+        if (e == cudaSuccess) e = launch_scan(v.codes, tab, bm, n, k, sh, sched, ScanOrder{false, true}, s);
+        if (e == cudaSuccess) e = launch_merge(sched, n, k, ids + q0 * k, dists + q0 * k, nullptr, nullptr, false, s);
         if (e != cudaSuccess) {
             cudaGetLastError();
             rc = report_error(IFVS_ERR_CUDA, "ifvs_scan_topk_static launch failed: %s", cudaGetErrorString(e));

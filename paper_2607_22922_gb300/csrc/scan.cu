@@ -164,7 +164,7 @@ __device__ __forceinline__ void scan_chunk(const uint8_t* __restrict__ codes,
 template <int KP, int MM, int MINB>
 __global__ void __launch_bounds__(kScanThreads, MINB)
 k_scan(const uint8_t* __restrict__ codes, const float* __restrict__ tables,
-       const uint32_t* __restrict__ bm, int k, ScanShape sh, ScanSched sched) {
+       const uint32_t* __restrict__ bm, int k, ScanShape sh, ScanSched sched, bool first) {
     extern __shared__ __align__(256) uint8_t smem[];
     const int S = MM > 0 ? 64 : sh.tab_words;
     float* tab = reinterpret_cast<float*>(smem);
@@ -175,6 +175,7 @@ k_scan(const uint8_t* __restrict__ codes, const float* __restrict__ tables,
     uint32_t* ring = ringbase + warp * kRing * 32;
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab);
     const bool fast = base == kDynSmemBase;
+    scan_begin(first);
     for (ItemLoop loop(sched, 1, ringbase + kScanWarps * kRing * 32); loop.more(); loop.next()) {
     const ScanItem item = loop.items[loop.at];
     const int64_t q = item.qa;
@@ -205,41 +206,42 @@ k_scan(const uint8_t* __restrict__ codes, const float* __restrict__ tables,
     // 3) merge the warps' lists pairwise; warp 0 writes the k best keys
     merge_warps<KP, kScanWarps>(tk, tkbuf, k, lane, warp, sched.partials + (int64_t)item.la * k);
     }
+    scan_end(first);
 }
 
 template <int KP, int MM, int MINB>
 static cudaError_t launch_one(const uint8_t* codes, const float* tab, const uint32_t* bm, int k, const ScanShape& sh,
-                              const ScanSched& sched, size_t smem, cudaStream_t s) {
+                              const ScanSched& sched, size_t smem, ScanOrder o, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_scan<KP, MM, MINB>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_scan<KP, MM, MINB><<<item_grid(sched.group[1]), kScanThreads, smem, s>>>(codes, tab, bm, k, sh, sched);
-    return cudaGetLastError();
+    return launch_kernel(k_scan<KP, MM, MINB>, dim3(item_grid(sched.group[1])), dim3(kScanThreads), smem, o.chain, s,
+                         codes, tab, bm, k, sh, sched, o.first);
 }
 
 template <int KP>
 static cudaError_t launch_scan_kp(const uint8_t* codes, const float* tab, const uint32_t* bm, int k,
-                                  const ScanShape& sh, const ScanSched& sched, cudaStream_t s) {
+                                  const ScanShape& sh, const ScanSched& sched, ScanOrder o, cudaStream_t s) {
     const int mm = fixed_m(sh);
     const size_t smem = scan_smem_bytes(sh.tab_words, KP);
     const bool two = scan_ctas_per_sm(sh.tab_words, KP) >= 2;
     if (mm == 16)
-        return two ? launch_one<KP, 16, 2>(codes, tab, bm, k, sh, sched, smem, s)
-                   : launch_one<KP, 16, 1>(codes, tab, bm, k, sh, sched, smem, s);
+        return two ? launch_one<KP, 16, 2>(codes, tab, bm, k, sh, sched, smem, o, s)
+                   : launch_one<KP, 16, 1>(codes, tab, bm, k, sh, sched, smem, o, s);
     if (mm == 12)
-        return two ? launch_one<KP, 12, 2>(codes, tab, bm, k, sh, sched, smem, s)
-                   : launch_one<KP, 12, 1>(codes, tab, bm, k, sh, sched, smem, s);
-    return launch_one<KP, 0, 1>(codes, tab, bm, k, sh, sched, smem, s);
+        return two ? launch_one<KP, 12, 2>(codes, tab, bm, k, sh, sched, smem, o, s)
+                   : launch_one<KP, 12, 1>(codes, tab, bm, k, sh, sched, smem, o, s);
+    return launch_one<KP, 0, 1>(codes, tab, bm, k, sh, sched, smem, o, s);
 }
 
 cudaError_t launch_scan(const uint8_t* codes, const float* tab, const uint32_t* bm, int64_t nq, int k,
-                        const ScanShape& sh, const ScanSched& sched, cudaStream_t s) {
+                        const ScanShape& sh, const ScanSched& sched, ScanOrder o, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     switch (scan_kp(k)) {
-        case 32: return launch_scan_kp<32>(codes, tab, bm, k, sh, sched, s);
-        case 64: return launch_scan_kp<64>(codes, tab, bm, k, sh, sched, s);
-        case 128: return launch_scan_kp<128>(codes, tab, bm, k, sh, sched, s);
-        default: return launch_scan_kp<256>(codes, tab, bm, k, sh, sched, s);
+        case 32: return launch_scan_kp<32>(codes, tab, bm, k, sh, sched, o, s);
+        case 64: return launch_scan_kp<64>(codes, tab, bm, k, sh, sched, o, s);
+        case 128: return launch_scan_kp<128>(codes, tab, bm, k, sh, sched, o, s);
+        default: return launch_scan_kp<256>(codes, tab, bm, k, sh, sched, o, s);
     }
 }
 

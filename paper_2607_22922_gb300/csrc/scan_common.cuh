@@ -603,13 +603,16 @@ struct ItemLoop {
     }
 };
 
-// The one-query scan overlaps the two-query scan before it in the stream: they
-// share no data, and the second fills the SMs that the first leaves at its end
-// (one CTA of the first fills an SM).  The first lets the second start
-// (start_dependents), the second's CTAs end only after the first (wait_before),
-// so that what follows the second sees both.
-__device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A batch's scans share no data and overlap: the first waits for the tables and
+// lets the next start, which fills the SMs that the first leaves at its end;
+// the others wait for the one before them at their end.
+__device__ __forceinline__ void scan_begin(bool first) {
+    if (first) wait_before();
+    start_dependents();
+}
+__device__ __forceinline__ void scan_end(bool first) {
+    if (!first) wait_before();
+}
 
 // CTAs to launch for a group: all that fit the device, or the items there can be
 inline unsigned item_grid(const SchedGroup& g) { return (unsigned)(g.cap < g.slots ? (g.cap < 1 ? 1 : g.cap) : g.slots); }

@@ -70,7 +70,7 @@ __device__ __forceinline__ void scan_positions(const uint8_t* __restrict__ codes
 template <int KP, int MM, int MINB>
 __global__ void __launch_bounds__(kScanThreads, MINB)
 k_scan_list(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __restrict__ plan, int k,
-            ScanSched sched) {
+            ScanSched sched, bool first) {
     extern __shared__ __align__(256) uint8_t smem[];
     constexpr int S = 64;
     float* tab = reinterpret_cast<float*>(smem);
@@ -78,6 +78,7 @@ k_scan_list(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __r
     uint64_t* share = tkbuf + kScanWarps * 2 * KP;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab);
+    scan_begin(first);
     for (ItemLoop loop(sched, 0, share + 1 + kScanWarps); loop.more(); loop.next()) {
         const ScanItem item = loop.items[loop.at];
         const ScanPlan p = plan[item.qa];
@@ -98,7 +99,7 @@ k_scan_list(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __r
             scan_positions<KP, MM, false>(codes, rows, p.a, p.b, item.a, item.b, base, tk, lane, warp);
         merge_warps<KP, kScanWarps>(tk, tkbuf, k, lane, warp, sched.partials + (int64_t)item.la * k);
     }
-    wait_before();
+    scan_end(first);
 }
 
 // ---- sorted-copy scan with bulk-copied code tiles (M = 16) ------------------
@@ -205,7 +206,7 @@ __device__ __forceinline__ bool scan_positions_bulk(const uint8_t* __restrict__ 
 template <int KP, int MM, int MINB>
 __global__ void __launch_bounds__(kScanThreads, MINB)
 k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __restrict__ plan, int k,
-                 ScanSched sched, uint32_t tx_extra, int* __restrict__ err) {
+                 ScanSched sched, uint32_t tx_extra, int* __restrict__ err, bool first) {
     extern __shared__ __align__(256) uint8_t smem[];
     float* tab = reinterpret_cast<float*>(smem);
     uint64_t* tkbuf = reinterpret_cast<uint64_t*>(smem + (size_t)256 * 64 * 4);
@@ -222,6 +223,7 @@ k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan
     }
     uint64_t* share = tkbuf + kScanWarps * 2 * KP;
     uint32_t phase = 0u, tphase = 0u;
+    scan_begin(first);
     for (ItemLoop loop(sched, 0, bars_all + kScanWarps + 1); loop.more(); loop.next()) {
         const ScanItem item = loop.items[loop.at];
         // the query's 64 KB table (rows replicated and rotated, as k_tables
@@ -256,7 +258,7 @@ k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan
         merge_warps<KP, kScanWarps>(tk, tkbuf, k, lane, warp, sched.partials + (int64_t)item.la * k);
         if (__syncthreads_or(ok ? 0 : 1)) break;   // the search reports a timeout; its lists are incomplete
     }
-    wait_before();
+    scan_end(first);
 }
 
 // ---- generic M ----------------------------------------------------------------
@@ -379,7 +381,7 @@ __device__ __forceinline__ void scan_positions_gen(const uint32_t* __restrict__ 
 template <int KP, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, WARPS > 12 ? 1 : 2)
 k_scan_list_gen(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __restrict__ plan, int k,
-                ScanShape sh, ScanSched sched) {
+                ScanShape sh, ScanSched sched, bool first) {
     extern __shared__ __align__(256) uint8_t smem[];
     const int S = sh.tab_words;
     float* tab = reinterpret_cast<float*>(smem);
@@ -387,6 +389,7 @@ k_scan_list_gen(const float* __restrict__ tables, SortedCols sc, const ScanPlan*
     uint64_t* share = tkbuf + WARPS * 2 * KP;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab);
+    scan_begin(first);
     for (ItemLoop loop(sched, 0, share + 1 + WARPS); loop.more(); loop.next()) {
         const ScanItem item = loop.items[loop.at];
         const ScanPlan p = plan[item.qa];
@@ -404,24 +407,16 @@ k_scan_list_gen(const float* __restrict__ tables, SortedCols sc, const ScanPlan*
                                       p.b, item.a, item.b, sh, base, tk, lane, warp);
         merge_warps<KP, WARPS>(tk, tkbuf, k, lane, warp, sched.partials + (int64_t)item.la * k);
     }
+    scan_end(first);
 }
 
 template <class Kernel, class... Args>
-static cudaError_t launch_items(Kernel kern, const ScanSched& sched, int threads, size_t smem, bool overlap,
+static cudaError_t launch_items(Kernel kern, const ScanSched& sched, int threads, size_t smem, ScanOrder o,
                                 cudaStream_t s, Args... args) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(item_grid(sched.group[0]));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
+    return launch_kernel(kern, dim3(item_grid(sched.group[0])), dim3((unsigned)threads), smem, o.chain, s, args...,
+                         o.first);
 }
 
 // The kernel for a shape.  M = 12 and 16: bulk copies where asked for, else
@@ -461,7 +456,8 @@ int scan_list_ctas_per_sm(const ScanShape& sh, int k, bool bulk) { return list_k
 
 template <int KP>
 static cudaError_t launch_list_kp(const float* tab, SortedCols sc, const ScanPlan* plan, int k, const ScanShape& sh,
-                                  const ScanSched& sched, const ListOpts& lo, cudaStream_t s) {
+                                  const ScanSched& sched, const ListOpts& lo, ScanOrder o,
+                                  cudaStream_t s) {
     const int mm = fixed_m(sh);
     const ListKernel lk = list_kernel(sh, KP, lo.bulk);
     const bool two = lk.ctas == 2;
@@ -469,27 +465,28 @@ static cudaError_t launch_list_kp(const float* tab, SortedCols sc, const ScanPla
     if (lk.kind == ListKernel::kBulk) {
         auto kern = mm == 16 ? (two ? k_scan_list_bulk<KP, 16, 2> : k_scan_list_bulk<KP, 16, 1>)
                              : (two ? k_scan_list_bulk<KP, 12, 2> : k_scan_list_bulk<KP, 12, 1>);
-        return launch_items(kern, sched, threads, lk.smem, lo.after_pairs, s, tab, sc, plan, k, sched, lo.tx_extra, lo.err);
+        return launch_items(kern, sched, threads, lk.smem, o, s, tab, sc, plan, k, sched, lo.tx_extra, lo.err);
     }
     if (lk.kind == ListKernel::kPlain) {
         auto kern = mm == 16 ? (two ? k_scan_list<KP, 16, 2> : k_scan_list<KP, 16, 1>)
                              : (two ? k_scan_list<KP, 12, 2> : k_scan_list<KP, 12, 1>);
-        return launch_items(kern, sched, threads, lk.smem, lo.after_pairs, s, tab, sc, plan, k, sched);
+        return launch_items(kern, sched, threads, lk.smem, o, s, tab, sc, plan, k, sched);
     }
     auto kern = lk.warps == 24   ? k_scan_list_gen<KP, 24>
                 : lk.warps == 12 ? k_scan_list_gen<KP, 12>
                                  : k_scan_list_gen<KP, 8>;
-    return launch_items(kern, sched, threads, lk.smem, lo.after_pairs, s, tab, sc, plan, k, sh, sched);
+    return launch_items(kern, sched, threads, lk.smem, o, s, tab, sc, plan, k, sh, sched);
 }
 
 cudaError_t launch_scan_list(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                             const ScanShape& sh, const ScanSched& sched, const ListOpts& lo, cudaStream_t s) {
+                             const ScanShape& sh, const ScanSched& sched, const ListOpts& lo, ScanOrder o,
+                                  cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     switch (scan_kp(k)) {
-        case 32: return launch_list_kp<32>(tab, sc, plan, k, sh, sched, lo, s);
-        case 64: return launch_list_kp<64>(tab, sc, plan, k, sh, sched, lo, s);
-        case 128: return launch_list_kp<128>(tab, sc, plan, k, sh, sched, lo, s);
-        default: return launch_list_kp<256>(tab, sc, plan, k, sh, sched, lo, s);
+        case 32: return launch_list_kp<32>(tab, sc, plan, k, sh, sched, lo, o, s);
+        case 64: return launch_list_kp<64>(tab, sc, plan, k, sh, sched, lo, o, s);
+        case 128: return launch_list_kp<128>(tab, sc, plan, k, sh, sched, lo, o, s);
+        default: return launch_list_kp<256>(tab, sc, plan, k, sh, sched, lo, o, s);
     }
 }
 }  // namespace ifvs

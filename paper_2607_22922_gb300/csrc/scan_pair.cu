@@ -479,22 +479,23 @@ __device__ __forceinline__ void pair_item(uint8_t* smem, const float* __restrict
 template <int KP>
 __global__ void __launch_bounds__(kPairThreads, 1)
 k_scan_list_pair(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __restrict__ plan, int k,
-                 ScanSched sched) {
+                 ScanSched sched, bool first) {
     extern __shared__ __align__(256) uint8_t smem[];
-    start_dependents();
+    scan_begin(first);
     for (ItemLoop loop(sched, 2, smem + scan_pair_item_offset(KP)); loop.more(); loop.next())
         pair_item<KP>(smem, tables, sc, plan, loop.items[loop.at], k, sched.partials);
+    scan_end(first);
 }
 
 template <int KP>
 static cudaError_t launch_pairs_kp(const float* tab, SortedCols sc, const ScanPlan* plan, int k,
-                                   const ScanSched& sched, cudaStream_t s) {
+                                   const ScanSched& sched, ScanOrder o, cudaStream_t s) {
     const size_t ps = scan_pair_smem_bytes(KP);
     const cudaError_t e =
         cudaFuncSetAttribute(k_scan_list_pair<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps);
     if (e != cudaSuccess) return e;
-    k_scan_list_pair<KP><<<item_grid(sched.group[2]), kPairThreads, ps, s>>>(tab, sc, plan, k, sched);
-    return cudaGetLastError();
+    return launch_kernel(k_scan_list_pair<KP>, dim3(item_grid(sched.group[2])), dim3(kPairThreads), ps, o.chain, s,
+                         tab, sc, plan, k, sched, o.first);
 }
 
 bool scan_pairs_fit(const ScanShape& sh, int k) {
@@ -502,13 +503,13 @@ bool scan_pairs_fit(const ScanShape& sh, int k) {
 }
 
 cudaError_t launch_scan_pairs(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                              const ScanShape&, const ScanSched& sched, cudaStream_t s) {
+                              const ScanShape&, const ScanSched& sched, ScanOrder o, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     switch (scan_kp(k)) {
-        case 32: return launch_pairs_kp<32>(tab, sc, plan, k, sched, s);
-        case 64: return launch_pairs_kp<64>(tab, sc, plan, k, sched, s);
-        case 128: return launch_pairs_kp<128>(tab, sc, plan, k, sched, s);
-        default: return launch_pairs_kp<256>(tab, sc, plan, k, sched, s);
+        case 32: return launch_pairs_kp<32>(tab, sc, plan, k, sched, o, s);
+        case 64: return launch_pairs_kp<64>(tab, sc, plan, k, sched, o, s);
+        case 128: return launch_pairs_kp<128>(tab, sc, plan, k, sched, o, s);
+        default: return launch_pairs_kp<256>(tab, sc, plan, k, sched, o, s);
     }
 }
 

@@ -126,6 +126,8 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
     int* pre = reinterpret_cast<int*>(key);
     const int tid = threadIdx.x, nt = blockDim.x;
     int n_pairs = 0;
+    wait_before();
+    start_dependents();   // prepare and filter are complete: the tables can start
 
     // no sort for a batch that cannot pair: 3/4 in common, a pair spans at most
     // 5/4 of its longer range
@@ -365,12 +367,12 @@ size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)
 }
 
 cudaError_t launch_schedule(const ScanPlan* plan, const unsigned long long* npass, int64_t nq, int64_t n_blocks,
-                            int64_t pair_min_rows, int64_t pair_min_total, const ScanSched& s, cudaStream_t st) {
+                            int64_t pair_min_rows, int64_t pair_min_total, const ScanSched& s, bool chain, cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
     int threads = 128;
     while (threads < kSchedThreads && threads < nq) threads <<= 1;
-    k_schedule<<<1, threads, 0, st>>>(plan, npass, nq, n_blocks, plan ? pair_min_rows : -1, pair_min_total, s);
-    return cudaGetLastError();
+    return launch_kernel(k_schedule, dim3(1), dim3((unsigned)threads), 0, chain, st, plan, npass, nq, n_blocks,
+                         plan ? pair_min_rows : (int64_t)-1, pair_min_total, s);
 }
 
 }  // namespace ifvs

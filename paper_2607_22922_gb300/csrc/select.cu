@@ -61,6 +61,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_merge(const uint64_t* __restrict
                                                       int64_t* __restrict__ npass_copy) {
     __shared__ uint64_t a[WARPS * 2 * KP];
     const int64_t q = blockIdx.x;
+    wait_before();
+    start_dependents();
     const int2 ql = qlist[q];
     const uint64_t* src = partials + (int64_t)ql.x * k;
     if (npass_copy != nullptr && threadIdx.x == 0) npass_copy[q] = (int64_t)npass[q];
@@ -92,22 +94,11 @@ __global__ void __launch_bounds__(WARPS * 32) k_merge(const uint64_t* __restrict
 }
 
 cudaError_t launch_merge(const ScanSched& sched, int64_t nq, int k, int64_t* ids, float* dists,
-                         const unsigned long long* npass, int64_t* npass_copy, cudaStream_t s) {
+                         const unsigned long long* npass, int64_t* npass_copy, bool chain, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
-    const unsigned g = (unsigned)nq;
-    if (k <= 32)
-        k_merge<32, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists, npass,
-                                                npass_copy);
-    else if (k <= 64)
-        k_merge<64, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists, npass,
-                                                npass_copy);
-    else if (k <= 128)
-        k_merge<128, 16><<<g, 512, 0, s>>>(sched.partials, sched.qlist, k, ids, dists, npass,
-                                                npass_copy);
-    else
-        k_merge<256, 8><<<g, 256, 0, s>>>(sched.partials, sched.qlist, k, ids, dists, npass,
-                                                npass_copy);
-    return cudaGetLastError();
+    auto kern = k <= 32 ? k_merge<32, 16> : (k <= 64 ? k_merge<64, 16> : (k <= 128 ? k_merge<128, 16> : k_merge<256, 8>));
+    return launch_kernel(kern, dim3((unsigned)nq), dim3(k <= 128 ? 512 : 256), 0, chain, s,
+                         (const uint64_t*)sched.partials, (const int2*)sched.qlist, k, ids, dists, npass, npass_copy);
 }
 
 constexpr int kShardMergeCap = 4096;   // G * k entries per query, at most
@@ -186,6 +177,7 @@ __global__ void __launch_bounds__(256) k_rerank(const float* __restrict__ X, int
     const int64_t qi = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < rp; i += blockDim.x) a[i] = ~0ull;
+    wait_before();
     __syncthreads();
     const float* qv = q + qi * D;
     for (int j = warp; j < R; j += 8) {
@@ -206,12 +198,11 @@ __global__ void __launch_bounds__(256) k_rerank(const float* __restrict__ X, int
 }
 
 cudaError_t launch_rerank(const float* X, int64_t N, int D, const float* q, const int64_t* cand,
-                          int64_t nq, int R, int k, int64_t* ids, float* dists, cudaStream_t s) {
+                          int64_t nq, int R, int k, int64_t* ids, float* dists, bool chain, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     int rp = 32;
     while (rp < R) rp <<= 1;
-    k_rerank<<<(unsigned)nq, 256, 0, s>>>(X, N, D, q, cand, R, k, rp, ids, dists);
-    return cudaGetLastError();
+    return launch_kernel(k_rerank, dim3((unsigned)nq), dim3(256), 0, chain, s, X, N, D, q, cand, R, k, rp, ids, dists);
 }
 
 }  // namespace ifvs
