@@ -93,6 +93,30 @@ struct AttrCols {
     int32_t n;
 };
 
+// ---- sums that carry their rounding errors (TwoSum, Knuth) -------------------
+// a + b = hi + lo exactly (hi the rounded sum)
+__device__ __forceinline__ void two_sum(float a, float b, float& hi, float& lo) {
+    hi = __fadd_rn(a, b);
+    const float bb = __fsub_rn(hi, a);
+    lo = __fadd_rn(__fsub_rn(a, __fsub_rn(hi, bb)), __fsub_rn(b, bb));
+}
+// a running sum as a pair of floats
+struct Sum2 {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        float e;
+        two_sum(hi, v, hi, e);
+        lo = __fadd_rn(lo, e);
+    }
+    __device__ __forceinline__ void add(float2 v) {
+        add(v.x);
+        lo = __fadd_rn(lo, v.y);
+    }
+    __device__ __forceinline__ bool finite() const { return isfinite(hi) && isfinite(lo); }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+
 // ---- overlapping launches ----------------------------------------------
 //
 // The kernels of a search follow each other in one stream.  Launched with

@@ -37,28 +37,6 @@ __device__ __forceinline__ unsigned long long far_key(float d, int64_t row) {
     return ((unsigned long long)__float_as_uint(d) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)row);
 }
 
-// a + b = hi + lo exactly (hi the rounded sum)
-__device__ __forceinline__ void two_sum(float a, float b, float& hi, float& lo) {
-    hi = __fadd_rn(a, b);
-    const float bb = __fsub_rn(hi, a);
-    lo = __fadd_rn(__fsub_rn(a, __fsub_rn(hi, bb)), __fsub_rn(b, bb));
-}
-// a running sum as a pair of floats
-struct Sum2 {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        float e;
-        two_sum(hi, v, hi, e);
-        lo = __fadd_rn(lo, e);
-    }
-    __device__ __forceinline__ void add(float2 v) {
-        add(v.x);
-        lo = __fadd_rn(lo, v.y);
-    }
-    __device__ __forceinline__ bool finite() const { return isfinite(hi) && isfinite(lo); }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // the block's maximum, in every thread
 __device__ __forceinline__ unsigned long long block_max(unsigned long long v, unsigned long long* scratch) {
 #pragma unroll

@@ -256,6 +256,70 @@ static __device__ __noinline__ uint64_t absorb32(uint64_t mine, uint64_t c, int 
     return mine;
 }
 
+// k <= 64: the same with two rows of 32 keys, every key of `lo` below those of
+// `hi`: the candidates meet `lo` first, what falls out of it meets `hi`.
+static __device__ __noinline__ ulonglong2 absorb64(uint64_t lo, uint64_t hi, uint64_t c, int lane) {
+    c = sort32_down(c, lane);
+    uint64_t out = c < lo ? lo : c;      // the 32 larger keys, bitonic
+    lo = c < lo ? c : lo;
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+        lo = min_max_step(lo, j, (lane & j) == 0);
+        out = min_max_step(out, j, (lane & j) != 0);   // descending
+    }
+    hi = out < hi ? out : hi;
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) hi = min_max_step(hi, j, (lane & j) == 0);
+    return make_ulonglong2(lo, hi);
+}
+
+template <int NW>
+struct WarpTopK<64, NW> {
+    uint64_t* buf;   // candidates, 64 slots (of 128)
+    uint64_t* share;
+    int cnt;
+    int k, kw;
+    uint64_t thr;
+    uint64_t lo, hi;   // the lane's keys of the sorted list
+
+    __device__ __forceinline__ void init(uint64_t* b, int k_, int, uint64_t* share_ = nullptr) {
+        buf = b;
+        share = share_;
+        k = k_;
+        kw = NW > 0 ? (k_ + NW - 1) / (NW > 0 ? NW : 1) - 1 : 0;
+        cnt = 0;
+        thr = ~0ull;
+        lo = hi = ~0ull;
+    }
+    __device__ __forceinline__ void refresh(int) {
+        if (NW == 0) return;
+        const uint64_t t = *reinterpret_cast<volatile uint64_t*>(share);
+        if (t < thr) thr = t;
+    }
+    __device__ __forceinline__ void drain(int n, int lane) {
+        cnt -= n;
+        __syncwarp();
+        const uint64_t c = lane < n ? buf[cnt + lane] : ~0ull;
+        __syncwarp();   // the drained slots take the next candidates
+        const ulonglong2 r = absorb64(lo, hi, c, lane);
+        lo = r.x;
+        hi = r.y;
+        thr = __shfl_sync(0xFFFFFFFFu, k > 32 ? hi : lo, (k - 1) & 31);
+        if (NW > 0) share_publish<(NW > 0 ? NW : 1)>(share, thr, __shfl_sync(0xFFFFFFFFu, lo, kw), lane);
+        refresh(lane);
+    }
+    __device__ __forceinline__ void flush(int lane) {
+        if (cnt > 0) drain(cnt, lane);
+    }
+    __device__ __forceinline__ void offer(uint64_t key, bool want, int lane) {
+        const unsigned ball = __ballot_sync(0xFFFFFFFFu, want);
+        if (ball == 0) return;
+        if (want) buf[cnt + __popc(ball & ((1u << lane) - 1u))] = key;
+        cnt += __popc(ball);
+        if (cnt >= 32) drain(32, lane);
+    }
+};
+
 template <int NW>
 struct WarpTopK<32, NW> {
     uint64_t* buf;   // candidates, 64 slots
@@ -456,6 +520,10 @@ __device__ __forceinline__ void merge_warps(TK& tk, uint64_t* tkbuf, int k, int 
     if constexpr (KP == 32) {
         __syncwarp();
         tk.buf[lane] = tk.mine;
+    } else if constexpr (KP == 64) {
+        __syncwarp();
+        tk.buf[lane] = tk.lo;
+        tk.buf[32 + lane] = tk.hi;
     }
 #pragma unroll 1
     for (int step = 1; step < WARPS; step <<= 1) {

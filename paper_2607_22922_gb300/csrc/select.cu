@@ -168,11 +168,15 @@ cudaError_t launch_merge_shards(const float* dists, const int64_t* ids, int64_t 
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(256) k_rerank(const float* __restrict__ X, int64_t N, int D,
-                                                const float* __restrict__ q,
-                                                const int64_t* __restrict__ cand, int R, int k,
-                                                int rp, int64_t* __restrict__ ids,
-                                                float* __restrict__ dists) {
+// 16 warps, two candidates of a warp in flight: the rows lie anywhere in DRAM
+// (100 candidates of 1 KB per query: 35 us with one at a time in 8 warps,
+// RERANK_FIGURES).
+constexpr int kRerankWarps = 16;
+__global__ void __launch_bounds__(kRerankWarps * 32) k_rerank(const float* __restrict__ X, int64_t N, int D,
+                                                              const float* __restrict__ q,
+                                                              const int64_t* __restrict__ cand, int R, int k,
+                                                              int rp, int64_t* __restrict__ ids,
+                                                              float* __restrict__ dists) {
     __shared__ uint64_t a[IFVS_MAX_K];
     const int64_t qi = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -180,18 +184,34 @@ __global__ void __launch_bounds__(256) k_rerank(const float* __restrict__ X, int
     wait_before();
     __syncthreads();
     const float* qv = q + qi * D;
-    for (int j = warp; j < R; j += 8) {
-        const int64_t id = cand[qi * R + j];
-        if (id < 0 || id >= N) continue;
-        const float* x = X + id * D;
-        float s = 0.f;
+    for (int j = warp; j < R; j += 2 * kRerankWarps) {
+        int64_t id[2];
+        const float* x[2];
+        float s[2] = {0.f, 0.f};
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int c = j + u * kRerankWarps;
+            id[u] = c < R ? cand[qi * R + c] : -1;
+            if (id[u] >= N) id[u] = -1;
+            x[u] = X + (id[u] < 0 ? 0 : id[u]) * D;
+        }
+        if (id[0] < 0 && id[1] < 0) continue;
+#pragma unroll 4
         for (int d = lane; d < D; d += 32) {
-            const float diff = qv[d] - x[d];
-            s = fmaf(diff, diff, s);
+            const float y = qv[d];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float diff = y - x[u][d];
+                s[u] = fmaf(diff, diff, s[u]);
+            }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-        if (lane == 0) a[j] = ((uint64_t)__float_as_uint(s) << 32) | (uint64_t)(uint32_t)id;
+        for (int u = 0; u < 2; ++u) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xFFFFFFFFu, s[u], o);
+            if (lane == 0 && id[u] >= 0)
+                a[j + u * kRerankWarps] = ((uint64_t)__float_as_uint(s[u]) << 32) | (uint64_t)(uint32_t)id[u];
+        }
     }
     block_sort(a, rp);
     for (int i = threadIdx.x; i < k; i += blockDim.x) write_key(a[i], ids + qi * k + i, dists + qi * k + i);
@@ -202,7 +222,7 @@ cudaError_t launch_rerank(const float* X, int64_t N, int D, const float* q, cons
     if (nq <= 0) return cudaSuccess;
     int rp = 32;
     while (rp < R) rp <<= 1;
-    return launch_kernel(k_rerank, dim3((unsigned)nq), dim3(256), 0, chain, s, X, N, D, q, cand, R, k, rp, ids, dists);
+    return launch_kernel(k_rerank, dim3((unsigned)nq), dim3(kRerankWarps * 32), 0, chain, s, X, N, D, q, cand, R, k, rp, ids, dists);
 }
 
 }  // namespace ifvs

@@ -61,88 +61,150 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_gram(const float* __res
 // scatter of dL/dC into the query's dense gC slice and dL/dw_f.  Each thread
 // owns the dimensions d = tid + i * blockDim, so every gC address (m, *, t)
 // is written by one thread only, in candidate order.
+//
+// What bounded it was latency and the float64 pipe (about two additions per SM
+// and cycle): one thread made the candidate list, every candidate waited for
+// the one before it (10 dependent loads each) and was summed over the CTA in
+// float64.  Now a warp makes the list by ballots, four candidates' code and W
+// values are loaded together, the differences go to shared memory and a few
+// threads per candidate add its terms as float pairs that carry the rounding
+// errors (about 48 bits), and so is dL/dw_f.  1024 queries with 42 candidates:
+// 228 us before, TRAIN_FIGURES.
+constexpr int kTrainDiffs = 8192;      // floats of the differences held at a time
+constexpr int kTrainBatch = 4;         // candidates whose loads are in flight together
+
+// floats shared by the differences (pass 1) and dL/dalpha per dimension (pass
+// 2), and the candidates whose differences they hold
+__host__ __device__ inline int train_floats(int D, int r) {
+    const int need = D * r > D + 1 ? D * r : D + 1;
+    return need > kTrainDiffs ? need : kTrainDiffs;
+}
+__host__ __device__ inline int train_chunk(int V, int D, int r) {
+    const int c = train_floats(D, r) / (D + 1);
+    return c < V ? c : V;
+}
+
 template <int RMAX>
 __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int V = a.P + a.n_neg;
     const int Mr = a.M * a.r;
+    const int CH = train_chunk(V, a.D, a.r);
     int64_t* cand = reinterpret_cast<int64_t*>(sm);
-    double* part = reinterpret_cast<double*>(cand + V);       // [V][warps]
-    double* dist = part + (size_t)V * kTrainWarps;            // [V]
+    double* dist = reinterpret_cast<double*>(cand + V);       // [V]
     double* gam = dist + V;                                   // [V]
-    double* red = gam + V;                                    // [warps]
-    float* alpha = reinterpret_cast<float*>(red + kTrainWarps);   // [Mr]
-    float* gas = alpha + Mr;                                      // [D][r]: dL/dalpha per dimension
+    double* red = gam + V;                                    // [warps + 1]
+    float* alpha = reinterpret_cast<float*>(red + kTrainWarps + 1);   // [Mr]
+    float* dfs = alpha + Mr;                                      // [CH][D + 1] differences
+    float* gas = dfs;                                             // [D][r]: dL/dalpha per dimension
     const int64_t q = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nwarps = blockDim.x >> 5;
+    const float* qv = a.q + q * a.D;
+    const float* wf = a.wf + q * a.D;
 
-    if (tid == 0) {
+    if (warp == 0) {
         const int64_t* pos = a.pos + q * a.pos_stride;
-        for (int g = 0; g < a.P; ++g) cand[g] = pos[g];
         const int64_t* src = a.negsrc + q * a.neg_stride;
+        bool bad = false;
+        auto checked = [&](int64_t id) {
+            const bool out = id < -1 || id >= a.N;
+            bad |= out;
+            return out ? (int64_t)-1 : id;
+        };
+        // positives as given while the mined list is compared with them
+        for (int g = lane; g < a.P; g += 32) cand[g] = pos[g];
+        __syncwarp();
         int got = 0;
-        for (int s = 0; s < a.S && got < a.n_neg; ++s) {
-            const int64_t id = src[s];
+        for (int s0 = 0; s0 < a.S && got < a.n_neg; s0 += 32) {
+            const int s = s0 + lane;
+            const int64_t id = s < a.S ? src[s] : -1;
+            bool keep = s < a.S;
+            unsigned end = 0u;
             if (a.exclude) {
-                if (id < 0) break;
-                bool is_pos = false;
-                for (int g = 0; g < a.P; ++g) is_pos |= pos[g] == id;
-                if (is_pos) continue;
+                end = __ballot_sync(0xFFFFFFFFu, s < a.S && id < 0);   // a mined list ends at its first -1
+                keep = keep && (end == 0u || lane < __ffs(end) - 1);
+                for (int g = 0; g < a.P; ++g) keep = keep && cand[g] != id;
             }
-            cand[a.P + got++] = id;
+            const unsigned ball = __ballot_sync(0xFFFFFFFFu, keep);
+            const int at = got + __popc(ball & ((1u << lane) - 1u));
+            if (keep && at < a.n_neg) cand[a.P + at] = checked(id);
+            got = min(a.n_neg, got + __popc(ball));
+            if (end != 0u) break;
         }
-        for (; got < a.n_neg; ++got) cand[a.P + got] = -1;
-        for (int v = 0; v < V; ++v)
-            if (cand[v] < -1 || cand[v] >= a.N) {
-                atomicOr(a.err, 2);
-                cand[v] = -1;
-            }
+        for (int n = got + lane; n < a.n_neg; n += 32) cand[a.P + n] = -1;
+        for (int g = lane; g < a.P; g += 32) cand[g] = checked(cand[g]);
+        if (bad) atomicOr(a.err, 2);
+        __syncwarp();
         if (a.neg_out)
-            for (int n = 0; n < a.n_neg; ++n) a.neg_out[q * a.n_neg + n] = cand[a.P + n];
+            for (int n = lane; n < a.n_neg; n += 32) a.neg_out[q * a.n_neg + n] = cand[a.P + n];
     }
     for (int e = tid; e < Mr; e += blockDim.x) alpha[e] = a.alpha[q * Mr + e];
     __syncthreads();
 
-    const float* qv = a.q + q * a.D;
-    const float* wf = a.wf + q * a.D;
     const int64_t KD = (int64_t)a.K * a.ds;
-
-    // C_iFVS[m][c][t] = C_PQ + sum_j alpha[m][j] W[m][j][c][t] for the code of
-    // candidate `id` in the subspace of dimension d; returns q_d - C
-    auto diff_of = [&](int64_t id, int d, int* code) -> float {
-        const int m = d / a.ds, t = d - m * a.ds;
-        const int rot = (int)(id & 31) % a.M;
-        int s = m - rot;
+    // code of candidate `id` in subspace m
+    auto code_of = [&](int64_t id, int m) -> int {
+        int s = m - (int)(id & 31) % a.M;
         if (s < 0) s += a.M;
-        const int c = a.codes[id * a.row_bytes + s];
-        *code = c;
-        const int64_t e = (int64_t)c * a.ds + t;
-        float C = a.C_pq[(int64_t)m * KD + e];
-        for (int j = 0; j < a.r; ++j) C += alpha[m * a.r + j] * a.W[((int64_t)m * a.r + j) * KD + e];
-        return qv[d] - C;
+        return a.codes[id * a.row_bytes + s];
     };
 
-    // pass 1: weighted distances (float32 terms, fp64 sums)
-    for (int v = 0; v < V; ++v) {
-        const int64_t id = cand[v];
-        double acc = 0.0;
-        if (id >= 0)
-            for (int d = tid; d < a.D; d += blockDim.x) {
-                int c;
-                const float df = diff_of(id, d, &c);
-                acc += (double)(wf[d] * df * df);
+    // pass 1: weighted distances (float32 terms of 48-bit sums).  The term of
+    // dimension d = m ds + t is w_f (q - C)^2 with C_iFVS[m][c][t] = C_PQ +
+    // sum_j alpha[m][j] W[m][j][c][t].
+    for (int v0 = 0; v0 < V; v0 += CH) {
+        const int nv = min(CH, V - v0);
+        for (int d = tid; d < a.D; d += blockDim.x) {
+            const int m = d / a.ds, t = d - m * a.ds;
+            const float* Cm = a.C_pq + (int64_t)m * KD + t;
+            const float* Wm = a.W + (int64_t)m * a.r * KD + t;
+            for (int i0 = 0; i0 < nv; i0 += kTrainBatch) {
+                int c[kTrainBatch];
+                float C[kTrainBatch];
+#pragma unroll
+                for (int u = 0; u < kTrainBatch; ++u) {
+                    const int64_t id = i0 + u < nv ? cand[v0 + i0 + u] : -1;
+                    c[u] = id >= 0 ? code_of(id, m) * a.ds : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < kTrainBatch; ++u) C[u] = __ldg(Cm + c[u]);
+#pragma unroll
+                for (int j = 0; j < RMAX; ++j)
+                    if (j < a.r) {
+                        const float al = alpha[m * a.r + j];
+#pragma unroll
+                        for (int u = 0; u < kTrainBatch; ++u) C[u] += al * __ldg(Wm + (int64_t)j * KD + c[u]);
+                    }
+#pragma unroll
+                for (int u = 0; u < kTrainBatch; ++u)
+                    if (i0 + u < nv) dfs[(i0 + u) * (a.D + 1) + d] = qv[d] - C[u];
             }
-        acc = warp_sum(acc);
-        if (lane == 0) part[v * kTrainWarps + warp] = acc;
+        }
+        __syncthreads();
+        // 4 neighbouring threads per candidate, every fourth dimension each
+        for (int x = tid; x < ((4 * nv + 31) & ~31); x += blockDim.x) {
+            const int i = x >> 2, p = x & 3;
+            Sum2 s;
+            if (i < nv)
+                for (int d = p; d < a.D; d += 4) {
+                    const float df = dfs[i * (a.D + 1) + d];
+                    s.add(__ldg(wf + d) * df * df);
+                }
+            double t = s.value();
+            if (i < nv && !s.finite()) {   // beyond float32, infinite or NaN
+                t = 0.0;
+                for (int d = p; d < a.D; d += 4) {
+                    const float df = dfs[i * (a.D + 1) + d];
+                    t += (double)(__ldg(wf + d) * df * df);
+                }
+            }
+            t += __shfl_xor_sync(0xFFFFFFFFu, t, 1);
+            t += __shfl_xor_sync(0xFFFFFFFFu, t, 2);
+            if (i < nv && p == 0) dist[v0 + i] = cand[v0 + i] >= 0 ? t : 0.0;
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int v = tid; v < V; v += blockDim.x) {
-        double s = 0.0;
-        for (int w = 0; w < nwarps; ++w) s += part[v * kTrainWarps + w];
-        dist[v] = s;
-    }
-    __syncthreads();
 
     // Softmax of each positive g against the negatives N, with the shift
     // m_g = min(dist_g, m_N), m_N = min over N:
@@ -182,26 +244,24 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a)
         const double inv = npos > 0 ? 1.0 / npos : 0.0;
         for (int n = a.P + lane; n < V; n += 32) gam[n] = -gam[n] * csum / a.tau * inv;
         for (int g = lane; g < a.P; g += 32) gam[g] *= inv;
-        if (lane == 0) red[0] = npos > 0 ? lpos * inv : 0.0;
+        if (lane == 0) red[kTrainWarps] = npos > 0 ? lpos * inv : 0.0;
     }
-    // anchor ||Delta||^2 = sum_m alpha[m]^T G_m alpha[m]
+    // anchor ||Delta||^2 = sum_m alpha[m]^T G_m alpha[m], a row of G_m per thread
     double an = 0.0;
-    for (int m = tid; m < a.M; m += blockDim.x) {
-        const float* Gm = a.G + (int64_t)m * a.r * a.r;
-        for (int j = 0; j < a.r; ++j)
-            for (int j2 = 0; j2 < a.r; ++j2)
-                an += (double)alpha[m * a.r + j] * (double)Gm[j * a.r + j2] * (double)alpha[m * a.r + j2];
+    for (int x = tid; x < Mr; x += blockDim.x) {
+        const int m = x / a.r;
+        double row = 0.0;
+        for (int j2 = 0; j2 < a.r; ++j2)
+            row += (double)a.G[(int64_t)x * a.r + j2] * (double)alpha[m * a.r + j2];
+        an += (double)alpha[x] * row;
     }
     an = warp_sum(an);
-    __syncthreads();
-    const double lpos = red[0];
-    __syncthreads();
     if (lane == 0) red[warp] = an;
     __syncthreads();
     if (tid == 0) {
         double s = 0.0;
         for (int w = 0; w < nwarps; ++w) s += red[w];
-        a.loss[q] = lpos + (double)a.lambda * s;
+        a.loss[q] = red[kTrainWarps] + (double)a.lambda * s;
     }
 
     // pass 2: gC scatter, dL/dw_f, and dL/dalpha through the same W values:
@@ -209,25 +269,63 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a)
     float* gC = a.gC + q * (int64_t)a.M * KD;
     for (int d = tid; d < a.D; d += blockDim.x) {
         const int m = d / a.ds, t = d - m * a.ds;
-        double gw = 0.0;
+        const float* Cm = a.C_pq + (int64_t)m * KD + t;
+        const float* Wm = a.W + (int64_t)m * a.r * KD + t;
+        float* gm = gC + (int64_t)m * KD + t;
+        Sum2 gw;
         float ga[RMAX];
 #pragma unroll
         for (int j = 0; j < RMAX; ++j) ga[j] = 0.f;
-        for (int v = 0; v < V; ++v) {
-            const int64_t id = cand[v];
-            if (id < 0) continue;
-            int c;
-            const float df = diff_of(id, d, &c);
-            const float ge = (float)gam[v] * (-2.f * wf[d] * df);
-            const int64_t e = (int64_t)c * a.ds + t;
-            gC[(int64_t)m * KD + e] += ge;
-            gw += gam[v] * (double)(df * df);
-            const float* Wc = a.W + (int64_t)m * a.r * KD + e;
+        constexpr int B = RMAX <= 8 ? kTrainBatch : 1;
+        for (int v0 = 0; v0 < V; v0 += B) {
+            int c[B];
+            float C[B], w[B][RMAX];
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                const int64_t id = v0 + u < V ? cand[v0 + u] : -1;
+                c[u] = id >= 0 ? code_of(id, m) * a.ds : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < B; ++u) C[u] = __ldg(Cm + max(c[u], 0));
 #pragma unroll
             for (int j = 0; j < RMAX; ++j)
-                if (j < a.r) ga[j] += ge * Wc[(int64_t)j * KD];
+                if (j < a.r)
+#pragma unroll
+                    for (int u = 0; u < B; ++u) w[u][j] = __ldg(Wm + (int64_t)j * KD + max(c[u], 0));
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                if (c[u] < 0) continue;
+#pragma unroll
+                for (int j = 0; j < RMAX; ++j)
+                    if (j < a.r) C[u] += alpha[m * a.r + j] * w[u][j];
+                const float df = qv[d] - C[u];
+                const double g = gam[v0 + u];
+                const float gf = (float)g;
+                const float ge = gf * (-2.f * __ldg(wf + d) * df);
+                gm[c[u]] += ge;
+                // gam (df df) to about 48 bits: gam as two floats, exact products
+                const float sq = df * df, p = __fmul_rn(gf, sq);
+                gw.add(p);
+                gw.lo = __fadd_rn(gw.lo, fmaf((float)(g - (double)gf), sq, fmaf(gf, sq, -p)));
+#pragma unroll
+                for (int j = 0; j < RMAX; ++j)
+                    if (j < a.r) ga[j] += ge * w[u][j];
+            }
         }
-        a.gw[q * a.D + d] = (float)gw;
+        double gwd = gw.value();
+        if (!gw.finite()) {   // beyond float32, infinite or NaN: in float64
+            gwd = 0.0;
+            for (int v = 0; v < V; ++v) {
+                const int64_t id = cand[v];
+                if (id < 0) continue;
+                const int c = code_of(id, m) * a.ds;
+                float C = Cm[c];
+                for (int j = 0; j < a.r; ++j) C += alpha[m * a.r + j] * Wm[(int64_t)j * KD + c];
+                const float df = qv[d] - C;
+                gwd += gam[v] * (double)(df * df);
+            }
+        }
+        a.gw[q * a.D + d] = (float)gwd;
 #pragma unroll
         for (int j = 0; j < RMAX; ++j)
             if (j < a.r) gas[d * a.r + j] = ga[j];
@@ -392,8 +490,8 @@ __global__ void k_sgd(float* __restrict__ theta, const float* __restrict__ g, in
 }
 
 size_t train_query_smem(int V, int Mr, int D, int r) {
-    return sizeof(int64_t) * V + sizeof(double) * ((size_t)V * kTrainWarps + 2 * V + kTrainWarps) +
-           sizeof(float) * (Mr + (size_t)D * r);
+    return sizeof(int64_t) * V + sizeof(double) * ((size_t)2 * V + kTrainWarps + 1) +
+           sizeof(float) * (Mr + (size_t)train_floats(D, r));
 }
 
 cudaError_t launch_train_gram(const float* W, int M, int r, int KD, float* G, cudaStream_t s) {
