@@ -1707,15 +1707,11 @@ int ifvs_train_step(ifvs_index* ix, const float* queries, const ifvs_predicate* 
     const int64_t nW = (int64_t)ix->M * ix->r * ix->K * ix->ds;
     {
         Stage st(ix, s, o.timing, IFVS_STAGE_TRAIN);
-        CUDA_TRY(st.end(launch_sgd(ix->d_bank, ix->t_gbank.as<float>(), ix->B * Mr, tp->lr, s)));
-    }
-    {
-        Stage st(ix, s, o.timing, IFVS_STAGE_TRAIN);
-        CUDA_TRY(st.end(launch_sgd(ix->d_W, ix->t_gW.as<float>(), nW, tp->lr, s)));
-    }
-    {
-        Stage st(ix, s, o.timing, IFVS_STAGE_TRAIN);
-        CUDA_TRY(st.end(launch_sgd(ix->t_wz.as<float>(), ix->t_gwz.as<float>(), ix->D, tp->lr_wz, s)));
+        SgdArgs sg{{ix->d_bank, ix->d_W, ix->t_wz.as<float>()},
+                   {ix->t_gbank.as<float>(), ix->t_gW.as<float>(), ix->t_gwz.as<float>()},
+                   {ix->B * Mr, nW, ix->D},
+                   {tp->lr, tp->lr, tp->lr_wz}};
+        CUDA_TRY(st.end(launch_sgd(sg, s)));
     }
     TRY(copy_out(s, o.dio, wz, ix->t_wz.p, sizeof(float) * ix->D));
     if (negatives && tp->n_neg > 0)

@@ -432,7 +432,13 @@ cudaError_t launch_train_bank(const uint32_t* idx, int64_t n, int h, int Mr, con
                               float inv_n, float* gbank, cudaStream_t s);
 cudaError_t launch_train_wz(const float* gw, int64_t n, int D, const float* wz, float inv_n, float* gwz,
                             cudaStream_t s);
-cudaError_t launch_sgd(float* theta, const float* g, int64_t n, float lr, cudaStream_t s);
+struct SgdArgs {
+    float* theta[3];
+    const float* g[3];
+    int64_t n[3];
+    float lr[3];
+};
+cudaError_t launch_sgd(const SgdArgs& a, cudaStream_t s);
 
 // Read-only view of a loaded index, for entry points defined outside api.cu.
 struct IndexView {

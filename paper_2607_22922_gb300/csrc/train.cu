@@ -69,7 +69,8 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_gram(const float* __res
 // values are loaded together, the differences go to shared memory and a few
 // threads per candidate add its terms as float pairs that carry the rounding
 // errors (about 48 bits), and so is dL/dw_f.  1024 queries with 42 candidates:
-// 228 us before, TRAIN_FIGURES.
+// 228 us before, 195 us now; what is left is the latency of those loads (pass 1
+// about 85 us, pass 2 75) at the 16 warps per SM that 128 registers leave.
 constexpr int kTrainDiffs = 8192;      // floats of the differences held at a time
 constexpr int kTrainBatch = 4;         // candidates whose loads are in flight together
 
@@ -84,7 +85,9 @@ __host__ __device__ inline int train_chunk(int V, int D, int r) {
     return c < V ? c : V;
 }
 
-template <int RMAX>
+// EXACT: r = RMAX, so no load is behind a test of r and a batch's are all in
+// flight at once.
+template <int RMAX, bool EXACT>
 __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int V = a.P + a.n_neg;
@@ -169,13 +172,25 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a)
                 }
 #pragma unroll
                 for (int u = 0; u < kTrainBatch; ++u) C[u] = __ldg(Cm + c[u]);
+                if constexpr (EXACT && RMAX <= 8) {
+                    float w[kTrainBatch][RMAX];
 #pragma unroll
-                for (int j = 0; j < RMAX; ++j)
-                    if (j < a.r) {
-                        const float al = alpha[m * a.r + j];
+                    for (int u = 0; u < kTrainBatch; ++u)
 #pragma unroll
-                        for (int u = 0; u < kTrainBatch; ++u) C[u] += al * __ldg(Wm + (int64_t)j * KD + c[u]);
-                    }
+                        for (int j = 0; j < RMAX; ++j) w[u][j] = __ldg(Wm + (int64_t)j * KD + c[u]);
+#pragma unroll
+                    for (int j = 0; j < RMAX; ++j)
+#pragma unroll
+                        for (int u = 0; u < kTrainBatch; ++u) C[u] += alpha[m * RMAX + j] * w[u][j];
+                } else {
+#pragma unroll
+                    for (int j = 0; j < RMAX; ++j)
+                        if (j < a.r) {
+                            const float al = alpha[m * a.r + j];
+#pragma unroll
+                            for (int u = 0; u < kTrainBatch; ++u) C[u] += al * __ldg(Wm + (int64_t)j * KD + c[u]);
+                        }
+                }
 #pragma unroll
                 for (int u = 0; u < kTrainBatch; ++u)
                     if (i0 + u < nv) dfs[(i0 + u) * (a.D + 1) + d] = qv[d] - C[u];
@@ -289,7 +304,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a)
             for (int u = 0; u < B; ++u) C[u] = __ldg(Cm + max(c[u], 0));
 #pragma unroll
             for (int j = 0; j < RMAX; ++j)
-                if (j < a.r)
+                if (EXACT || j < a.r)
 #pragma unroll
                     for (int u = 0; u < B; ++u) w[u][j] = __ldg(Wm + (int64_t)j * KD + max(c[u], 0));
 #pragma unroll
@@ -297,7 +312,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a)
                 if (c[u] < 0) continue;
 #pragma unroll
                 for (int j = 0; j < RMAX; ++j)
-                    if (j < a.r) C[u] += alpha[m * a.r + j] * w[u][j];
+                    if (EXACT || j < a.r) C[u] += alpha[m * a.r + j] * w[u][j];
                 const float df = qv[d] - C[u];
                 const double g = gam[v0 + u];
                 const float gf = (float)g;
@@ -309,7 +324,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a)
                 gw.lo = __fadd_rn(gw.lo, fmaf((float)(g - (double)gf), sq, fmaf(gf, sq, -p)));
 #pragma unroll
                 for (int j = 0; j < RMAX; ++j)
-                    if (j < a.r) ga[j] += ge * w[u][j];
+                    if (EXACT || j < a.r) ga[j] += ge * w[u][j];
             }
         }
         double gwd = gw.value();
@@ -328,7 +343,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a)
         a.gw[q * a.D + d] = (float)gwd;
 #pragma unroll
         for (int j = 0; j < RMAX; ++j)
-            if (j < a.r) gas[d * a.r + j] = ga[j];
+            if (EXACT || j < a.r) gas[d * a.r + j] = ga[j];
     }
     __syncthreads();
     // sum over the subspace's dimensions in order, plus the anchor 2 lambda G_m alpha[m]
@@ -471,8 +486,17 @@ __global__ void __launch_bounds__(1024) k_train_wz(const float* __restrict__ gw,
     __shared__ double part[32][33];
     const int d = blockIdx.x * 32 + threadIdx.x;
     double s = 0.0;
-    if (d < D)
-        for (int64_t q = threadIdx.y; q < n; q += 32) s += (double)gw[q * D + d];
+    if (d < D) {
+        // float pairs: the float64 adders took 22 us for 1024 queries at D = 128
+        Sum2 p;
+#pragma unroll 8
+        for (int64_t q = threadIdx.y; q < n; q += 32) p.add(gw[q * D + d]);
+        s = p.value();
+        if (!p.finite()) {
+            s = 0.0;
+            for (int64_t q = threadIdx.y; q < n; q += 32) s += (double)gw[q * D + d];
+        }
+    }
     part[threadIdx.y][threadIdx.x] = s;
     __syncthreads();
     if (threadIdx.y != 0 || d >= D) return;
@@ -483,10 +507,15 @@ __global__ void __launch_bounds__(1024) k_train_wz(const float* __restrict__ gw,
     gwz[d] = (float)t * sg * inv_n;
 }
 
-// theta <- theta - lr * g
-__global__ void k_sgd(float* __restrict__ theta, const float* __restrict__ g, int64_t n, float lr) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) theta[e] = theta[e] - lr * g[e];
+// theta <- theta - lr * g for the bank, W and w_z
+__global__ void k_sgd(SgdArgs a) {
+    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        if (e < a.n[i]) a.theta[i][e] = a.theta[i][e] - a.lr[i] * a.g[i][e];
+        if (e < a.n[i]) return;
+        e -= a.n[i];
+    }
 }
 
 size_t train_query_smem(int V, int Mr, int D, int r) {
@@ -503,7 +532,8 @@ cudaError_t launch_train_query(const TrainQueryArgs& a, cudaStream_t s) {
     const size_t smem = train_query_smem(a.P + a.n_neg, a.M * a.r, a.D, a.r);
     // threads own dimensions: no more threads than (32-rounded) dimensions
     const int threads = a.D >= kTrainThreads ? kTrainThreads : ((a.D + 31) / 32) * 32;
-    auto kern = a.r <= 8 ? k_train_query<8> : k_train_query<kTrainMaxR>;
+    auto kern = a.r == 8 ? k_train_query<8, true>
+                         : (a.r < 8 ? k_train_query<8, false> : k_train_query<kTrainMaxR, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)a.n, threads, smem, s>>>(a);
@@ -550,9 +580,10 @@ cudaError_t launch_train_wz(const float* gw, int64_t n, int D, const float* wz, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_sgd(float* theta, const float* g, int64_t n, float lr, cudaStream_t s) {
+cudaError_t launch_sgd(const SgdArgs& a, cudaStream_t s) {
+    const int64_t n = a.n[0] + a.n[1] + a.n[2];
     if (n <= 0) return cudaSuccess;
-    k_sgd<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(theta, g, n, lr);
+    k_sgd<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
