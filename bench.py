@@ -47,9 +47,10 @@ if ROOT not in sys.path:
 
 WORKLOAD = "gmm100m-d128-m16"
 LIST_DEFAULT_PPM = 1000000   # the library's default sorted-copy threshold (always)
-# the library's automatic pairing: rows a pair spans and rows a batch's ranges
-# hold together, at least, for k <= 32 and above
-PAIR_AUTO = {True: (160_000, 30_000_000), False: (300_000, 90_000_000)}
+# the library's automatic pairing for k <= 32 and above: rows a pair spans and
+# rows a batch's ranges hold together, at least; of bitmap queries the share of
+# the rows passing (forty parts) and rows times queries, at least
+PAIR_AUTO = {True: (160_000, 30_000_000, 9, 30_000_000), False: (300_000, 90_000_000, 12, 128_000_000)}
 TRAIN_WORKLOAD = "sift1m-d128-m16"
 CPU_SAMPLE_ROWS = 10_000_000
 
@@ -508,14 +509,16 @@ def sorted_path(preds, attrs, npass, list_rows):
     return out
 
 
-def scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, pair_total=0, seg=2048):
+def scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, pair_total=0, bm_pass=-1, bm_total=0, seg=2048):
     """Shared-memory look-ups the scan stage executes for one batch, by the
-    library's pairing rule for one-column ranges of the sorted copy (M = 16;
+    library's pairing rule for one-column ranges of the sorted copy (M = 12, 16;
     sort by (column, range start, query) per 2048-query segment; neighbours
     2j, 2j+1 pair when 3/4 of the longer range is common and the two span at
     least pair_rows, in batches whose ranges hold pair_total rows or more): a
     pair costs the union of its ranges x M (one load
-    serves both queries), any other query its pool x M."""
+    serves both queries), any other query its pool x M.  Bitmap queries that
+    at least bm_pass rows pass pair in their order when their number times the
+    rows reaches bm_total: all rows x M per pair."""
     n = len(qs.q)
     a = np.zeros(n, np.int64)
     b = np.zeros(n, np.int64)
@@ -543,7 +546,7 @@ def scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, pair_total=0, se
         span = max(b[x], b[y]) - min(a[x], a[y])
         return 4 * common >= 3 * max(lx, ly) and span >= pair_rows
 
-    if w.M == 16 and pair_rows >= 0 and (b - a).sum() >= pair_total:
+    if w.M in (12, 16) and pair_rows >= 0 and (b - a).sum() >= pair_total:
         for s0 in range(0, n, seg):
             idx = [i for i in range(s0, min(n, s0 + seg)) if on_list[i]]
             idx.sort(key=lambda i: (col[i], a[i], i))
@@ -552,6 +555,11 @@ def scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, pair_total=0, se
                 if pair_ok(x, y):
                     paired[x] = paired[y] = True
                     union += max(b[x], b[y]) - min(a[x], a[y])
+    dense = np.flatnonzero(~on_list & (npass > 0) & (npass >= bm_pass))
+    rows = (w.N + 1023) // 1024 * 1024
+    if w.M in (12, 16) and bm_pass >= 0 and len(dense) > 1 and len(dense) * rows >= bm_total:
+        paired[dense[:len(dense) // 2 * 2]] = True
+        union += rows * (len(dense) // 2)
     single = float(npass[~paired].sum())
     return {"lookups": (single + union) * w.M, "paired_share": float(paired.mean())}
 
@@ -659,7 +667,10 @@ def run_ifvs(args):
     n_blocks = (w.N + 1023) // 1024
     ppm = args.list_max_ppm if args.list_max_ppm != 0 else LIST_DEFAULT_PPM
     list_rows = -1 if ppm < 0 else w.N * ppm // 1000000
-    pair_rows, pair_total = (args.pair_min_rows, 0) if args.pair_min_rows != 0 else PAIR_AUTO[w.k <= 32]
+    pair_rows, pair_total, bm_pass, bm_total = args.pair_min_rows, 0, args.pair_min_rows, 0
+    if args.pair_min_rows == 0:
+        pair_rows, pair_total, bm_pass, bm_total = PAIR_AUTO[w.k <= 32]
+        bm_pass = w.N // 40 * bm_pass
     lookups_total = code_bytes_total = 0.0
     sorted_vals = [np.sort(a) for a in ix.attrs]
     for b, qs in enumerate(batches):
@@ -667,7 +678,7 @@ def run_ifvs(args):
         npass = dev_out[b][2].cpu().numpy().astype(np.float64)
         nsteps_b = len(ms_b)
         on_list = sorted_path(qs.preds, ix.attrs, npass, list_rows)
-        lk = scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, pair_total)
+        lk = scan_lookups(w, qs, sorted_vals, on_list, npass, pair_rows, pair_total, bm_pass, bm_total)
         lookups_total += nsteps_b * lk["lookups"]
         code_bytes_total += nsteps_b * float(npass.sum()) * w.M
         per_bin[str(qs.sel)] = {
@@ -676,8 +687,8 @@ def run_ifvs(args):
             "mean_selectivity": float(npass.mean() / w.N),
             "sorted_path_share": float(on_list.mean()),
             "paired_share": lk["paired_share"]}
-    # The scan stage (per batch: k_pair_items, k_scan_list_pair, k_scan_list
-    # and k_scan, one launch of each) is the unit.  Its binding resource is
+    # The scan stage (per batch: k_schedule, k_scan_list_pair, the one-query
+    # sorted-copy kernel and k_scan, one launch of each) is the unit.  Its binding resource is
     # the shared-memory look-up rate: one conflict-free 32-lane load per SM
     # per cycle.  Executed look-ups per batch: passing positions x M for a
     # query scanned alone, and for a pair of queries the positions of the
@@ -692,7 +703,7 @@ def run_ifvs(args):
     achieved = (lookups_total / nbatch) / (scan_ms / nbatch / 1000.0) if scan_ms > 0 else None
     hbm_peak, peak_kind = measured_peaks()
     dram = scan_dram(w.name, hbm_peak)
-    roofline = {"kernel": "scan stage (k_pair_items + k_scan_list_pair + k_scan_list_bulk; k_scan_list and"
+    roofline = {"kernel": "scan stage (k_schedule + k_scan_list_pair + k_scan_list_bulk; k_scan_list and"
                           " k_scan where a query takes them)",
                 "bound": "smem", "achieved": achieved, "peak": peak, "unit": "look-ups/s",
                 "frac": achieved / peak if achieved else None,

@@ -135,16 +135,19 @@ typedef struct {
                            0: default (1000000: always); -1: never.  The two
                            paths sum a row's entries in different orders, so
                            distances agree to float32 rounding.              */
-    int32_t pair_min_rows; /* M = 16 sorted-copy scan: two queries on the same
+    int32_t pair_min_rows; /* M = 12 and 16: two queries on the same sorted
                            column whose ranges share 3/4 of the longer one
-                           and together span at least this many rows share a
-                           CTA and one shared-memory look-up per code byte
-                           (tables quantised to 11 bits; every row that can
-                           reach a top-k is rescored exactly, so results
+                           and together span at least this many rows, or two
+                           bitmap queries that at least this many rows pass,
+                           share a CTA and one shared-memory look-up per code
+                           byte (tables quantised to 11 bits; every row that
+                           can reach a top-k is rescored exactly, so results
                            equal those of one query per CTA bit for bit).
                            0: automatic (spans of at least 160000 rows in
                            batches whose ranges hold 3e7 together, 300000
-                           and 9e7 for k > 32); -1: never pair.            */
+                           and 9e7 for k > 32; 22.5 % of the rows passing in
+                           batches of 3e7 rows times queries, 30 % and
+                           1.28e8 for k > 32); -1: never pair.             */
     void* stream;       /* cudaStream_t to run on; NULL: the index's stream   */
 } ifvs_search_params;
 

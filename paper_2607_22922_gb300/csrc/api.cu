@@ -445,13 +445,18 @@ constexpr int32_t kListDefaultPpm = 1000000;
 // 64 queries: 4 x 10^5 165 / 174, 5 x 10^5 170 / 156, 10^6 262 / 193.
 // k = 100, 1024 queries: 2 x 10^5 912 / 985, 4 x 10^5 1541 / 1443; 64
 // queries: 4 x 10^5 233 / 320, 10^6 337 / 325, 2 x 10^6 561 / 466.
-struct PairRule {
-    int64_t span;      // rows a pair spans, at least
-    int64_t total;     // rows of the batch's ranges together, at least
-};
-PairRule pair_rule(int32_t pair_min_rows, int k) {
-    if (pair_min_rows > 0) return {pair_min_rows, 0};
-    return k <= 32 ? PairRule{160000, 30000000} : PairRule{300000, 90000000};
+//
+// Bitmap queries (any two share every block): a pair's time does not depend on
+// how many rows pass, a single one's does.  Measured (us per batch, single /
+// paired) on 4 x 10^6 rows of 16 codes, 256 queries, k = 10: 20 % passing 1767
+// / 1965, 30 % 2345 / 1933, 50 % 2887 / 1947; 64 queries of 10^6: 20 % 190 /
+// 199, 30 % 225 / 196; 16 of 10^6: 40 % 110 / 107.  k = 100: 512 queries of
+// 2 x 10^6, 20 % 1912 / 2219, 30 % 2356 / 2168, 40 % 2860 / 2186; 64 of 10^6,
+// 40 % 328 / 333.
+PairRule pair_rule(int32_t pair_min_rows, int64_t N, int k) {
+    if (pair_min_rows > 0) return {pair_min_rows, 0, pair_min_rows, 0};
+    return k <= 32 ? PairRule{160000, 30000000, N / 40 * 9, 30000000}
+                   : PairRule{300000, 90000000, N / 40 * 12, 128000000};
 }
 
 int parse_opts(const ifvs_search_params* p, Opts* o) {
@@ -502,11 +507,12 @@ ScanShape scan_shape(const ifvs_index* ix) {
 // Work lists of n queries (k keys per list) in w_part; groups that the batch
 // cannot use get no room.
 int make_sched(ifvs_index* ix, const ScanShape& sh, int64_t n, int k, const Opts& o, bool lists, bool bitmaps,
-               bool pairs, ScanSched* s) {
-    const int slots[3] = {ix->num_sms * scan_list_ctas_per_sm(sh, k, !o.plain_loads),
-                          ix->num_sms * scan_ctas_per_sm(ix->tab_words, scan_kp(k)), ix->num_sms};
+               bool pairs, bool bm_pairs, ScanSched* s) {
+    const int slots[kGroups] = {ix->num_sms * scan_list_ctas_per_sm(sh, k, !o.plain_loads),
+                                ix->num_sms * scan_ctas_per_sm(ix->tab_words, scan_kp(k)), ix->num_sms,
+                                ix->num_sms};
     const int64_t any = (int64_t)1 << 40;
-    const int64_t most[3] = {lists ? any : 0, bitmaps ? any : 0, pairs ? any : 0};
+    const int64_t most[kGroups] = {lists ? any : 0, bitmaps ? any : 0, pairs ? any : 0, bm_pairs ? any : 0};
     TRY(ensure(ix->w_part, scan_sched_layout(n, k, ix->n_blocks, slots, o.chunk_blocks, most, nullptr, s)));
     scan_sched_layout(n, k, ix->n_blocks, slots, o.chunk_blocks, most, ix->w_part.as<uint8_t>(), s);
     return 0;
@@ -566,11 +572,16 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     const ScanShape sh = scan_shape(ix);
     // where no pair can arise its kernel is not launched (with stage timing
     // every kernel of the path is)
-    const PairRule pr = pair_rule(o.pair_min_rows, kk);
-    const bool pairs = list_on && o.pair_min_rows >= 0 && scan_pairs_fit(sh, kk) &&
-                       (o.timing || (n > 1 && ix->N >= pr.span && n * ix->N >= pr.total));
+    PairRule pr = pair_rule(o.pair_min_rows, ix->N, kk);
+    const bool may_pair = o.pair_min_rows >= 0 && scan_pairs_fit(sh, kk);
+    const bool pairs = list_on && may_pair &&
+                       ((o.timing && ix->M == 16) || (n > 1 && ix->N >= pr.span && n * ix->N >= pr.total));
+    const bool bm_pairs =
+        bitmaps && may_pair && n > 1 && ix->N >= pr.bm_pass && n * ix->n_blocks * kBlockRows >= pr.bm_total;
+    if (!pairs) pr.span = -1;
+    if (!bm_pairs) pr.bm_pass = -1;
     ScanSched sched;
-    TRY(make_sched(ix, sh, n, kk, o, list_on, bitmaps, pairs, &sched));
+    TRY(make_sched(ix, sh, n, kk, o, list_on, bitmaps, pairs, bm_pairs, &sched));
     if (o.R > 0) {
         TRY(ensure(ix->w_cand, sizeof(int64_t) * n * kk));
         TRY(ensure(ix->w_cdist, sizeof(float) * n * kk));
@@ -610,9 +621,8 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     }
     const bool chain = !o.timing && cond_tables_fit(ix->ds, ix->r, cond);
     {
-        Stage st(ix, s, o.timing, pairs ? IFVS_STAGE_SCAN : IFVS_STAGE_LAYOUT);
-        CUDA_TRY(st.end(launch_schedule(plan, npass_u64, n, ix->n_blocks, pairs ? pr.span : -1, pr.total, sched, chain,
-                                        s)));
+        Stage st(ix, s, o.timing, pairs || bm_pairs ? IFVS_STAGE_SCAN : IFVS_STAGE_LAYOUT);
+        CUDA_TRY(st.end(launch_schedule(plan, npass_u64, n, ix->n_blocks, pr, sched, chain, s)));
     }
     const float* alpha = cond ? ix->w_alpha.as<float>() : nullptr;
     if (chain) {
@@ -637,9 +647,10 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
                                     order, s)));
         order.first = false;
     }
-    if (pairs) {
+    if (pairs || bm_pairs) {
         Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);
-        CUDA_TRY(st.end(launch_scan_pairs(ix->w_tab.as<float>(), ix->sorted(), plan, n, kk, sh, sched, order, s)));
+        CUDA_TRY(st.end(launch_scan_pairs(ix->w_tab.as<float>(), ix->sorted(), plan, ix->d_codes,
+                                          ix->w_bm.as<uint32_t>(), n, kk, sh, sched, order, s)));
         order.first = false;
     }
     if (plan) {
@@ -1344,7 +1355,7 @@ int ifvs_scan_topk(ifvs_index* ix, const float* lut, const uint32_t* bitmaps, in
         }
         const ScanShape sh = scan_shape(ix);
         ScanSched sched;
-        TRY(make_sched(ix, sh, n, k, o, false, true, false, &sched));
+        TRY(make_sched(ix, sh, n, k, o, false, true, false, false, &sched));
         TRY(ensure(ix->w_tab, sizeof(float) * n * 256 * ix->tab_words));
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_LUT);
@@ -1352,7 +1363,8 @@ int ifvs_scan_topk(ifvs_index* ix, const float* lut, const uint32_t* bitmaps, in
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_LAYOUT);
-            CUDA_TRY(st.end(launch_schedule(nullptr, nullptr, n, ix->n_blocks, -1, 0, sched, false, s)));
+            CUDA_TRY(st.end(launch_schedule(nullptr, nullptr, n, ix->n_blocks, PairRule{-1, 0, -1, 0}, sched, false,
+                                            s)));
         }
         {
             Stage st(ix, s, o.timing, IFVS_STAGE_SCAN);

@@ -296,25 +296,33 @@ struct SchedGroup {
     int64_t fixed;     // units per item set by the caller (0: automatic)
     int64_t cap;       // most items
 };
-// Groups 0, 1, 2: one-query sorted-copy scan, bitmap scan, pairs.
+// Groups: one-query sorted-copy scan, bitmap scan, pairs on a sorted copy, pairs
+// of bitmap queries.
+constexpr int kGroups = 4;
+__host__ __device__ constexpr bool pair_group(int g) { return g >= 2; }
 struct ScanSched {
-    SchedGroup group[3];
-    ScanItem* items[3];
-    int* ctl;              // [0, 3): items per group; [3, 6): work counters
+    SchedGroup group[kGroups];
+    ScanItem* items[kGroups];
+    int* ctl;              // items per group, then work counters
     int2* qlist;           // [nq] (first list, lists) of a query
-    int2* pairs;           // pairs of queries
+    int2* pairs;           // pairs of queries: on sorted copies, then of bitmap queries
     uint8_t* paired;       // [nq]
     uint64_t* partials;    // [lists][k]
 };
 // fills s (pointers from `base`, which may be null); returns the bytes needed.
 // most[g] bounds group g's items (0: the group is not used).
-size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)[3], int64_t chunk_blocks,
-                         const int64_t (&most)[3], uint8_t* base, ScanSched* s);
-// plan null: every query on the bitmap path; npass null: pass counts unknown;
-// pair_min_rows < 0: no pairs; nor where the sorted-copy ranges together hold
-// fewer than pair_min_total rows
+size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)[kGroups], int64_t chunk_blocks,
+                         const int64_t (&most)[kGroups], uint8_t* base, ScanSched* s);
+// What two queries must bring to be paired (pair_rule, api.cu); < 0: no pairs.
+struct PairRule {
+    int64_t span;       // rows a pair on a sorted copy spans, at least
+    int64_t total;      // rows of the batch's ranges together, at least
+    int64_t bm_pass;    // passing rows of a bitmap query, at least
+    int64_t bm_total;   // index rows times such queries, at least
+};
+// plan null: every query on the bitmap path; npass null: pass counts unknown
 cudaError_t launch_schedule(const ScanPlan* plan, const unsigned long long* npass, int64_t nq, int64_t n_blocks,
-                            int64_t pair_min_rows, int64_t pair_min_total, const ScanSched& s, bool chain, cudaStream_t st);
+                            PairRule rule, const ScanSched& s, bool chain, cudaStream_t st);
 
 // How a scan is launched: `chain` as above; first: it is the batch's first scan
 // (waits at its start, the others at their end)
@@ -339,10 +347,12 @@ struct ListOpts {
 cudaError_t launch_scan_list(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
                              const ScanShape& sh, const ScanSched& sched, const ListOpts& lo, ScanOrder o,
                              cudaStream_t s);
-// Rank over the pair group's items (M = 16): two queries per CTA
+// Rank over the pair groups' items (M = 12 and 16): two queries per CTA, on a
+// sorted copy or, by their bitmaps bm, on the index layout `codes`
 bool scan_pairs_fit(const ScanShape& sh, int k);
-cudaError_t launch_scan_pairs(const float* tab, SortedCols sc, const ScanPlan* plan, int64_t nq, int k,
-                              const ScanShape& sh, const ScanSched& sched, ScanOrder o, cudaStream_t s);
+cudaError_t launch_scan_pairs(const float* tab, SortedCols sc, const ScanPlan* plan, const uint8_t* codes,
+                              const uint32_t* bm, int64_t nq, int k, const ScanShape& sh, const ScanSched& sched,
+                              ScanOrder o, cudaStream_t s);
 // the sorted copy of the codes: dst position p <- row rows[p] of the index
 // layout `src`, re-rotated by (p mod 32) mod M; positions >= N are zero
 cudaError_t launch_relayout_sorted(const uint8_t* src, const uint32_t* rows, int64_t N, int M,

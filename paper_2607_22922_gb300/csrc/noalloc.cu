@@ -57,8 +57,8 @@ size_t one_query(const IndexView& v, int k) {
 size_t layout(const IndexView& v, int64_t n, int64_t items, int k, uint8_t* base, ScanSched* s) {
     const size_t bm = (size_t)n * v.n_blocks * 128;
     const size_t tab = (size_t)n * 256 * v.tab_words * sizeof(float);
-    const int slots[3] = {1, v.num_sms * scan_ctas_per_sm(v.tab_words, scan_kp(k)), 1};
-    const int64_t most[3] = {0, items, 0};
+    const int slots[kGroups] = {1, v.num_sms * scan_ctas_per_sm(v.tab_words, scan_kp(k)), 1, 1};
+    const int64_t most[kGroups] = {0, items, 0, 0};
     const size_t head = (bm + tab + 255) / 256 * 256;
     return head + scan_sched_layout(n, k, v.n_blocks, slots, 0, most, base ? base + head : nullptr, s);
 }
@@ -127,7 +127,7 @@ extern "C" int ifvs_scan_topk_static(ifvs_index* ix, const float* lut, const uin
         sh.tab_words = v.tab_words;
         cudaError_t e = launch_bitmap_layout(bitmaps + q0 * wrows, bm, n, v.n_blocks, wrows, false, s);
         if (e == cudaSuccess) e = launch_tables(lut + q0 * lut_n, n, v.M, v.K, v.tab_words, tab, s);
-        if (e == cudaSuccess) e = launch_schedule(nullptr, nullptr, n, v.n_blocks, -1, 0, sched, false, s);
+        if (e == cudaSuccess) e = launch_schedule(nullptr, nullptr, n, v.n_blocks, PairRule{-1, 0, -1, 0}, sched, false, s);
         if (e == cudaSuccess) e = launch_scan(v.codes, tab, bm, n, k, sh, sched, ScanOrder{false, true}, s);
         if (e == cudaSuccess) e = launch_merge(sched, n, k, ids + q0 * k, dists + q0 * k, nullptr, nullptr, false, s);
         if (e != cudaSuccess) {

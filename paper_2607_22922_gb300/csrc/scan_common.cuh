@@ -458,22 +458,6 @@ __device__ __forceinline__ void lookup2(const uint4 ca, const uint4 cb, uint32_t
     unpack_f32x2(acc, da, db);
 }
 
-// Distance of one row for any M (runtime loop; row_bytes a multiple of 4);
-// w0 = the row's index mod 32.
-__device__ __forceinline__ float lookup_any(const uint8_t* rp, bool pass, int M, int S,
-                                            const float* tab, int w0) {
-    float acc = 0.f;
-    for (int w = 0; w * 4 < M; ++w) {
-        const uint32_t wd = pass ? __ldg(reinterpret_cast<const uint32_t*>(rp) + w) : 0u;
-#pragma unroll
-        for (int bb = 0; bb < 4; ++bb) {
-            const int s = 4 * w + bb;
-            if (s < M) acc += tab[(int)((wd >> (8 * bb)) & 0xFFu) * S + w0 + s];
-        }
-    }
-    return acc;
-}
-
 // Distances of NU rows for any M, all owned by one lane (so they share the
 // table word offset w0 = the lane): the rows' code words are read together
 // and their look-ups go into NU/2 packed f32x2 chains, independent of each
@@ -649,7 +633,8 @@ inline int fixed_m(const ScanShape& sh) {
 }
 
 // A scan kernel's CTA takes items from its group's list until it is empty: the
-// first by its block index, the others from the work counter.  `slot`: a word
+// first by its block index, the others from the work counter (after another
+// group's items, the first one too).  `slot`: a word
 // of the CTA's dynamic shared memory (static shared memory would move the
 // dynamic window off the base that the look-ups' immediate offsets assume).
 struct ItemLoop {
@@ -657,14 +642,17 @@ struct ItemLoop {
     int n;
     int* counter;
     volatile int* slot;
+    int own;   // items given out by block index
     int at;
-    __device__ __forceinline__ ItemLoop(const ScanSched& s, int group, void* slot_)
-        : items(s.items[group]), n(s.ctl[group]), counter(s.ctl + 3 + group),
-          slot(reinterpret_cast<volatile int*>(slot_)), at((int)blockIdx.x) {}
+    __device__ __forceinline__ ItemLoop(const ScanSched& s, int group, void* slot_, bool later = false)
+        : items(s.items[group]), n(s.ctl[group]), counter(s.ctl + kGroups + group),
+          slot(reinterpret_cast<volatile int*>(slot_)), own(later ? 0 : (int)gridDim.x), at((int)blockIdx.x) {
+        if (later && n > 0) next();
+    }
     __device__ __forceinline__ bool more() const { return at < n; }
     // all threads; a barrier on both sides: shared memory may be reused after it
     __device__ __forceinline__ void next() {
-        if (threadIdx.x == 0) *slot = (int)gridDim.x + atomicAdd(counter, 1);
+        if (threadIdx.x == 0) *slot = own + atomicAdd(counter, 1);
         __syncthreads();
         at = *slot;
         __syncthreads();

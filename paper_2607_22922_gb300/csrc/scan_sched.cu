@@ -21,9 +21,11 @@
 // k keys (two for a pair), numbered so that a query's lists are contiguous;
 // k_merge reads (first list, count) per query.
 //
-// The pairing of overlapping ranges (M = 16) comes first in the same kernel:
-// see scan_pair.cu for what a pair is worth.  Its sort covers the next power
-// of two of the queries (2048 keys for any batch took 14 us).
+// The pairing of overlapping ranges (M = 12 and 16) comes first in the same
+// kernel: see scan_pair.cu for what a pair is worth.  Its sort covers the next
+// power of two of the queries (2048 keys for any batch took 14 us).  Bitmap
+// queries that many rows pass are paired in their order: any two share every
+// block.
 #include "scan_common.cuh"
 
 namespace ifvs {
@@ -36,38 +38,48 @@ static_assert(kSeg == 2 * kSchedThreads, "one neighbour pair per thread");
 static_assert(kSortedCopies <= 8, "the pairing key keeps 3 bits of the sorted copy");
 
 // exclusive prefix of v over the block's threads (in thread order) and the
-// total; wsum holds one value per warp
-__device__ __forceinline__ int block_prefix(int v, int* wsum, int& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
+// total; wsum holds one value per warp, which every warp adds up by itself, a
+// lane per warp (a loop over 32 warps' values in every thread took half a
+// microsecond of shared-memory reads)
+__device__ __forceinline__ int warp_prefix(int v, int lane) {   // inclusive
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += t;
+        const int t = __shfl_up_sync(0xFFFFFFFFu, v, o);
+        if (lane >= o) v += t;
     }
+    return v;
+}
+
+__device__ __forceinline__ int block_prefix(int v, int* wsum, int& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int incl = warp_prefix(v, lane);
     __syncthreads();
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
-    int before = 0;
-    total = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        const int t = wsum[w];
-        before += w < warp ? t : 0;
-        total += t;
-    }
-    return before + incl - v;
+    const int w = warp_prefix(lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0, lane);
+    total = __shfl_sync(0xFFFFFFFFu, w, 31);
+    const int before = __shfl_sync(0xFFFFFFFFu, w, (warp + 31) & 31);
+    return (warp > 0 ? before : 0) + incl - v;
 }
 
-__device__ __forceinline__ int64_t block_sum(int64_t v, int64_t* wsum) {
+// v[i] <- its sum over the block's threads; wsum holds N values per warp
+template <int N>
+__device__ __forceinline__ void block_sums(int64_t (&v)[N], int64_t (*wsum)[32]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto warp_sum = [](int64_t x) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+        return x;
+    };
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = warp_sum(v[i]);
     __syncthreads();
-    if (lane == 0) wsum[warp] = v;
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < N; ++i) wsum[i][warp] = v[i];
     __syncthreads();
-    int64_t t = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
-    return t;
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = warp_sum(lane < (int)(blockDim.x >> 5) ? wsum[i][lane] : 0);
 }
 
 __device__ __forceinline__ bool pairable(const ScanPlan& x, const ScanPlan& y, int64_t min_rows) {
@@ -118,30 +130,29 @@ __device__ __forceinline__ Cut cut_of(int64_t work, int64_t n, const SchedGroup&
 
 __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __restrict__ plan,
                                                             const unsigned long long* __restrict__ npass, int64_t nq,
-                                                            int64_t n_blocks, int64_t pair_min_rows,
-                                                            int64_t pair_min_total, ScanSched s) {
+                                                            int64_t n_blocks, PairRule rule, ScanSched s) {
     __shared__ uint64_t key[kSeg];          // pairing; then the items' prefix counts
     __shared__ int wsum[32];
-    __shared__ int64_t wsum64[32];
+    __shared__ int64_t wsum64[2 * kGroups][32];
     int* pre = reinterpret_cast<int*>(key);
     const int tid = threadIdx.x, nt = blockDim.x;
-    int n_pairs = 0;
+    int n_pairs = 0, n_bm_pairs = 0;
+    int64_t pair_min_rows = plan != nullptr ? rule.span : -1;
     wait_before();
     start_dependents();   // prepare and filter are complete: the tables can start
 
     // no sort for a batch that cannot pair: 3/4 in common, a pair spans at most
     // 5/4 of its longer range
     if (pair_min_rows >= 0) {
-        int64_t rows = 0, wide = 0;
+        int64_t t[2] = {0, 0};   // rows, ranges wide enough
         for (int64_t q = tid; q < nq; q += nt)
             if (plan[q].list) {
                 const int64_t len = plan[q].b - plan[q].a;
-                rows += len;
-                wide += 5 * len >= 4 * pair_min_rows;
+                t[0] += len;
+                t[1] += 5 * len >= 4 * pair_min_rows;
             }
-        rows = block_sum(rows, wsum64);
-        wide = block_sum(wide, wsum64);
-        if (rows < pair_min_total || wide == 0) pair_min_rows = -1;
+        block_sums(t, wsum64);
+        if (t[0] < rule.total || t[1] == 0) pair_min_rows = -1;
     }
 
     // ---- pairs: sorted by (copy, range start, query), neighbours (2j, 2j + 1)
@@ -200,6 +211,34 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
         __syncthreads();
     }
 
+    // ---- bitmap queries with enough passing rows, two by two
+    bool bm_pairs = rule.bm_pass >= 0 && npass != nullptr;
+    if (bm_pairs) {
+        int* of = reinterpret_cast<int*>(s.pairs + n_pairs);
+        auto dense = [&](int64_t q) {
+            return (plan == nullptr || !plan[q].list) && npass[q] > 0 && (int64_t)npass[q] >= rule.bm_pass;
+        };
+        int64_t n[1] = {0};
+        for (int64_t q = tid; q < nq; q += nt) n[0] += dense(q);
+        block_sums(n, wsum64);
+        bm_pairs = n[0] > 1 && n[0] * n_blocks * kBlockRows >= rule.bm_total;
+        if (bm_pairs) {
+            n_bm_pairs = (int)(n[0] / 2);
+            int done = 0;
+            for (int64_t q0 = 0; q0 < nq; q0 += nt) {
+                const int64_t q = q0 + tid;
+                const bool d = q < nq && dense(q);
+                int total = 0;
+                const int at = done + block_prefix(d, wsum, total);
+                const bool in = d && at < 2 * n_bm_pairs;   // an odd one stays alone
+                if (in) of[at] = (int)q;
+                if (q < nq && (plan == nullptr || !plan[q].list)) s.paired[q] = in;
+                done += total;
+            }
+            __syncthreads();
+        }
+    }
+
     // lengths in units of work
     auto list_len = [&](int64_t q) -> int64_t {
         if (plan == nullptr) return 0;
@@ -208,7 +247,7 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
         return (p.b + kRoundRows - 1) / kRoundRows - p.a / kRoundRows;
     };
     auto bm_len = [&](int64_t q) -> int64_t {
-        if (plan != nullptr && plan[q].list) return 0;
+        if ((plan != nullptr && plan[q].list) || (bm_pairs && s.paired[q])) return 0;
         if (s.group[1].fixed > 0) return n_blocks;
         if (npass == nullptr) return n_blocks;
         const int64_t np = (int64_t)npass[q];
@@ -220,7 +259,8 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
         lo = min(x.a, y.a) / kBlockRows;
         hi = (max(x.b, y.b) + kBlockRows - 1) / kBlockRows;
     };
-    int64_t work[3] = {0, 0, 0}, cnt[3] = {0, 0, 0};
+    int64_t sums[2 * kGroups] = {};
+    int64_t *work = sums, *cnt = sums + kGroups;
     for (int64_t q = tid; q < nq; q += nt) {
         const int64_t l = list_len(q), b = bm_len(q);
         work[0] += l;
@@ -234,12 +274,14 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
         work[2] += hi - lo;
         cnt[2] += 1;
     }
-    Cut cut[3];
-#pragma unroll
-    for (int g = 0; g < 3; ++g) {
-        const int64_t w = block_sum(work[g], wsum64), c = block_sum(cnt[g], wsum64);
-        cut[g] = cut_of(w, c, s.group[g]);
+    if (tid == 0) {
+        work[3] = n_bm_pairs * n_blocks;
+        cnt[3] = n_bm_pairs;
     }
+    block_sums(sums, wsum64);
+    Cut cut[kGroups];
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) cut[g] = cut_of(work[g], cnt[g], s.group[g]);
 
     // no lists for queries that nothing passes
     for (int64_t q = tid; q < nq; q += nt) s.qlist[q] = make_int2(0, 0);
@@ -248,9 +290,14 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
     // items, numbered segment by segment
     int lists = 0;
 #pragma unroll
-    for (int g = 0; g < 3; ++g) {
+    for (int g = 0; g < kGroups; ++g) {
         int items = 0;
-        const int64_t n_el = g == 2 ? n_pairs : nq;
+        const int64_t n_el = g == 2 ? n_pairs : (g == 3 ? n_bm_pairs : nq);
+        const int2* pairs = s.pairs + (g == 3 ? n_pairs : 0);
+        if (cnt[g] == 0) {   // the same in every thread
+            if (tid == 0) s.ctl[g] = s.ctl[kGroups + g] = 0;
+            continue;
+        }
         for (int64_t e0 = 0; e0 < n_el; e0 += kSeg) {
             const int n = (int)min((int64_t)kSeg, n_el - e0);
             int total = 0, done = 0;
@@ -262,6 +309,8 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
                         len = list_len(e0 + i);
                     } else if (g == 1) {
                         len = bm_len(e0 + i);
+                    } else if (g == 3) {
+                        len = n_blocks;
                     } else {
                         int64_t lo, hi;
                         pair_span(e0 + i, lo, hi);
@@ -273,8 +322,8 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
                 done += total;
                 if (i >= n) continue;
                 pre[i] = at;
-                if (g == 2) {
-                    const int2 p = s.pairs[e0 + i];
+                if (pair_group(g)) {
+                    const int2 p = pairs[e0 + i];
                     s.qlist[p.x] = make_int2(lists + 2 * at, c);
                     s.qlist[p.y] = make_int2(lists + 2 * at + c, c);
                 } else if (c > 0) {
@@ -295,9 +344,11 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
                 const int nc = (lo + 1 < n ? pre[lo + 1] : done) - pre[lo];
                 ScanItem w;
                 int64_t a, b;
-                if (g == 2) {
-                    const int2 p = s.pairs[e0 + lo];
-                    pair_span(e0 + lo, a, b);
+                if (pair_group(g)) {
+                    const int2 p = pairs[e0 + lo];
+                    a = 0;
+                    b = n_blocks;
+                    if (g == 2) pair_span(e0 + lo, a, b);
                     w.qa = p.x;
                     w.qb = p.y;
                     w.la = lists + 2 * pre[lo] + c;
@@ -322,18 +373,18 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
             }
             __syncthreads();   // pre is rewritten
             items += done;
-            lists += (g == 2 ? 2 : 1) * done;
+            lists += (pair_group(g) ? 2 : 1) * done;
         }
         if (tid == 0) {
             s.ctl[g] = items;        // items of the list
-            s.ctl[3 + g] = 0;        // work counter
+            s.ctl[kGroups + g] = 0;  // work counter
         }
     }
 }
 
 // Bounds of the lists and the workspace's layout (offsets from `base`).
-size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)[3], int64_t chunk_blocks,
-                         const int64_t (&most)[3], uint8_t* base, ScanSched* s) {
+size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)[kGroups], int64_t chunk_blocks,
+                         const int64_t (&most)[kGroups], uint8_t* base, ScanSched* s) {
     size_t at = 0;
     auto take = [&](size_t bytes) {
         uint8_t* p = base + at;
@@ -341,9 +392,9 @@ size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)
         return p;
     };
     int64_t lists = 0;
-    for (int g = 0; g < 3; ++g) {
+    for (int g = 0; g < kGroups; ++g) {
         SchedGroup& G = s->group[g];
-        const int64_t el = g == 2 ? nq / 2 : nq;
+        const int64_t el = pair_group(g) ? nq / 2 : nq;
         G.slots = slots[g];
         G.least = g == 0 ? kScanWarps : (g == 1 ? 2 : 64);
         G.fixed = chunk_blocks > 0 ? chunk_blocks * (g == 0 ? kBlockRows / kRoundRows : 1) : 0;
@@ -356,9 +407,9 @@ size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)
         if (cap > most[g]) cap = most[g];
         G.cap = cap;
         s->items[g] = reinterpret_cast<ScanItem*>(take(sizeof(ScanItem) * (size_t)cap));
-        lists += (g == 2 ? 2 : 1) * cap;
+        lists += (pair_group(g) ? 2 : 1) * cap;
     }
-    s->ctl = reinterpret_cast<int*>(take(6 * sizeof(int)));
+    s->ctl = reinterpret_cast<int*>(take(2 * kGroups * sizeof(int)));
     s->qlist = reinterpret_cast<int2*>(take(sizeof(int2) * (size_t)nq));
     s->pairs = reinterpret_cast<int2*>(take(sizeof(int2) * (size_t)(nq / 2 + 1)));
     s->paired = take((size_t)nq);
@@ -367,12 +418,12 @@ size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)
 }
 
 cudaError_t launch_schedule(const ScanPlan* plan, const unsigned long long* npass, int64_t nq, int64_t n_blocks,
-                            int64_t pair_min_rows, int64_t pair_min_total, const ScanSched& s, bool chain, cudaStream_t st) {
+                            PairRule rule, const ScanSched& s, bool chain, cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
     int threads = 128;
     while (threads < kSchedThreads && threads < nq) threads <<= 1;
     return launch_kernel(k_schedule, dim3(1), dim3((unsigned)threads), 0, chain, st, plan, npass, nq, n_blocks,
-                         plan ? pair_min_rows : (int64_t)-1, pair_min_total, s);
+                         rule, s);
 }
 
 }  // namespace ifvs

@@ -81,3 +81,33 @@ def test_results_do_not_depend_on_the_split(ifvs, M, k):
     for j in range(3):
         np.testing.assert_array_equal(base[j][few], np.concatenate([o[j] for o in one]))
     g.close()
+
+
+@pytest.mark.parametrize("M,k", [(12, 1), (12, 64), (16, 10), (16, 128), (12, 256), (16, 256)])
+@pytest.mark.parametrize("lists", [True, False])
+def test_bitmap_pairs_equal_single_queries(ifvs, M, k, lists):
+    """Two bitmap queries per CTA (any density, an odd one out, ties in distance,
+    an index that ends inside a block; with the sorted-copy scan off every
+    query is one): bit for bit what one query per CTA returns."""
+    rng = np.random.default_rng(M + k)
+    N, nq, ds = 33_333, 61, 4
+    codes = rng.integers(0, 256, (N, M), dtype=np.uint8)
+    codes[20_000:24_000] = codes[:4_000]                          # equal rows: ids decide
+    attr = rng.integers(0, 1000, N, dtype=np.int32)
+    other = rng.integers(0, 50, N).astype(np.int16)
+    other[8_192:16_384] = 49                                      # blocks few queries pass
+    g = ifvs.Index(codes, [attr, other], D=M * ds)
+    g.load_codebooks(rng.standard_normal((M, 256, ds)).astype(np.float32))
+    q = rng.standard_normal((nq, M * ds)).astype(np.float32)
+    p = synth.empty_predicates(nq)
+    for i in range(nq):
+        synth.set_clause(p[i], 0, 0, synth.OP_LT, int(rng.choice([0, 1, 5, 100, 500, 1001])))
+        synth.set_clause(p[i], 1, 1, synth.OP_LT, int(rng.choice([2, 25, 49, 60])))
+        p[i]["n_clauses"] = 2
+    kw = dict(list_max_ppm=0 if lists else -1)
+    base = g.search(q, p, k, pair_min_rows=-1, **kw)
+    for more in (dict(pair_min_rows=1), dict(pair_min_rows=9000), dict(pair_min_rows=1, chunk_blocks=3),
+                 dict(pair_min_rows=1, sub_batch=2), dict(pair_min_rows=1, flags=ifvs.IFVS_F_STAGE_TIMING)):
+        for x, y in zip(base, g.search(q, p, k, **more, **kw)):
+            np.testing.assert_array_equal(x, y)
+    g.close()

@@ -176,3 +176,24 @@ def test_the_margins_are_needed():
             d, S, sl, inv = rows_of(L, codes, rot)
             dropped += int((S > quant_bound(d, sl, inv, margin=0.0)).sum())
     assert dropped > 0
+
+
+@pytest.mark.parametrize("kind", ["gaussian", "wide_subspace", "tiny_range", "huge", "tiny",
+                                  "few_values", "zero_range", "ulp_spaced"])
+def test_twelve_subspaces_with_wider_entries(kind, monkeypatch):
+    """M = 12: entries up to floor(32767 / 12), twelve additions; the same bound."""
+    monkeypatch.setitem(globals(), "QMAX", 32767 // 12)
+    rng = np.random.default_rng(zlib.crc32(kind.encode()) + 12)
+    L = tables(kind, rng)[:12]
+    codes = rng.integers(0, 256, size=(60000, 12))
+    lo, inv, sl = quant_params(L)
+    Q = quantise(L, lo, inv)
+    for rot in (0, 7, 11):
+        d, S = np.zeros(len(codes), F), np.zeros(len(codes), np.int64)
+        for s in range(12):
+            m = (s + rot) % 12
+            with np.errstate(over="ignore"):
+                d = (d + L[m, codes[:, s]]).astype(F)
+            S += Q[m, codes[:, s]]
+        assert S.max() < 1 << 15
+        assert np.all(S <= quant_bound(d, sl, inv))
