@@ -144,7 +144,10 @@ __device__ __forceinline__ uint64_t sort32_down(uint64_t c, int lane) {
 template <int NW>
 __device__ __forceinline__ void share_publish(uint64_t* share, uint64_t own_kth, uint64_t own_kw, int lane) {
     const int warp = (int)(threadIdx.x >> 5);
-    if (lane == 0) *reinterpret_cast<volatile uint64_t*>(share + 1 + warp) = own_kw;
+    if (lane == 0) {
+        volatile uint64_t* mine = reinterpret_cast<volatile uint64_t*>(share + 1 + warp);
+        if (own_kw < *mine) *mine = own_kw;
+    }
     __syncwarp();
     uint64_t b = lane < NW ? *reinterpret_cast<volatile uint64_t*>(share + 1 + lane) : 0ull;
 #pragma unroll
@@ -154,6 +157,34 @@ __device__ __forceinline__ void share_publish(uint64_t* share, uint64_t own_kth,
     }
     b = own_kth < b ? own_kth : b;
     if (lane == 0 && b != ~0ull) atomicMin(reinterpret_cast<unsigned long long*>(share), b);
+}
+
+// The bound before anything is offered.  Each lane brings the smallest distance
+// (as bits) of its rows of the warp's first round; the lanes' minima are 32
+// distinct rows, so the sorted minima bound the warp's k-th (k <= 32) and
+// (kw + 1)-th key.  All warps of the CTA call it, or prime_none, once per item;
+// after the barrier in it the CTA's bound holds over all their first rounds.
+// Without it every row of a warp's first rounds went through its list: eight
+// sorts of 32 keys per warp and item.  BM_PRIME
+__device__ __forceinline__ void prime_none() { __syncthreads(); }
+
+template <int NW, class TK>
+__device__ __forceinline__ void prime_bound(TK& tk, uint32_t smallest, int lane) {
+    uint32_t c = smallest;
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+        for (int j = size >> 1; j > 0; j >>= 1) {
+            const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, c, j);
+            c = ((lane & j) == 0) == ((lane & size) == 0) ? min(c, y) : max(c, y);
+        }
+    // the last key of a distance: rows at it are offered
+    auto key = [&](int i) { return (uint64_t)__shfl_sync(0xFFFFFFFFu, c, i) << 32 | 0xFFFFFFFFull; };
+    const uint64_t own = tk.k <= 32 ? key(tk.k - 1) : ~0ull;
+    share_publish<NW>(tk.share, own, key(tk.kw), lane);
+    tk.primed(own);
+    __syncthreads();
+    tk.refresh(lane);
 }
 
 constexpr size_t share_bytes(int warps) { return (size_t)(1 + warps) * 8; }
@@ -218,8 +249,13 @@ struct WarpTopK {
         const uint64_t t = *reinterpret_cast<volatile uint64_t*>(share);
         if (t < thr) thr = t;
     }
+    __device__ __forceinline__ void primed(uint64_t own) {
+        if (own < thr) thr = own;
+        first = false;
+    }
     __device__ __forceinline__ void flush(int lane) {
-        thr = flush_list<KP, NW>(buf, k, kw, share, lane);
+        const uint64_t t = flush_list<KP, NW>(buf, k, kw, share, lane);
+        if (t < thr) thr = t;
         cnt = 0;
         first = false;
         refresh(lane);
@@ -296,6 +332,9 @@ struct WarpTopK<64, NW> {
         const uint64_t t = *reinterpret_cast<volatile uint64_t*>(share);
         if (t < thr) thr = t;
     }
+    __device__ __forceinline__ void primed(uint64_t own) {
+        if (own < thr) thr = own;
+    }
     __device__ __forceinline__ void drain(int n, int lane) {
         cnt -= n;
         __syncwarp();
@@ -304,7 +343,8 @@ struct WarpTopK<64, NW> {
         const ulonglong2 r = absorb64(lo, hi, c, lane);
         lo = r.x;
         hi = r.y;
-        thr = __shfl_sync(0xFFFFFFFFu, k > 32 ? hi : lo, (k - 1) & 31);
+        const uint64_t t = __shfl_sync(0xFFFFFFFFu, k > 32 ? hi : lo, (k - 1) & 31);
+        if (t < thr) thr = t;
         if (NW > 0) share_publish<(NW > 0 ? NW : 1)>(share, thr, __shfl_sync(0xFFFFFFFFu, lo, kw), lane);
         refresh(lane);
     }
@@ -343,13 +383,17 @@ struct WarpTopK<32, NW> {
         const uint64_t t = *reinterpret_cast<volatile uint64_t*>(share);
         if (t < thr) thr = t;
     }
+    __device__ __forceinline__ void primed(uint64_t own) {
+        if (own < thr) thr = own;
+    }
     __device__ __forceinline__ void drain(int n, int lane) {
         cnt -= n;
         __syncwarp();
         const uint64_t c = lane < n ? buf[cnt + lane] : ~0ull;
         __syncwarp();   // the drained slots take the next candidates
         mine = absorb32(mine, c, lane);
-        thr = __shfl_sync(0xFFFFFFFFu, mine, k - 1);
+        const uint64_t t = __shfl_sync(0xFFFFFFFFu, mine, k - 1);
+        if (t < thr) thr = t;
         if (NW > 0) share_publish<(NW > 0 ? NW : 1)>(share, thr, __shfl_sync(0xFFFFFFFFu, mine, kw), lane);
         refresh(lane);
     }

@@ -23,6 +23,15 @@ size_t scan_list_smem_bytes(int tab_words, int kp) {
     return (size_t)256 * tab_words * 4 + (size_t)kScanWarps * 2 * kp * 8 + share_bytes(kScanWarps) + 24;
 }
 
+// the smallest distance (as bits) of the rows with a bit in `valid`
+template <int NU>
+__device__ __forceinline__ uint32_t smallest(const float (&d)[NU], unsigned valid) {
+    uint32_t m = 0xFFFFFFFFu;
+#pragma unroll
+    for (int u = 0; u < NU; ++u) m = (valid >> u & 1u) ? min(m, __float_as_uint(d[u])) : m;
+    return m;
+}
+
 template <int KP, int MM, bool FAST, class TK>
 __device__ __forceinline__ void scan_positions(const uint8_t* __restrict__ codes, const uint32_t* __restrict__ rows,
                                                int64_t a, int64_t b, uint32_t r0, uint32_t r1, uint32_t base,
@@ -31,8 +40,10 @@ __device__ __forceinline__ void scan_positions(const uint8_t* __restrict__ codes
     const uint64_t keep = policy_evict_last();
     // positions fit in 32 bits: N < 2^32 - 2048
     const uint32_t a32 = (uint32_t)a, b32 = (uint32_t)b;
+    const uint32_t first = r0 + (uint32_t)warp;
+    if (first >= r1) prime_none();
 #pragma unroll 1
-    for (uint32_t r = r0 + (uint32_t)warp; r < r1; r += kScanWarps) {
+    for (uint32_t r = first; r < r1; r += kScanWarps) {
         const uint32_t P = r * kRoundRows;
         const bool full = P >= a32 && P + kRoundRows <= b32;
         tk.refresh(lane);
@@ -50,19 +61,22 @@ __device__ __forceinline__ void scan_positions(const uint8_t* __restrict__ codes
             c[u] = (valid >> u & 1u) ? ldg_nc_v4(codes + (size_t)pos[u] * 16, keep) : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int u = 0; u < kU; u += 2) lookup2<MM, FAST>(c[u], c[u + 1], tb, tb, base, d[u], d[u + 1]);
+        if (r == first) prime_bound<kScanWarps>(tk, smallest(d, valid), lane);
         // a position can enter the top-k only if its distance is at most the
         // current k-th one; only those load their row id
         const uint32_t thr_hi = (uint32_t)(tk.thr >> 32);
-        bool cand_any = false;
+        unsigned cand = 0u;
 #pragma unroll
-        for (int u = 0; u < kU; ++u) cand_any |= (valid >> u & 1u) && __float_as_uint(d[u]) <= thr_hi;
-        if (!__any_sync(0xFFFFFFFFu, cand_any)) continue;
+        for (int u = 0; u < kU; ++u) cand |= (unsigned)(__float_as_uint(d[u]) <= thr_hi) << u;
+        cand &= valid;
+        if (!__any_sync(0xFFFFFFFFu, cand != 0u)) continue;
+        uint32_t row[kU];   // loaded together: a load per offer waited eight times
+#pragma unroll
+        for (int u = 0; u < kU; ++u) row[u] = (cand >> u & 1u) ? __ldg(rows + pos[u]) : 0u;
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
-            const bool cand = (valid >> u & 1u) && __float_as_uint(d[u]) <= thr_hi;
-            const uint32_t row = cand ? __ldg(rows + pos[u]) : 0u;
-            const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | row;
-            tk.offer(key, cand && key < tk.thr, lane);
+            const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | row[u];
+            tk.offer(key, (cand >> u & 1u) && key < tk.thr, lane);
         }
     }
 }
@@ -156,11 +170,13 @@ __device__ __forceinline__ bool scan_positions_bulk(const uint8_t* __restrict__ 
         fence_proxy_async_smem();   // the tile's readers of the previous item are past a barrier
         issue(first);
     }
+    if (first >= r1) prime_none();
 #pragma unroll 1
     for (uint32_t r = first; r < r1; r += kScanWarps) {
         if (!mbar_wait_warp(bar_s, phase)) {
             if (lane == 0) atomicOr(err, 4);
             mbar_wait_warp(bar_s, phase);   // this round's copy may still be in flight
+            if (r == first) prime_none();
             return false;
         }
         phase ^= 1u;
@@ -186,18 +202,21 @@ __device__ __forceinline__ bool scan_positions_bulk(const uint8_t* __restrict__ 
         float d[kU];
 #pragma unroll
         for (int u = 0; u < kU; u += 2) lookup2<MM, FAST>(c[u], c[u + 1], tb, tb, base, d[u], d[u + 1]);
+        if (r == first) prime_bound<kScanWarps>(tk, smallest(d, valid), lane);
         // as in scan_positions: only candidates load their row id
         const uint32_t thr_hi = (uint32_t)(tk.thr >> 32);
-        bool cand_any = false;
+        unsigned cand = 0u;
 #pragma unroll
-        for (int u = 0; u < kU; ++u) cand_any |= (valid >> u & 1u) && __float_as_uint(d[u]) <= thr_hi;
-        if (!__any_sync(0xFFFFFFFFu, cand_any)) continue;
+        for (int u = 0; u < kU; ++u) cand |= (unsigned)(__float_as_uint(d[u]) <= thr_hi) << u;
+        cand &= valid;
+        if (!__any_sync(0xFFFFFFFFu, cand != 0u)) continue;
+        uint32_t row[kU];   // loaded together: a load per offer waited eight times
+#pragma unroll
+        for (int u = 0; u < kU; ++u) row[u] = (cand >> u & 1u) ? __ldg(rows + pos[u]) : 0u;
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
-            const bool cand = (valid >> u & 1u) && __float_as_uint(d[u]) <= thr_hi;
-            const uint32_t row = cand ? __ldg(rows + pos[u]) : 0u;
-            const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | row;
-            tk.offer(key, cand && key < tk.thr, lane);
+            const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | row[u];
+            tk.offer(key, (cand >> u & 1u) && key < tk.thr, lane);
         }
     }
     return true;
@@ -254,6 +273,8 @@ k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan
             else
                 ok = scan_positions_bulk<KP, MM, false>(codes, rows, p.a, p.b, item.a, item.b, tab, tile, bar, phase,
                                                         tx_extra, err, tk, lane, warp);
+        } else {
+            prime_none();
         }
         merge_warps<KP, kScanWarps>(tk, tkbuf, k, lane, warp, sched.partials + (int64_t)item.la * k);
         if (__syncthreads_or(ok ? 0 : 1)) break;   // the search reports a timeout; its lists are incomplete
@@ -335,7 +356,11 @@ __device__ __forceinline__ void scan_positions_gen(const uint32_t* __restrict__ 
     const uint32_t* p = codes + (size_t)g * 2 * nw * 32 + lane;    // the block to load next
     const size_t step = (size_t)(WARPS * 2 * nw) * 32 - (size_t)(nblk - 1) * kGenWords * 32;
     uint32_t wa[kGenWords], wb[kGenWords];
-    if (g < last) load(p, nw, wa, wb);
+    const uint32_t first = g;
+    if (g < last)
+        load(p, nw, wa, wb);
+    else
+        prime_none();
 #pragma unroll 1
     for (; g < last; g += WARPS) {
         tk.refresh(lane);
@@ -361,18 +386,24 @@ __device__ __forceinline__ void scan_positions_gen(const uint32_t* __restrict__ 
         float d[2];
         unpack_f32x2(acc, d[0], d[1]);
         const uint32_t pos = 64u * g + (uint32_t)lane;
-        const uint32_t thr_hi = (uint32_t)(tk.thr >> 32);
-        bool cand[2];
+        unsigned valid = 0u;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const uint32_t p = pos + 32u * (uint32_t)u;
-            cand[u] = p >= a32 && p < b32 && __float_as_uint(d[u]) <= thr_hi;
+            valid |= (unsigned)(p >= a32 && p < b32) << u;
         }
+        if (g == first) prime_bound<WARPS>(tk, smallest(d, valid), lane);
+        const uint32_t thr_hi = (uint32_t)(tk.thr >> 32);
+        bool cand[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) cand[u] = (valid >> u & 1u) && __float_as_uint(d[u]) <= thr_hi;
         if (!__any_sync(0xFFFFFFFFu, cand[0] || cand[1])) continue;
+        uint32_t id[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) id[u] = cand[u] ? __ldg(rows + pos + 32u * (uint32_t)u) : 0u;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const uint32_t id = cand[u] ? __ldg(rows + pos + 32u * (uint32_t)u) : 0u;
-            const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | id;
+            const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | id[u];
             tk.offer(key, cand[u] && key < tk.thr, lane);
         }
     }
