@@ -295,6 +295,8 @@ struct SchedGroup {
     int64_t least;     // fewest units per item
     int64_t fixed;     // units per item set by the caller (0: automatic)
     int64_t cap;       // most items
+    int64_t per_slot;  // items per slot aimed at (large batches)
+    int64_t start;     // what an item costs beside its units, in units
 };
 // Groups: one-query sorted-copy scan, bitmap scan, pairs on a sorted copy, pairs
 // of bitmap queries.

@@ -33,12 +33,13 @@
 // then the warp walks its 32 columns, 32 neighbouring rows per load, with
 // the lanes whose row fails masked.
 //
-// Top-k.  Each warp keeps a sorted list of its KP best keys and a candidate
-// area of KP slots; a key (dist bits << 32 | row) enters the area when it
-// is below the warp's current k-th key, and a full area is merged by a warp
-// bitonic sort.  Keys are unique (row ids are), so the result is exact and
-// independent of scheduling.  At the end the warps' lists are merged
-// pairwise and warp 0 writes the CTA's k keys.
+// Top-k.  Each warp keeps a sorted list of its KP best keys (in registers for
+// k <= 64, a key or two per lane) and a candidate area; a key (dist bits << 32 |
+// row) enters the area when it is below the bound of its CTA (the smallest of
+// the warps' k-th keys and the largest of their ceil(k / warps)-th ones), and a
+// full area is sorted and merged.  Keys are unique (row ids are), so the result
+// is exact and independent of scheduling.  At the end the warps' lists are
+// merged pairwise and warp 0 writes the CTA's k keys.
 //
 // The tile constants (warps per CTA, ring depth, rows per round) were chosen
 // by measurement on the 10^8-row workload; the macros below only exist to
@@ -165,7 +166,11 @@ __device__ __forceinline__ void share_publish(uint64_t* share, uint64_t own_kth,
 // (kw + 1)-th key.  All warps of the CTA call it, or prime_none, once per item;
 // after the barrier in it the CTA's bound holds over all their first rounds.
 // Without it every row of a warp's first rounds went through its list: eight
-// sorts of 32 keys per warp and item.  BM_PRIME
+// sorts of 32 keys per warp and item (with each candidate's row id loaded by
+// itself; 512 queries of 40,000 rows, M = 12: 113 us, 90 now; 16 of 100,000
+// at k = 100: 46, 35; 1024 of 100,000 at k = 42: 374, 332).  k_scan_list_gen, with 24 warps
+// of 64 rows, gained nothing (484 us with and without).  The two-query kernel:
+// 512 pairs of 10^6 rows at k = 100 2109 -> 1869 us per batch.
 __device__ __forceinline__ void prime_none() { __syncthreads(); }
 
 template <int NW, class TK>
@@ -195,6 +200,14 @@ __device__ __forceinline__ void share_init(uint64_t* share) {
     if (threadIdx.x <= NW) share[threadIdx.x] = ~0ull;
 }
 
+// A candidate whose low word is a position of a sorted copy -> its key.  The row
+// ids of a scan's candidates are loaded when their list takes them, 32 at a
+// time: loaded round by round, half of a warp's rounds waited for one (512 queries of 40,000 rows 157 ->
+// 150 us per batch).
+__device__ __forceinline__ uint64_t row_key(const uint32_t* rows, uint64_t c) {
+    return c == ~0ull ? c : ((c & 0xFFFFFFFF00000000ull) | __ldg(rows + (uint32_t)c));
+}
+
 // Merges a warp's candidates [KP, 2KP) of buf into its sorted list [0, KP),
 // clears the candidates, publishes (NW > 0) and returns the new k-th key.  The
 // candidates are sorted and the KP smallest of both runs kept by one bitonic
@@ -204,7 +217,13 @@ __device__ __forceinline__ void share_init(uint64_t* share) {
 // keeps their code small (instruction-fetch stalls led the two-query kernel's
 // profile).
 template <int KP, int NW>
-__device__ __noinline__ uint64_t flush_list(uint64_t* buf, int k, int kw, uint64_t* share, int lane) {
+__device__ __noinline__ uint64_t flush_list(uint64_t* buf, int k, int kw, uint64_t* share, const uint32_t* rows,
+                                            int lane) {
+    if (rows != nullptr) {
+        __syncwarp();
+#pragma unroll
+        for (int i = KP + lane; i < 2 * KP; i += 32) buf[i] = row_key(rows, buf[i]);
+    }
     warp_sort(buf + KP, KP, lane);
     warp_merge_low(buf, KP, lane);
     const uint64_t thr = buf[k - 1];
@@ -225,14 +244,17 @@ template <int KP, int NW = 0>
 struct WarpTopK {
     uint64_t* buf;   // [0, KP): sorted best keys; [KP, 2KP): candidates
     uint64_t* share; // the CTA's shared bound for this query (NW > 0)
+    const uint32_t* rows;   // null: candidates are keys; else (distance, position)
     int cnt;
     int k, kw;
     bool first;      // nothing published yet
     uint64_t thr;    // keys below thr are offered: min(own k-th key, shared bound)
 
-    __device__ __forceinline__ void init(uint64_t* b, int k_, int lane, uint64_t* share_ = nullptr) {
+    __device__ __forceinline__ void init(uint64_t* b, int k_, int lane, uint64_t* share_ = nullptr,
+                                         const uint32_t* rows_ = nullptr) {
         buf = b;
         share = share_;
+        rows = rows_;
         k = k_;
         kw = NW > 0 ? (k_ + NW - 1) / (NW > 0 ? NW : 1) - 1 : 0;
         cnt = 0;
@@ -254,7 +276,7 @@ struct WarpTopK {
         first = false;
     }
     __device__ __forceinline__ void flush(int lane) {
-        const uint64_t t = flush_list<KP, NW>(buf, k, kw, share, lane);
+        const uint64_t t = flush_list<KP, NW>(buf, k, kw, share, rows, lane);
         if (t < thr) thr = t;
         cnt = 0;
         first = false;
@@ -313,14 +335,17 @@ template <int NW>
 struct WarpTopK<64, NW> {
     uint64_t* buf;   // candidates, 64 slots (of 128)
     uint64_t* share;
+    const uint32_t* rows;
     int cnt;
     int k, kw;
     uint64_t thr;
     uint64_t lo, hi;   // the lane's keys of the sorted list
 
-    __device__ __forceinline__ void init(uint64_t* b, int k_, int, uint64_t* share_ = nullptr) {
+    __device__ __forceinline__ void init(uint64_t* b, int k_, int, uint64_t* share_ = nullptr,
+                                         const uint32_t* rows_ = nullptr) {
         buf = b;
         share = share_;
+        rows = rows_;
         k = k_;
         kw = NW > 0 ? (k_ + NW - 1) / (NW > 0 ? NW : 1) - 1 : 0;
         cnt = 0;
@@ -338,7 +363,8 @@ struct WarpTopK<64, NW> {
     __device__ __forceinline__ void drain(int n, int lane) {
         cnt -= n;
         __syncwarp();
-        const uint64_t c = lane < n ? buf[cnt + lane] : ~0ull;
+        uint64_t c = lane < n ? buf[cnt + lane] : ~0ull;
+        if (rows != nullptr) c = row_key(rows, c);
         __syncwarp();   // the drained slots take the next candidates
         const ulonglong2 r = absorb64(lo, hi, c, lane);
         lo = r.x;
@@ -364,14 +390,17 @@ template <int NW>
 struct WarpTopK<32, NW> {
     uint64_t* buf;   // candidates, 64 slots
     uint64_t* share;
+    const uint32_t* rows;
     int cnt;
     int k, kw;
     uint64_t thr;
     uint64_t mine;   // the lane's key of the sorted list
 
-    __device__ __forceinline__ void init(uint64_t* b, int k_, int, uint64_t* share_ = nullptr) {
+    __device__ __forceinline__ void init(uint64_t* b, int k_, int, uint64_t* share_ = nullptr,
+                                         const uint32_t* rows_ = nullptr) {
         buf = b;
         share = share_;
+        rows = rows_;
         k = k_;
         kw = NW > 0 ? (k_ + NW - 1) / (NW > 0 ? NW : 1) - 1 : 0;
         cnt = 0;
@@ -389,7 +418,8 @@ struct WarpTopK<32, NW> {
     __device__ __forceinline__ void drain(int n, int lane) {
         cnt -= n;
         __syncwarp();
-        const uint64_t c = lane < n ? buf[cnt + lane] : ~0ull;
+        uint64_t c = lane < n ? buf[cnt + lane] : ~0ull;
+        if (rows != nullptr) c = row_key(rows, c);
         __syncwarp();   // the drained slots take the next candidates
         mine = absorb32(mine, c, lane);
         const uint64_t t = __shfl_sync(0xFFFFFFFFu, mine, k - 1);

@@ -32,6 +32,29 @@ __device__ __forceinline__ uint32_t smallest(const float (&d)[NU], unsigned vali
     return m;
 }
 
+// The candidates of a round (bits of `cand`: distance at most the bound's).  Their
+// row ids are looked up when the list takes them (row_key), except where the
+// distance equals the bound's: there the id decides now, so that rows of equal
+// distance do not all go through the list.
+template <class TK>
+__device__ __forceinline__ void offer_round(TK& tk, const float (&d)[kU], const uint32_t (&pos)[kU], unsigned cand,
+                                            uint32_t thr_hi, const uint32_t* __restrict__ rows, int lane) {
+    unsigned tie = 0u;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) tie |= (unsigned)(__float_as_uint(d[u]) == thr_hi) << u;
+    tie &= cand;
+    if (__any_sync(0xFFFFFFFFu, tie != 0u)) {
+        const uint32_t thr_lo = (uint32_t)tk.thr;
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if ((tie >> u & 1u) && __ldg(rows + pos[u]) >= thr_lo) cand &= ~(1u << u);
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+        tk.offer(((uint64_t)__float_as_uint(d[u]) << 32) | pos[u],
+                 (cand >> u & 1u) && __float_as_uint(d[u]) <= (uint32_t)(tk.thr >> 32), lane);
+}
+
 template <int KP, int MM, bool FAST, class TK>
 __device__ __forceinline__ void scan_positions(const uint8_t* __restrict__ codes, const uint32_t* __restrict__ rows,
                                                int64_t a, int64_t b, uint32_t r0, uint32_t r1, uint32_t base,
@@ -70,14 +93,7 @@ __device__ __forceinline__ void scan_positions(const uint8_t* __restrict__ codes
         for (int u = 0; u < kU; ++u) cand |= (unsigned)(__float_as_uint(d[u]) <= thr_hi) << u;
         cand &= valid;
         if (!__any_sync(0xFFFFFFFFu, cand != 0u)) continue;
-        uint32_t row[kU];   // loaded together: a load per offer waited eight times
-#pragma unroll
-        for (int u = 0; u < kU; ++u) row[u] = (cand >> u & 1u) ? __ldg(rows + pos[u]) : 0u;
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | row[u];
-            tk.offer(key, (cand >> u & 1u) && key < tk.thr, lane);
-        }
+        offer_round(tk, d, pos, cand, thr_hi, rows, lane);
     }
 }
 
@@ -103,7 +119,7 @@ k_scan_list(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __r
         }
         share_init<kScanWarps>(share);
         WarpTopK<KP, kScanWarps> tk;
-        tk.init(tkbuf + warp * 2 * KP, k, lane, share);
+        tk.init(tkbuf + warp * 2 * KP, k, lane, share, sc.rows_of(p.col));
         __syncthreads();
         const uint8_t* codes = sc.codes_of(p.col);
         const uint32_t* rows = sc.rows_of(p.col);
@@ -210,14 +226,7 @@ __device__ __forceinline__ bool scan_positions_bulk(const uint8_t* __restrict__ 
         for (int u = 0; u < kU; ++u) cand |= (unsigned)(__float_as_uint(d[u]) <= thr_hi) << u;
         cand &= valid;
         if (!__any_sync(0xFFFFFFFFu, cand != 0u)) continue;
-        uint32_t row[kU];   // loaded together: a load per offer waited eight times
-#pragma unroll
-        for (int u = 0; u < kU; ++u) row[u] = (cand >> u & 1u) ? __ldg(rows + pos[u]) : 0u;
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | row[u];
-            tk.offer(key, (cand >> u & 1u) && key < tk.thr, lane);
-        }
+        offer_round(tk, d, pos, cand, thr_hi, rows, lane);
     }
     return true;
 }
@@ -256,7 +265,7 @@ k_scan_list_bulk(const float* __restrict__ tables, SortedCols sc, const ScanPlan
         share_init<kScanWarps>(share);
         const ScanPlan p = plan[item.qa];
         WarpTopK<KP, kScanWarps> tk;
-        tk.init(tkbuf + warp * 2 * KP, k, lane, share);
+        tk.init(tkbuf + warp * 2 * KP, k, lane, share, sc.rows_of(p.col));
         __syncthreads();
         bool ok = mbar_wait_warp(tbar, tphase);
         if (!ok) {
@@ -359,8 +368,6 @@ __device__ __forceinline__ void scan_positions_gen(const uint32_t* __restrict__ 
     const uint32_t first = g;
     if (g < last)
         load(p, nw, wa, wb);
-    else
-        prime_none();
 #pragma unroll 1
     for (; g < last; g += WARPS) {
         tk.refresh(lane);
@@ -392,7 +399,6 @@ __device__ __forceinline__ void scan_positions_gen(const uint32_t* __restrict__ 
             const uint32_t p = pos + 32u * (uint32_t)u;
             valid |= (unsigned)(p >= a32 && p < b32) << u;
         }
-        if (g == first) prime_bound<WARPS>(tk, smallest(d, valid), lane);
         const uint32_t thr_hi = (uint32_t)(tk.thr >> 32);
         bool cand[2];
 #pragma unroll

@@ -14,9 +14,16 @@
 // `slots` CTAs resident and n queries:
 //   n <= slots / 2   one wave: items of ceil(w / (slots - n)) units, so that
 //                    at most `slots` items arise;
-//   otherwise        about four items per slot, a query's count rounded to
-//                    nearest (equal queries stay whole: every item pays its
-//                    table, lists and merge).
+//   otherwise        three to six items per slot (per_slot), a query's count
+//                    rounded to nearest (every item pays its table, lists and
+//                    merge);
+//   pairs of about equal ranges: the count c per pair of the least
+//                    ceil(n c / slots) (length / c + start), waves times an
+//                    item's time.  Measured, c = 1 / 2: 512 pairs of 5 x 10^6
+//                    rows at k = 100 7410 / 7010 us, of 10^6 rows 1869 / 2064;
+//                    c = 5 / 7 / 14: 128 bitmap pairs of 4 x 10^6 rows at k =
+//                    10 1242 / 1123 / 1178 us.  start = 128 blocks for k <= 32 and
+//                    400 above fit these.
 // A query's items are equal parts of its range.  Each item writes one list of
 // k keys (two for a pair), numbered so that a query's lists are contiguous;
 // k_merge reads (first list, count) per query.
@@ -34,6 +41,10 @@ namespace {
 
 constexpr int kSeg = 2048;              // queries sorted and numbered together
 constexpr int kSchedThreads = 1024;
+// items per slot aimed at in large batches: one-query lists 4 -> 3: 1024 mixed
+// ranges of 10^6 rows 700 -> 686 us, 512 of 40,000 157 -> 150; pairs 4 -> 6:
+// nothing but where the waves below decide
+constexpr int kListPerSlot = 3, kPairPerSlot = 6, kBitmapPerSlot = 4;
 static_assert(kSeg == 2 * kSchedThreads, "one neighbour pair per thread");
 static_assert(kSortedCopies <= 8, "the pairing key keeps 3 bits of the sorted copy");
 
@@ -102,7 +113,7 @@ struct Cut {
     }
 };
 
-__device__ __forceinline__ Cut cut_of(int64_t work, int64_t n, const SchedGroup& g) {
+__device__ __forceinline__ Cut cut_of(int64_t work, int64_t n, const SchedGroup& g, bool equal) {
     Cut c;
     c.up = false;
     if (n <= 0) {
@@ -115,8 +126,17 @@ __device__ __forceinline__ Cut cut_of(int64_t work, int64_t n, const SchedGroup&
     } else if (2 * n <= g.slots) {
         c.L = max((work + g.slots - n - 1) / (g.slots - n), g.least);
         c.up = true;
+    } else if (equal) {
+        // a count per lane (64-bit divisions: one lane for all took 10 us)
+        const int64_t len = work / n;
+        const int i = (int)(threadIdx.x & 15) + 1;
+        int64_t t = i == 1 || len / i >= g.least ? (n * i + g.slots - 1) / g.slots * (len / i + g.start) : INT64_MAX;
+        t = (t < INT64_MAX >> 4 ? t : INT64_MAX >> 4) << 4 | (i - 1);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) t = min(t, __shfl_xor_sync(0xFFFFFFFFu, t, o));
+        c.L = max(len / ((t & 15) + 1), (int64_t)1);
     } else {
-        c.L = max(work / (4 * g.slots), 8 * g.least);
+        c.L = max(work / (g.per_slot * g.slots), 8 * g.least);
     }
     // at most `cap` items in all: each query has at most len / L + 1
     if (g.cap <= n)
@@ -279,9 +299,19 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
         cnt[3] = n_bm_pairs;
     }
     block_sums(sums, wsum64);
+    bool longer = false;   // a pair's span is more than 5/4 of the mean
+    for (int64_t j = tid; j < n_pairs; j += nt) {
+        int64_t lo, hi;
+        pair_span(j, lo, hi);
+        longer |= 4 * (hi - lo) * cnt[2] > 5 * work[2];
+    }
+    const bool equal = n_pairs > 0 && __syncthreads_or(longer ? 1 : 0) == 0;   // n_pairs: the same in every thread
     Cut cut[kGroups];
 #pragma unroll
-    for (int g = 0; g < kGroups; ++g) cut[g] = cut_of(work[g], cnt[g], s.group[g]);
+    for (int g = 0; g < kGroups; ++g) {
+        cut[g] = {1, false};
+        if (cnt[g] > 0) cut[g] = cut_of(work[g], cnt[g], s.group[g], g == 3 || (g == 2 && equal));
+    }
 
     // no lists for queries that nothing passes
     for (int64_t q = tid; q < nq; q += nt) s.qlist[q] = make_int2(0, 0);
@@ -398,7 +428,9 @@ size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)
         G.slots = slots[g];
         G.least = g == 0 ? kScanWarps : (g == 1 ? 2 : 64);
         G.fixed = chunk_blocks > 0 ? chunk_blocks * (g == 0 ? kBlockRows / kRoundRows : 1) : 0;
-        int64_t cap = 4 * (int64_t)slots[g] + el;
+        G.per_slot = g == 0 ? kListPerSlot : (pair_group(g) ? kPairPerSlot : kBitmapPerSlot);
+        G.start = k <= 32 ? 128 : 400;
+        int64_t cap = G.per_slot * (int64_t)slots[g] + el;
         if (chunk_blocks > 0) {
             int64_t per = (n_blocks + chunk_blocks - 1) / chunk_blocks + 1;
             if (per > 1024) per = 1024;
