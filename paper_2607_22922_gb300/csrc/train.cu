@@ -65,14 +65,18 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_gram(const float* __res
 // What bounded it was latency and the float64 pipe (about two additions per SM
 // and cycle): one thread made the candidate list, every candidate waited for
 // the one before it (10 dependent loads each) and was summed over the CTA in
-// float64.  Now a warp makes the list by ballots, four candidates' code and W
+// float64.  Now a warp makes the list by ballots, two candidates' code and W
 // values are loaded together, the differences go to shared memory and a few
 // threads per candidate add its terms as float pairs that carry the rounding
 // errors (about 48 bits), and so is dL/dw_f.  1024 queries with 42 candidates:
-// 228 us before, 195 us now; what is left is the latency of those loads (pass 1
-// about 85 us, pass 2 75) at the 16 warps per SM that 128 registers leave.
-constexpr int kTrainDiffs = 8192;      // floats of the differences held at a time
-constexpr int kTrainBatch = 4;         // candidates whose loads are in flight together
+// 228 us before.  What is left is the latency of those loads, so CTAs per SM
+// count for more than loads per thread: at 128 registers, four candidates in
+// flight and 36 KB the grid ran as 1.7 waves of four CTAs per SM (195 us); at 72
+// registers, two in flight and 26 KB seven fit (the training step 735 -> 665 us;
+// six with two 738, six with four, which spill, 764).
+constexpr int kQueryThreads = 128;
+constexpr int kTrainDiffs = 5632;      // floats of the differences held at a time
+constexpr int kTrainBatch = 2;         // candidates whose loads are in flight together
 
 // floats shared by the differences (pass 1) and dL/dalpha per dimension (pass
 // 2), and the candidates whose differences they hold
@@ -88,7 +92,7 @@ __host__ __device__ inline int train_chunk(int V, int D, int r) {
 // EXACT: r = RMAX, so no load is behind a test of r and a batch's are all in
 // flight at once.
 template <int RMAX, bool EXACT>
-__global__ void __launch_bounds__(kTrainThreads) k_train_query(TrainQueryArgs a) {
+__global__ void __launch_bounds__(kQueryThreads, RMAX <= 8 ? 7 : 3) k_train_query(TrainQueryArgs a) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int V = a.P + a.n_neg;
     const int Mr = a.M * a.r;
@@ -531,7 +535,7 @@ cudaError_t launch_train_gram(const float* W, int M, int r, int KD, float* G, cu
 cudaError_t launch_train_query(const TrainQueryArgs& a, cudaStream_t s) {
     const size_t smem = train_query_smem(a.P + a.n_neg, a.M * a.r, a.D, a.r);
     // threads own dimensions: no more threads than (32-rounded) dimensions
-    const int threads = a.D >= kTrainThreads ? kTrainThreads : ((a.D + 31) / 32) * 32;
+    const int threads = a.D >= kQueryThreads ? kQueryThreads : ((a.D + 31) / 32) * 32;
     auto kern = a.r == 8 ? k_train_query<8, true>
                          : (a.r < 8 ? k_train_query<8, false> : k_train_query<kTrainMaxR, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
