@@ -132,7 +132,7 @@ k_scan_list(const float* __restrict__ tables, SortedCols sc, const ScanPlan* __r
     scan_end(first);
 }
 
-// ---- sorted-copy scan with bulk-copied code tiles (M = 16) ------------------
+// ---- sorted-copy scan with bulk-copied code tiles (M = 12, 16) --------------
 //
 // The walk of k_scan_list with the code rows of every round brought into
 // shared memory by the bulk-copy engine (cp.async.bulk, the untiled form of

@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_gram(const float* __res
 // 228 us before.  What is left is the latency of those loads, so CTAs per SM
 // count for more than loads per thread: at 128 registers, four candidates in
 // flight and 36 KB the grid ran as 1.7 waves of four CTAs per SM (195 us); at 72
-// registers, two in flight and 26 KB seven fit (the training step 735 -> 665 us;
-// six with two 738, six with four, which spill, 764).
+// registers, two in flight and 26 KB seven fit (111 us; the training step 735 ->
+// 665 us; six with two 738, six with four, which spill, 764).
 constexpr int kQueryThreads = 128;
 constexpr int kTrainDiffs = 5632;      // floats of the differences held at a time
 constexpr int kTrainBatch = 2;         // candidates whose loads are in flight together
