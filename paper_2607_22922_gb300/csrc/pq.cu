@@ -8,12 +8,15 @@
 // k_pq_accumulate: CTA (row chunk, subspace).  The chunk's rows are sorted by
 // codeword (counting sort in shared memory, 4096 rows at a time), then thread
 // (codeword, dimension) adds its members' values, in registers, into its own
-// shared accumulator.  Sums are pairs of floats with the rounding error of
-// every addition carried along (TwoSum, Knuth), about 48 bits: this part adds
-// some two float64 values per SM and cycle, which bound the same kernel with
-// float64 sums (77 us for 65 536 rows x 16 subspaces, 40 us with pairs;
-// 140 us with float64 atomics on shared memory, which are compare-and-swap
-// loops).  A sum that leaves the float32 range is taken again in float64, so
+// float64 accumulator in shared memory.  Float64 additions bound the same kernel
+// with one per member (this part adds some two per SM and cycle: 77 us for
+// 65 536 rows x 16 subspaces; 140 us with float64 atomics on shared memory,
+// which are compare-and-swap loops), so up to 32 members go into a pair of
+// floats with the rounding error of every addition carried along (TwoSum,
+// Knuth) before it is added (sum_f64): three Lloyd steps of those rows, with
+// their call, take 512 us (529 us with one pair per codeword and chunk, which
+// was up to 1500 float32 ulp off on long runs of alike values).  A sum that
+// leaves the float32 range is taken again in float64, so
 // infinite, huge and NaN values give what float64 sums give.  The same CTA
 // adds up the chunk's distances and finds its farthest row.
 //
@@ -53,7 +56,7 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long v, un
 
 __global__ void __launch_bounds__(kLloydThreads) k_pq_accumulate(const float* __restrict__ X, int64_t n, int D, int M,
                                                                  int K, int ds, LloydBufs b) {
-    extern __shared__ __align__(16) float2 acc[];   // [K * ds]
+    extern __shared__ __align__(16) double acc[];   // [K * ds]
     __shared__ uint16_t order[kSortRows];
     __shared__ int cnt[256], start[257], wsum[kLloydThreads / 32];
     __shared__ unsigned total[256];
@@ -66,7 +69,7 @@ __global__ void __launch_bounds__(kLloydThreads) k_pq_accumulate(const float* __
     const int KD = K * ds;
     const uint8_t* codes = b.codes + (int64_t)m * n;
     const float* dmin = b.dmin + (int64_t)m * n;
-    for (int e = tid; e < KD; e += kLloydThreads) acc[e] = make_float2(0.f, 0.f);
+    for (int e = tid; e < KD; e += kLloydThreads) acc[e] = 0.0;
     total[tid] = 0u;
     constexpr int PER = kSortRows / kLloydThreads;
     for (int64_t s0 = r0; s0 < r1; s0 += kSortRows) {
@@ -106,32 +109,20 @@ __global__ void __launch_bounds__(kLloydThreads) k_pq_accumulate(const float* __
         const float* base = X + s0 * D + m * ds;
         for (int e = tid; e < KD; e += kLloydThreads) {
             const int k = e / ds, t = e - k * ds;
-            const int j1 = start[k + 1];
-            Sum2 s{acc[e].x, acc[e].y};
-            for (int j = start[k]; j < j1; j += 8) {   // 8 loads in flight
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (j + u < j1) v[u] = __ldg(base + (int64_t)order[j + u] * D + t);
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (j + u < j1) s.add(v[u]);
-            }
-            acc[e] = make_float2(s.hi, s.lo);
+            const int j0 = start[k];
+            acc[e] = sum_f64(acc[e], start[k + 1] - j0,
+                             [&](int j) { return __ldg(base + (int64_t)order[j0 + j] * D + t); });
         }
         __syncthreads();   // order and the counts are rewritten
     }
-    Sum2 mine;
+    double obj = 0.0;
     unsigned long long far = 0ull;
     for (int64_t r = r0 + tid; r < r1; r += kLloydThreads) {
         const float d = dmin[r];
         const unsigned long long key = far_key(d, r);
         far = key > far ? key : far;
-        mine.add(d);
+        obj += (double)d;
     }
-    double obj = mine.finite() ? mine.value() : 0.0;
-    if (!mine.finite())
-        for (int64_t r = r0 + tid; r < r1; r += kLloydThreads) obj += (double)dmin[r];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) obj += __shfl_xor_sync(0xFFFFFFFFu, obj, o);
     if (lane == 0) dred[warp] = obj;
@@ -163,14 +154,13 @@ __global__ void k_pq_finalize(const float* __restrict__ X, int64_t n, int D, Llo
     if (e >= all) return;
     const int64_t mk = e / ds;
     unsigned long long c = 0ull;
-    Sum2 s;
+    double v = 0.0;
 #pragma unroll 8
     for (int ch = 0; ch < b.chunks; ++ch) {
-        s.add(b.sums[ch * all + e]);
+        v += b.sums[ch * all + e];
         c += b.counts[(int64_t)ch * M * K + mk];
     }
-    double v = s.value();
-    if (!s.finite()) {   // beyond float32, infinite or NaN: over the rows again, in float64
+    if (!isfinite(v)) {   // beyond float32, infinite or NaN: over the rows again, in float64
         const int m = (int)(mk / K), k = (int)(mk - (int64_t)m * K), t = (int)(e - mk * ds);
         v = 0.0;
         for (int64_t i = 0; i < n; ++i)
@@ -227,7 +217,7 @@ void lloyd_plan(int64_t n, int M, int K, int ds, int num_sms, LloydBufs* b, size
         return p;
     };
     uint8_t* p = b->base;
-    b->sums = reinterpret_cast<float2*>(p + take(sizeof(float2) * (size_t)(cm * KD)));
+    b->sums = reinterpret_cast<double*>(p + take(sizeof(double) * (size_t)(cm * KD)));
     b->obj = reinterpret_cast<double*>(p + take(sizeof(double) * (size_t)cm));
     b->far = reinterpret_cast<unsigned long long*>(p + take(sizeof(unsigned long long) * (size_t)cm));
     b->counts = reinterpret_cast<unsigned*>(p + take(sizeof(unsigned) * (size_t)(cm * K)));
@@ -240,7 +230,7 @@ void lloyd_plan(int64_t n, int M, int K, int ds, int num_sms, LloydBufs* b, size
 cudaError_t launch_pq_update(const float* X, int64_t n, int D, int M, int K, const LloydBufs& b, const float* C_in,
                              float* C_out, double* objective, cudaStream_t s) {
     const int ds = D / M;
-    const size_t smem = (size_t)K * ds * sizeof(float2);
+    const size_t smem = (size_t)K * ds * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_pq_accumulate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_pq_accumulate<<<dim3((unsigned)b.chunks, (unsigned)M), kLloydThreads, smem, s>>>(X, n, D, M, K, ds, b);

@@ -133,6 +133,31 @@ def test_one_lloyd_step_edges(ifvs, orc, n, M, K, ds):
     np.testing.assert_allclose(obj[0], robj, rtol=1e-12)
 
 
+def test_lloyd_sums_of_long_lopsided_runs(ifvs, orc):
+    """Runs of half a million members per chunk whose rounding errors do not
+    cancel (a constant, nearly one value, one sign): the float64 means to one
+    ulp, and the objective (errors of 10^6 additions of one sign, sqrt(n)
+    2^-53 to n 2^-53 = 1e-13 to 1e-10, exact for the alike values)."""
+    rng = np.random.default_rng(12)
+    n, M = 1_000_000, 120
+    X = rng.standard_normal((n, M), dtype=np.float32)
+    X[:, 0] = 0.1
+    X[:, 1] = 0.3
+    X[:, 2] = 0.3 + 1e-4 * X[:, 2]
+    X[:, 3] = 1.7 + 0.025 * rng.random(n, dtype=np.float32)
+    X[:, 4] = np.abs(X[:, 4])
+    X[:, 5] = np.exp(2.0 * X[:, 5])
+    C0 = np.zeros((M, 2, 1), np.float32)
+    C0[:, 0] = 0.45
+    C0[:, 1] = 2000.0                            # takes nothing, or the tail of the lognormal
+    C1, obj = ifvs.ifvs_pq_train(X, C0, 1)
+    R1, codes, robj = orc.lloyd_step(X, C0)
+    assert (codes[:, :5] == 0).all()
+    assert _ulp_close(C1, R1).all(), np.argwhere(~_ulp_close(C1, R1))
+    np.testing.assert_allclose(obj[0, :4], robj[:4], rtol=1e-12)
+    np.testing.assert_allclose(obj[0], robj, rtol=1e-10)
+
+
 def test_empty_codewords_take_the_farthest_points(ifvs, orc):
     rng = np.random.default_rng(5)
     X = rng.standard_normal((4000, 16)).astype(np.float32)
