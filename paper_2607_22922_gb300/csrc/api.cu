@@ -1181,12 +1181,15 @@ int ifvs_search_batch(ifvs_index* ix, const float* queries, const ifvs_predicate
                          wz ? (const float*)(di + pad(bq) + pad(bp)) : nullptr, ix->D, nq, k, (int64_t*)od,
                          (float*)(od + pad(bi)), ix->w_npass.as<unsigned long long>(),
                          npass ? (int64_t*)(od + pad(bi) + pad(bd)) : nullptr));
-            TRY(finish(ix, s, true));
+            // an error found on the device (a malformed predicate) takes no
+            // other query's results away: they go out with the status
+            const int rc = finish(ix, s, true);
+            if (ix->open) return rc;   // the work did not complete
             const uint8_t* ho = ix->page + kPageHead + kPageHalf;
             memcpy(ids, ho, bi);
             memcpy(dists, ho + pad(bi), bd);
             if (npass) memcpy(npass, ho + pad(bi) + pad(bd), bn);
-            return IFVS_OK;
+            return rc;
         }
     }
     TRY(ensure(ix->w_npass, sizeof(unsigned long long) * sb));

@@ -111,3 +111,35 @@ def test_bitmap_pairs_equal_single_queries(ifvs, M, k, lists):
         for x, y in zip(base, g.search(q, p, k, **more, **kw)):
             np.testing.assert_array_equal(x, y)
     g.close()
+
+
+def test_a_malformed_predicate_takes_no_other_results_away(ifvs):
+    """One malformed predicate: IFVS_ERR_ARG, and the other queries' ids,
+    distances and counts all the same, whether a host call is small (results
+    in the index's page-locked block), larger, or device I/O."""
+    import torch
+    rng = np.random.default_rng(3)
+    N, M, ds, nq, k = 5001, 16, 8, 9, 10
+    g = ifvs.Index(rng.integers(0, 256, (N, M), dtype=np.uint8), [rng.integers(0, 1000, N, dtype=np.int32)], D=M * ds)
+    g.load_codebooks(rng.standard_normal((M, 256, ds)).astype(np.float32))
+    q = rng.standard_normal((nq, M * ds)).astype(np.float32)
+    p = synth.empty_predicates(nq)
+    p["n_clauses"] = 1
+    p["c"][:, 0]["op"] = synth.OP_LT
+    p["c"][:, 0]["lo"] = 500
+    want = [x.copy() for x in g.search(q, p, k)]
+    p[4]["reserved"] = 1
+    want[0][4], want[1][4], want[2][4] = -1, np.inf, 0
+    for kw in (dict(), dict(sub_batch=4), dict(flags=ifvs.IFVS_F_DEVICE_IO)):
+        out = [np.full((nq, k), -7, np.int64), np.full((nq, k), -7, np.float32), np.full(nq, -7, np.int64)]
+        args = [q, p.view(np.uint8).reshape(nq, -1)] + out
+        if kw.get("flags"):
+            args = [torch.from_numpy(x).cuda() for x in args]
+        else:
+            args[1] = p
+        with pytest.raises(ifvs.IfvsError) as e:
+            g.search(args[0], args[1], k, ids=args[2], dists=args[3], npass=args[4], **kw)
+        assert e.value.code == ifvs.IFVS_ERR_ARG
+        for x, y in zip(want, args[2:]):
+            np.testing.assert_array_equal(x, y.cpu().numpy() if kw.get("flags") else y)
+    g.close()
