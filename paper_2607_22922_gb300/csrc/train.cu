@@ -66,9 +66,10 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_gram(const float* __res
 // and cycle): one thread made the candidate list, every candidate waited for
 // the one before it (10 dependent loads each) and was summed over the CTA in
 // float64.  Now a warp makes the list by ballots, two candidates' code and W
-// values are loaded together, the differences go to shared memory and a few
-// threads per candidate add its terms as float pairs that carry the rounding
-// errors (about 48 bits), and so is dL/dw_f.  1024 queries with 42 candidates:
+// values are loaded together, the differences go to shared memory and four
+// threads per candidate add its terms (sum_f64).  dL/dw_f, a float32 result, is
+// summed over the at most 512 candidates as one float pair (Sum2: within 2^-30 of
+// the terms' magnitudes; each term holds a square rounded to float32).  1024 queries with 42 candidates:
 // 228 us before.  What is left is the latency of those loads, so CTAs per SM
 // count for more than loads per thread: at 128 registers, four candidates in
 // flight and 36 KB the grid ran as 1.7 waves of four CTAs per SM (195 us); at 72
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(kQueryThreads, RMAX <= 8 ? 7 : 3) k_train_quer
         return a.codes[id * a.row_bytes + s];
     };
 
-    // pass 1: weighted distances (float32 terms of 48-bit sums).  The term of
+    // pass 1: weighted distances (float32 terms, sum_f64).  The term of
     // dimension d = m ds + t is w_f (q - C)^2 with C_iFVS[m][c][t] = C_PQ +
     // sum_j alpha[m][j] W[m][j][c][t].
     for (int v0 = 0; v0 < V; v0 += CH) {
@@ -204,19 +205,16 @@ __global__ void __launch_bounds__(kQueryThreads, RMAX <= 8 ? 7 : 3) k_train_quer
         // 4 neighbouring threads per candidate, every fourth dimension each
         for (int x = tid; x < ((4 * nv + 31) & ~31); x += blockDim.x) {
             const int i = x >> 2, p = x & 3;
-            Sum2 s;
-            if (i < nv)
-                for (int d = p; d < a.D; d += 4) {
-                    const float df = dfs[i * (a.D + 1) + d];
-                    s.add(__ldg(wf + d) * df * df);
-                }
-            double t = s.value();
-            if (i < nv && !s.finite()) {   // beyond float32, infinite or NaN
+            auto term = [&](int u) {
+                const int d = p + 4 * u;
+                const float df = dfs[i * (a.D + 1) + d];
+                return __ldg(wf + d) * df * df;
+            };
+            const int terms = i < nv && p < a.D ? (a.D - p + 3) / 4 : 0;
+            double t = sum_f64(0.0, terms, term);
+            if (!isfinite(t)) {   // beyond float32, infinite or NaN
                 t = 0.0;
-                for (int d = p; d < a.D; d += 4) {
-                    const float df = dfs[i * (a.D + 1) + d];
-                    t += (double)(__ldg(wf + d) * df * df);
-                }
+                for (int u = 0; u < terms; ++u) t += (double)term(u);
             }
             t += __shfl_xor_sync(0xFFFFFFFFu, t, 1);
             t += __shfl_xor_sync(0xFFFFFFFFu, t, 2);

@@ -297,3 +297,35 @@ def test_argument_errors(ifvs, orc, case):
     rc = ifvs.lib().ifvs_train_grad(plain.h, None, None, 1, None, None, ifvs.C.byref(tp), None,
                                     None, None, None)
     assert rc == ifvs.IFVS_ERR_STATE
+
+
+def test_distance_sums_do_not_depend_on_the_dimension(ifvs):
+    """D = 8192: 2048 terms per thread, four of them large and the rest alike
+    and small, so that a sum's rounding errors add up.  One positive against
+    one negative at distance 0 and a temperature at which the softmax is
+    saturated: the loss is the positive's distance over tau, within
+    2^-38 of the sum (32-term float pairs added in float64) and e^-200."""
+    M, ds, K, r, N, nq = 128, 64, 2, 2, 64, 3
+    D = M * ds
+    rng = np.random.default_rng(8)
+    codes = np.zeros((N, M), np.uint8)
+    codes[1] = 1
+    C = np.zeros((M, K, ds), np.float32)
+    C[:, 0] = 0.0011                             # codeword 0: small differences, alike
+    C[0, 0, :4] = 1.0
+    g = ifvs.Index(codes, [np.zeros(N, np.int32)], D=D, K=K)
+    g.load_codebooks(C, bank=np.zeros((16, M * r), np.float32),
+                     W=rng.standard_normal((M, r, K, ds)).astype(np.float32), hash_seeds=np.array([3], np.uint64))
+    q = np.zeros((nq, D), np.float32)
+    p = synth.empty_predicates(nq)
+    cand = np.tile(np.array([[0, 1]], np.int64), (nq, 1))
+    for w in (0.3, -0.7):
+        wz = np.full(D, w, np.float32)
+        wf = g.condition(q, p, wz=np.tile(wz, (nq, 1)))["wf"][0]
+        df = q[0] - C[:, 0].reshape(-1)
+        terms = (wf * df).astype(np.float32) * df
+        dist = math.fsum(terms.astype(np.float64))
+        tau = np.float32(dist / 200.0)
+        loss = g.train_grad(q, p, wz, cand, 1, float(tau), 0.0)[0]
+        assert abs(loss - dist / float(tau)) <= 2.0 ** -38 * dist / float(tau), loss * float(tau) / dist - 1.0
+    g.close()
