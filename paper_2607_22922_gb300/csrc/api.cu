@@ -172,7 +172,7 @@ struct ifvs_index {
     // small host calls, which would take three pageable copies each way.
     uint8_t* page = nullptr;
     uint8_t* page_dev = nullptr;
-    bool open = false;      // a call began and did not reach its synchronisation
+    bool open = false;      // a call began (begin_call) and did not reach its synchronisation
     int* err() const { return reinterpret_cast<int*>(page_dev); }
     // timing
     double stage_ms[IFVS_N_STAGES] = {0};
@@ -230,6 +230,7 @@ void free_index(ifvs_index* ix) {
     if (!ix) return;
     DeviceGuard g(ix->device);
     if (ix->stream) cudaStreamSynchronize(ix->stream);
+    if (ix->open) cudaDeviceSynchronize();   // work of a call that failed midway, on another stream
     for (int i = 0; i < IFVS_MAX_ATTRS; ++i) {
         if (ix->d_attr[i]) cudaFree(ix->d_attr[i]);
         if (ix->d_srt_vals[i]) cudaFree(ix->d_srt_vals[i]);
@@ -757,12 +758,26 @@ int finish(ifvs_index* ix, cudaStream_t s, bool check_preds) {
     return 0;
 }
 
-// A call that reads the error word begins.  Work of an earlier call that failed
-// midway may still be running and may still write the word.
-int reset_err_flag(ifvs_index* ix, cudaStream_t) {
+// Work of an earlier call that failed midway may still be running, on whatever
+// stream that call had, and may still use the model, the workspace and the
+// page-locked block.
+int settle(ifvs_index* ix) {
     if (ix->open) CUDA_TRY(cudaDeviceSynchronize());
-    *reinterpret_cast<volatile int*>(ix->page) = 0;
+    ix->open = false;
+    return 0;
+}
+
+// A call that uses the index's workspace begins (finish ends it).
+int begin_call(ifvs_index* ix) {
+    TRY(settle(ix));
     ix->open = true;
+    return 0;
+}
+
+// The same for a call that reads the error word.
+int reset_err_flag(ifvs_index* ix) {
+    TRY(begin_call(ix));
+    *reinterpret_cast<volatile int*>(ix->page) = 0;
     return 0;
 }
 
@@ -1104,6 +1119,7 @@ int ifvs_load_codebooks(ifvs_index* ix, const float* C_pq, int32_t ds, const flo
     }
     DeviceGuard g(ix->device);
     cudaStream_t s = ix->stream;
+    TRY(settle(ix));
     CUDA_TRY(cudaStreamSynchronize(s));
     void* old[] = {ix->d_cpq, ix->d_bank, ix->d_W, ix->d_seeds};
     for (void* p : old)
@@ -1159,7 +1175,7 @@ int ifvs_search_batch(ifvs_index* ix, const float* queries, const ifvs_predicate
     DeviceGuard g(ix->device);
     cudaStream_t s = o.stream ? o.stream : ix->stream;
     const int64_t sb = pick_sub_batch(ix, o, nq);
-    TRY(reset_err_flag(ix, s));
+    TRY(reset_err_flag(ix));
     if (!o.dio && nq <= sb) {
         // a small host call: its inputs go over in one copy from the index's
         // page-locked block and the kernels write the results into it
@@ -1230,7 +1246,7 @@ int ifvs_filter(ifvs_index* ix, const ifvs_predicate* preds, int64_t nq, const i
     cudaStream_t s = o.stream ? o.stream : ix->stream;
     const int64_t sb = pick_sub_batch(ix, o, nq);
     const int64_t wrows = (ix->N + 31) / 32;
-    TRY(reset_err_flag(ix, s));
+    TRY(reset_err_flag(ix));
     TRY(ensure(ix->w_npass, sizeof(unsigned long long) * sb));
     TRY(ensure(ix->w_canon, sizeof(CanonPred) * sb));
     TRY(ensure(ix->w_bm, (size_t)sb * ix->n_blocks * 128));
@@ -1277,7 +1293,7 @@ int ifvs_condition(ifvs_index* ix, const float* queries, const ifvs_predicate* p
     const bool cond = !o.plain && ix->d_bank != nullptr;
     const int Mr = ix->M * ix->r;
     const int64_t sb = nq < 1024 ? nq : 1024;
-    TRY(reset_err_flag(ix, s));
+    TRY(reset_err_flag(ix));
     TRY(ensure(ix->w_idx, sizeof(uint32_t) * sb * (ix->h > 0 ? ix->h : 1)));
     TRY(ensure(ix->w_alpha, sizeof(float) * sb * (Mr > 0 ? Mr : 1)));
     TRY(ensure(ix->w_wf, sizeof(float) * sb * ix->D));
@@ -1334,6 +1350,7 @@ int ifvs_scan_topk(ifvs_index* ix, const float* lut, const uint32_t* bitmaps, in
     const int64_t sb = pick_sub_batch(ix, o, nq);
     const int64_t wrows = (ix->N + 31) / 32;
     const size_t lut_n = (size_t)ix->M * ix->K;
+    TRY(begin_call(ix));
     TRY(ensure(ix->w_bm, (size_t)sb * ix->n_blocks * 128));
     if (!o.dio) {
         TRY(ensure(ix->w_rows, (size_t)sb * wrows * 4));
@@ -1407,6 +1424,7 @@ int ifvs_rerank(ifvs_index* ix, const float* queries, const int64_t* cand, int64
     const int64_t* dc = cand;
     int64_t* oid = ids;
     float* odi = dists;
+    TRY(begin_call(ix));
     if (!o.dio) {
         TRY(ensure(ix->w_q, sizeof(float) * nq * ix->D));
         TRY(ensure(ix->w_cand, sizeof(int64_t) * nq * R));
@@ -1635,7 +1653,7 @@ int ifvs_train_grad(ifvs_index* ix, const float* queries, const ifvs_predicate* 
     cudaStream_t s = o.stream ? o.stream : ix->stream;
     const int V = tp->n_pos + tp->n_neg;
     const int64_t Mr = (int64_t)ix->M * ix->r;
-    TRY(reset_err_flag(ix, s));
+    TRY(reset_err_flag(ix));
     const float* dq;
     const ifvs_predicate* dp;
     TRY(train_stage(ix, s, o, nq, queries, preds, wz, &dq, &dp));
@@ -1685,7 +1703,7 @@ int ifvs_train_step(ifvs_index* ix, const float* queries, const ifvs_predicate* 
     cudaStream_t s = o.stream ? o.stream : ix->stream;
     const int P = tp->n_pos, kk = tp->n_pos + tp->n_neg;
     const int64_t Mr = (int64_t)ix->M * ix->r;
-    TRY(reset_err_flag(ix, s));
+    TRY(reset_err_flag(ix));
     const float* dq;
     const ifvs_predicate* dp;
     TRY(train_stage(ix, s, o, nq, queries, preds, wz, &dq, &dp));
@@ -1744,6 +1762,7 @@ int ifvs_get_conditioning(ifvs_index* ix, float* bank, float* W, uint32_t flags)
     const bool dio = flags & IFVS_F_DEVICE_IO;
     DeviceGuard g(ix->device);
     cudaStream_t s = ix->stream;
+    TRY(settle(ix));
     const size_t nW = sizeof(float) * (size_t)ix->M * ix->r * ix->K * ix->ds;
     if (bank) TRY(copy_out(s, dio, bank, ix->d_bank, sizeof(float) * ix->B * ix->M * ix->r));
     if (W) TRY(copy_out(s, dio, W, ix->d_W, nW));
