@@ -121,7 +121,9 @@ struct Sum2 {
 // (constant, low-variance, normal, lognormal) the total was as near the exact sum
 // as float64 additions one by one.
 constexpr int kPairTerms = 32;
-// s + get(0) + ... + get(n - 1) to float64 accuracy, 8 terms fetched at a time
+// s + get(0) + ... + get(n - 1) to float64 accuracy, 8 terms fetched at a time.
+// Terms that a pair cannot hold (infinite, NaN, or a sum beyond float32) are
+// fetched again and added in float64: the result is what float64 additions give.
 template <class Get>
 __device__ __forceinline__ double sum_f64(double s, int n, const Get& get) {
     for (int i0 = 0; i0 < n; i0 += kPairTerms) {
@@ -136,7 +138,12 @@ __device__ __forceinline__ double sum_f64(double s, int n, const Get& get) {
             for (int u = 0; u < 8; ++u)
                 if (i + u < i1) p.add(v[u]);
         }
-        s += p.value();
+        double t = p.value();
+        if (!p.finite()) {
+            t = 0.0;
+            for (int i = i0; i < i1; ++i) t += (double)get(i);
+        }
+        s += t;
     }
     return s;
 }

@@ -15,9 +15,8 @@
 // floats with the rounding error of every addition carried along (TwoSum,
 // Knuth) before it is added (sum_f64): three Lloyd steps of those rows, with
 // their call, take 512 us (529 us with one pair per codeword and chunk, which
-// was up to 1500 float32 ulp off on long runs of alike values).  A sum that
-// leaves the float32 range is taken again in float64, so
-// infinite, huge and NaN values give what float64 sums give.  The same CTA
+// was up to 1500 float32 ulp off on long runs of alike values).  Infinite, huge
+// and NaN values give what float64 sums give.  The same CTA
 // adds up the chunk's distances and finds its farthest row.
 //
 // k_pq_finalize: the chunks' sums, in order, to float32 means; the objective.
@@ -140,9 +139,8 @@ __global__ void __launch_bounds__(kLloydThreads) k_pq_accumulate(const float* __
 
 // thread (m, k, t): float32 mean of the members; thread m of the first CTA:
 // the objective of subspace m
-__global__ void k_pq_finalize(const float* __restrict__ X, int64_t n, int D, LloydBufs b, int M, int K, int ds,
-                              const float* __restrict__ C_in, float* __restrict__ C_out,
-                              double* __restrict__ objective) {
+__global__ void k_pq_finalize(LloydBufs b, int M, int K, int ds, const float* __restrict__ C_in,
+                              float* __restrict__ C_out, double* __restrict__ objective) {
     if (blockIdx.x == 0 && objective != nullptr)
         for (int m = threadIdx.x; m < M; m += blockDim.x) {
             double t = 0.0;
@@ -159,12 +157,6 @@ __global__ void k_pq_finalize(const float* __restrict__ X, int64_t n, int D, Llo
     for (int ch = 0; ch < b.chunks; ++ch) {
         v += b.sums[ch * all + e];
         c += b.counts[(int64_t)ch * M * K + mk];
-    }
-    if (!isfinite(v)) {   // beyond float32, infinite or NaN: over the rows again, in float64
-        const int m = (int)(mk / K), k = (int)(mk - (int64_t)m * K), t = (int)(e - mk * ds);
-        v = 0.0;
-        for (int64_t i = 0; i < n; ++i)
-            if (b.codes[(int64_t)m * n + i] == k) v += (double)X[i * D + m * ds + t];
     }
     C_out[e] = c > 0 ? (float)(v / (double)c) : C_in[e];
     if (e - mk * ds == 0) b.used[mk] = c > 0 ? 1 : 0;
@@ -236,7 +228,7 @@ cudaError_t launch_pq_update(const float* X, int64_t n, int D, int M, int K, con
     k_pq_accumulate<<<dim3((unsigned)b.chunks, (unsigned)M), kLloydThreads, smem, s>>>(X, n, D, M, K, ds, b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int64_t total = (int64_t)M * K * ds;
-    k_pq_finalize<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(X, n, D, b, M, K, ds, C_in, C_out, objective);
+    k_pq_finalize<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(b, M, K, ds, C_in, C_out, objective);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_pq_reseed<<<(unsigned)M, kLloydThreads, 0, s>>>(X, n, D, M, K, ds, b, C_out);
     return cudaGetLastError();

@@ -212,10 +212,6 @@ __global__ void __launch_bounds__(kQueryThreads, RMAX <= 8 ? 7 : 3) k_train_quer
             };
             const int terms = i < nv && p < a.D ? (a.D - p + 3) / 4 : 0;
             double t = sum_f64(0.0, terms, term);
-            if (!isfinite(t)) {   // beyond float32, infinite or NaN
-                t = 0.0;
-                for (int u = 0; u < terms; ++u) t += (double)term(u);
-            }
             t += __shfl_xor_sync(0xFFFFFFFFu, t, 1);
             t += __shfl_xor_sync(0xFFFFFFFFu, t, 2);
             if (i < nv && p == 0) dist[v0 + i] = cand[v0 + i] >= 0 ? t : 0.0;

@@ -158,6 +158,39 @@ def test_lloyd_sums_of_long_lopsided_runs(ifvs, orc):
     np.testing.assert_allclose(obj[0], robj, rtol=1e-10)
 
 
+def _step_ms(ifvs, X, C, iters=2):
+    """Fastest of three calls of `iters` Lloyd steps on device data, in ms per step."""
+    import time
+    import torch
+    out = torch.empty_like(C)
+    best = 1e9
+    for _ in range(4):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        ifvs.ifvs_pq_train(X, C, iters, C_out=out, flags=ifvs.IFVS_F_DEVICE_IO)
+        best = min(best, time.perf_counter() - t0)
+    return best * 1000.0 / iters
+
+
+def test_a_lloyd_step_is_not_slowed_down_by_an_infinite_value(ifvs, orc):
+    """One infinite value per sub-vector of 2^20 rows: the sums that hold it are
+    infinite, the others right, and the step takes no multiple of its time
+    (a thread that went over all rows again took 17 times as long)."""
+    import torch
+    rng = np.random.default_rng(4)
+    n, M, K, ds = 1 << 20, 4, 256, 8
+    X = rng.standard_normal((n, M * ds), dtype=np.float32)
+    C = np.ascontiguousarray(X[:K].reshape(K, M, ds).transpose(1, 0, 2))
+    plain = _step_ms(ifvs, torch.from_numpy(X).cuda(), torch.from_numpy(C).cuda())
+    X[1234, ::ds] = np.inf
+    assert _step_ms(ifvs, torch.from_numpy(X).cuda(), torch.from_numpy(C).cuda()) < 4.0 * plain
+    G, obj = ifvs.ifvs_pq_train(X, C, 1)
+    R, _, robj = orc.lloyd_step(X, C)
+    with np.errstate(invalid="ignore"):
+        assert (_ulp_close(G, R) | (G == R) | (np.isnan(G) & np.isnan(R))).all()
+    assert np.isinf(G).any() and np.isinf(obj).all() and np.isinf(robj).all()
+
+
 def test_empty_codewords_take_the_farthest_points(ifvs, orc):
     rng = np.random.default_rng(5)
     X = rng.standard_normal((4000, 16)).astype(np.float32)
