@@ -18,14 +18,30 @@
 // float32 accumulation of up to 64 products at most 64 x 2^-24 x 3 of it; the
 // float32 distance it stands for is within 20 x 2^-24 x 2 (|x|^2 + |c|^2) of
 // the true one.  So the float32 argmin's score is within
-// 2 (1.2e-5 + 1.2e-5 + 2.4e-6) (|x|^2 + max|c|^2) of the smallest score, and
-// every codeword within kMargin = 2^-14 (6.1e-5) of it is a candidate.  The
+// 2 (1.2e-5 + 1.2e-5 + 2.4e-6) (|x|^2 + max|c|^2) = 5.3e-5 of the smallest
+// score, and every codeword within kMargin = 2^-14 (6.1e-5) of it is a
+// candidate; kFloor covers what underflow takes (64 products and three parts of
+// |c|^2 on either side, 2^-126 each).  The
 // unit is a group of 4 codewords: the groups whose smallest score is a
 // candidate (one for almost every row) are compared exactly, codewords
-// ascending; data whose offset from the origin is tens of times its spread
-// would see several.  Rows for which the bound does not hold (non-finite or
-// huge values, all values below 1e-12) and rows with more than kMaxCand
-// candidate groups take all codewords exactly.
+// ascending.
+//
+// Data that would have many candidates, or none that the bound vouches for
+// (2^19 rows x 16 subspaces of 8: ordinary data 0.42 ms; every codeword evaluated
+// for every row 1.84 ms; each of these up to 2.73 ms before it had its rule):
+//  * A codebook far from the origin (is_far) is ranked relative to its mean mu,
+//    whose rounding adds 4 x 2^-24 (|x - mu|^2 + |c - mu|^2) to a score's error:
+//    0.58 ms (offset 30 times the spread or more).
+//  * A codeword that is not finite is at an infinite or NaN distance, never
+//    smaller than another, unless it is the first, whose distance stands until
+//    a smaller one is found: it gets the score of the columns beyond K.  A row
+//    that is not finite takes codeword 0 for the same reason: 0.38 ms.
+//  * Rows with more than kMaxCand candidate groups (equal codewords: padding,
+//    codebooks trained on few distinct values) and rows for which the bound does
+//    not hold (huge values) take scan_all, which measures one codeword of each
+//    class of equal ones: 0.50 ms for zeros against zeros, 1.56 ms with 16
+//    distinct codewords.  Codebooks of nearly equal codewords and values below
+//    1e-18 are left: 2.7 ms.
 //
 // A thread owns a row.  It reads its scores from TMEM once, keeps the minimum
 // of every four (half an ALU operation per score with the three-input min),
@@ -33,9 +49,10 @@
 // groups and one funnel shift each that collects the sign).  A CTA of 128
 // threads works on half a codebook (128 TMEM columns) at a time, so that four
 // CTAs share an SM's 512 columns: their decisions cover each other's MMAs.
-// The issue slots are the bound (58 % used; tensor pipe 14 %).  Measured,
+// The rows being decided wait in shared memory: in registers they made the
+// main loop spill (0.75 ms).  The issue slots are the bound (58 % used; tensor pipe 14 %).  Measured,
 // 2^20 rows x 16 subspaces: 3.49 ms with every codeword evaluated in float32,
-// 0.69 ms now; with whole codebooks (256 columns, two CTAs per SM) 0.80 ms;
+// 0.68 ms now; with whole codebooks (256 columns, two CTAs per SM) 0.80 ms;
 // with two passes over the scores and a bit per codeword 1.22 ms.
 #include "scan_common.cuh"
 
@@ -46,6 +63,9 @@ namespace {
 constexpr int kTile = 128;              // rows per MMA (TMEM lanes), threads per CTA
 constexpr int kMaxTiles = 4;            // tiles per CTA: one codebook image serves them
 constexpr float kMargin = 0x1p-14f;
+constexpr float kFloor = 0x1p-116f;
+constexpr float kHuge = 1e28f;          // |x|^2 + max|c|^2 from which the bound does not hold
+constexpr float kAbsent = 0x1p100f;     // |c|^2 of a column that can never be a candidate
 constexpr int kHalf2 = 128;             // codewords (TMEM columns) per MMA: half a codebook
 constexpr int kMaxCand = 8;             // candidate groups per row; more: all codewords
 
@@ -164,6 +184,14 @@ __device__ __forceinline__ void load_vec(const float* __restrict__ p, bool vec, 
     }
 }
 
+template <int DS>
+__device__ __forceinline__ bool finite_vec(const float (&x)[DS]) {
+    bool ok = true;
+#pragma unroll
+    for (int t = 0; t < DS; ++t) ok &= fabsf(x[t]) < INFINITY;   // false for NaN
+    return ok;
+}
+
 // the float32 distance, in its defined order
 template <int DS>
 __device__ __forceinline__ float exact_dist(const float (&x)[DS], const float* c) {
@@ -181,6 +209,28 @@ __device__ __forceinline__ float exact_dist(const float (&x)[DS], const float* c
     return s;
 }
 
+// Codeword k's column of the operand image, from g = -2 c and n = |c|^2.
+template <int DS>
+__device__ __forceinline__ void store_column(uint8_t* B, int k, const float (&g)[DS], float n) {
+    using S = AssignShape<DS>;
+#pragma unroll
+    for (int b = 0; b < S::NB; ++b) {
+        uint4 h, l;
+        split8<(DS < 8 ? DS : 8)>(g + 8 * b, h, l);
+        *reinterpret_cast<uint4*>(B + (size_t)(b * 256 + k) * 16) = h;
+        *reinterpret_cast<uint4*>(B + (size_t)((S::NB + b) * 256 + k) * 16) = h;
+        *reinterpret_cast<uint4*>(B + (size_t)((2 * S::NB + b) * 256 + k) * 16) = l;
+    }
+    const uint32_t p1 = bf16x2(n, 0.f);   // |c|^2 in three parts
+    const float r1 = n - bf16_lo(p1);
+    const uint32_t p2 = bf16x2(r1, 0.f);
+    const uint32_t p3 = bf16x2(r1 - bf16_lo(p2), 0.f);
+    *reinterpret_cast<uint4*>(B + (size_t)(3 * S::NB * 256 + k) * 16) =
+        make_uint4((p1 & 0xFFFFu) | (p2 << 16), p3 & 0xFFFFu, 0u, 0u);
+    if (S::B_CHUNKS > 3 * S::NB + 1)
+        *reinterpret_cast<uint4*>(B + (size_t)((3 * S::NB + 1) * 256 + k) * 16) = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // Codewords `tid` and `tid + 128` of one subspace, in registers.
 template <int DS>
 struct CodeRegs {
@@ -196,12 +246,12 @@ struct CodeRegs {
                 for (int t = 0; t < DS; ++t) c[i][t] = 0.f;
         }
     }
-    // the float32 codebook, the operand image, and the largest |c|^2 (as
-    // float bits: order-preserving for values >= 0; +inf when a codeword is
-    // not finite or too large for the error bound)
-    __device__ __forceinline__ void store(int K, int tid, float* cbf, uint8_t* B, unsigned* cmax) const {
-        using S = AssignShape<DS>;
-        unsigned mx = 0u;
+    // the float32 codebook, the operand image, and the largest and the smallest
+    // |c|^2 (as float bits: order-preserving for values >= 0; the largest +inf
+    // when the error bound does not hold for a codeword)
+    __device__ __forceinline__ void store(int K, int tid, float* cbf, uint8_t* B, unsigned* cmax,
+                                          unsigned* cmin) const {
+        unsigned mx = 0u, mn = 0x7F800000u;
         const float nan = __uint_as_float(0x7FC00000u);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -216,33 +266,142 @@ struct CodeRegs {
                 n += c[i][t] * c[i][t] + c[i][t + 1] * c[i][t + 1];
                 n += c[i][t + 2] * c[i][t + 2] + c[i][t + 3] * c[i][t + 3];
             }
-            if (k < K) mx = max(mx, n < 1e28f ? __float_as_uint(n) : 0x7F800000u);
             float g[DS];
 #pragma unroll
             for (int t = 0; t < DS; ++t) g[t] = -2.f * c[i][t];
+            if (k >= K || !(n < kHuge)) {
+                // not finite: only the first can be the answer
+                const bool absent = k >= K || (k > 0 && !finite_vec<DS>(c[i]));
+                if (!absent) mx = 0x7F800000u;
+                n = kAbsent;
 #pragma unroll
-            for (int b = 0; b < S::NB; ++b) {
-                uint4 h, l;
-                split8<(DS < 8 ? DS : 8)>(g + 8 * b, h, l);
-                *reinterpret_cast<uint4*>(B + (size_t)(b * 256 + k) * 16) = h;
-                *reinterpret_cast<uint4*>(B + (size_t)((S::NB + b) * 256 + k) * 16) = h;
-                *reinterpret_cast<uint4*>(B + (size_t)((2 * S::NB + b) * 256 + k) * 16) = l;
+                for (int t = 0; t < DS; ++t) g[t] = 0.f;
+            } else {
+                mx = max(mx, __float_as_uint(n));
+                mn = min(mn, __float_as_uint(n));
             }
-            // |c|^2 in three parts; columns beyond K can never be candidates
-            const float nn = k < K ? n : 0x1p100f;
-            const uint32_t p1 = bf16x2(nn, 0.f);
-            const float r1 = nn - bf16_lo(p1);
-            const uint32_t p2 = bf16x2(r1, 0.f);
-            const uint32_t p3 = bf16x2(r1 - bf16_lo(p2), 0.f);
-            *reinterpret_cast<uint4*>(B + (size_t)(3 * S::NB * 256 + k) * 16) =
-                make_uint4((p1 & 0xFFFFu) | (p2 << 16), p3 & 0xFFFFu, 0u, 0u);
-            if (S::B_CHUNKS > 3 * S::NB + 1)
-                *reinterpret_cast<uint4*>(B + (size_t)((3 * S::NB + 1) * 256 + k) * 16) = make_uint4(0u, 0u, 0u, 0u);
+            store_column<DS>(B, k, g, n);
         }
         mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-        if ((tid & 31) == 0) atomicMax(cmax, mx);
+        mn = __reduce_min_sync(0xFFFFFFFFu, mn);
+        if ((tid & 31) == 0) {
+            atomicMax(cmax, mx);
+            atomicMin(cmin, mn);
+        }
     }
 };
+
+// A codebook far from the origin: every score carries the offset, and the margin
+// that follows it takes in more groups than kMaxCand in some row of every warp
+// from about 20 times the spread.  The smallest |c|^2 is above 3/4 of the largest from 12
+// to 15 times (normal data, ds = 8), where a second image costs 0.07 ms of 0.50.
+__device__ __forceinline__ bool is_far(unsigned cmax, unsigned cmin, int K) {
+    return K > 4 * kMaxCand && cmax < 0x7F800000u && __uint_as_float(cmin) > 0.75f * __uint_as_float(cmax);
+}
+// The whole CTA calls this: the operand image again, relative to mu, the mean of
+// 32 of the codewords, and the largest |c - mu|^2.
+template <int DS>
+__device__ __noinline__ void recentre(int K, const float* cbf, uint8_t* B, float* mu, unsigned* far_max) {
+    const int tid = threadIdx.x;
+    if (tid < DS) {
+        float s = 0.f;
+        for (int i = 0; i < 32; ++i) {
+            const int k = i * K / 32;
+            const float v = cbf[k * DS + (k >> 2) * 4 + tid];
+            s += fabsf(v) < 1e14f ? v : 0.f;
+        }
+        mu[tid] = s * (1.f / 32.f);
+    }
+    if (tid == 0) *far_max = 0u;
+    __syncthreads();
+    unsigned mx = 0u;
+#pragma unroll 1
+    for (int k = tid; k < K; k += kTile) {
+        const float* c = cbf + k * DS + (k >> 2) * 4;
+        float g[DS], n = 0.f;
+        bool finite = true;
+#pragma unroll
+        for (int t = 0; t < DS; ++t) {
+            const float d = c[t] - mu[t];
+            finite &= fabsf(c[t]) < INFINITY;
+            n = fmaf(d, d, n);
+            g[t] = -2.f * d;
+        }
+        if (!(n < kHuge)) {
+            if (k == 0 || finite) mx = 0x7F800000u;
+            n = kAbsent;
+#pragma unroll
+            for (int t = 0; t < DS; ++t) g[t] = 0.f;
+        } else {
+            mx = max(mx, __float_as_uint(n));
+        }
+        store_column<DS>(B, k, g, n);
+    }
+    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    if ((tid & 31) == 0) atomicMax(far_max, mx);
+}
+
+// The float32 decision over all codewords, for the lanes that ask; the whole
+// warp calls it.  While whole classes of equal codewords are met (padding, a
+// codebook trained on few distinct values) only the first of each is measured:
+// the others lose the tie.  NaN distances as in the definition: the first
+// codeword stands until a smaller distance is found, so that a row that is not
+// finite (every distance infinite or NaN) needs no other.
+template <int DS>
+struct Vec {
+    float v[DS];
+};
+// (distance, codeword)
+template <int DS>
+__device__ __noinline__ float2 scan_all(const Vec<DS> row, const float* cb, int K, bool ask) {
+    const int lane = threadIdx.x & 31;
+    float x[DS];
+#pragma unroll
+    for (int t = 0; t < DS; ++t) x[t] = row.v[t];
+    float best = exact_dist<DS>(x, cb);
+    int bk = 0;
+    if (!__any_sync(0xFFFFFFFFu, ask && finite_vec<DS>(x))) return make_float2(best, __int_as_float(0));
+    uint32_t left[8];    // bit l of left[j]: codeword 32 j + l
+#pragma unroll
+    for (int j = 0; j < 8; ++j) left[j] = K >= 32 * j + 32 ? 0xFFFFFFFFu : (K > 32 * j ? (1u << (K - 32 * j)) - 1u : 0u);
+    auto measure = [&](int k) {
+        const float s = exact_dist<DS>(x, cb + k * DS + (k >> 2) * 4);
+        if (s < best) {
+            best = s;
+            bk = k;
+        }
+    };
+    // a class at a time, while that is cheaper than measuring its members (a
+    // round costs about four distances)
+    for (int k = 0, gone = 4; gone >= 4;) {
+        const float* e = cb + k * DS + (k >> 2) * 4;
+        if (k > 0) measure(k);
+        gone = 0;
+        int next = -1;
+#pragma unroll
+        for (int j = 7; j >= 0; --j) {
+            const int o = 32 * j + lane;
+            const float* c = cb + (left[j] >> lane & 1u ? o * DS + (o >> 2) * 4 : 0);
+            bool same = true;
+#pragma unroll
+            for (int t = 0; t < DS; ++t) same &= c[t] == e[t];
+            const uint32_t drop = __ballot_sync(0xFFFFFFFFu, same || o == k) & left[j];
+            gone += __popc(drop);
+            left[j] &= ~drop;
+            if (left[j] != 0u) next = 32 * j + __ffs(left[j]) - 1;
+        }
+        if (next < 0) break;
+        k = next;
+    }
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) {
+        uint32_t w = left[0];
+#pragma unroll
+        for (int i = 1; i < 8; ++i) w = j == i ? left[i] : w;
+        for (; w != 0u; w &= w - 1u) measure(32 * j + __ffs(w) - 1);
+    }
+    return make_float2(best, __int_as_float(bk));
+}
 
 }  // namespace
 
@@ -256,7 +415,10 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
     extern __shared__ __align__(1024) uint8_t sm[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tmem_base;
-    __shared__ unsigned cmax[3];   // slots as the float32 codebooks
+    __shared__ unsigned cmax[3], cmin[3];   // slots as the float32 codebooks
+    __shared__ float mu[DS];                // of a subspace far from the origin
+    __shared__ unsigned far_max;
+    __shared__ float4 xs[DS / 4][kTile];    // the rows being decided
     const int nslots = code_slots(K);
     uint8_t* A = sm;
     uint8_t* B = sm + S::A_BYTES;
@@ -281,6 +443,7 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
         mbar_init(smem_u32(&bar), 1u);
         fence_mbar_init();
         cmax[0] = cmax[1] = cmax[2] = 0u;
+        cmin[0] = cmin[1] = cmin[2] = 0x7F800000u;
     }
     // the constant chunks of A: ones against the parts of |c|^2, zeros
     *reinterpret_cast<uint4*>(A + (size_t)(2 * S::NB * kTile + tid) * 16) =
@@ -290,27 +453,29 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
     __syncthreads();
 
     CodeRegs<DS> cr;
-    float x[DS], x1[DS];   // this tile's row, the next one's (loading)
-    // the row pointer runs ahead of the tile being decided: tile xt of subspace xm
+    float x1[DS];   // the next tile's row (loading)
+    // the rows run ahead of the tile being decided: tile xt of subspace xm is next
+    const int rows = (int)min((int64_t)tiles * kTile, n - row0);
     int xm = 0, xt = 0;
-    const float* xp = X + (row0 + tid) * D + m0 * DS;
-    int64_t left = n - row0 - tid;   // rows from this thread's on
     auto load_x = [&](float (&v)[DS]) {
-        if (left > 0)
-            load_vec<DS>(xp, vec != 0, v);
+        const int r = xt * kTile + tid;
+        if (r < rows)
+            load_vec<DS>(X + (row0 + r) * D + (m0 + xm) * DS, vec != 0, v);
         else
 #pragma unroll
             for (int t = 0; t < DS; ++t) v[t] = 0.f;
-        xp += (int64_t)kTile * D;
-        left -= kTile;
         if (++xt == nt) {
             xt = 0;
             ++xm;
-            xp = X + (row0 + tid) * D + (m0 + xm) * DS;
-            left = n - row0 - tid;
         }
     };
-    auto store_a = [&](const float (&v)[DS]) {
+    auto store_a = [&](const float (&u)[DS], bool centred) {
+        float v[DS];
+#pragma unroll
+        for (int t = 0; t < DS; ++t) v[t] = u[t];
+        if (centred)
+#pragma unroll
+            for (int t = 0; t < DS; ++t) v[t] -= mu[t];
 #pragma unroll
         for (int b = 0; b < S::NB; ++b) {
             uint4 h, l;
@@ -318,6 +483,20 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
             *reinterpret_cast<uint4*>(A + (size_t)(b * kTile + tid) * 16) = h;
             *reinterpret_cast<uint4*>(A + (size_t)((S::NB + b) * kTile + tid) * 16) = l;
         }
+    };
+    // the row becomes this tile's; its squared norm (relative to the centre)
+    auto keep = [&](const float (&v)[DS], bool centred) -> float {
+        float s = 0.f;
+#pragma unroll
+        for (int t = 0; t < DS; t += 4) xs[t / 4][tid] = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
+        if (centred) {
+#pragma unroll
+            for (int t = 0; t < DS; ++t) s = fmaf(v[t] - mu[t], v[t] - mu[t], s);
+        } else {
+#pragma unroll
+            for (int t = 0; t < DS; ++t) s = fmaf(v[t], v[t], s);
+        }
+        return s;
     };
     // A's chunk of K chunk j of B: (ch, xh), (ch, xl), (cl, xh), (|c|^2, ones), (0, zeros)
     auto a_chunk = [](int j) { return j < 2 * S::NB ? j : (j < 3 * S::NB ? j - 2 * S::NB : j - S::NB); };
@@ -334,12 +513,20 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
 
     const int iters = g * nt;
     cr.load(C, m0, K, tid, vec != 0);
-    load_x(x);
-    cr.store(K, tid, cbf, B, &cmax[0]);
-    store_a(x);
-    if (iters > 1) load_x(x1);
+    load_x(x1);
+    cr.store(K, tid, cbf, B, &cmax[0], &cmin[0]);
+    store_a(x1, false);
     fence_proxy_async_smem();
     __syncthreads();
+    bool far = is_far(cmax[0], cmin[0], K);
+    if (far) {   // the same in every thread
+        recentre<DS>(K, cbf, B, mu, &far_max);
+        store_a(x1, true);
+        fence_proxy_async_smem();
+        __syncthreads();
+    }
+    float nx = keep(x1, far);
+    if (iters > 1) load_x(x1);
     const uint32_t tm = tmem_base + ((uint32_t)(warp * 32) << 16);
     if (tid == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -355,12 +542,11 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
     for (int it = 0; it < iters; ++it) {
         const bool more = it + 1 < iters;
         const bool new_m = more && ti + 1 == nt;
-        float nx = 0.f;
-#pragma unroll
-        for (int t = 0; t < DS; ++t) nx = fmaf(x[t], x[t], nx);
-        const float span = nx + __uint_as_float(cmax[slot]);
-        const float margin = kMargin * span;
-        bool all = !(span > 1e-24f && span < 1e28f);
+        const float span = nx + __uint_as_float(far ? far_max : cmax[slot]);
+        const float margin = kMargin * span + kFloor;
+        bool all = !(span < kHuge);
+        const int next = new_m ? (slot + 1 == nslots ? 0 : slot + 1) : slot;
+        bool next_far = far;
         // per half: the smallest score and the groups within the margin of
         // it (bit j: group j of the half)
         uint32_t mask[2] = {0u, 0u};
@@ -391,18 +577,19 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
             // replace this one's now that its MMAs are done
             const bool last = h + 1 == halves;
             if (last && more) {
-                store_a(x1);
+                store_a(x1, far && !new_m);
                 if (new_m) {
-                    const int next = slot + 1 == nslots ? 0 : slot + 1;
                     cr.load(C, m0 + mi + 1, K, tid, vec != 0);
-                    cr.store(K, tid, cbf + next * code_floats(DS, K), B, &cmax[next]);
+                    cr.store(K, tid, cbf + next * code_floats(DS, K), B, &cmax[next], &cmin[next]);
                 }
                 fence_proxy_async_smem();
             }
             if (__syncthreads_or(mma_ok ? 0 : 1) != 0 && late < 0) late = (int)phase;
             mma_ok = late < 0;
             phase ^= 1u;
-            if (mma_ok && (!last || more) && tid == 0) {
+            // a subspace far from the origin starts when this tile is decided
+            if (last && new_m) next_far = is_far(cmax[next], cmin[next], K);
+            if (mma_ok && (!last || (more && !(new_m && next_far))) && tid == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 issue(last ? 0 : 1);
             }
@@ -441,18 +628,24 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
         const float* cb = cbf + slot * code_floats(DS, K);
         float best = INFINITY;
         int bk = 0;
-        if (all) {
-            // every codeword exactly; NaN distances as in the definition
-            // (the first codeword stands until a smaller distance is found)
-            mask[0] = mask[1] = 0u;
-            best = exact_dist<DS>(x, cb);
-#pragma unroll 1
-            for (int k = 1; k < K; ++k) {
-                const float s = exact_dist<DS>(x, cb + k * DS + (k >> 2) * 4);
-                if (s < best) {
-                    best = s;
-                    bk = k;
-                }
+        float x[DS];
+#pragma unroll
+        for (int t = 0; t < DS; t += 4) {
+            const float4 v = xs[t / 4][tid];
+            x[t] = v.x;
+            x[t + 1] = v.y;
+            x[t + 2] = v.z;
+            x[t + 3] = v.w;
+        }
+        if (__any_sync(0xFFFFFFFFu, all)) {
+            Vec<DS> row;
+#pragma unroll
+            for (int t = 0; t < DS; ++t) row.v[t] = x[t];
+            const float2 r = scan_all<DS>(row, cb, K, all);
+            if (all) {
+                mask[0] = mask[1] = 0u;
+                best = r.x;
+                bk = __float_as_int(r.y);
             }
         }
         // the float32 decision over the candidate groups, codewords
@@ -479,11 +672,24 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
         }
         const int lr = ti * kTile + tid;
         out[BY_SUBSPACE ? mi * (nt * kTile) + lr : lr * g + mi] = (uint8_t)bk;
-        if (dmin != nullptr && row0 + lr < n)
+        if (dmin != nullptr && lr < rows)
             dmin[BY_SUBSPACE ? (m0 + mi) * n + row0 + lr : (row0 + lr) * M + m0 + mi] = best;
-        if (new_m && tid == 0) cmax[slot] = 0u;   // its last readers passed the barrier above
-#pragma unroll
-        for (int t = 0; t < DS; ++t) x[t] = x1[t];
+        if (new_m && tid == 0) {   // its last readers passed the barrier above
+            cmax[slot] = 0u;
+            cmin[slot] = 0x7F800000u;
+        }
+        far = next_far;
+        if (new_m && far) {   // mu and far_max: their last readers are past the barrier above
+            recentre<DS>(K, cbf + next * code_floats(DS, K), B, mu, &far_max);
+            store_a(x1, true);
+            fence_proxy_async_smem();
+            __syncthreads();
+            if (mma_ok && tid == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                issue(0);
+            }
+        }
+        if (more) nx = keep(x1, far);
         if (it + 2 < iters) load_x(x1);
         if (++ti == nt) {
             ti = 0;
@@ -498,13 +704,12 @@ k_pq_assign_mma(const float* __restrict__ X, int64_t n, int D, int M, int K, con
     }
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem_base));
-    const int64_t rows = min((int64_t)nt * kTile, n - row0);
     if (BY_SUBSPACE) {
         for (int j = 0; j < g; ++j)
-            for (int r = tid; r < (int)rows; r += kTile)
+            for (int r = tid; r < rows; r += kTile)
                 codes[(m0 + j) * n + row0 + r] = out[j * nt * kTile + r];
     } else {
-        for (int e = tid; e < (int)rows * g; e += kTile) {
+        for (int e = tid; e < rows * g; e += kTile) {
             const int r = e / g;
             codes[(row0 + r) * M + m0 + (e - r * g)] = out[e];
         }

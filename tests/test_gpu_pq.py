@@ -85,6 +85,76 @@ def test_encode_edges_of_the_tensor_core_path(ifvs, orc, ds, n, M, K):
     np.testing.assert_array_equal(ifvs.ifvs_pq_encode(X, C), rc)   # without distances: fewer exact evaluations
 
 
+def _hard_subspaces(rng, n, K, ds):
+    """Seven subspaces: ordinary; far from the origin; very far; all zeros
+    (either sign); three distinct codewords, one of them at the rows' place;
+    some codewords not finite; the first codeword not finite."""
+    X = rng.standard_normal((n, 7, ds), dtype=np.float32)
+    C = rng.standard_normal((7, K, ds)).astype(np.float32)
+    X[:, 1] += 40.0
+    C[1] += 40.0
+    X[:, 2] = X[:, 2] * 0.1 - 3000.0
+    C[2] = C[2] * 0.1 - 3000.0
+    X[:, 3] = np.copysign(0.0, X[:, 3])
+    C[3] = np.copysign(0.0, C[3])
+    C[4] = C[4, rng.integers(0, 3, K)]
+    X[::3, 4] = C[4, K - 1]
+    C[5, 3::5, ds - 1] = np.inf
+    C[5, 4::9, 0] = np.nan
+    C[6, 0, 1] = rng.choice([np.nan, np.inf])
+    X[::1001] = np.inf
+    X[5::1001, :, ds // 2] = np.nan
+    return X.reshape(n, 7 * ds), C
+
+
+@pytest.mark.parametrize("ds,K,n", [(4, 33, 1_250_000), (4, 256, 640_000), (8, 129, 70_001), (8, 256, 127), (16, 256, 30_001),
+                                    (16, 128, 2_000)])
+def test_encode_far_and_degenerate_subspaces(ifvs, orc, ds, K, n):
+    """Bit for bit, several tiles per CTA and one, in the encoder's layout and
+    (through a Lloyd step's objective) by subspace."""
+    rng = np.random.default_rng(ds * K)
+    X, C = _hard_subspaces(rng, n, K, ds)
+    codes, dmin = ifvs.ifvs_pq_encode(X, C, want_dmin=True)
+    rc, rd = orc.pq_encode_f32(X, C)
+    np.testing.assert_array_equal(codes, rc)
+    np.testing.assert_array_equal(dmin, rd)
+    fin = np.isfinite(X).all(1)
+    X[~fin] = 1.0                                # finite rows: finite objectives where the codebook is
+    _, obj = ifvs.ifvs_pq_train(X, C, 1)
+    robj = orc.pq_encode_f32(X, C)[1].astype(np.float64).sum(0)
+    np.testing.assert_allclose(obj[0], robj, rtol=1e-12)
+
+
+def test_encode_time_does_not_hang_on_the_data(ifvs):
+    """Data that the ranking has rules for take no multiple of the time of
+    ordinary data (they took six times as long when every row went through
+    all codewords)."""
+    import time
+    import torch
+    n, M, K, ds = 1 << 18, 16, 256, 8
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    X = torch.randn((n, M * ds), device="cuda", generator=g)
+    C = torch.randn((M, K, ds), device="cuda", generator=g)
+    codes = torch.empty((n, M), dtype=torch.uint8, device="cuda")
+
+    def ms(x, c):
+        best = 1e9
+        for _ in range(5):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            ifvs.ifvs_pq_encode(x, c, codes=codes, flags=ifvs.IFVS_F_DEVICE_IO)
+            best = min(best, time.perf_counter() - t0)
+        return best * 1000.0
+
+    plain = ms(X, C)
+    inf = C.clone()
+    inf[:, 7, 3] = float("inf")
+    for x, c in ((X + 100.0, C + 100.0), (X * 0.0, C * 0.0), (X * float("nan"), C), (X, inf),
+                 (X, C[:, torch.arange(K, device="cuda") % 3].contiguous())):
+        assert ms(x, c) < 2.5 * plain
+
+
 def test_encode_unaligned_device_pointers(ifvs, orc):
     import torch
     rng = np.random.default_rng(9)
