@@ -75,6 +75,17 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_gram(const float* __res
 // flight and 36 KB the grid ran as 1.7 waves of four CTAs per SM (195 us); at 72
 // registers, two in flight and 26 KB seven fit (111 us; the training step 735 ->
 // 665 us; six with two 738, six with four, which spill, 764).
+//
+// Twice the threads per query (three CTAs per SM, two for r > 8) where the
+// batch leaves room for them or the shared memory (D r floats) holds fewer than
+// seven CTAs anyway; a gradient call in us with 128 / 256 threads, 42 candidates:
+//   D = 256, r = 8: 1 query 188 / 151, 400 298 / 254, 1024 421 / 504
+//   D = 960, r = 8: 128 queries 820 / 541, 1024 2171 / 1823
+//   D = 960, r = 4: 128 queries 819 / 536, 1024 1384 / 1769
+//   D = 960, r = 16: 128 queries 1522 / 987, 1024 5081 / 4005
+//   D = 2048, r = 8: 1024 queries 4297 / 3118
+// At D = 960 the 128 threads alone were slower than the kernel before them, which
+// had 256 (r = 4, 128 queries: 641 us).
 constexpr int kQueryThreads = 128;
 constexpr int kTrainDiffs = 5632;      // floats of the differences held at a time
 constexpr int kTrainBatch = 2;         // candidates whose loads are in flight together
@@ -92,8 +103,9 @@ __host__ __device__ inline int train_chunk(int V, int D, int r) {
 
 // EXACT: r = RMAX, so no load is behind a test of r and a batch's are all in
 // flight at once.
-template <int RMAX, bool EXACT>
-__global__ void __launch_bounds__(kQueryThreads, RMAX <= 8 ? 7 : 3) k_train_query(TrainQueryArgs a) {
+template <int RMAX, bool EXACT, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == kQueryThreads ? (RMAX <= 8 ? 7 : 3) : (RMAX <= 8 ? 3 : 2))
+k_train_query(TrainQueryArgs a) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int V = a.P + a.n_neg;
     const int Mr = a.M * a.r;
@@ -528,11 +540,21 @@ cudaError_t launch_train_gram(const float* W, int M, int r, int KD, float* G, cu
 
 cudaError_t launch_train_query(const TrainQueryArgs& a, cudaStream_t s) {
     const size_t smem = train_query_smem(a.P + a.n_neg, a.M * a.r, a.D, a.r);
+    int dev = 0, sms = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    const bool wide = a.D > kQueryThreads && (a.n <= 3 * (int64_t)sms || 7 * (smem + 1024) > 233472);
     // threads own dimensions: no more threads than (32-rounded) dimensions
-    const int threads = a.D >= kQueryThreads ? kQueryThreads : ((a.D + 31) / 32) * 32;
-    auto kern = a.r == 8 ? k_train_query<8, true>
-                         : (a.r < 8 ? k_train_query<8, false> : k_train_query<kTrainMaxR, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int most = wide ? 2 * kQueryThreads : kQueryThreads;
+    const int threads = a.D >= most ? most : ((a.D + 31) / 32) * 32;
+    auto kern = wide ? (a.r == 8  ? k_train_query<8, true, 2 * kQueryThreads>
+                        : a.r < 8 ? k_train_query<8, false, 2 * kQueryThreads>
+                                  : k_train_query<kTrainMaxR, false, 2 * kQueryThreads>)
+                     : (a.r == 8  ? k_train_query<8, true, kQueryThreads>
+                        : a.r < 8 ? k_train_query<8, false, kQueryThreads>
+                                  : k_train_query<kTrainMaxR, false, kQueryThreads>);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)a.n, threads, smem, s>>>(a);
     return cudaGetLastError();

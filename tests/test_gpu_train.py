@@ -329,3 +329,34 @@ def test_distance_sums_do_not_depend_on_the_dimension(ifvs):
         loss = g.train_grad(q, p, wz, cand, 1, float(tau), 0.0)[0]
         assert abs(loss - dist / float(tau)) <= 2.0 ** -38 * dist / float(tau), loss * float(tau) / dist - 1.0
     g.close()
+
+
+@pytest.mark.parametrize("M,ds,r,nq", [(16, 8, 8, 5), (17, 8, 8, 5), (17, 8, 3, 500), (33, 8, 1, 70), (120, 8, 16, 3),
+                                       (120, 8, 8, 500), (30, 8, 32, 500)])
+def test_gradients_at_every_thread_count(ifvs, orc, M, ds, r, nq):
+    """Dimensions around the thread counts, batches on either side of the
+    rule (three CTAs per SM), rows of shared memory that hold seven CTAs or fewer."""
+    rng = np.random.default_rng(M + r + nq)
+    N, K, B = 3000, 16, 64
+    D = M * ds
+    codes = rng.integers(0, K, (N, M), dtype=np.uint8)
+    attr = rng.integers(0, 100, N, dtype=np.int32)
+    C = rng.standard_normal((M, K, ds)).astype(np.float32)
+    bank = (0.1 * rng.standard_normal((B, M * r))).astype(np.float32)
+    W = (0.1 * rng.standard_normal((M, r, K, ds))).astype(np.float32)
+    seeds = np.array([3, 5, 9], np.uint64)
+    q = rng.standard_normal((nq, D)).astype(np.float32)
+    wz = (0.2 * rng.standard_normal(D)).astype(np.float32)
+    p = synth.empty_predicates(nq)
+    cand = rng.integers(0, N, (nq, P + 5))
+    cand[0, 1] = cand[0, P + 1] = -1
+    tau = float(D) / 8.0
+    L, gb, gW, gz = orc.train_loss(codes, C, bank, W, seeds, wz, q, p, cand, P, tau, LAM)
+    g = ifvs.Index(codes, [attr], D=D, K=K)
+    g.load_codebooks(C, bank=bank, W=W, hash_seeds=seeds)
+    Lg, gbg, gWg, gzg = g.train_grad(q, p, wz, cand, P, tau, LAM)
+    assert abs(Lg - L) <= 1e-6 * abs(L)
+    _close(gbg, gb)
+    _close(gWg, gW)
+    _close(gzg, gz)
+    g.close()
