@@ -168,15 +168,21 @@ cudaError_t launch_merge_shards(const float* dists, const int64_t* ids, int64_t 
     return cudaGetLastError();
 }
 
-// 16 warps, two candidates of a warp in flight: the rows lie anywhere in DRAM
-// (100 candidates of 1 KB per query: 35 us with one at a time in 8 warps,
-// 26 us with two in each of 16).
-constexpr int kRerankWarps = 16;
-__global__ void __launch_bounds__(kRerankWarps * 32) k_rerank(const float* __restrict__ X, int64_t N, int D,
-                                                              const float* __restrict__ q,
-                                                              const int64_t* __restrict__ cand, int R, int k,
-                                                              int rp, int64_t* __restrict__ ids,
-                                                              float* __restrict__ dists) {
+// WARPS warps, U candidates of a warp in flight: the rows lie anywhere in DRAM.
+// While all queries' CTAs are resident at once (four of 16 warps per SM), 16 warps
+// with two candidates, from 256 dimensions on one (eight loads of a row are there
+// to be in flight); for more queries 8 warps with one.  us per call, 8 warps with
+// one / 16 with two / 16 with one:
+//   D = 128, 256 candidates: 1 query 32.2 / 25.3 / 24.5, 600 36.4 / 32.5 / 34.5,
+//     1024 49.6 / 52.8 / 54.0
+//   D = 192, 256 candidates: 600 queries - / 35.9 / 39.2; D = 256: - / 47.1 / 44.1
+//   D = 960, 100 candidates: 150 queries 42.5 / 40.5 / 30.8, 1024 82 / 140 / 92,
+//     4000 265 / 431 / 280
+template <int WARPS, int U>
+__global__ void __launch_bounds__(WARPS * 32) k_rerank(const float* __restrict__ X, int64_t N, int D,
+                                                       const float* __restrict__ q,
+                                                       const int64_t* __restrict__ cand, int R, int k, int rp,
+                                                       int64_t* __restrict__ ids, float* __restrict__ dists) {
     __shared__ uint64_t a[IFVS_MAX_K];
     const int64_t qi = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -184,33 +190,35 @@ __global__ void __launch_bounds__(kRerankWarps * 32) k_rerank(const float* __res
     wait_before();
     __syncthreads();
     const float* qv = q + qi * D;
-    for (int j = warp; j < R; j += 2 * kRerankWarps) {
-        int64_t id[2];
-        const float* x[2];
-        float s[2] = {0.f, 0.f};
+    for (int j = warp; j < R; j += U * WARPS) {
+        int64_t id[U];
+        const float* x[U];
+        float s[U] = {};
+        bool any = false;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int c = j + u * kRerankWarps;
+        for (int u = 0; u < U; ++u) {
+            const int c = j + u * WARPS;
             id[u] = c < R ? cand[qi * R + c] : -1;
             if (id[u] >= N) id[u] = -1;
             x[u] = X + (id[u] < 0 ? 0 : id[u]) * D;
+            any |= id[u] >= 0;
         }
-        if (id[0] < 0 && id[1] < 0) continue;
+        if (!any) continue;
 #pragma unroll 4
         for (int d = lane; d < D; d += 32) {
             const float y = qv[d];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const float diff = y - x[u][d];
                 s[u] = fmaf(diff, diff, s[u]);
             }
         }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < U; ++u) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xFFFFFFFFu, s[u], o);
             if (lane == 0 && id[u] >= 0)
-                a[j + u * kRerankWarps] = ((uint64_t)__float_as_uint(s[u]) << 32) | (uint64_t)(uint32_t)id[u];
+                a[j + u * WARPS] = ((uint64_t)__float_as_uint(s[u]) << 32) | (uint64_t)(uint32_t)id[u];
         }
     }
     block_sort(a, rp);
@@ -222,7 +230,14 @@ cudaError_t launch_rerank(const float* X, int64_t N, int D, const float* q, cons
     if (nq <= 0) return cudaSuccess;
     int rp = 32;
     while (rp < R) rp <<= 1;
-    return launch_kernel(k_rerank, dim3((unsigned)nq), dim3(kRerankWarps * 32), 0, chain, s, X, N, D, q, cand, R, k, rp, ids, dists);
+    int dev = 0, sms = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    const bool many = nq > 4 * (int64_t)sms;
+    auto kern = many ? k_rerank<8, 1> : (D < 256 ? k_rerank<16, 2> : k_rerank<16, 1>);
+    return launch_kernel(kern, dim3((unsigned)nq), dim3(many ? 256 : 512), 0, chain, s, X, N, D, q, cand, R, k, rp,
+                         ids, dists);
 }
 
 }  // namespace ifvs

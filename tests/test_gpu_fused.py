@@ -143,3 +143,30 @@ def test_a_malformed_predicate_takes_no_other_results_away(ifvs):
         for x, y in zip(want, args[2:]):
             np.testing.assert_array_equal(x, y.cpu().numpy() if kw.get("flags") else y)
     g.close()
+
+
+@pytest.mark.parametrize("M,ds", [(4, 8), (31, 8), (32, 8), (120, 8)])
+@pytest.mark.parametrize("R", [1, 17, 256])
+def test_rerank_of_many_queries_equals_few(ifvs, M, ds, R):
+    """A batch on either side of the rule for the warps per query, at
+    dimensions on either side of the candidates in flight: the same bits, and
+    the exact order (the distances to a float32 sum's rounding, D 2^-24)."""
+    rng = np.random.default_rng(M + R)
+    N, nq, k, D = 2000, 650, min(R, 7), M * ds
+    X = rng.standard_normal((N, D)).astype(np.float32)
+    g = ifvs.Index(rng.integers(0, 256, (N, M), dtype=np.uint8), [np.zeros(N, np.int32)], vectors=X)
+    q = rng.standard_normal((nq, D)).astype(np.float32)
+    cand = np.stack([rng.permutation(N)[:R] for _ in range(nq)]).astype(np.int64)
+    cand[rng.random((nq, R)) < 0.1] = -1
+    cand[5] = -1
+    ids, d = g.rerank(q, cand, k)
+    for a in range(0, nq, 300):
+        i2, d2 = g.rerank(q[a:a + 300], cand[a:a + 300], k)
+        np.testing.assert_array_equal(ids[a:a + 300], i2)
+        np.testing.assert_array_equal(d[a:a + 300], d2)
+    for i in (0, 5, 649):
+        ok = cand[i][cand[i] >= 0]
+        e = np.sort(((q[i].astype(np.float64) - X[ok]) ** 2).sum(1))[:k]
+        np.testing.assert_allclose(d[i, :len(e)], e, rtol=D * 2.0 ** -24)
+        assert (ids[i, len(e):] == -1).all() and np.isinf(d[i, len(e):]).all()
+    g.close()
