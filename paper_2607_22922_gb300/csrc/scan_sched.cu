@@ -24,7 +24,13 @@
 //                    c = 5 / 7 / 14: 128 bitmap pairs of 4 x 10^6 rows at k =
 //                    10 1242 / 1123 / 1178 us.  start = 128 blocks for k <= 32 and
 //                    400 above fit these.
-// A query's items are equal parts of its range.  Each item writes one list of
+// A query's items are equal parts of its range.  Where the bitmap scan's are more
+// than one wave, the first parts of all queries come first, then the second ones
+// (up to the fourth): CTAs that work at the same time read the same part of the
+// codes and share it in the L2, which 8 x 10^6 rows fill (512 queries of M = 16
+// that 21 and 32 % of them pass, k = 200: 8946 and 12344 us query by query, 8602 and
+// 11866 so; k = 10 8647 and 8470 us at 32 %).  The other groups gained nothing
+// from it.  Each item writes one list of
 // k keys (two for a pair), numbered so that a query's lists are contiguous;
 // k_merge reads (first list, count) per query.
 //
@@ -52,25 +58,27 @@ static_assert(kSortedCopies <= 8, "the pairing key keeps 3 bits of the sorted co
 // total; wsum holds one value per warp, which every warp adds up by itself, a
 // lane per warp (a loop over 32 warps' values in every thread took half a
 // microsecond of shared-memory reads)
-__device__ __forceinline__ int warp_prefix(int v, int lane) {   // inclusive
+template <class T>
+__device__ __forceinline__ T warp_prefix(T v, int lane) {   // inclusive
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xFFFFFFFFu, v, o);
+        const T t = __shfl_up_sync(0xFFFFFFFFu, v, o);
         if (lane >= o) v += t;
     }
     return v;
 }
 
-__device__ __forceinline__ int block_prefix(int v, int* wsum, int& total) {
+template <class T>
+__device__ __forceinline__ T block_prefix(T v, T* wsum, T& total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int incl = warp_prefix(v, lane);
+    const T incl = warp_prefix(v, lane);
     __syncthreads();
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
-    const int w = warp_prefix(lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0, lane);
+    const T w = warp_prefix(lane < (int)(blockDim.x >> 5) ? wsum[lane] : T(0), lane);
     total = __shfl_sync(0xFFFFFFFFu, w, 31);
-    const int before = __shfl_sync(0xFFFFFFFFu, w, (warp + 31) & 31);
-    return (warp > 0 ? before : 0) + incl - v;
+    const T before = __shfl_sync(0xFFFFFFFFu, w, (warp + 31) & 31);
+    return (warp > 0 ? before : T(0)) + incl - v;
 }
 
 // v[i] <- its sum over the block's threads; wsum holds N values per warp
@@ -152,7 +160,9 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
                                                             const unsigned long long* __restrict__ npass, int64_t nq,
                                                             int64_t n_blocks, PairRule rule, ScanSched s) {
     __shared__ uint64_t key[kSeg];          // pairing; then the items' prefix counts
+    __shared__ uint64_t rank[kSeg];         // of an element among those with more than c parts, c = 0..3
     __shared__ int wsum[32];
+    __shared__ uint64_t wsum_rank[32];
     __shared__ int64_t wsum64[2 * kGroups][32];
     int* pre = reinterpret_cast<int*>(key);
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -249,7 +259,7 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
                 const int64_t q = q0 + tid;
                 const bool d = q < nq && dense(q);
                 int total = 0;
-                const int at = done + block_prefix(d, wsum, total);
+                const int at = done + block_prefix((int)d, wsum, total);
                 const bool in = d && at < 2 * n_bm_pairs;   // an odd one stays alone
                 if (in) of[at] = (int)q;
                 if (q < nq && (plan == nullptr || !plan[q].list)) s.paired[q] = in;
@@ -328,9 +338,11 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
             if (tid == 0) s.ctl[g] = s.ctl[kGroups + g] = 0;
             continue;
         }
+        const bool by_part = g == 1 && (s.group[g].fixed > 0 || 2 * cnt[g] > s.group[g].slots);
         for (int64_t e0 = 0; e0 < n_el; e0 += kSeg) {
             const int n = (int)min((int64_t)kSeg, n_el - e0);
             int total = 0, done = 0;
+            uint64_t ranks = 0ull;   // 16 bits per part
             for (int i0 = 0; i0 < n; i0 += nt) {
                 const int i = i0 + tid;
                 int64_t len = 0;
@@ -350,6 +362,14 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
                 const int c = i < n ? cut[g].count(len) : 0;
                 const int at = done + block_prefix(c, wsum, total);
                 done += total;
+                if (by_part) {
+                    const uint64_t has = (uint64_t)(c > 0) | (uint64_t)(c > 1) << 16 | (uint64_t)(c > 2) << 32 |
+                                         (uint64_t)(c > 3) << 48;
+                    uint64_t all = 0ull;
+                    const uint64_t r = ranks + block_prefix(has, wsum_rank, all);
+                    ranks += all;
+                    if (i < n) rank[i] = r;
+                }
                 if (i >= n) continue;
                 pre[i] = at;
                 if (pair_group(g)) {
@@ -361,6 +381,8 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
                 }
             }
             __syncthreads();
+            auto field = [](uint64_t v, int c) { return (int)(v >> (16 * c) & 0xFFFFu); };
+            const int f1 = field(ranks, 0), f2 = f1 + field(ranks, 1), f3 = f2 + field(ranks, 2), f4 = f3 + field(ranks, 3);
             for (int it = tid; it < done; it += nt) {
                 int lo = 0, hi = n;              // the last element whose prefix is <= it
                 while (hi - lo > 1) {
@@ -399,7 +421,16 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
                 }
                 w.a = (uint32_t)(a + (b - a) * c / nc);
                 w.b = (uint32_t)(a + (b - a) * (c + 1) / nc);
-                s.items[g][items + it] = w;
+                int to = it;
+                if (by_part) {
+                    const uint64_t r = rank[lo];
+                    to = c == 0   ? field(r, 0)
+                         : c == 1 ? f1 + field(r, 1)
+                         : c == 2 ? f2 + field(r, 2)
+                         : c == 3 ? f3 + field(r, 3)
+                                  : f4 + it - 4 - field(r, 0) - field(r, 1) - field(r, 2) - field(r, 3);
+                }
+                s.items[g][items + to] = w;
             }
             __syncthreads();   // pre is rewritten
             items += done;
