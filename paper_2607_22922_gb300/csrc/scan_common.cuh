@@ -173,9 +173,9 @@ __device__ __forceinline__ void share_publish(uint64_t* share, uint64_t own_kth,
 // 512 pairs of 10^6 rows at k = 100 2109 -> 1869 us per batch.
 __device__ __forceinline__ void prime_none() { __syncthreads(); }
 
-template <int NW, class TK>
-__device__ __forceinline__ void prime_bound(TK& tk, uint32_t smallest, int lane) {
-    uint32_t c = smallest;
+// the lanes' minima sorted and published; the warp's own k-th key (k <= 32)
+template <int NW>
+__device__ __forceinline__ uint64_t prime_publish(uint32_t c, int k, int kw, uint64_t* share, int lane) {
 #pragma unroll
     for (int size = 2; size <= 32; size <<= 1)
 #pragma unroll
@@ -185,10 +185,27 @@ __device__ __forceinline__ void prime_bound(TK& tk, uint32_t smallest, int lane)
         }
     // the last key of a distance: rows at it are offered
     auto key = [&](int i) { return (uint64_t)__shfl_sync(0xFFFFFFFFu, c, i) << 32 | 0xFFFFFFFFull; };
-    const uint64_t own = tk.k <= 32 ? key(tk.k - 1) : ~0ull;
-    share_publish<NW>(tk.share, own, key(tk.kw), lane);
-    tk.primed(own);
+    const uint64_t own = k <= 32 ? key(k - 1) : ~0ull;
+    share_publish<NW>(share, own, key(kw), lane);
     __syncthreads();
+    return own;
+}
+
+// The same out of line, for the scan by per-lane loads: inlined in its loop it
+// left the loads of a round waiting for one another at M = 12 (512 queries of
+// 8 x 10^6 rows: k = 50 10333 us, 8923 so; k = 100 13017, 9093).  The other kernels
+// measured the same or 1 % slower with it.
+template <int NW>
+__device__ __noinline__ uint64_t prime_publish_out(uint32_t c, int k, int kw, uint64_t* share, int lane) {
+    return prime_publish<NW>(c, k, kw, share, lane);
+}
+
+template <int NW, bool OUT = false, class TK>
+__device__ __forceinline__ void prime_bound(TK& tk, uint32_t smallest, int lane) {
+    if constexpr (OUT)
+        tk.primed(prime_publish_out<NW>(smallest, tk.k, tk.kw, tk.share, lane));
+    else
+        tk.primed(prime_publish<NW>(smallest, tk.k, tk.kw, tk.share, lane));
     tk.refresh(lane);
 }
 

@@ -84,7 +84,7 @@ __device__ __forceinline__ void scan_positions(const uint8_t* __restrict__ codes
             c[u] = (valid >> u & 1u) ? ldg_nc_v4(codes + (size_t)pos[u] * 16, keep) : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int u = 0; u < kU; u += 2) lookup2<MM, FAST>(c[u], c[u + 1], tb, tb, base, d[u], d[u + 1]);
-        if (r == first) prime_bound<kScanWarps>(tk, smallest(d, valid), lane);
+        if (r == first) prime_bound<kScanWarps, true>(tk, smallest(d, valid), lane);
         // a position can enter the top-k only if its distance is at most the
         // current k-th one; only those load their row id
         const uint32_t thr_hi = (uint32_t)(tk.thr >> 32);
