@@ -47,7 +47,7 @@ if ROOT not in sys.path:
 
 WORKLOAD = "gmm100m-d128-m16"
 LIST_DEFAULT_PPM = 1000000   # the library's default sorted-copy threshold (always)
-# the library's automatic pairing for k <= 32 and above: rows a pair spans and
+# the library's automatic pairing for k <= 32 and for k <= 128: rows a pair spans and
 # rows a batch's ranges hold together, at least; of bitmap queries the share of
 # the rows passing (forty parts) and rows times queries, at least
 PAIR_AUTO = {True: (160_000, 30_000_000, 9, 30_000_000), False: (300_000, 90_000_000, 12, 128_000_000)}

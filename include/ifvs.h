@@ -147,7 +147,8 @@ typedef struct {
                            batches whose ranges hold 3e7 together, 300000
                            and 9e7 for k > 32; 22.5 % of the rows passing in
                            batches of 3e7 rows times queries, 30 % and
-                           1.28e8 for k > 32); -1: never pair.             */
+                           1.28e8 for k > 32, 5e8 and an index of 2e6 rows
+                           for k > 128); -1: never pair.                   */
     void* stream;       /* cudaStream_t to run on; NULL: the index's stream   */
 } ifvs_search_params;
 

@@ -453,11 +453,16 @@ constexpr int32_t kListDefaultPpm = 1000000;
 // / 1965, 30 % 2345 / 1933, 50 % 2887 / 1947; 64 queries of 10^6: 20 % 190 /
 // 199, 30 % 225 / 196; 16 of 10^6: 40 % 110 / 107.  k = 100: 512 queries of
 // 2 x 10^6, 20 % 1912 / 2219, 30 % 2356 / 2168, 40 % 2860 / 2186; 64 of 10^6,
-// 40 % 328 / 333.
+// 40 % 328 / 333.  Above k = 128 a pair rescores in place (no room for the
+// candidate buffers): time paired over single at 45 % passing, M = 12, k = 136 /
+// 256: 1024 queries of 5 x 10^5 1.21 / 1.24, of 10^6 1.18 / 1.06, of 2 x 10^6 0.96 /
+// 0.96; 128 of 2 x 10^6 1.09 / 0.99, of 4 x 10^6 0.89 / 0.90; 512 of 2 x 10^6
+// 0.88 / 0.86.
 PairRule pair_rule(int32_t pair_min_rows, int64_t N, int k) {
     if (pair_min_rows > 0) return {pair_min_rows, 0, pair_min_rows, 0};
-    return k <= 32 ? PairRule{160000, 30000000, N / 40 * 9, 30000000}
-                   : PairRule{300000, 90000000, N / 40 * 12, 128000000};
+    if (k <= 32) return {160000, 30000000, N / 40 * 9, 30000000};
+    if (k <= 128) return {300000, 90000000, N / 40 * 12, 128000000};
+    return {300000, 90000000, N >= 2000000 ? N / 40 * 12 : -1, 500000000};
 }
 
 int parse_opts(const ifvs_search_params* p, Opts* o) {
@@ -577,8 +582,8 @@ int run_path(ifvs_index* ix, cudaStream_t s, const Opts& o, const float* dq,
     const bool may_pair = o.pair_min_rows >= 0 && scan_pairs_fit(sh, kk);
     const bool pairs = list_on && may_pair &&
                        ((o.timing && ix->M == 16) || (n > 1 && ix->N >= pr.span && n * ix->N >= pr.total));
-    const bool bm_pairs =
-        bitmaps && may_pair && n > 1 && ix->N >= pr.bm_pass && n * ix->n_blocks * kBlockRows >= pr.bm_total;
+    const bool bm_pairs = bitmaps && may_pair && n > 1 && pr.bm_pass >= 0 && ix->N >= pr.bm_pass &&
+                          n * ix->n_blocks * kBlockRows >= pr.bm_total;
     if (!pairs) pr.span = -1;
     if (!bm_pairs) pr.bm_pass = -1;
     ScanSched sched;
