@@ -5,7 +5,7 @@
 // Training keeps the codes and distances of an iteration by subspace
 // ([M][n]), so that every pass over one subspace is coalesced.
 //
-// k_pq_accumulate: CTA (row chunk, subspace).  The chunk's rows are sorted by
+// k_pq_accumulate: CTA (row chunk, subspace), the subspaces of a chunk in a row.  The chunk's rows are sorted by
 // codeword (counting sort in shared memory, 4096 rows at a time), then thread
 // (codeword, dimension) adds its members' values, in registers, into its own
 // float64 accumulator in shared memory.  Float64 additions bound the same kernel
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kLloydThreads) k_pq_accumulate(const float* __
     __shared__ unsigned total[256];
     __shared__ unsigned long long red[kLloydThreads / 32];
     __shared__ double dred[kLloydThreads / 32];
-    const int m = blockIdx.y, ch = blockIdx.x, tid = threadIdx.x;
+    const int m = (int)(blockIdx.x % (unsigned)M), ch = (int)(blockIdx.x / (unsigned)M), tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
     const int64_t r0 = (int64_t)ch * b.rows_per_chunk;
     const int64_t r1 = min(n, r0 + b.rows_per_chunk);
@@ -225,7 +225,8 @@ cudaError_t launch_pq_update(const float* X, int64_t n, int D, int M, int K, con
     const size_t smem = (size_t)K * ds * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_pq_accumulate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_pq_accumulate<<<dim3((unsigned)b.chunks, (unsigned)M), kLloydThreads, smem, s>>>(X, n, D, M, K, ds, b);
+    // one grid dimension: M may be above the 65535 of the second
+    k_pq_accumulate<<<(unsigned)((int64_t)b.chunks * M), kLloydThreads, smem, s>>>(X, n, D, M, K, ds, b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int64_t total = (int64_t)M * K * ds;
     k_pq_finalize<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(b, M, K, ds, C_in, C_out, objective);

@@ -769,6 +769,7 @@ static cudaError_t launch_assign_mma(const float* X, int64_t n, int D, int M, in
     if (groups > M) groups = M;
     int group = (int)((M + groups - 1) / groups);
     if (group > (DS > 8 ? 8 : 32)) group = DS > 8 ? 8 : 32;   // two CTAs' shared memory per SM
+    if ((M + group - 1) / group > 65535) group = (M + 65534) / 65535;   // the grid's second dimension
     groups = (M + group - 1) / group;
     const bool vec = ((uintptr_t)X | (uintptr_t)C) % 16 == 0;   // ds is a multiple of 4: so are D and every offset
     const size_t smem = assign_smem_bytes<DS>(K, tiles, group);

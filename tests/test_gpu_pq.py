@@ -261,6 +261,18 @@ def test_a_lloyd_step_is_not_slowed_down_by_an_infinite_value(ifvs, orc):
     assert np.isinf(G).any() and np.isinf(obj).all() and np.isinf(robj).all()
 
 
+def test_a_lloyd_step_of_more_subspaces_than_a_grid_dimension_has(ifvs, orc):
+    import torch
+    rng = np.random.default_rng(6)
+    M = 66_000
+    X = rng.standard_normal((40, M)).astype(np.float32)
+    C = rng.standard_normal((M, 2, 1)).astype(np.float32)
+    out = torch.empty((M, 2, 1), device="cuda")
+    ifvs.ifvs_pq_train(torch.from_numpy(X).cuda(), torch.from_numpy(C).cuda(), 1, C_out=out, flags=ifvs.IFVS_F_DEVICE_IO)
+    R, _, _ = orc.lloyd_step(X, C)
+    assert _ulp_close(out.cpu().numpy(), R).all()
+
+
 def test_empty_codewords_take_the_farthest_points(ifvs, orc):
     rng = np.random.default_rng(5)
     X = rng.standard_normal((4000, 16)).astype(np.float32)
