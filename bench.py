@@ -214,7 +214,7 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-SCAN_SOURCES = ("scan_common.cuh", "scan.cu", "scan_list.cu", "scan_pair.cu")
+SCAN_SOURCES = ("scan_common.cuh", "scan.cu", "scan_list.cu", "scan_pair.cu", "scan_sched.cu")
 
 
 def sources_sha256(sources):
@@ -870,21 +870,18 @@ def run_pq(args):
     max_ms = reduce_max(dist, total_ms, device)
     launch_ms = total_ms / args.steps
 
-    # roofline: three rounded float32 operations (sub, mul, add) per row,
-    # codeword and dimension; the FP32 pipes of 152 SMs x 128 lanes at the
-    # SM clock (one operation per lane per cycle)
-    props = torch.cuda.get_device_properties(device)
-    sms = props.multi_processor_count
-    mhz = (clk or {}).get("sm_max_mhz") or 2070.0
-    ops = 3.0 * rows * w.K * w.D
-    achieved = ops / (launch_ms / 1000.0) / 1e12
-    peak = sms * 128 * mhz * 1e6 / 1e12
-    roofline = {"kernel": "k_pq_assign", "bound": "alu", "achieved": achieved, "peak": peak,
-                "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": kernel_traffic("pq_encode_traffic.json", ("pq.cu",)),
-                "peak_kind": "derived: %d SMs x 128 FP32 lanes x %.0f MHz (max SM clock)" % (sms, mhz),
-                "avg_launch_ms": launch_ms, "algorithmic_flop_per_launch": ops,
-                "algorithmic_bytes_per_launch": rows * (w.D * 4 + w.M)}
+    # roofline: the bytes of the vectors and codes against the measured copy
+    # bandwidth (the tensor cores rank the codewords; what the kernel spends its
+    # time on is issue slots, for the scores' way back from tensor memory)
+    hbm_peak, peak_kind = measured_peaks()
+    nbytes = rows * (w.D * 4 + w.M)
+    achieved = nbytes / (launch_ms / 1000.0) / 1e9
+    roofline = {"kernel": "k_pq_assign_mma", "bound": "hbm", "achieved": achieved, "peak": hbm_peak,
+                "unit": "GB/s", "frac": achieved / hbm_peak if hbm_peak else None,
+                "traffic": kernel_traffic("pq_encode_traffic.json", ("pq_assign.cu",)),
+                "peak_kind": peak_kind, "avg_launch_ms": launch_ms,
+                "algorithmic_flop_per_launch": 3.0 * rows * w.K * w.D,
+                "algorithmic_bytes_per_launch": nbytes}
 
     # Lloyd training on a sample (device I/O, 25 iterations by default)
     n_tr = min(args.pq_train_rows, rows)

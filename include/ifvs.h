@@ -110,7 +110,7 @@ typedef struct {
                                      on the launching stream (ifvs_stage_times) */
 #define IFVS_F_PLAIN_PQ     0x4u  /* ignore the memory bank: Delta = 0 (plain PQ
                                      ADC, baseline Pre_IndexPQ_ADC of §3.2)   */
-#define IFVS_F_PLAIN_LOADS  0x8u  /* search, M = 16 sorted-copy scan: one-query
+#define IFVS_F_PLAIN_LOADS  0x8u  /* search, M = 12 and 16, sorted-copy scan: one-query
                                      CTAs read code rows with per-lane vector
                                      loads instead of bulk copies (TMA) into
                                      shared memory; same results              */
@@ -140,7 +140,8 @@ typedef struct {
                            and together span at least this many rows, or two
                            bitmap queries that at least this many rows pass,
                            share a CTA and one shared-memory look-up per code
-                           byte (tables quantised to 11 bits; every row that
+                           byte (tables quantised to floor(32767 / M)
+                           levels; every row that
                            can reach a top-k is rescored exactly, so results
                            equal those of one query per CTA bit for bit).
                            0: automatic (spans of at least 160000 rows in
@@ -355,7 +356,8 @@ int ifvs_pq_encode(int32_t device, const float* X, int64_t n, int32_t D, int32_t
  * ifvs_pq_train — `iters` Lloyd iterations per subspace from C_init
  * (k-means training of the PQ codebook).  Each iteration assigns every row
  * as ifvs_pq_encode does, then replaces each codeword used by at least one
- * row by the fp64 mean of its rows rounded to float32; each unused
+ * row by the mean of its rows, summed to fp64 accuracy (within 2^-38 of the
+ * sum of the magnitudes) and rounded to float32; each unused
  * codeword, in increasing order, takes the row farthest from its codeword
  * (largest distance, ties to the smallest row), whose distance then counts
  * as 0.
@@ -388,7 +390,8 @@ int ifvs_pq_train(int32_t device, const float* X, int64_t n, int32_t D, int32_t 
  * own for w_z (at a fixed temperature, shrinking every weight lowers this
  * loss whenever positives trail hard negatives, so a jointly learned w_f
  * can collapse toward 0).  Distances are float32
- * terms summed in fp64; gradients are float32; every sum runs in a fixed
+ * terms summed to fp64 accuracy (within 2^-38 of the sum of their magnitudes);
+ * gradients are float32; every sum runs in a fixed
  * order, so results are deterministic.  One call handles one mini-batch of
  * at most 1024 queries; the index must hold a bank, W and seeds with
  * r <= 32.

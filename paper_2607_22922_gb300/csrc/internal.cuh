@@ -425,7 +425,7 @@ struct LloydBufs {
 };
 // sets the plan and the pointers (relative to b->base, which may be null) and the bytes needed
 void lloyd_plan(int64_t n, int M, int K, int ds, int num_sms, LloydBufs* b, size_t* bytes);
-// Lloyd update from b's codes and dmin: fp64 means of the members, unused
+// Lloyd update from b's codes and dmin: means of the members (sum_f64), unused
 // codewords on the farthest rows; objective [M] (may be null)
 cudaError_t launch_pq_update(const float* X, int64_t n, int D, int M, int K, const LloydBufs& b, const float* C_in,
                              float* C_out, double* objective, cudaStream_t s);

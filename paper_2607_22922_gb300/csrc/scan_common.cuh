@@ -552,8 +552,8 @@ __device__ __forceinline__ void lookup2(const uint4 ca, const uint4 cb, uint32_t
 // Distances of NU rows for any M, all owned by one lane (so they share the
 // table word offset w0 = the lane): the rows' code words are read together
 // and their look-ups go into NU/2 packed f32x2 chains, independent of each
-// other; each row's entries are still added for s ascending, as in
-// lookup_any.  Rows whose bit in `valid` is clear read no codes.
+// other; each row's entries are still added one by one for s ascending, from
+// subspace w0 mod M on.  Rows whose bit in `valid` is clear read no codes.
 template <int NU>
 __device__ __forceinline__ void lookup_rows(const uint8_t* __restrict__ codes, const uint32_t (&idx)[NU],
                                             unsigned valid, int row_bytes, int M, int S, const float* tab,
@@ -753,6 +753,14 @@ struct ItemLoop {
 // A batch's scans share no data and overlap: the first waits for the tables and
 // lets the next start, which fills the SMs that the first leaves at its end;
 // the others wait for the one before them at their end.
+//
+// The others read the work lists, the plan and the tables without a wait of their
+// own, which PTX does not promise to be enough: it speaks of what a grid sees
+// after its own griddepcontrol.wait.  They rely on the grids that wrote these
+// having completed, and their writes being in memory, before the first scan's
+// wait returned, and on the first scan letting them start only after that; no
+// CTA of theirs has read those addresses earlier.  A wait of their own would hold
+// them until the first scan has ended, which is what the overlap avoids.
 __device__ __forceinline__ void scan_begin(bool first) {
     if (first) wait_before();
     start_dependents();

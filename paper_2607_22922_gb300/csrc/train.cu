@@ -328,7 +328,7 @@ k_train_query(TrainQueryArgs a) {
                 const float gf = (float)g;
                 const float ge = gf * (-2.f * __ldg(wf + d) * df);
                 gm[c[u]] += ge;
-                // gam (df df) to about 48 bits: gam as two floats, exact products
+                // gam (df df) to 48 bits: gam as two floats, exact products
                 const float sq = df * df, p = __fmul_rn(gf, sq);
                 gw.add(p);
                 gw.lo = __fadd_rn(gw.lo, fmaf((float)(g - (double)gf), sq, fmaf(gf, sq, -p)));
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(1024) k_train_wz(const float* __restrict__ gw,
     const int d = blockIdx.x * 32 + threadIdx.x;
     double s = 0.0;
     if (d < D) {
-        // float pairs: the float64 adders took 22 us for 1024 queries at D = 128
+        // a float pair over at most 32 terms (1024 queries): the float64 adders took 22 us at D = 128
         Sum2 p;
 #pragma unroll 8
         for (int64_t q = threadIdx.y; q < n; q += 32) p.add(gw[q * D + d]);
