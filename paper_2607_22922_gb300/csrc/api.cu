@@ -519,8 +519,8 @@ int make_sched(ifvs_index* ix, const ScanShape& sh, int64_t n, int k, const Opts
                                 ix->num_sms};
     const int64_t any = (int64_t)1 << 40;
     const int64_t most[kGroups] = {lists ? any : 0, bitmaps ? any : 0, pairs ? any : 0, bm_pairs ? any : 0};
-    TRY(ensure(ix->w_part, scan_sched_layout(n, k, ix->n_blocks, slots, o.chunk_blocks, most, nullptr, s)));
-    scan_sched_layout(n, k, ix->n_blocks, slots, o.chunk_blocks, most, ix->w_part.as<uint8_t>(), s);
+    TRY(ensure(ix->w_part, scan_sched_layout(n, k, ix->n_blocks, ix->row_bytes, slots, o.chunk_blocks, most, nullptr, s)));
+    scan_sched_layout(n, k, ix->n_blocks, ix->row_bytes, slots, o.chunk_blocks, most, ix->w_part.as<uint8_t>(), s);
     return 0;
 }
 

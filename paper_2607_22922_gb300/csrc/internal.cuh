@@ -336,6 +336,7 @@ constexpr int kGroups = 4;
 __host__ __device__ constexpr bool pair_group(int g) { return g >= 2; }
 struct ScanSched {
     SchedGroup group[kGroups];
+    bool by_part;          // the bitmap group's items part by part (scan_sched.cu)
     ScanItem* items[kGroups];
     int* ctl;              // items per group, then work counters
     int2* qlist;           // [nq] (first list, lists) of a query
@@ -345,8 +346,9 @@ struct ScanSched {
 };
 // fills s (pointers from `base`, which may be null); returns the bytes needed.
 // most[g] bounds group g's items (0: the group is not used).
-size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)[kGroups], int64_t chunk_blocks,
-                         const int64_t (&most)[kGroups], uint8_t* base, ScanSched* s);
+// row_bytes: of a code row.
+size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, int row_bytes, const int (&slots)[kGroups],
+                         int64_t chunk_blocks, const int64_t (&most)[kGroups], uint8_t* base, ScanSched* s);
 // What two queries must bring to be paired (pair_rule, api.cu); < 0: no pairs.
 struct PairRule {
     int64_t span;       // rows a pair on a sorted copy spans, at least

@@ -60,7 +60,7 @@ size_t layout(const IndexView& v, int64_t n, int64_t items, int k, uint8_t* base
     const int slots[kGroups] = {1, v.num_sms * scan_ctas_per_sm(v.tab_words, scan_kp(k)), 1, 1};
     const int64_t most[kGroups] = {0, items, 0, 0};
     const size_t head = (bm + tab + 255) / 256 * 256;
-    return head + scan_sched_layout(n, k, v.n_blocks, slots, 0, most, base ? base + head : nullptr, s);
+    return head + scan_sched_layout(n, k, v.n_blocks, v.row_bytes, slots, 0, most, base ? base + head : nullptr, s);
 }
 
 }  // namespace

@@ -29,8 +29,8 @@
 // (up to the fourth): CTAs that work at the same time read the same part of the
 // codes and share it in the L2, which 8 x 10^6 rows fill (512 queries of M = 16
 // that 21 and 32 % of them pass, k = 200: 8946 and 12344 us query by query, 8602 and
-// 11866 so; k = 10 8647 and 8470 us at 32 %).  The other groups gained nothing
-// from it.  Each item writes one list of
+// 11866 so; k = 10 8647 and 8470 us at 32 %; 2 x 10^6 rows the same either way).  The
+// other groups gained nothing from it.  Each item writes one list of
 // k keys (two for a pair), numbered so that a query's lists are contiguous;
 // k_merge reads (first list, count) per query.
 //
@@ -156,11 +156,14 @@ __device__ __forceinline__ Cut cut_of(int64_t work, int64_t n, const SchedGroup&
 
 }  // namespace
 
+// PARTS: the bitmap group's items part by part (a kernel of its own: the ranks'
+// code cost a batch without them 3 us).
+template <bool PARTS>
 __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __restrict__ plan,
                                                             const unsigned long long* __restrict__ npass, int64_t nq,
                                                             int64_t n_blocks, PairRule rule, ScanSched s) {
     __shared__ uint64_t key[kSeg];          // pairing; then the items' prefix counts
-    __shared__ uint64_t rank[kSeg];         // of an element among those with more than c parts, c = 0..3
+    __shared__ uint64_t rank[PARTS ? kSeg : 1];   // of an element among those with more than c parts, c = 0..3
     __shared__ int wsum[32];
     __shared__ uint64_t wsum_rank[32];
     __shared__ int64_t wsum64[2 * kGroups][32];
@@ -338,7 +341,7 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
             if (tid == 0) s.ctl[g] = s.ctl[kGroups + g] = 0;
             continue;
         }
-        const bool by_part = g == 1 && (s.group[g].fixed > 0 || 2 * cnt[g] > s.group[g].slots);
+        const bool by_part = PARTS && g == 1 && (s.group[g].fixed > 0 || 2 * cnt[g] > s.group[g].slots);
         for (int64_t e0 = 0; e0 < n_el; e0 += kSeg) {
             const int n = (int)min((int64_t)kSeg, n_el - e0);
             int total = 0, done = 0;
@@ -444,8 +447,9 @@ __global__ void __launch_bounds__(kSchedThreads) k_schedule(const ScanPlan* __re
 }
 
 // Bounds of the lists and the workspace's layout (offsets from `base`).
-size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, const int (&slots)[kGroups], int64_t chunk_blocks,
-                         const int64_t (&most)[kGroups], uint8_t* base, ScanSched* s) {
+size_t scan_sched_layout(int64_t nq, int k, int64_t n_blocks, int row_bytes, const int (&slots)[kGroups],
+                         int64_t chunk_blocks, const int64_t (&most)[kGroups], uint8_t* base, ScanSched* s) {
+    s->by_part = n_blocks * kBlockRows * row_bytes > (int64_t)1 << 26;   // half of the L2
     size_t at = 0;
     auto take = [&](size_t bytes) {
         uint8_t* p = base + at;
@@ -485,8 +489,8 @@ cudaError_t launch_schedule(const ScanPlan* plan, const unsigned long long* npas
     if (nq <= 0) return cudaSuccess;
     int threads = 128;
     while (threads < kSchedThreads && threads < nq) threads <<= 1;
-    return launch_kernel(k_schedule, dim3(1), dim3((unsigned)threads), 0, chain, st, plan, npass, nq, n_blocks,
-                         rule, s);
+    return launch_kernel(s.by_part ? k_schedule<true> : k_schedule<false>, dim3(1), dim3((unsigned)threads), 0, chain,
+                         st, plan, npass, nq, n_blocks, rule, s);
 }
 
 }  // namespace ifvs
