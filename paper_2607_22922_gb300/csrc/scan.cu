@@ -151,11 +151,16 @@ __device__ __forceinline__ void scan_chunk(const uint8_t* __restrict__ codes,
         } else {
             float d[kU];
             lookup_rows<kU>(codes, row, (1u << kU) - 1u, row_bytes, M, S, tab, lane, d);
+            uint64_t key[kU];
+            bool want = false;
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
-                const bool pass = valid >> u & 1u;
-                const uint64_t key = ((uint64_t)__float_as_uint(d[u]) << 32) | row[u];
-                tk.offer(key, pass && key < tk.thr, lane);
+                key[u] = ((uint64_t)__float_as_uint(d[u]) << 32) | row[u];
+                want |= (valid >> u & 1u) && key[u] < tk.thr;
+            }
+            if (__any_sync(0xFFFFFFFFu, want)) {
+#pragma unroll
+                for (int u = 0; u < kU; ++u) tk.offer(key[u], (valid >> u & 1u) && key[u] < tk.thr, lane);
             }
         }
     }
