@@ -1095,7 +1095,7 @@ def run_train(args):
     mhz = (clk or {}).get("sm_max_mhz") or 2070.0
     peak = sms * 32 * mhz * 1e6
     achieved = (lookups / scan_n) / (scan_ms / scan_n / 1000.0) if scan_n else None
-    roofline = {"kernel": "k_scan (mining)", "bound": "smem", "achieved": achieved, "peak": peak,
+    roofline = {"kernel": "scan stage (mining)", "bound": "smem", "achieved": achieved, "peak": peak,
                 "unit": "look-ups/s", "frac": achieved / peak if achieved else None, "traffic": None,
                 "peak_kind": "derived: %d SMs x 32 lanes x %.0f MHz (one conflict-free shared load "
                              "per SM per cycle)" % (sms, mhz),

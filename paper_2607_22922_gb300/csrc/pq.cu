@@ -13,9 +13,9 @@
 // 65 536 rows x 16 subspaces; 140 us with float64 atomics on shared memory,
 // which are compare-and-swap loops), so up to 32 members go into a pair of
 // floats with the rounding error of every addition carried along (TwoSum,
-// Knuth) before it is added (sum_f64): three Lloyd steps of those rows, with
-// their call, take 512 us (529 us with one pair per codeword and chunk, which
-// was up to 1500 float32 ulp off on long runs of alike values).  Infinite, huge
+// Knuth) before it is added (sum_f64): 39 us, as with one pair per codeword and
+// chunk, which was up to 1500 float32 ulp off on long runs of alike values.  The
+// latency of the members' loads is what is left (issue slots 32 % used).  Infinite, huge
 // and NaN values give what float64 sums give.  The same CTA
 // adds up the chunk's distances and finds its farthest row.
 //

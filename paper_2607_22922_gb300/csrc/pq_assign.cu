@@ -50,7 +50,7 @@
 // threads works on half a codebook (128 TMEM columns) at a time, so that four
 // CTAs share an SM's 512 columns: their decisions cover each other's MMAs.
 // The rows being decided wait in shared memory: in registers they made the
-// main loop spill (0.75 ms).  The issue slots are the bound (58 % used; tensor pipe 14 %).  Measured,
+// main loop spill (0.75 ms).  The issue slots are the bound (63 % used; tensor pipe 18 %).  Measured,
 // 2^20 rows x 16 subspaces: 3.49 ms with every codeword evaluated in float32,
 // 0.68 ms now; with whole codebooks (256 columns, two CTAs per SM) 0.80 ms;
 // with two passes over the scores and a bit per codeword 1.22 ms.

@@ -73,8 +73,9 @@ __global__ void __launch_bounds__(kTrainThreads) k_train_gram(const float* __res
 // 228 us before.  What is left is the latency of those loads, so CTAs per SM
 // count for more than loads per thread: at 128 registers, four candidates in
 // flight and 36 KB the grid ran as 1.7 waves of four CTAs per SM (195 us); at 72
-// registers, two in flight and 26 KB seven fit (111 us; the training step 735 ->
-// 665 us; six with two 738, six with four, which spill, 764).
+// registers, two in flight and 26 KB seven fit (114 us, 40 % of the issue slots, the
+// loads' latency still first; the training step 735 -> 673 us; six with two 738, six
+// with four, which spill, 764).
 //
 // Twice the threads per query (three CTAs per SM, two for r > 8) where the
 // batch leaves room for them or the shared memory (D r floats) holds fewer than
